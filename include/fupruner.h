@@ -222,6 +222,9 @@ typedef enum {
                                 minus launches 0..i-1), each prefix replayed as a CUDA graph `index` times (0 = 10)
                                 between two events; a layer inside a fused run reports 0 except the run's first;
                                 synchronises */,
+    FP_Q_ALL_MASKS = 16,     /* index 0: int32, the filters of all convolutions together (n); index 1: the masks and ranks of all
+                                convolutions in one call - int32[N_CONVS] filters per convolution (0 if absorbed),
+                                int32[n] ranks, uint8[n] masks, in description order                   */
     FP_Q_CONV_BANK_ELEMS = 15 /* int64: weights in the fused fp32 bank of conv `index` (K_fused*C_fused*R*S), 0 if absorbed */
 } fp_query_what;
 

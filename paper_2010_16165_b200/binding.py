@@ -22,7 +22,7 @@ FP_COMPUTE_BF16_TC, FP_COMPUTE_FP32, FP_COMPUTE_BF16_SIMT = 0, 1, 2
 FP_NORM_L1, FP_NORM_L2 = 0, 1
 (FP_Q_N_CONVS, FP_Q_CONV_K_FUSED, FP_Q_CONV_K_KEPT, FP_Q_CONV_C_KEPT, FP_Q_MASK, FP_Q_RANK, FP_Q_N_CLASSES,
  FP_Q_FLOPS, FP_Q_BYTES, FP_Q_N_OPS, FP_Q_OP_INFO, FP_Q_OP_OUTPUT, FP_Q_DEVICE_STATUS, FP_Q_N_LAUNCHES,
- FP_Q_OP_TIMES, FP_Q_CONV_BANK_ELEMS) = range(16)
+ FP_Q_OP_TIMES, FP_Q_CONV_BANK_ELEMS, FP_Q_ALL_MASKS) = range(17)
 
 EXPORTS = ["fp_fuse", "fp_prune", "fp_forward", "fp_forward_host", "fp_forward_host_async", "fp_score", "fp_query", "fp_destroy",
            "fp_last_error", "fp_rank_filters_static", "fp_soft_prune_epoch", "fp_soft_prune_finish",
@@ -256,13 +256,15 @@ def fp_destroy(h):
 
 
 def masks_and_ranks(h):
-    out = {}
-    for ci in range(fp_query_int(h, FP_Q_N_CONVS)):
-        K = fp_query_int(h, FP_Q_CONV_K_FUSED, ci)
-        if K == 0:
-            out[ci] = (None, None)
-            continue
-        out[ci] = (fp_query_array(h, FP_Q_MASK, ci, np.uint8, K), fp_query_array(h, FP_Q_RANK, ci, np.int32, K))
+    n_convs, n = fp_query_int(h, FP_Q_N_CONVS), fp_query_int(h, FP_Q_ALL_MASKS, 0)
+    raw = fp_query_array(h, FP_Q_ALL_MASKS, 1, np.uint8, 4 * n_convs + 5 * n)
+    ints = raw[:4 * (n_convs + n)].view(np.int32)
+    masks = raw[4 * (n_convs + n):]
+    out, at = {}, 0
+    for ci, K in enumerate(ints[:n_convs].tolist()):
+        end = at + K
+        out[ci] = (masks[at:end], ints[n_convs + at:n_convs + end]) if K else (None, None)
+        at = end
     return out
 
 

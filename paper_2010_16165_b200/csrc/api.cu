@@ -78,18 +78,18 @@ struct FConv {
     int compact = 0;           // 1: pruned filters are physically removed from the output tensor
     int scatter = 0;           // 1: only kept filters are computed, scattered into a full-width output (residual stream)
     int n_tile_forced = 0;     // scatter: filters per CTA tile the packed bank was laid out for
-    int32_t* d_out_map = nullptr;   // scatter: output channel -> packed filter row (-1 = no filter kept)
-    int32_t* d_chunk0 = nullptr;    // scatter: first output chunk of every filter tile, and the end
+    int map_off = -1;          // scatter: output channel -> packed filter row (-1 = no filter kept), in the index array
+    int chunk0_off = -1;       // scatter: first output chunk of every filter tile, and the end, in the index array
     int n_mult = 1;            // 4: a 1x1 layer over a parity-split tensor runs on its 4 N half-size images
     int proj = -1;             // >= 0: the projection shortcut (index into convs) that this layer computes itself
     int proj_kind = 0;         // 1: filters stacked along the channels (1x1 layer); 2: extra centre-tap K groups (streamed 3x3 layer)
     int absorbed = 0;          // 1: this projection runs inside the layer that adds its result; its operator launches nothing
-    void* d_wp_plain = nullptr;     // the packed bank before any re-blocking ([tap][chunk][K_pad][8])
+    int plain_bank = 0;        // 1: an absorbed projection whose bank is read as [chunk][K_pad][8] (proj_kind 2)
     int K_kept = 0, K_rows = 0, K_pad = 0, C_kept = 0, C_pad = 0;
-    void* d_wp = nullptr;      // packed filters in the compute type, K_pad x R x S x C_pad
+    void* d_wp = nullptr;      // packed filters in the compute type, in the order the plan reads them (fp::PackJob)
     float* d_bp = nullptr;
-    int32_t* d_row = nullptr;  // packed filter row -> fused filter (-1 = zero row)
-    int32_t* d_chan = nullptr; // packed input channel -> fused input channel (-1 = zero channel)
+    int row_off = -1;          // packed filter row -> fused filter (-1 = zero row), in the index array
+    int chan_off = -1;         // packed input channel -> fused input channel (-1 = zero channel), in the index array
     fp::ConvArgs args;
     fp::ConvPlanTC tc;
 };
@@ -103,7 +103,11 @@ struct Chain {
     fp::ChainArgs args;
     fp::ChainPlan plan;
     uint8_t* d_blob = nullptr;
+    size_t blob_bytes = 0;
 };
+
+// One device allocation that is kept from one planning to the next while it is large enough.
+struct Region { void* p = nullptr; size_t cap = 0; };
 
 struct Op { int kind; int idx; };
 constexpr int kHostPieces = 8;     // fp_forward_host copies the input in up to this many pieces   // kind: 0 conv, 1 pool, 2 head, 3 input conversion
@@ -139,11 +143,15 @@ struct fp_handle_s {
     int head_src = -1, n_classes = 0, fc_C = 0;
     const float* d_fcw = nullptr;          // classes x fc_C (copy of the description's FC weights)
     const float* d_fcb = nullptr;
+    const int32_t* d_idx = nullptr;        // the plan's index arrays (part of meta_region)
     float* d_fcw_packed = nullptr;         // classes x C_pad, scaled by 1/(H*W)
     float* d_pool = nullptr;               // max_batch x C_pad channel sums (between the two head kernels)
     // buffers
-    std::vector<void*> act_buffers;        // activation storage (re-planned by fp_prune)
-    std::vector<void*> pack_buffers;       // packed filters / biases / index arrays
+    Region act_region;                     // activation storage (re-planned by fp_prune)
+    Region pack_region;                    // packed filters, biases, FC matrix, channel sums
+    Region meta_region;                    // packing jobs and index arrays
+    void* pinned = nullptr;                // host side of uploads (jobs, index arrays, bank table) and of the masks' way back
+    size_t pinned_cap = 0;
     std::vector<void*> fixed_buffers;      // fused fp32 filters etc. (live until fp_destroy)
     void* d_in_stage = nullptr;            // device staging for fp_forward_host
     float* d_logits_stage = nullptr;
@@ -154,14 +162,17 @@ struct fp_handle_s {
     cudaStream_t copy_stream = nullptr;    // fp_forward_host: input pieces are copied here while earlier pieces are converted
     int stage_used = 0;                    // the staging buffer has been read by a kernel queued behind copy_events[kHostPieces]
     cudaEvent_t copy_events[kHostPieces + 1] = {};
-    double* d_scores = nullptr; int32_t* d_rank = nullptr; uint8_t* d_mask = nullptr;
+    double* d_scores = nullptr;            // fp_score
     std::map<GraphKey, cudaGraphExec_t> graphs;
     const void* last_input = nullptr; int last_batch = 0;
     int soft_epochs = 0;                   // passes of fp_soft_prune_epoch since fp_fuse
-    // dynamic pruning over all banks at once: bank table, filter -> bank map, scores / ranks / masks of all filters
-    fp::SoftBank* d_soft_banks = nullptr; int32_t* d_soft_map = nullptr;
-    double* d_soft_scores = nullptr; int32_t* d_soft_rank = nullptr; uint8_t* d_soft_mask = nullptr;
-    int soft_total = 0;
+    // selection over all banks at once (fp_prune, fp_soft_prune_epoch): bank table, filter -> bank map, scores, and ranks with
+    // the masks right behind them; filters are numbered bank by bank in description order
+    std::vector<fp::SoftBank> banks;
+    std::vector<int> bank_conv;            // bank -> index into convs
+    int n_filters = 0;
+    fp::SoftBank* d_banks = nullptr; int32_t* d_bank_map = nullptr;
+    double* d_bank_scores = nullptr; int32_t* d_bank_rank = nullptr; uint8_t* d_bank_mask = nullptr;
     int stem_packed = 0;                   // network input stored in the packed form of a 7x7/2 first convolution
     int stem_fused = 0;                    // operators 0-2 (input conversion, 7x7/2 convolution, 3x3/2 max pooling) run as one kernel
     fp::StemPoolArgs stem_args;
@@ -220,6 +231,32 @@ fp_status dev_alloc(fp_handle h, std::vector<void*>& owner, void** out, size_t b
     *out = p;
     return FP_OK;
 }
+
+// Room for `bytes`: what the region holds is given up.  The allocation of an earlier plan is used again where it is large
+// enough - cudaMalloc and cudaFree of every packed array cost fp_prune of ResNet-50 more than 20 ms - except with a
+// caller's allocator: that memory goes back first, for the caller's pool to place as it likes.
+fp_status region_reserve(fp_handle h, Region& r, size_t bytes) {
+    if (r.p && (h->dealloc || r.cap < bytes)) {
+        dev_free(h, r.p);
+        r.p = nullptr; r.cap = 0;
+    }
+    if (!r.p) {
+        TRY(dev_alloc_raw(h, &r.p, bytes));
+        r.cap = bytes;
+    }
+    return FP_OK;
+}
+
+fp_status pinned_reserve(fp_handle h, size_t bytes) {
+    if (h->pinned_cap >= bytes) return FP_OK;
+    if (h->pinned) cudaFreeHost(h->pinned);
+    h->pinned = nullptr; h->pinned_cap = 0;
+    CK(cudaMallocHost(&h->pinned, bytes));
+    h->pinned_cap = bytes;
+    return FP_OK;
+}
+
+inline size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // ---------------------------------------------------------------------------------------
 // description -> fused operators
@@ -644,14 +681,8 @@ bool compactable(fp_handle h, const std::vector<std::vector<Use>>& uses, int tid
     return true;
 }
 
-fp_status upload_i32(fp_handle h, const std::vector<int32_t>& v, int32_t** out) {
-    TRY(dev_alloc(h, h->pack_buffers, (void**)out, v.size() * sizeof(int32_t)));
-    CK(cudaMemcpy(*out, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    return FP_OK;
-}
-
 bool chain_candidate(fp_handle h, const FConv& f) {
-    if (h->compute != FP_COMPUTE_BF16_TC || h->keep_outputs || f.scatter) return false;
+    if (h->compute != FP_COMPUTE_BF16_TC || h->keep_outputs || f.scatter || f.proj >= 0) return false;
     if (f.R != 3 || f.S != 3 || f.stride != 1 || f.pad != 1) return false;
     if ((h->stem_packed || h->stem_fused) && f.src == 0) return false;
     if (h->tensors[f.src].split || h->tensors[f.out].split) return false;
@@ -661,8 +692,8 @@ bool chain_candidate(fp_handle h, const FConv& f) {
 
 // Finds runs of consecutive operators that are stride-1 3x3 convolutions where each reads the previous
 // one's output, a shortcut operand (other than the first layer's) is the tensor two layers back, and no
-// tensor inside the run is read from outside it; packs their filters for the fused kernel.
-fp_status find_chains(fp_handle h, const std::vector<std::vector<Use>>& uses) {
+// tensor inside the run is read from outside it.
+void find_chains(fp_handle h, const std::vector<std::vector<Use>>& uses) {
     h->chains.clear();
     h->op_chain.assign(h->ops.size(), -1);
     const int n_ops = (int)h->ops.size();
@@ -717,16 +748,7 @@ fp_status find_chains(fp_handle h, const std::vector<std::vector<Use>>& uses) {
             Chain ch;
             ch.first_op = i; ch.last_op = i + len - 1; ch.args = a; ch.plan = plan;
             for (int j = 0; j < len; ++j) ch.convs.push_back(h->ops[i + j].idx);
-            TRY(dev_alloc(h, h->pack_buffers, (void**)&ch.d_blob, (size_t)off));
-            for (int j = 0; j < len; ++j) {
-                const FConv& f = h->convs[ch.convs[j]];
-                const fp::ChainLayer& ly = a.layers[j];
-                fp::launch_repack_chain(f.d_w32, f.C, f.d_row, f.K_pad, f.d_chan, f.C_pad,
-                                        (__nv_bfloat16*)(ch.d_blob + ly.blob_off), 0);
-                fp::launch_pack_bias(f.d_b32, f.d_row, f.K_pad,
-                                     (float*)(ch.d_blob + ly.blob_off + (size_t)9 * f.C_pad * f.K_pad * 2), 0);
-            }
-            CK(cudaGetLastError());
+            ch.blob_bytes = (size_t)off;
             for (int j = 0; j < len; ++j) h->op_chain[i + j] = (int)h->chains.size();
             h->chains.push_back(ch);
             break;
@@ -743,7 +765,6 @@ fp_status find_chains(fp_handle h, const std::vector<std::vector<Use>>& uses) {
             h->input_fused = 1;
         }
     }
-    return FP_OK;
 }
 
 // How a convolution reads a parity-split input tensor: 0 it cannot, 'A' 3x3 / stride 2 / pad 1 (nine taps over the four
@@ -818,11 +839,12 @@ fp_status replan(fp_handle h) {
     h->planned = 0;
     drop_graphs(h);
     CK(cudaDeviceSynchronize());
-    free_list(h, h->act_buffers);
-    free_list(h, h->pack_buffers);
     const auto uses = tensor_uses(h);
     const int bf16 = h->act_is_bf16();
     cudaStream_t st = 0;
+    std::vector<int32_t> idx;                    // all index arrays of the plan, one behind the other
+    auto add_idx = [&](const std::vector<int32_t>& v) { const int o = (int)idx.size(); idx.insert(idx.end(), v.begin(), v.end()); return o; };
+    int head_chan = 0;
 
     // --- shapes in execution order ---
     {
@@ -841,7 +863,7 @@ fp_status replan(fp_handle h) {
     decide_splits(h, uses);
     for (FConv& f : h->convs) {
         f.n_mult = (h->tensors[f.src].split && split_reader(f) == 'C') ? 4 : 1;
-        f.proj = -1; f.proj_kind = 0; f.absorbed = 0;
+        f.proj = -1; f.proj_kind = 0; f.absorbed = 0; f.plain_bank = 0;
     }
     // ... and, where a 3x3 / stride-2 max pooling is the only reader of that convolution and the input is bf16, input
     // conversion, convolution and pooling run as one kernel (decided below, once the filter count is known).
@@ -869,7 +891,7 @@ fp_status replan(fp_handle h) {
             // output channels: other layers write them too.  On the tensor-core path it still computes only its kept
             // filters and scatters them into the full-width tensor in the epilogue; layers that can join a fused run of
             // layers, and the validation paths, keep pruned filters as zero rows instead.
-            f.scatter = 0; f.n_tile_forced = 0; f.d_out_map = nullptr; f.d_chunk0 = nullptr;
+            f.scatter = 0; f.n_tile_forced = 0; f.map_off = -1; f.chunk0_off = -1;
             if (!f.compact && h->compute == FP_COMPUTE_BF16_TC && round_up(f.K_kept, 16) < round_up(f.K, 16)) {
                 const bool runs_fused = !h->keep_outputs && f.R == 3 && f.S == 3 && f.stride == 1 && f.pad == 1 &&
                                         !(h->stem_packed && f.src == 0) &&
@@ -931,8 +953,8 @@ fp_status replan(fp_handle h) {
                 f.K_rows = f.K; f.K_pad = n_tiles * n_tile; f.n_tile_forced = n_tile;
                 out.keep.resize(f.K);
                 for (int k = 0; k < f.K; ++k) out.keep[k] = k;
-                TRY(upload_i32(h, out_map, &f.d_out_map));
-                TRY(upload_i32(h, chunk0, &f.d_chunk0));
+                f.map_off = add_idx(out_map);
+                f.chunk0_off = add_idx(chunk0);
                 out.C = f.K; out.C_pad = out_C_pad;
             } else {
                 if (f.compact) {
@@ -952,13 +974,7 @@ fp_status replan(fp_handle h) {
             if (f.src == 0 && stem_candidate && !f.scatter && fp::stem_pool_supported(f.C, h->in_H, h->in_W, f.K_pad)) {
                 h->stem_fused = 1;
                 h->stem_packed = 0;
-                int32_t* d_row;
-                TRY(upload_i32(h, row_src, &d_row));
-                f.d_row = d_row; f.d_chan = nullptr;
-                TRY(dev_alloc(h, h->pack_buffers, &f.d_wp, (size_t)256 * f.K_pad * 2));
-                TRY(dev_alloc(h, h->pack_buffers, (void**)&f.d_bp, (size_t)f.K_pad * sizeof(float)));
-                fp::launch_repack_stem_direct(f.d_w32, f.C, d_row, f.K_pad, (__nv_bfloat16*)f.d_wp, st);
-                fp::launch_pack_bias(f.d_b32, d_row, f.K_pad, f.d_bp, st);
+                f.row_off = add_idx(row_src); f.chan_off = -1;
                 f.tc.valid = 0;
                 continue;
             }
@@ -979,7 +995,7 @@ fp_status replan(fp_handle h) {
                     const FConv& q = h->convs[cand];
                     const Tensor& X = h->tensors[q.src];
                     if (q.R == 1 && q.S == 1 && q.pad == 0 && q.res_mode == 0 && !q.relu && !q.scatter && !q.compact && q.K == f.K &&
-                        q.K_pad == f.K_pad && q.n_mult == 1 && q.tc.valid && q.d_wp_plain && !(h->stem_packed && q.src == 0) &&
+                        q.K_pad == f.K_pad && q.n_mult == 1 && q.tc.valid && !(h->stem_packed && q.src == 0) &&
                         ((q.stride == 1 && !X.split) || (q.stride == 2 && X.split)))
                         pj = cand;
                 }
@@ -996,33 +1012,8 @@ fp_status replan(fp_handle h) {
                 if (fp::plan_conv_tc(ga, &f.tc, msg, sizeof(msg)) != 0)
                     return fail(FP_ERR_UNSUPPORTED, "convolution %d: %s", f.conv_index, msg);
             }
-            // pack filters and bias
-            int32_t *d_row, *d_chan;
-            TRY(upload_i32(h, row_src, &d_row));
-            TRY(upload_i32(h, chan_src, &d_chan));
-            f.d_row = d_row; f.d_chan = d_chan;
-            const bool packed_stem = h->stem_packed && f.src == 0;
-            const size_t cnt = packed_stem ? (size_t)f.K_pad * 3 * 80 : (size_t)f.K_pad * f.R * f.S * f.C_pad;
-            TRY(dev_alloc(h, h->pack_buffers, &f.d_wp, cnt * h->act_elem()));
-            TRY(dev_alloc(h, h->pack_buffers, (void**)&f.d_bp, (size_t)f.K_pad * sizeof(float)));
-            if (packed_stem) fp::launch_repack_stem(f.d_w32, f.C, d_row, f.K_pad, (__nv_bfloat16*)f.d_wp, st);
-            else fp::launch_repack_conv(f.d_w32, f.C, f.R * f.S, d_row, f.K_pad, d_chan, f.C_pad,
-                                   bf16 ? (__nv_bfloat16*)f.d_wp : nullptr, bf16 ? nullptr : (float*)f.d_wp, st);
-            fp::launch_pack_bias(f.d_b32, d_row, f.K_pad, f.d_bp, st);
-            f.d_wp_plain = f.d_wp;
-            if (pj >= 0) {
-                // [chunk][K_pad][8]: this layer's chunks, then the projection's; the biases add up
-                FConv& q = h->convs[pj];
-                const size_t b1 = (size_t)f.C_pad * f.K_pad * h->act_elem(), b2 = (size_t)q.C_pad * f.K_pad * h->act_elem();
-                void* cat; float* bsum;
-                TRY(dev_alloc(h, h->pack_buffers, &cat, b1 + b2));
-                TRY(dev_alloc(h, h->pack_buffers, (void**)&bsum, (size_t)f.K_pad * sizeof(float)));
-                CK(cudaMemcpyAsync(cat, f.d_wp, b1, cudaMemcpyDeviceToDevice, st));
-                CK(cudaMemcpyAsync((uint8_t*)cat + b1, q.d_wp_plain, b2, cudaMemcpyDeviceToDevice, st));
-                fp::launch_add_bias(f.d_bp, q.d_bp, f.K_pad, bsum, st);
-                f.d_wp = cat; f.d_bp = bsum;
-                f.proj = pj; f.proj_kind = 1; q.absorbed = 1;
-            }
+            f.row_off = add_idx(row_src); f.chan_off = add_idx(chan_src);
+            if (pj >= 0) { f.proj = pj; f.proj_kind = 1; h->convs[pj].absorbed = 1; }
             // The same for a 3x3 / stride-1 layer with streamed filters (the second layer of a basic block that changes the
             // resolution): the projection becomes extra K groups with a centre tap only, read from its own packed bank.
             if (pj < 0 && h->compute == FP_COMPUTE_BF16_TC && !h->keep_outputs && f.res_mode == 1 && f.R == 3 && f.S == 3 &&
@@ -1034,28 +1025,11 @@ fp_status replan(fp_handle h) {
                     FConv& q = h->convs[cand];
                     const Tensor& X = h->tensors[q.src];
                     if (q.R == 1 && q.S == 1 && q.pad == 0 && q.res_mode == 0 && !q.relu && !q.scatter && !q.compact && q.K == f.K &&
-                        q.K_pad == f.K_pad && q.n_mult == 1 && q.tc.valid && q.d_wp_plain && !(h->stem_packed && q.src == 0) &&
+                        q.K_pad == f.K_pad && q.n_mult == 1 && q.tc.valid && !(h->stem_packed && q.src == 0) &&
                         ((q.stride == 1 && !X.split) || (q.stride == 2 && X.split))) {
-                        float* bsum;
-                        TRY(dev_alloc(h, h->pack_buffers, (void**)&bsum, (size_t)f.K_pad * sizeof(float)));
-                        fp::launch_add_bias(f.d_bp, q.d_bp, f.K_pad, bsum, st);
-                        f.d_bp = bsum;
-                        f.proj = cand; f.proj_kind = 2; q.absorbed = 1;
+                        f.proj = cand; f.proj_kind = 2; q.absorbed = 1; q.plain_bank = 1;
                     }
                 }
-            }
-            if (f.tc.valid && f.tc.blocked_bank) {
-                // the streamed form of the kernel reads its bank block by block: one copy per pipeline stage
-                const int taps = packed_stem ? 3 : f.R * f.S, cchunks = (packed_stem ? 80 : C_pad_total) / 8;
-                void* blocked;
-                TRY(dev_alloc(h, h->pack_buffers, &blocked, (size_t)f.tc.n_tiles * taps * cchunks * f.tc.n_tile * 16));
-                if (f.tc.blocked_bank == 1)          // 1x1 layer, unified stages: [tile][K group][tap][chunk][row]
-                    fp::launch_reblock_bank((const __nv_bfloat16*)f.d_wp, taps, cchunks, f.K_pad, f.tc.n_tile, f.tc.n_tiles, f.tc.cg,
-                                            (__nv_bfloat16*)blocked, st);
-                else                                 // gathered layer with several filter tiles: [tile][(tap, chunk) plane][row]
-                    fp::launch_reblock_bank((const __nv_bfloat16*)f.d_wp, 1, taps * cchunks, f.K_pad, f.tc.n_tile, f.tc.n_tiles,
-                                            taps * cchunks, (__nv_bfloat16*)blocked, st);
-                f.d_wp = blocked;
             }
         } else if (op.kind == 1) {
             const Pool& p = h->pools[op.idx];
@@ -1066,17 +1040,114 @@ fp_status replan(fp_handle h) {
             const Tensor& src = h->tensors[h->head_src];
             std::vector<int32_t> chan_src(src.C_pad, -1);
             for (int c = 0; c < src.C; ++c) chan_src[c] = src.keep[c];
-            int32_t* d_chan;
-            TRY(upload_i32(h, chan_src, &d_chan));
-            TRY(dev_alloc(h, h->pack_buffers, (void**)&h->d_fcw_packed, (size_t)h->n_classes * src.C_pad * sizeof(float)));
-            TRY(dev_alloc(h, h->pack_buffers, (void**)&h->d_pool, (size_t)h->max_batch * src.C_pad * sizeof(float)));
-            // the average's 1/(H*W) is folded into the FC weights
-            fp::launch_repack_fc(h->d_fcw, h->fc_C, h->n_classes, d_chan, src.C_pad, 1.0f / (float)(src.H * src.W),
-                                 h->d_fcw_packed, st);
+            head_chan = add_idx(chan_src);
         }
     }
-    CK(cudaGetLastError());
-    TRY(find_chains(h, uses));
+    find_chains(h, uses);
+
+    // --- packed filters, biases, FC matrix: sizes and jobs, then one region, one upload and one launch ---
+    {
+        struct Want { void** slot; size_t bytes; };
+        std::vector<Want> wants;
+        std::vector<fp::PackJob> jobs;
+        struct Out { int job; void** slot; size_t off; };
+        std::vector<Out> outs;                   // where each job writes: a slot of `wants`, known once the region exists
+        auto add_job = [&](fp::PackJob j, void** slot, size_t off) { outs.push_back({(int)jobs.size(), slot, off}); jobs.push_back(j); };
+        auto filters = [&](const FConv& f, int kind) {
+            fp::PackJob j;
+            memset(&j, 0, sizeof(j));
+            j.kind = kind; j.w = f.d_w32; j.f32 = !bf16; j.C = f.C; j.RS = f.R * f.S;
+            j.rows = j.K_pad = j.n_tile = f.K_pad;
+            j.chunks = j.chunks1 = j.cg = f.C_pad / 8;
+            j.row = f.row_off; j.chan = f.chan_off;
+            return j;
+        };
+        auto bias = [&](const FConv& f) {
+            fp::PackJob j;
+            memset(&j, 0, sizeof(j));
+            j.kind = fp::PACK_BIAS; j.w = f.d_b32; j.units = f.K_pad; j.row = f.row_off;
+            if (f.proj >= 0) { j.w2 = h->convs[f.proj].d_b32; j.row2 = h->convs[f.proj].row_off; }
+            return j;
+        };
+        for (int i = 0; i < (int)h->ops.size(); ++i) {
+            if (h->ops[i].kind != 0) continue;
+            FConv& f = h->convs[h->ops[i].idx];
+            f.d_wp = nullptr; f.d_bp = nullptr;
+            if (h->op_chain[i] >= 0) continue;                           // packed for its run below
+            if (f.absorbed && !f.plain_bank) continue;                   // stacked into the layer that adds it
+            fp::PackJob j = filters(f, fp::PACK_CONV);
+            size_t vecs;
+            if (h->stem_fused && i == 1) {
+                j.kind = fp::PACK_STEM_DIRECT;
+                j.units = 32 * f.K_pad; vecs = (size_t)j.units;
+            } else if (h->stem_packed && f.src == 0) {
+                j.kind = fp::PACK_STEM;
+                j.units = 30 * f.K_pad; vecs = (size_t)j.units;
+            } else {
+                if (f.proj_kind == 1) {
+                    const FConv& q = h->convs[f.proj];
+                    j.w2 = q.d_w32; j.C2 = q.C; j.row2 = q.row_off; j.chan2 = q.chan_off;
+                    j.chunks += q.C_pad / 8;
+                    j.cg = j.chunks;
+                }
+                if (f.tc.valid && f.tc.blocked_bank && !f.plain_bank) {
+                    // the streamed form of the kernel reads its bank block by block, one copy per pipeline stage; gathered and
+                    // resident layers with several filter tiles read it tile by tile
+                    j.n_tile = f.tc.n_tile; j.rows = f.tc.n_tile * f.tc.n_tiles;
+                    if (f.tc.blocked_bank == 1) j.cg = f.tc.cg;
+                }
+                j.units = j.rows * j.chunks;
+                vecs = (size_t)j.units * j.RS;
+            }
+            wants.push_back({&f.d_wp, vecs * 8 * h->act_elem()});
+            add_job(j, &f.d_wp, 0);
+            wants.push_back({(void**)&f.d_bp, (size_t)f.K_pad * sizeof(float)});
+            add_job(bias(f), (void**)&f.d_bp, 0);
+        }
+        for (Chain& ch : h->chains) {
+            wants.push_back({(void**)&ch.d_blob, ch.blob_bytes});
+            for (size_t l = 0; l < ch.convs.size(); ++l) {
+                const FConv& f = h->convs[ch.convs[l]];
+                fp::PackJob j = filters(f, fp::PACK_CHAIN);
+                j.units = j.rows * j.chunks;
+                add_job(j, (void**)&ch.d_blob, (size_t)ch.args.layers[l].blob_off);
+                add_job(bias(f), (void**)&ch.d_blob, (size_t)ch.args.layers[l].blob_off + (size_t)9 * f.C_pad * f.K_pad * 2);
+            }
+        }
+        {
+            const Tensor& src = h->tensors[h->head_src];
+            fp::PackJob j;
+            memset(&j, 0, sizeof(j));
+            j.kind = fp::PACK_FC; j.f32 = 1; j.w = h->d_fcw; j.C = h->fc_C; j.chan = head_chan; j.chunks = src.C_pad / 8;
+            j.units = h->n_classes * j.chunks;
+            j.scale = 1.0f / (float)(src.H * src.W);                     // the average's 1/(H*W) is folded into the FC weights
+            wants.push_back({(void**)&h->d_fcw_packed, (size_t)h->n_classes * src.C_pad * sizeof(float)});
+            add_job(j, (void**)&h->d_fcw_packed, 0);
+            wants.push_back({(void**)&h->d_pool, (size_t)h->max_batch * src.C_pad * sizeof(float)});
+        }
+        size_t total = 0;
+        for (const Want& w : wants) total += align256(w.bytes ? w.bytes : 16);
+        TRY(region_reserve(h, h->pack_region, total));
+        size_t at = 0;
+        for (const Want& w : wants) { *w.slot = (uint8_t*)h->pack_region.p + at; at += align256(w.bytes ? w.bytes : 16); }
+        for (const Out& o : outs) jobs[o.job].out = (uint8_t*)*o.slot + o.off;
+        int n_blocks = 0;
+        for (fp::PackJob& j : jobs) { j.first_block = n_blocks; n_blocks += (j.units + fp::kPackThreads - 1) / fp::kPackThreads; }
+        const size_t o_blocks = align256(jobs.size() * sizeof(fp::PackJob)), o_idx = o_blocks + align256((size_t)n_blocks * 4);
+        const size_t meta = o_idx + align256(idx.size() * 4 + 4);
+        TRY(region_reserve(h, h->meta_region, meta));
+        TRY(pinned_reserve(h, meta));
+        uint8_t *hm = (uint8_t*)h->pinned, *dm = (uint8_t*)h->meta_region.p;
+        memcpy(hm, jobs.data(), jobs.size() * sizeof(fp::PackJob));
+        int32_t* bj = (int32_t*)(hm + o_blocks);
+        for (size_t k = 0; k < jobs.size(); ++k)
+            for (int b = 0; b < (jobs[k].units + fp::kPackThreads - 1) / fp::kPackThreads; ++b) *bj++ = (int32_t)k;
+        memcpy(hm + o_idx, idx.data(), idx.size() * 4);
+        h->d_idx = (const int32_t*)(dm + o_idx);
+        CK(cudaMemcpyAsync(dm, hm, meta, cudaMemcpyHostToDevice, st));
+        fp::launch_pack((const fp::PackJob*)dm, (const int32_t*)(dm + o_blocks), n_blocks, h->d_idx, st);
+        CK(cudaGetLastError());
+    }
 
     // --- activation memory: buffers are reused once their last reader has run ---
     {
@@ -1089,8 +1160,10 @@ fp_status replan(fp_handle h) {
                 const int x = h->convs[h->convs[h->ops[i].idx].proj].src;
                 last_use[x] = std::max(last_use[x], i);
             }
-        struct Buf { void* p; size_t bytes; int free_after; };
+        struct Buf { size_t bytes; int free_after; };
         std::vector<Buf> bufs;
+        std::vector<std::pair<int, int>> placed;         // (tensor, buffer)
+        const size_t vec_bytes = 8 * h->act_elem();
         for (int i = 0; i < (int)h->ops.size(); ++i) {
             const Op& op = h->ops[i];
             int tid = -1;
@@ -1116,7 +1189,6 @@ fp_status replan(fp_handle h) {
             if (tid < 0) continue;
             Tensor& t = h->tensors[tid];
             // planar-8 with border, plus guard vectors before and after (halo reads of the first/last tiles)
-            const size_t vec_bytes = 8 * h->act_elem();
             t.bytes = ((size_t)(t.C_pad / 8) * h->max_batch * (t.H + 2) * (t.W + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
             if (t.split)
                 t.bytes = ((size_t)(t.C_pad / 8) * 4 * h->max_batch * (t.H / 2 + 2) * (t.W / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
@@ -1127,15 +1199,19 @@ fp_status replan(fp_handle h) {
                 for (int b = 0; b < (int)bufs.size(); ++b)
                     if (bufs[b].free_after < i && bufs[b].bytes >= t.bytes && (best < 0 || bufs[b].bytes < bufs[best].bytes)) best = b;
             if (best < 0) {
-                void* p;
-                TRY(dev_alloc(h, h->act_buffers, &p, t.bytes));
-                CK(cudaMemsetAsync(p, 0, t.bytes, st));
-                bufs.push_back({p, t.bytes, 0});
+                bufs.push_back({t.bytes, 0});
                 best = (int)bufs.size() - 1;
             }
-            t.d = (uint8_t*)bufs[best].p + (size_t)fp::kGuardVectors * vec_bytes;
+            placed.push_back({tid, best});
             bufs[best].free_after = std::max(last_use[tid], i);
         }
+        std::vector<size_t> start(bufs.size());
+        size_t total = 0;
+        for (size_t b = 0; b < bufs.size(); ++b) { start[b] = total; total += align256(bufs[b].bytes); }
+        TRY(region_reserve(h, h->act_region, total));
+        CK(cudaMemsetAsync(h->act_region.p, 0, total, st));
+        for (const auto& pl : placed)
+            h->tensors[pl.first].d = (uint8_t*)h->act_region.p + start[pl.second] + (size_t)fp::kGuardVectors * vec_bytes;
     }
 
     // --- launch arguments and tensor-core plans ---
@@ -1148,7 +1224,8 @@ fp_status replan(fp_handle h) {
         conv_geometry(h, f, &a);
         a.C_pad = (h->stem_packed && f.src == 0) ? 80 : f.C_pad;
         a.K_pad = f.K_pad;
-        a.scatter = f.scatter; a.out_C_pad = out.C_pad; a.out_map = f.d_out_map; a.tile_chunk0 = f.d_chunk0;
+        a.scatter = f.scatter; a.out_C_pad = out.C_pad;
+        a.out_map = f.map_off >= 0 ? h->d_idx + f.map_off : nullptr; a.tile_chunk0 = f.chunk0_off >= 0 ? h->d_idx + f.chunk0_off : nullptr;
         a.n_tile_forced = f.n_tile_forced;
         a.res_mode = f.res_mode;
         if (f.proj >= 0) {
@@ -1156,7 +1233,7 @@ fp_status replan(fp_handle h) {
             const Tensor& X = h->tensors[q.src];
             a.x2 = X.d; a.x2_plane_mult = X.split ? 4 : 1;
             if (f.proj_kind == 1) { a.C_pad = f.C_pad + q.C_pad; a.x2_chunk0 = f.C_pad / 8; }
-            else { a.w2 = q.d_wp_plain; a.x2_C_pad = q.C_pad; }
+            else { a.w2 = q.d_wp; a.x2_C_pad = q.C_pad; }
             a.res_mode = 0;
         } else if (f.res_mode) {
             const Tensor& r = h->tensors[f.res_tid];
@@ -1271,9 +1348,9 @@ extern "C" fp_status fp_destroy(fp_handle h) {
         cudaStreamDestroy(h->copy_stream);
         for (cudaEvent_t e : h->copy_events) if (e) cudaEventDestroy(e);
     }
-    free_list(h, h->act_buffers);
-    free_list(h, h->pack_buffers);
+    for (Region* r : {&h->act_region, &h->pack_region, &h->meta_region}) dev_free(h, r->p);
     free_list(h, h->fixed_buffers);
+    if (h->pinned) cudaFreeHost(h->pinned);
     delete h;
     return FP_OK;
 }
@@ -1336,8 +1413,6 @@ extern "C" fp_status fp_fuse_with_allocator(const fp_model_desc* desc, const flo
         for (const FConv& f : h->convs) max_K = std::max(max_K, f.K);
         if ((size_t)max_K * sizeof(double) > 48 * 1024) return fail(FP_ERR_UNSUPPORTED, "fp_fuse: more than 6144 filters in one convolution");
         TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_scores, (size_t)max_K * sizeof(double)));
-        TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_rank, (size_t)max_K * sizeof(int32_t)));
-        TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_mask, (size_t)max_K));
         TRY(dev_alloc(h, h->fixed_buffers, &h->d_in_stage, (size_t)max_batch * h->in_C * h->in_H * h->in_W * h->in_elem()));
         TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_logits_stage, (size_t)max_batch * h->n_classes * sizeof(float)));
         all_ones_masks(h);
@@ -1372,41 +1447,96 @@ extern "C" fp_status fp_score(fp_handle h, int32_t conv_index, int32_t norm, dou
     return FP_OK;
 }
 
+// The bank table (description order, which is also the order of fp_soft_prune_epoch's update array) and the buffers of a
+// selection over all banks; made at the first selection.
+static fp_status ensure_banks(fp_handle h) {
+    if (!h->banks.empty()) return FP_OK;
+    std::vector<fp::SoftBank> banks;
+    std::vector<int> bank_conv;
+    std::vector<int32_t> map;
+    long long off = 0;
+    for (int ci = 0; ci < h->n_desc_convs; ++ci) {
+        if (h->conv_to_fused[ci] < 0) continue;
+        const FConv& f = h->convs[h->conv_to_fused[ci]];
+        fp::SoftBank b;
+        b.w = f.d_w32; b.dw_off = off; b.K = f.K; b.per = f.C * f.R * f.S; b.q = 0; b.k_off = (int)map.size();
+        map.insert(map.end(), (size_t)f.K, (int32_t)banks.size());
+        banks.push_back(b);
+        bank_conv.push_back(h->conv_to_fused[ci]);
+        off += (long long)f.K * b.per;
+    }
+    const size_t n = map.size();
+    TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_banks, banks.size() * sizeof(fp::SoftBank)));
+    TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_bank_map, n * sizeof(int32_t)));
+    TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_bank_scores, n * sizeof(double)));
+    TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_bank_rank, n * (sizeof(int32_t) + 1)));
+    h->d_bank_mask = (uint8_t*)(h->d_bank_rank + n);
+    CK(cudaMemcpy(h->d_bank_map, map.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice));
+    h->n_filters = (int)n;
+    h->bank_conv = bank_conv;
+    h->banks = banks;
+    return FP_OK;
+}
+
+// How many filters of every convolution a selection masks: n - m of a fused operator (back to its original filter count),
+// floor(ratio * n) of the others.
+static fp_status filters_to_mask(fp_handle h, const FConv& f, const double* h_ratios, const char* who, int* q) {
+    if (f.role != 0) { *q = f.K - f.n_orig; return FP_OK; }
+    const double r = h_ratios ? h_ratios[f.conv_index] : 0.0;
+    if (!(r >= 0.0) || r > 1.0) return fail(FP_ERR_ARG, "%s: ratio of convolution %d outside [0,1]", who, f.conv_index);
+    *q = (int)std::floor(r * (double)f.K + 1e-9);
+    return FP_OK;
+}
+
+// Scores (after adding `d_updates`, if given), ranks and masks of all banks: two launches and one copy back; h->pinned then
+// holds the ranks and, behind them, the masks.  q: one count per fused convolution.
+static fp_status select_all(fp_handle h, int norm, const std::vector<int>& q, const float* d_updates, int zeroize,
+                            const int32_t** ranks, const uint8_t** masks) {
+    const size_t n = (size_t)h->n_filters, table = h->banks.size() * sizeof(fp::SoftBank);
+    TRY(pinned_reserve(h, align256(table) + n * 5));
+    for (size_t i = 0; i < h->banks.size(); ++i) h->banks[i].q = q[h->bank_conv[i]];
+    memcpy(h->pinned, h->banks.data(), table);
+    int32_t* back = (int32_t*)((uint8_t*)h->pinned + align256(table));
+    CK(cudaMemcpyAsync(h->d_banks, h->pinned, table, cudaMemcpyHostToDevice, 0));
+    fp::launch_bank_score(h->d_banks, h->d_bank_map, (int)n, d_updates, norm, h->d_bank_scores, 0);
+    fp::launch_bank_rank(h->d_banks, h->d_bank_map, (int)n, h->d_bank_scores, zeroize, h->d_bank_rank, h->d_bank_mask, 0);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(back, h->d_bank_rank, n * 5, cudaMemcpyDeviceToHost, 0));
+    CK(cudaStreamSynchronize(0));
+    *ranks = back;
+    *masks = (const uint8_t*)(back + n);
+    return FP_OK;
+}
+
 extern "C" fp_status fp_prune(fp_handle h, int32_t norm, const double* h_ratios, const uint8_t* const* h_masks) {
     if (!h) return fail(FP_ERR_ARG, "fp_prune: NULL handle");
     if (norm != FP_NORM_L1 && norm != FP_NORM_L2) return fail(FP_ERR_ARG, "fp_prune: bad norm");
-    // select every mask first (all scores are taken on the unpruned fused weights), then apply
-    std::vector<std::vector<uint8_t>> masks(h->convs.size());
-    std::vector<std::vector<int32_t>> ranks(h->convs.size());
+    // check every argument and select every mask first (all scores are taken on the unpruned fused weights), then apply
+    std::vector<int> q(h->convs.size(), 0);
     for (size_t i = 0; i < h->convs.size(); ++i) {
         const FConv& f = h->convs[i];
-        masks[i].resize(f.K);
-        ranks[i].resize(f.K);
-        TRY(score_conv(h, f, norm));
         const uint8_t* given = h_masks ? h_masks[f.conv_index] : nullptr;
-        int q;
-        if (f.role != 0) q = f.K - f.n_orig;               // fused operator: back to its original filter count
-        else {
-            const double r = h_ratios ? h_ratios[f.conv_index] : 0.0;
-            if (!(r >= 0.0) || r > 1.0) return fail(FP_ERR_ARG, "fp_prune: ratio of convolution %d outside [0,1]", f.conv_index);
-            q = (int)std::floor(r * (double)f.K + 1e-9);
-        }
-        fp::launch_rank_mask(h->d_scores, f.K, q, h->d_rank, h->d_mask, 0);
-        CK(cudaGetLastError());
-        CK(cudaMemcpy(ranks[i].data(), h->d_rank, (size_t)f.K * sizeof(int32_t), cudaMemcpyDeviceToHost));
+        TRY(filters_to_mask(h, f, h_ratios, "fp_prune", &q[i]));
+        int kept = f.K - q[i];
         if (given) {
+            kept = 0;
             for (int k = 0; k < f.K; ++k) {
                 if (given[k] > 1) return fail(FP_ERR_ARG, "fp_prune: mask of convolution %d has a value other than 0/1", f.conv_index);
-                masks[i][k] = given[k];
+                kept += given[k];
             }
-        } else {
-            CK(cudaMemcpy(masks[i].data(), h->d_mask, (size_t)f.K, cudaMemcpyDeviceToHost));
         }
-        int kept = 0;
-        for (int k = 0; k < f.K; ++k) kept += masks[i][k];
         if (kept == 0) return fail(FP_ERR_EMPTY_LAYER, "fp_prune: convolution %d would keep no filter", f.conv_index);
     }
-    for (size_t i = 0; i < h->convs.size(); ++i) { h->convs[i].mask = masks[i]; h->convs[i].rank = ranks[i]; }
+    TRY(ensure_banks(h));
+    const int32_t* ranks;
+    const uint8_t* masks;
+    TRY(select_all(h, norm, q, nullptr, 0, &ranks, &masks));
+    for (size_t bi = 0; bi < h->banks.size(); ++bi) {
+        FConv& f = h->convs[h->bank_conv[bi]];
+        const uint8_t* m = h_masks && h_masks[f.conv_index] ? h_masks[f.conv_index] : masks + h->banks[bi].k_off;
+        f.rank.assign(ranks + h->banks[bi].k_off, ranks + h->banks[bi].k_off + f.K);
+        f.mask.assign(m, m + f.K);
+    }
     return replan(h);
 }
 
@@ -1418,55 +1548,18 @@ extern "C" fp_status fp_soft_prune_epoch(fp_handle h, int32_t norm, const double
     std::vector<int> q(h->convs.size(), 0);
     for (size_t i = 0; i < h->convs.size(); ++i) {
         const FConv& f = h->convs[i];
-        if (f.role != 0) q[i] = f.K - f.n_orig;
-        else {
-            const double r = h_ratios ? h_ratios[f.conv_index] : 0.0;
-            if (!(r >= 0.0) || r > 1.0) return fail(FP_ERR_ARG, "fp_soft_prune_epoch: ratio of convolution %d outside [0,1]", f.conv_index);
-            q[i] = (int)std::floor(r * (double)f.K + 1e-9);
-        }
+        TRY(filters_to_mask(h, f, h_ratios, "fp_soft_prune_epoch", &q[i]));
         if (q[i] >= f.K) return fail(FP_ERR_EMPTY_LAYER, "fp_soft_prune_epoch: convolution %d would keep no filter", f.conv_index);
     }
-    // bank table in description order (the order of the update array), filters numbered bank by bank
-    std::vector<fp::SoftBank> banks;
-    std::vector<int32_t> map;
-    std::vector<size_t> fused_of;
-    long long off = 0;
-    int k_off = 0, max_K = 1;
-    for (int ci = 0; ci < h->n_desc_convs; ++ci) {
-        if (h->conv_to_fused[ci] < 0) continue;
-        const size_t i = (size_t)h->conv_to_fused[ci];
-        const FConv& f = h->convs[i];
-        fp::SoftBank b;
-        b.w = f.d_w32; b.dw_off = off; b.K = f.K; b.per = f.C * f.R * f.S; b.q = q[i]; b.k_off = k_off;
-        for (int k = 0; k < f.K; ++k) map.push_back((int32_t)banks.size());
-        banks.push_back(b);
-        fused_of.push_back(i);
-        off += (long long)f.K * b.per;
-        k_off += f.K;
-        max_K = std::max(max_K, f.K);
-    }
-    if (!h->d_soft_banks) {
-        h->soft_total = k_off;
-        TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_soft_banks, banks.size() * sizeof(fp::SoftBank)));
-        TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_soft_map, map.size() * sizeof(int32_t)));
-        TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_soft_scores, (size_t)k_off * sizeof(double)));
-        TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_soft_rank, (size_t)k_off * sizeof(int32_t)));
-        TRY(dev_alloc(h, h->fixed_buffers, (void**)&h->d_soft_mask, (size_t)k_off));
-        CK(cudaMemcpy(h->d_soft_map, map.data(), map.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    }
-    CK(cudaMemcpy(h->d_soft_banks, banks.data(), banks.size() * sizeof(fp::SoftBank), cudaMemcpyHostToDevice));
-    fp::launch_soft_update_score(h->d_soft_banks, h->d_soft_map, k_off, d_updates, norm, h->d_soft_scores, 0);
-    fp::launch_soft_rank(h->d_soft_banks, (int)banks.size(), max_K, h->d_soft_scores, h->d_soft_rank, h->d_soft_mask, 0);
-    fp::launch_soft_zeroize(h->d_soft_banks, h->d_soft_map, k_off, h->d_soft_mask, 0);
-    CK(cudaGetLastError());
-    std::vector<int32_t> all_rank(k_off);
-    std::vector<uint8_t> all_mask(k_off);
-    CK(cudaMemcpy(all_rank.data(), h->d_soft_rank, (size_t)k_off * sizeof(int32_t), cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(all_mask.data(), h->d_soft_mask, (size_t)k_off, cudaMemcpyDeviceToHost));
-    for (size_t bi = 0; bi < banks.size(); ++bi) {
-        FConv& f = h->convs[fused_of[bi]];
-        f.rank.assign(all_rank.begin() + banks[bi].k_off, all_rank.begin() + banks[bi].k_off + f.K);
-        f.mask.assign(all_mask.begin() + banks[bi].k_off, all_mask.begin() + banks[bi].k_off + f.K);
+    TRY(ensure_banks(h));
+    const int32_t* ranks;
+    const uint8_t* masks;
+    TRY(select_all(h, norm, q, d_updates, 1, &ranks, &masks));
+    for (size_t bi = 0; bi < h->banks.size(); ++bi) {
+        FConv& f = h->convs[h->bank_conv[bi]];
+        const int o = h->banks[bi].k_off;
+        f.rank.assign(ranks + o, ranks + o + f.K);
+        f.mask.assign(masks + o, masks + o + f.K);
     }
     ++h->soft_epochs;
     return FP_OK;
@@ -1677,6 +1770,27 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             TRY(conv_of(&f));
             if (!f) return fail(FP_ERR_ARG, "fp_query: convolution %d was absorbed by fusion", index);
             TRY(need((size_t)f->K * 4)); memcpy(h_out, f->rank.data(), (size_t)f->K * 4); return FP_OK;
+        case FP_Q_ALL_MASKS: {
+            // [K of every convolution][ranks of all filters][masks of all filters], description order
+            size_t total = 0;
+            for (int ci = 0; ci < h->n_desc_convs; ++ci)
+                if (h->conv_to_fused[ci] >= 0) total += (size_t)h->convs[h->conv_to_fused[ci]].K;
+            if (index == 0) { TRY(need(4)); *(int32_t*)h_out = (int32_t)total; return FP_OK; }
+            TRY(need((size_t)h->n_desc_convs * 4 + total * 5));
+            int32_t* Ks = (int32_t*)h_out;
+            int32_t* r = Ks + h->n_desc_convs;
+            uint8_t* m = (uint8_t*)(r + total);
+            for (int ci = 0; ci < h->n_desc_convs; ++ci) {
+                Ks[ci] = 0;
+                if (h->conv_to_fused[ci] < 0) continue;
+                const FConv& c = h->convs[h->conv_to_fused[ci]];
+                Ks[ci] = c.K;
+                memcpy(r, c.rank.data(), (size_t)c.K * 4);
+                memcpy(m, c.mask.data(), (size_t)c.K);
+                r += c.K; m += c.K;
+            }
+            return FP_OK;
+        }
         case FP_Q_FLOPS: {
             TRY(need(8));
             double s = 0;

@@ -93,44 +93,43 @@ void launch_identity_filters(float* dst, int C_dst, int R, int S, int k0, int c0
                              cudaStream_t st);
 void launch_count_nonfinite(const float* p, size_t n, int* d_count, cudaStream_t st);
 void launch_score_filters(const float* w, int K, int per_filter, int norm, double* scores, cudaStream_t st);
-void launch_rank_mask(const double* scores, int K, int q, int32_t* rank, uint8_t* mask, cudaStream_t st);
-// Algorithm 1's loop body over ALL filter banks of a model in three launches.  One SoftBank per convolution;
+// score, rank and mask one bank; `scores` has room for K
+void launch_score_rank(const float* w, int K, int per_filter, int norm, int q, double* scores, int32_t* rank, uint8_t* mask,
+                       cudaStream_t st);
+// Selection over ALL filter banks of a model (fp_prune, and the loop body of Algorithm 1).  One SoftBank per convolution;
 // filter_bank[g] names the bank of global filter g (filters of all banks numbered consecutively, bank by bank).
 struct SoftBank {
-    float* w;             // K x per fp32, updated and zeroized in place
+    float* w;             // K x per fp32
     long long dw_off;     // element offset of the bank's addends in the update array
-    int K, per, q;        // filters, weights per filter, filters to zeroize
+    int K, per, q;        // filters, weights per filter, filters to mask
     int k_off;            // global number of the bank's first filter
 };
-// w += dw (one fp32 addition per weight; dw may be nullptr) and the filter scores of the updated weights, in the
-// fixed summation order of launch_score_filters
-void launch_soft_update_score(const SoftBank* banks, const int32_t* filter_bank, int total_filters, const float* dw,
-                              int norm, double* scores, cudaStream_t st);
-// per bank: rank by (score, index) ascending, mask the first q (one block per bank)
-void launch_soft_rank(const SoftBank* banks, int n_banks, int max_K, const double* scores, int32_t* rank, uint8_t* mask,
-                      cudaStream_t st);
-// masked filters become zero
-void launch_soft_zeroize(const SoftBank* banks, const int32_t* filter_bank, int total_filters, const uint8_t* mask,
-                         cudaStream_t st);
-// Convolution filters: packed[rs][cp/8][kr][cp%8] = w[row_src[kr]][chan_src[cp]][rs] (zero where an index is -1)
-void launch_repack_conv(const float* w, int C, int RS, const int32_t* row_src, int K_pad, const int32_t* chan_src,
-                        int C_pad, __nv_bfloat16* out_bf16, float* out_f32, cudaStream_t st);
-// Streamed filter bank: from packed[rs][cp/8][K_pad][8] to blocks in the order the tensor-core kernel streams them,
-// blocked[filter tile t][K group g][rs][chunk in group][row in tile][8] (groups of `cg` chunks, the last one shorter;
-// tiles of `n_tile` rows, rows past K_pad zero): n_tiles * RS * (C_pad/8) * n_tile * 8 elements
-void launch_reblock_bank(const __nv_bfloat16* packed, int RS, int cchunks, int K_pad, int n_tile, int n_tiles, int cg,
-                         __nv_bfloat16* blocked, cudaStream_t st);
-// FC matrix: packed[k][cp] = w[k][chan_src[cp]] * scale
-void launch_repack_fc(const float* w, int C, int K, const int32_t* chan_src, int C_pad, float scale, float* out,
-                      cudaStream_t st);
-// 7x7 first convolution as a 3x1 convolution over the packed network input (80 channels)
-void launch_repack_stem(const float* w, int C, const int32_t* row_src, int K_pad, __nv_bfloat16* out, cudaStream_t st);
-void launch_add_bias(const float* a, const float* b, int n, float* out, cudaStream_t st);          // out = a + b (fp32)
-void launch_pack_bias(const float* b, const int32_t* row_src, int K_pad, float* out, cudaStream_t st);
-// 3x3 filters of one layer of a fused run: blob[r][cp/8][48*(kr/16) + 16*s + kr%16][cp%8], the three
-// horizontal taps stacked along the filter (N) axis of the MMA (see chain_tc.cu)
-void launch_repack_chain(const float* w, int C, const int32_t* row_src, int K_pad, const int32_t* chan_src, int C_pad,
-                         __nv_bfloat16* out, cudaStream_t st);
+// w += dw (one fp32 addition per weight; dw may be nullptr: the weights stay) and the scores of the weights that result, in
+// the fixed summation order of launch_score_filters
+void launch_bank_score(const SoftBank* banks, const int32_t* filter_bank, int total_filters, const float* dw, int norm,
+                       double* scores, cudaStream_t st);
+// per bank: rank by (score, index) ascending, mask the first q - and, with zeroize, set their weights to zero
+void launch_bank_rank(const SoftBank* banks, const int32_t* filter_bank, int total_filters, const double* scores, int zeroize,
+                      int32_t* rank, uint8_t* mask, cudaStream_t st);
+
+// Packing of a planned graph's filters, biases and FC matrix: all jobs in one launch.  Index arrays (packed row -> fused
+// filter, packed channel -> fused channel, -1 = zeros) are parts of one array, named by their offsets.
+enum { PACK_CONV = 0, PACK_CHAIN = 1, PACK_STEM = 2, PACK_STEM_DIRECT = 3, PACK_FC = 4, PACK_BIAS = 5 };
+constexpr int kPackThreads = 256;
+struct PackJob {
+    const float* w;       // fused fp32 filters K x C x RS (PACK_FC: the FC matrix; PACK_BIAS: the shifts)
+    const float* w2;      // a second bank stacked behind the first along the channels / a second shift to add, or nullptr
+    void* out;
+    int kind, f32;        // f32: fp32 vectors instead of bf16
+    int units, first_block;
+    int C, C2, RS;        // channels of the fused banks (row pitches), taps
+    int rows, K_pad;      // packed rows with and without the last filter tile's padding
+    int chunks, chunks1;  // packed channel chunks, those of the first bank
+    int n_tile, cg;       // PACK_CONV: rows per filter tile, chunks per K group
+    int row, chan, row2, chan2;
+    float scale;          // PACK_FC
+};
+void launch_pack(const PackJob* jobs, const int32_t* block_job, int n_blocks, const int32_t* idx, cudaStream_t st);
 
 // Memory-bound operators ------------------------------------------------------------------
 // Both convert images n0 .. n0 + n_count - 1 of a batch of N images (`in` and `out` are the whole batch's buffers).
@@ -156,8 +155,8 @@ struct ConvPlanTC {
     int flat;             // 1: stride-1 "same" convolution, activation tiles fetched as contiguous runs
                           //    of flat positions (bulk copies); 0: gathered by loader threads
     int b_resident;       // flat only: the whole filter bank stays in shared memory
-    int blocked_bank;     // 1: 1x1 layer with unified stages, bank stored block by block; 2: gathered layer with several
-                          // filter tiles, bank stored tile by tile (launch_reblock_bank either way)
+    int blocked_bank;     // 1: 1x1 layer with unified stages, bank stored block by block; 2: gathered or resident layer with
+                          // several filter tiles, bank stored tile by tile (PackJob either way)
     int cg;               // channel chunks (of 8) per K block
     int groups;           // K blocks per filter tap = ceil((C_pad/8) / cg)
     int halo;             // flat: vectors fetched before and after the 128 positions of a tile
@@ -185,7 +184,7 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
 struct StemPoolArgs {
     const void* x;        // network input, N x C x H x W, NCHW, bf16
     void* y;              // pooled tensor, planar-8 with border, (H/4) x (W/4) pixels, K_pad channels, N images
-    const void* w;        // filters [16 taps (ta, tb)][2 chunks of 8][K_pad rows][8] bf16 over the parity channels (launch_repack_stem_direct)
+    const void* w;        // filters [16 taps (ta, tb)][2 chunks of 8][K_pad rows][8] bf16 over the parity channels (PACK_STEM_DIRECT)
     const float* bias;    // [K_pad]
     int N, C, H, W, K_pad;
     int n0, n_count;      // the images this launch handles (the tensor's plane pitch is that of all N)
@@ -194,8 +193,6 @@ struct StemPoolPlan { int valid, tiles, tmem_cols; unsigned smem_bytes; };
 bool stem_pool_supported(int C, int H, int W, int K_pad);
 int plan_stem_pool(const StemPoolArgs& a, StemPoolPlan* plan, char* err, size_t err_len);
 void launch_stem_pool(const StemPoolPlan& plan, const StemPoolArgs& a, int* d_status, cudaStream_t st);
-// its filters: out[k / 8][kr][k % 8] = w[row_src[kr]][c][r][s] with k = (r * C + c) * 7 + s (zero rows / zero k padding)
-void launch_repack_stem_direct(const float* w, int C, const int32_t* row_src, int K_pad, __nv_bfloat16* out, cudaStream_t st);
 
 // A run of stride-1 3x3 convolutions executed by one kernel with the activations in shared memory.
 constexpr int kChainMaxLayers = 40;

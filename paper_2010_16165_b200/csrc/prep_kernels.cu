@@ -5,6 +5,10 @@
 
 namespace fp {
 
+constexpr int kSmallRank = 512;        // filters that one cluster scores and ranks in a single launch,
+constexpr int kSmallBank = 1 << 17;    // if the bank has no more weights than this: eight SMs read half a megabyte in about a microsecond
+constexpr int kRankCtas = 8;
+
 // omega_k with one rounded fp32 operation per step: t = var + eps; r = sqrt(t); omega = gamma / r.
 __device__ __forceinline__ float bn_omega(const float* bn, int K, int k, float eps) {
     const float t = __fadd_rn(bn[3 * K + k], eps);
@@ -55,227 +59,265 @@ __global__ void count_nonfinite_kernel(const float* __restrict__ p, size_t n, in
     if (bad) atomicAdd(count, bad);
 }
 
-// One warp per filter.  Lane l accumulates elements l, l+32, ... in increasing order in fp64
-// (each |w| or w*w is exact in fp64), then the 32 partial sums are combined pairwise with
-// partners at distance 16, 8, 4, 2, 1.  The order is part of the definition of the score, so
-// that the resulting double - and therefore the ranking - does not depend on the launch shape.
-__global__ void score_filters_kernel(const float* __restrict__ w, int K, int per, int norm, double* __restrict__ scores) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= K) return;
-    const float* f = w + (size_t)warp * per;
+// A filter's score by one warp.  Lane l accumulates elements l, l+32, ... in increasing order in fp64 (each |w| or
+// w*w is exact in fp64), then the 32 partial sums are combined pairwise with partners at distance 16, 8, 4, 2, 1.  The
+// order is part of the definition of the score, so that the resulting double - and therefore the ranking - does not
+// depend on the launch shape.  A lane's additions are one chain, but its loads are not: a batch of them is in flight at
+// once (with one load per addition a filter of 4608 weights waited for 144 memory latencies one after the other).
+constexpr int kScoreBatch = 16;
+template <bool UPDATE>
+__device__ __forceinline__ double score_filter(float* __restrict__ f, const float* __restrict__ d, int per, int norm, int lane) {
     double s = 0.0;
-    for (int t = lane; t < per; t += 32) {
-        const double v = (double)f[t];
-        s = __dadd_rn(s, norm ? __dmul_rn(v, v) : fabs(v));
-    }
+    for (int t0 = lane; t0 < per; t0 += 32 * kScoreBatch) {
+        float v[kScoreBatch];
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, d));
-    if (lane == 0) scores[warp] = s;
-}
-
-// rank[k] = number of filters ordered before k in ascending (score, index) order; the first q are masked.
-__global__ void rank_mask_kernel(const double* __restrict__ scores, int K, int q, int32_t* __restrict__ rank,
-                                 uint8_t* __restrict__ mask) {
-    extern __shared__ double sh[];
-    for (int i = threadIdx.x; i < K; i += blockDim.x) sh[i] = scores[i];
-    __syncthreads();
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        const double sk = sh[k];
-        int before = 0;
-        for (int j = 0; j < K; ++j) {
-            const double sj = sh[j];
-            before += (sj < sk) || (sj == sk && j < k);
+        for (int i = 0; i < kScoreBatch; ++i) v[i] = t0 + 32 * i < per ? f[t0 + 32 * i] : 0.0f;
+        if (UPDATE) {
+            float u[kScoreBatch];
+#pragma unroll
+            for (int i = 0; i < kScoreBatch; ++i) u[i] = t0 + 32 * i < per ? __ldg(d + t0 + 32 * i) : 0.0f;
+#pragma unroll
+            for (int i = 0; i < kScoreBatch; ++i) v[i] = __fadd_rn(v[i], u[i]);
+#pragma unroll
+            for (int i = 0; i < kScoreBatch; ++i)
+                if (t0 + 32 * i < per) f[t0 + 32 * i] = v[i];
         }
-        rank[k] = before;
-        mask[k] = before >= q ? 1 : 0;
-    }
-}
-
-// Algorithm 1's loop body over all banks.  One warp per filter: lane l updates and accumulates elements l, l+32, ...
-// in increasing order, then the 32 partial sums are combined pairwise at distances 16, 8, 4, 2, 1 - the order
-// that defines a score (see score_filters_kernel).
-__global__ void soft_update_score_kernel(const SoftBank* __restrict__ banks, const int32_t* __restrict__ filter_bank,
-                                         int total_filters, const float* __restrict__ dw, int norm,
-                                         double* __restrict__ scores) {
-    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (g >= total_filters) return;
-    const SoftBank b = banks[filter_bank[g]];
-    const int k = g - b.k_off;
-    float* f = b.w + (size_t)k * b.per;
-    const float* d = dw ? dw + b.dw_off + (size_t)k * b.per : nullptr;
-    double s = 0.0;
-    for (int t = lane; t < b.per; t += 32) {
-        float v = f[t];
-        if (d) { v = __fadd_rn(v, d[t]); f[t] = v; }
-        const double x = (double)v;
-        s = __dadd_rn(s, norm ? __dmul_rn(x, x) : fabs(x));
+#pragma unroll
+        for (int i = 0; i < kScoreBatch; ++i) {      // behind the filter's end: + 0.0, which changes no bit of a sum of non-negative terms
+            const double x = (double)v[i];
+            s = __dadd_rn(s, norm ? __dmul_rn(x, x) : fabs(x));
+        }
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
+    return s;
+}
+
+__global__ void score_filters_kernel(const float* __restrict__ w, int K, int per, int norm, double* __restrict__ scores) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (warp >= K) return;
+    const double s = score_filter<false>(const_cast<float*>(w) + (size_t)warp * per, nullptr, per, norm, lane);
+    if (lane == 0) scores[warp] = s;
+}
+
+// How many of a bank's K scores come before filter k's in ascending (score, index) order, counted by a whole warp.  (One
+// block per bank, every thread counting for its own filters, took 60-130 us for a bank of 2048 filters: K * K / 256
+// comparisons one after the other on one SM.)
+__device__ __forceinline__ int rank_of(const double* __restrict__ scores, int K, int k, int lane) {
+    const double sk = scores[k];
+    int before = 0;
+#pragma unroll 4
+    for (int j = lane; j < K; j += 32) {
+        const double sj = scores[j];
+        before += (sj < sk) || (sj == sk && j < k);
+    }
+    return __reduce_add_sync(0xffffffffu, before);
+}
+
+// rank[k] = number of filters ordered before k in ascending (score, index) order; the first q are masked.
+__global__ void rank_mask_kernel(const double* scores, int K, int q, int32_t* __restrict__ rank, uint8_t* __restrict__ mask) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (k >= K) return;
+    const int before = rank_of(scores, K, k, lane);
+    if (lane == 0) { rank[k] = before; mask[k] = before >= q ? 1 : 0; }
+}
+
+// Score, rank and mask of a small bank in one launch: a cluster of eight CTAs, every warp scores filters and puts each
+// score into all eight CTAs' shared memory; behind the cluster's barrier every CTA ranks an eighth of the filters, several
+// threads per filter.  No second launch and no scratch in global memory.
+__global__ void __cluster_dims__(kRankCtas, 1, 1) __launch_bounds__(256)
+score_rank_cluster_kernel(const float* __restrict__ w, int K, int per, int norm, int q, int32_t* __restrict__ rank,
+                          uint8_t* __restrict__ mask) {
+    __shared__ double sh[kSmallRank];
+    const int warp = (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    // nobody writes into another CTA's shared memory before that CTA runs
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    for (int k = (int)blockIdx.x * 8 + warp; k < K; k += 8 * kRankCtas) {
+        const double s = score_filter<false>(const_cast<float*>(w) + (size_t)k * per, nullptr, per, norm, lane);
+        if (lane < kRankCtas) {
+            uint32_t dst;
+            const uint32_t own = (uint32_t)__cvta_generic_to_shared(sh + k);
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(own), "r"(lane));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(s) : "memory");
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const int mine = (K + kRankCtas - 1) / kRankCtas;          // <= 64 filters of this CTA
+    int share = 1;                                             // threads of one warp per filter, a power of two
+    while (share < 32 && 2 * share * mine <= 256) share *= 2;
+    const int i = threadIdx.x / share, k = (int)blockIdx.x * mine + i, part = threadIdx.x & (share - 1);
+    const bool live = i < mine && k < K;
+    int before = 0;
+    if (live) {
+        const double sk = sh[k];
+        for (int j = part; j < K; j += share) before += (sh[j] < sk) || (sh[j] == sk && j < k);
+    }
+    for (int o = share >> 1; o >= 1; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (live && part == 0) { rank[k] = before; mask[k] = before >= q ? 1 : 0; }
+}
+
+// The same for all filter banks of a model at once, one warp per filter: (update and) score ...
+template <bool UPDATE>
+__global__ void bank_score_kernel(const SoftBank* __restrict__ banks, const int32_t* __restrict__ filter_bank, int total_filters,
+                                  const float* __restrict__ dw, int norm, double* __restrict__ scores) {
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (g >= total_filters) return;
+    const SoftBank& b = banks[filter_bank[g]];
+    const size_t first = (size_t)(g - b.k_off) * b.per;
+    const double s = score_filter<UPDATE>(b.w + first, UPDATE ? dw + b.dw_off + first : nullptr, b.per, norm, lane);
     if (lane == 0) scores[g] = s;
 }
 
-__global__ void soft_rank_kernel(const SoftBank* __restrict__ banks, const double* __restrict__ scores,
-                                 int32_t* __restrict__ rank, uint8_t* __restrict__ mask) {
-    extern __shared__ double sh[];
-    const SoftBank b = banks[blockIdx.x];
-    for (int i = threadIdx.x; i < b.K; i += blockDim.x) sh[i] = scores[b.k_off + i];
-    __syncthreads();
-    for (int k = threadIdx.x; k < b.K; k += blockDim.x) {
-        const double sk = sh[k];
-        int before = 0;
-        for (int j = 0; j < b.K; ++j) {
-            const double sj = sh[j];
-            before += (sj < sk) || (sj == sk && j < k);
-        }
-        rank[b.k_off + k] = before;
-        mask[b.k_off + k] = before >= b.q ? 1 : 0;
-    }
-}
-
-__global__ void soft_zeroize_kernel(const SoftBank* __restrict__ banks, const int32_t* __restrict__ filter_bank,
-                                    int total_filters, const uint8_t* __restrict__ mask) {
+// ... then rank, mask and, where asked, zeroize the masked filter in place.
+__global__ void bank_rank_kernel(const SoftBank* __restrict__ banks, const int32_t* __restrict__ filter_bank, int total_filters,
+                                 const double* __restrict__ scores, int zeroize, int32_t* __restrict__ rank, uint8_t* __restrict__ mask) {
     const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (g >= total_filters || mask[g]) return;
-    const SoftBank b = banks[filter_bank[g]];
-    float* f = b.w + (size_t)(g - b.k_off) * b.per;
-    for (int t = lane; t < b.per; t += 32) f[t] = 0.0f;
-}
-
-// Filters of one convolution in the order the MMA wants them: tap-major, then chunks of 8 input
-// channels, then the filter, then the channel within the chunk.  For a fixed tap and chunk the
-// K_pad x 8 block is a stack of 16-byte rows - the canonical K-major operand layout without swizzle.
-__global__ void repack_conv_kernel(const float* __restrict__ w, int C, int RS, const int32_t* __restrict__ row_src,
-                                   int K_pad, const int32_t* __restrict__ chan_src, int C_pad,
-                                   __nv_bfloat16* __restrict__ out_bf16, float* __restrict__ out_f32) {
-    const size_t total = (size_t)RS * C_pad * K_pad;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int e = (int)(i % 8);
-        size_t t = i / 8;
-        const int kr = (int)(t % K_pad); t /= K_pad;
-        const int chunk = (int)(t % (C_pad / 8));
-        const int rs = (int)(t / (C_pad / 8));
-        const int cp = chunk * 8 + e;
-        const int ks = row_src[kr], cs = chan_src[cp];
-        float v = 0.0f;
-        if (ks >= 0 && cs >= 0) v = w[((size_t)ks * C + cs) * RS + rs];
-        if (out_bf16) out_bf16[i] = __float2bfloat16_rn(v);
-        if (out_f32) out_f32[i] = v;
+    if (g >= total_filters) return;
+    const SoftBank& b = banks[filter_bank[g]];
+    const int before = rank_of(scores + b.k_off, b.K, g - b.k_off, lane);
+    if (lane == 0) { rank[g] = before; mask[g] = before >= b.q ? 1 : 0; }
+    if (zeroize && before < b.q) {
+        float* f = b.w + (size_t)(g - b.k_off) * b.per;
+        for (int t = lane; t < b.per; t += 32) f[t] = 0.0f;
     }
 }
 
-// Filters of a 3x3 convolution for a fused run of layers: for tap row r and channel chunk the operand is
-// a stack of 3*K_pad 16-byte rows; filter kr at horizontal tap s is row 48*(kr/16) + 16*s + kr%16.
-__global__ void repack_chain_kernel(const float* __restrict__ w, int C, const int32_t* __restrict__ row_src, int K_pad,
-                                    const int32_t* __restrict__ chan_src, int C_pad, __nv_bfloat16* __restrict__ out) {
-    const size_t total = (size_t)9 * C_pad * K_pad;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int e = (int)(i % 8);
-        size_t t = i / 8;
-        const int n = (int)(t % (3 * K_pad)); t /= 3 * K_pad;
-        const int chunk = (int)(t % (C_pad / 8));
-        const int r = (int)(t / (C_pad / 8));
-        const int kr = (n / 48) * 16 + n % 16, sx = (n % 48) / 16;
-        const int ks = row_src[kr], cs = chan_src[chunk * 8 + e];
-        float v = 0.0f;
-        if (ks >= 0 && cs >= 0) v = w[((size_t)ks * C + cs) * 9 + r * 3 + sx];
-        out[i] = __float2bfloat16_rn(v);
+// ---- everything a (re)planned graph reads besides activations, packed by ONE launch: a table of jobs, and for every block
+// the job it works for.  (One launch, one allocation and one upload per array made fp_prune of ResNet-50 take 25-45 ms.)
+__device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
+    uint4 o;
+    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    return o;
+}
+
+__device__ __forceinline__ void store8(const PackJob& j, size_t vec, const float (&v)[8]) {
+    if (j.f32) {
+        float4* o = reinterpret_cast<float4*>(j.out) + 2 * vec;
+        o[0] = make_float4(v[0], v[1], v[2], v[3]);
+        o[1] = make_float4(v[4], v[5], v[6], v[7]);
+    } else {
+        reinterpret_cast<uint4*>(j.out)[vec] = pack8(v);
     }
 }
 
-// Filters of a 7x7 first convolution in the order the packed network input wants them (see
-// input_to_stem_planar_kernel): a 3x1 convolution over 80 packed channels.  Tap dr (0..2 = offsets
-// -1,0,+1), chunk 0-2 (group E) take filter row r = 2*dr + 1, chunks 3-5 (O') take r = 2*dr at dr = 0, 1,
-// chunks 6-8 (O) take r = 2*dr + 2 at dr = 1, 2; packed channel j = s*C + c within a group; everything else
-// zero.  (Input row 2p+1 is held twice, as O of packed row p and as O' of row p+1; it is taken from row p,
-// because below the last image row there is only the zero border.)
-__global__ void repack_stem_kernel(const float* __restrict__ w, int C, const int32_t* __restrict__ row_src, int K_pad,
-                                   __nv_bfloat16* __restrict__ out) {
-    const size_t total = (size_t)3 * 10 * K_pad * 8;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int e = (int)(i % 8);
-        size_t t = i / 8;
-        const int kr = (int)(t % K_pad); t /= K_pad;
-        const int chunk = (int)(t % 10);
-        const int dr = (int)(t / 10);
-        float v = 0.0f;
-        const int ks = row_src[kr];
-        if (ks >= 0 && chunk < 9) {
-            const int group = chunk / 3;
-            const int j = (chunk % 3) * 8 + e;
-            const int sx = j / C, c = j - sx * C;
-            int r = -1;
-            if (group == 0) r = 2 * dr + 1;
-            else if (group == 1) { if (dr < 2) r = 2 * dr; }
-            else if (dr >= 1) r = 2 * dr + 2;
-            if (r >= 0 && sx < 7) v = w[(((size_t)ks * C + c) * 7 + r) * 7 + sx];
+// The filters of a convolution: unit = (filter row, chunk of 8 input channels), all taps of it - one thread reads
+// 8 * RS consecutive weights of a filter where no channel was removed, and neighbouring threads write neighbouring
+// 16-byte vectors.  Where the vector of (row k, chunk c, tap) goes is the kernels' affair:
+//   PACK_CONV   [filter tile][K group][tap][chunk in group][row in tile]: with one tile and one group the plain layout
+//               [tap][chunk][row], otherwise a block per pipeline stage / a contiguous part per filter tile (conv_tc.cu).
+//               Chunks >= chunks1 are the second bank's (a projection shortcut stacked along the channels).
+//   PACK_CHAIN  a fused run's layer: per tap row and chunk a stack of 3 * K_pad rows, row 48 * (k / 16) + 16 * s + k % 16
+//               for horizontal tap s (chain_tc.cu)
+__device__ __forceinline__ void pack_filters(const PackJob& j, const int32_t* __restrict__ idx, int u) {
+    const int c = u / j.rows, k = u - c * j.rows;
+    const bool second = c >= j.chunks1;
+    const float* __restrict__ w = second ? j.w2 : j.w;
+    const int C = second ? j.C2 : j.C, RS = j.RS;
+    const int ks = k < j.K_pad ? idx[(second ? j.row2 : j.row) + k] : -1;
+    const int32_t* chan = idx + (second ? j.chan2 + (c - j.chunks1) * 8 : j.chan + c * 8);
+    int cs[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) cs[e] = chan[e];
+    size_t base, step;
+    if (j.kind == PACK_CHAIN) {
+        base = (size_t)c * 3 * j.K_pad + 48 * (k >> 4) + (k & 15);
+        step = 0;
+    } else {
+        const int t = k / j.n_tile, row = k - t * j.n_tile;
+        const int g = c / j.cg, cgg = min(j.cg, j.chunks - g * j.cg);
+        base = (size_t)t * RS * j.chunks * j.n_tile + (size_t)g * RS * j.cg * j.n_tile + (size_t)(c - g * j.cg) * j.n_tile + row;
+        step = (size_t)cgg * j.n_tile;
+    }
+    const float* __restrict__ wk = w + (size_t)(ks < 0 ? 0 : ks) * C * RS;
+    for (int rs = 0; rs < RS; ++rs) {
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = ks >= 0 && cs[e] >= 0 ? __ldg(wk + (size_t)cs[e] * RS + rs) : 0.0f;
+        const size_t vec = j.kind == PACK_CHAIN ? base + (size_t)(rs / 3) * j.chunks * 3 * j.K_pad + 16 * (rs % 3) : base + rs * step;
+        store8(j, vec, v);
+    }
+}
+
+// A 7x7 first convolution in the order the packed network input wants it (see input_to_stem_planar_kernel): a 3x1
+// convolution over 80 packed channels.  Tap dr (0..2 = offsets -1,0,+1), chunk 0-2 (group E) take filter row
+// r = 2*dr + 1, chunks 3-5 (O') take r = 2*dr at dr = 0, 1, chunks 6-8 (O) take r = 2*dr + 2 at dr = 1, 2; packed channel
+// j = s*C + c within a group; everything else zero.  (Input row 2p+1 is held twice, as O of packed row p and as O' of row
+// p+1; it is taken from row p, because below the last image row there is only the zero border.)
+__device__ __forceinline__ void pack_stem_vec(const PackJob& j, const int32_t* __restrict__ idx, int u) {
+    const int k = u % j.K_pad, chunk = u / j.K_pad % 10, dr = u / j.K_pad / 10;
+    const int ks = idx[j.row + k];
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        v[e] = 0.0f;
+        if (ks < 0 || chunk >= 9) continue;
+        const int group = chunk / 3, q = (chunk % 3) * 8 + e;
+        const int sx = q / j.C, c = q - sx * j.C;
+        int r = -1;
+        if (group == 0) r = 2 * dr + 1;
+        else if (group == 1) { if (dr < 2) r = 2 * dr; }
+        else if (dr >= 1) r = 2 * dr + 2;
+        if (r >= 0 && sx < 7) v[e] = j.w[(((size_t)ks * j.C + c) * 7 + r) * 7 + sx];
+    }
+    store8(j, u, v);
+}
+
+// A 7x7 first convolution for the kernel that fuses it with the pooling: the 7x7 / stride-2 window over C channels as a
+// 4x4 window over the 4 C parity channels of the half-resolution input - tap (ta, tb), channel (2a + b) C + c takes
+// w[k][c][2 ta + a - 1][2 tb + b - 1] (zero where an index is -1) - as [tap][chunk of 8][filter][8].
+__device__ __forceinline__ void pack_stem_direct_vec(const PackJob& j, const int32_t* __restrict__ idx, int u) {
+    const int k = u % j.K_pad, chunk = u / j.K_pad % 2, tap = u / (2 * j.K_pad);
+    const int ta = tap >> 2, tb = tap & 3;
+    const int ks = idx[j.row + k];
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const int ch = chunk * 8 + e;
+        v[e] = 0.0f;
+        if (ks < 0 || ch >= 4 * j.C) continue;
+        const int par = ch / j.C, c = ch - par * j.C;
+        const int r = 2 * ta + (par >> 1) - 1, s = 2 * tb + (par & 1) - 1;
+        if (r >= 0 && s >= 0) v[e] = j.w[(((size_t)ks * j.C + c) * 7 + r) * 7 + s];
+    }
+    store8(j, u, v);
+}
+
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(const PackJob* __restrict__ jobs, const int32_t* __restrict__ block_job,
+                                                            const int32_t* __restrict__ idx) {
+    const PackJob& j = jobs[block_job[blockIdx.x]];
+    const int u = ((int)blockIdx.x - j.first_block) * kPackThreads + threadIdx.x;
+    if (u >= j.units) return;
+    switch (j.kind) {
+        case PACK_CONV:
+        case PACK_CHAIN: pack_filters(j, idx, u); break;
+        case PACK_STEM: pack_stem_vec(j, idx, u); break;
+        case PACK_STEM_DIRECT: pack_stem_direct_vec(j, idx, u); break;
+        case PACK_FC: {              // out[k][cp] = w[k][chan[cp]] * scale, fp32
+            const int chunks = j.chunks, k = u / chunks, c = u - k * chunks;
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int cs = idx[j.chan + c * 8 + e];
+                v[e] = cs >= 0 ? j.w[(size_t)k * j.C + cs] * j.scale : 0.0f;
+            }
+            store8(j, u, v);
+            break;
         }
-        out[i] = __float2bfloat16_rn(v);
-    }
-}
-
-// Filters of the first convolution for the kernel that fuses it with the pooling: the 7x7 / stride-2 window over C
-// channels as a 4x4 window over the 4 C parity channels of the half-resolution input - tap (ta, tb), channel
-// (2a + b) C + c takes w[k][c][2 ta + a - 1][2 tb + b - 1] (zero where an index is -1) - as [tap][chunk of 8][filter][8].
-__global__ void repack_stem_direct_kernel(const float* __restrict__ w, int C, const int32_t* __restrict__ row_src, int K_pad,
-                                          __nv_bfloat16* __restrict__ out) {
-    const int total = 16 * 2 * K_pad * 8;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int e = i % 8, kr = (i / 8) % K_pad, chunk = (i / (8 * K_pad)) % 2, tap = i / (16 * K_pad);
-        const int ch = chunk * 8 + e, ta = tap >> 2, tb = tap & 3;
-        float v = 0.0f;
-        const int ks = row_src[kr];
-        if (ks >= 0 && ch < 4 * C) {
-            const int par = ch / C, c = ch - par * C;
-            const int r = 2 * ta + (par >> 1) - 1, s = 2 * tb + (par & 1) - 1;
-            if (r >= 0 && s >= 0) v = w[(((size_t)ks * C + c) * 7 + r) * 7 + s];
+        default: {                   // PACK_BIAS: the kept filters' shifts, a taken-in projection's added
+            const int r1 = idx[j.row + u];
+            float b = r1 >= 0 ? j.w[r1] : 0.0f;
+            if (j.w2) { const int r2 = idx[j.row2 + u]; b += r2 >= 0 ? j.w2[r2] : 0.0f; }
+            reinterpret_cast<float*>(j.out)[u] = b;
         }
-        out[i] = __float2bfloat16_rn(v);
     }
-}
-
-__global__ void reblock_bank_kernel(const uint4* __restrict__ packed, int RS, int cchunks, int K_pad, int n_tile, int n_tiles,
-                                    int cg, uint4* __restrict__ blocked) {
-    const size_t total = (size_t)n_tiles * RS * cchunks * n_tile;          // 16-byte rows
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        // i = ((t * cchunks*RS ... decoded block by block: tile t, then group g (cgg chunks), tap, chunk, row
-        const size_t per_tile = (size_t)RS * cchunks * n_tile;
-        const int t = (int)(i / per_tile);
-        size_t r = i - (size_t)t * per_tile;
-        const size_t full_group = (size_t)RS * cg * n_tile;
-        const int g = (int)(r / full_group);
-        r -= (size_t)g * full_group;
-        int cgg = cchunks - g * cg;
-        if (cgg > cg) cgg = cg;
-        const int tap = (int)(r / ((size_t)cgg * n_tile));
-        r -= (size_t)tap * cgg * n_tile;
-        const int c = (int)(r / n_tile), row = (int)(r - (size_t)c * n_tile);
-        const int k = t * n_tile + row;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (k < K_pad) v = packed[((size_t)tap * cchunks + (g * cg + c)) * K_pad + k];
-        blocked[i] = v;
-    }
-}
-
-__global__ void repack_fc_kernel(const float* __restrict__ w, int C, int K, const int32_t* __restrict__ chan_src,
-                                 int C_pad, float scale, float* __restrict__ out) {
-    const size_t total = (size_t)K * C_pad;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int cp = (int)(i % C_pad);
-        const int k = (int)(i / C_pad);
-        const int cs = chan_src[cp];
-        out[i] = cs >= 0 ? w[(size_t)k * C + cs] * scale : 0.0f;
-    }
-}
-
-__global__ void pack_bias_kernel(const float* __restrict__ b, const int32_t* __restrict__ row_src, int K_pad,
-                                 float* __restrict__ out) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K_pad) return;
-    out[k] = row_src[k] >= 0 ? b[row_src[k]] : 0.0f;
 }
 
 static inline int blocks_for(size_t n, int threads) {
@@ -306,72 +348,41 @@ void launch_count_nonfinite(const float* p, size_t n, int* d_count, cudaStream_t
 }
 
 void launch_score_filters(const float* w, int K, int per_filter, int norm, double* scores, cudaStream_t st) {
-    const int warps_per_block = 8;
-    score_filters_kernel<<<(K + warps_per_block - 1) / warps_per_block, warps_per_block * 32, 0, st>>>(w, K, per_filter, norm, scores);
+    score_filters_kernel<<<(K + 7) / 8, 256, 0, st>>>(w, K, per_filter, norm, scores);
 }
 
-void launch_rank_mask(const double* scores, int K, int q, int32_t* rank, uint8_t* mask, cudaStream_t st) {
-    rank_mask_kernel<<<1, 256, (size_t)K * sizeof(double), st>>>(scores, K, q, rank, mask);
+void launch_score_rank(const float* w, int K, int per_filter, int norm, int q, double* scores, int32_t* rank, uint8_t* mask,
+                       cudaStream_t st) {
+    if (K <= kSmallRank && (long long)K * per_filter <= kSmallBank) {
+        score_rank_cluster_kernel<<<kRankCtas, 256, 0, st>>>(w, K, per_filter, norm, q, rank, mask);
+        return;
+    }
+    launch_score_filters(w, K, per_filter, norm, scores, st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((K + 7) / 8));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, rank_mask_kernel, (const double*)scores, K, q, rank, mask);
 }
 
-void launch_soft_update_score(const SoftBank* banks, const int32_t* filter_bank, int total_filters, const float* dw,
-                              int norm, double* scores, cudaStream_t st) {
-    const int warps_per_block = 8;
-    soft_update_score_kernel<<<(total_filters + warps_per_block - 1) / warps_per_block, warps_per_block * 32, 0, st>>>(
-        banks, filter_bank, total_filters, dw, norm, scores);
+void launch_bank_score(const SoftBank* banks, const int32_t* filter_bank, int total_filters, const float* dw, int norm,
+                       double* scores, cudaStream_t st) {
+    const int blocks = (total_filters + 7) / 8;
+    if (dw) bank_score_kernel<true><<<blocks, 256, 0, st>>>(banks, filter_bank, total_filters, dw, norm, scores);
+    else bank_score_kernel<false><<<blocks, 256, 0, st>>>(banks, filter_bank, total_filters, nullptr, norm, scores);
 }
-void launch_soft_rank(const SoftBank* banks, int n_banks, int max_K, const double* scores, int32_t* rank, uint8_t* mask,
-                      cudaStream_t st) {
-    soft_rank_kernel<<<n_banks, 256, (size_t)max_K * sizeof(double), st>>>(banks, scores, rank, mask);
-}
-void launch_soft_zeroize(const SoftBank* banks, const int32_t* filter_bank, int total_filters, const uint8_t* mask,
-                         cudaStream_t st) {
-    const int warps_per_block = 8;
-    soft_zeroize_kernel<<<(total_filters + warps_per_block - 1) / warps_per_block, warps_per_block * 32, 0, st>>>(
-        banks, filter_bank, total_filters, mask);
+void launch_bank_rank(const SoftBank* banks, const int32_t* filter_bank, int total_filters, const double* scores, int zeroize,
+                      int32_t* rank, uint8_t* mask, cudaStream_t st) {
+    bank_rank_kernel<<<(total_filters + 7) / 8, 256, 0, st>>>(banks, filter_bank, total_filters, scores, zeroize, rank, mask);
 }
 
-void launch_repack_conv(const float* w, int C, int RS, const int32_t* row_src, int K_pad, const int32_t* chan_src,
-                        int C_pad, __nv_bfloat16* out_bf16, float* out_f32, cudaStream_t st) {
-    const size_t n = (size_t)K_pad * RS * C_pad;
-    repack_conv_kernel<<<blocks_for(n, 256), 256, 0, st>>>(w, C, RS, row_src, K_pad, chan_src, C_pad, out_bf16, out_f32);
-}
-
-void launch_repack_chain(const float* w, int C, const int32_t* row_src, int K_pad, const int32_t* chan_src, int C_pad,
-                         __nv_bfloat16* out, cudaStream_t st) {
-    repack_chain_kernel<<<blocks_for((size_t)9 * C_pad * K_pad, 256), 256, 0, st>>>(w, C, row_src, K_pad, chan_src, C_pad, out);
-}
-
-void launch_repack_stem(const float* w, int C, const int32_t* row_src, int K_pad, __nv_bfloat16* out, cudaStream_t st) {
-    repack_stem_kernel<<<blocks_for((size_t)240 * K_pad, 256), 256, 0, st>>>(w, C, row_src, K_pad, out);
-}
-
-void launch_repack_stem_direct(const float* w, int C, const int32_t* row_src, int K_pad, __nv_bfloat16* out, cudaStream_t st) {
-    repack_stem_direct_kernel<<<blocks_for((size_t)256 * K_pad, 256), 256, 0, st>>>(w, C, row_src, K_pad, out);
-}
-
-void launch_reblock_bank(const __nv_bfloat16* packed, int RS, int cchunks, int K_pad, int n_tile, int n_tiles, int cg,
-                         __nv_bfloat16* blocked, cudaStream_t st) {
-    const size_t n = (size_t)n_tiles * RS * cchunks * n_tile;
-    reblock_bank_kernel<<<blocks_for(n, 256), 256, 0, st>>>((const uint4*)packed, RS, cchunks, K_pad, n_tile, n_tiles, cg, (uint4*)blocked);
-}
-
-void launch_repack_fc(const float* w, int C, int K, const int32_t* chan_src, int C_pad, float scale, float* out,
-                      cudaStream_t st) {
-    repack_fc_kernel<<<blocks_for((size_t)K * C_pad, 256), 256, 0, st>>>(w, C, K, chan_src, C_pad, scale, out);
-}
-
-__global__ void add_bias_kernel(const float* __restrict__ a, const float* __restrict__ b, int n, float* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = a[i] + b[i];
-}
-
-void launch_add_bias(const float* a, const float* b, int n, float* out, cudaStream_t st) {
-    add_bias_kernel<<<(n + 127) / 128, 128, 0, st>>>(a, b, n, out);
-}
-
-void launch_pack_bias(const float* b, const int32_t* row_src, int K_pad, float* out, cudaStream_t st) {
-    pack_bias_kernel<<<(K_pad + 127) / 128, 128, 0, st>>>(b, row_src, K_pad, out);
+void launch_pack(const PackJob* jobs, const int32_t* block_job, int n_blocks, const int32_t* idx, cudaStream_t st) {
+    if (n_blocks > 0) pack_kernel<<<n_blocks, kPackThreads, 0, st>>>(jobs, block_job, idx);
 }
 
 }  // namespace fp

@@ -1,9 +1,10 @@
 // fp_rank_filters_static: filter scoring + ranking + masking for one filter bank without any
-// device allocation.  The only intermediate the two kernels need - one fp64 score per filter -
-// lives in a fixed array that is part of the library image.
+// device allocation.  The only intermediate - one fp64 score per filter - lives in a fixed array
+// that is part of the library image.
 #include "../../include/fupruner.h"
 #include "fp_internal.h"
 
+#include <atomic>
 #include <mutex>
 
 namespace {
@@ -14,7 +15,7 @@ static __device__ __align__(256) double g_static_scores[FP_STATIC_RANK_MAX_FILTE
 
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_mutex;
-double* g_scores_ptr[kMaxDevices] = {};   // device address of g_static_scores, per device ordinal
+std::atomic<double*> g_scores_ptr[kMaxDevices];   // device address of g_static_scores, per device ordinal
 
 }  // namespace
 
@@ -31,26 +32,20 @@ extern "C" fp_status fp_rank_filters_static(const float* d_filters, int32_t K, i
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
         return fp_detail::set_error(FP_ERR_CUDA, "fp_rank_filters_static: cannot identify the current device");
-    double* scores = nullptr;
-    {
+    double* scores = g_scores_ptr[dev].load(std::memory_order_acquire);
+    if (!scores) {
         // One-time set-up per device, with that device current: in host code the array's name is only a
         // handle; the address a kernel can use has to be asked for.
         std::lock_guard<std::mutex> lock(g_setup_mutex);
-        if (!g_scores_ptr[dev]) {
-            double* p = nullptr;
-            cudaError_t e = cudaGetSymbolAddress((void**)&p, g_static_scores);
-            if (e != cudaSuccess || !p) {
-                cudaGetLastError();
-                return fp_detail::set_error(FP_ERR_CUDA, "fp_rank_filters_static: cudaGetSymbolAddress failed");
-            }
-            g_scores_ptr[dev] = p;
+        cudaError_t e = cudaGetSymbolAddress((void**)&scores, g_static_scores);
+        if (e != cudaSuccess || !scores) {
+            cudaGetLastError();
+            return fp_detail::set_error(FP_ERR_CUDA, "fp_rank_filters_static: cudaGetSymbolAddress failed");
         }
-        scores = g_scores_ptr[dev];
+        g_scores_ptr[dev].store(scores, std::memory_order_release);
     }
-    cudaStream_t st = (cudaStream_t)stream;
-    // Both kernels overwrite everything they later read (scores[0..K)), so nothing has to be cleared.
-    fp::launch_score_filters(d_filters, K, per_filter, norm, scores, st);
-    fp::launch_rank_mask(scores, K, q, d_rank, d_mask, st);
+    // Everything the kernels later read (scores[0..K)) is written first, so nothing has to be cleared.
+    fp::launch_score_rank(d_filters, K, per_filter, norm, q, scores, d_rank, d_mask, (cudaStream_t)stream);
     if (cudaGetLastError() != cudaSuccess) return fp_detail::set_error(FP_ERR_CUDA, "fp_rank_filters_static: kernel launch failed");
     return FP_OK;
 }

@@ -138,6 +138,12 @@ struct fp_handle_s {
     std::vector<Op> ops;
     std::vector<Chain> chains;             // re-derived by fp_prune
     std::vector<int> op_chain;             // operator -> chain number, -1 = launched on its own
+    // the whole network as one kernel (find_net): one placement per way of giving images to CTAs
+    int net_on = 0;
+    std::vector<fp::NetPlan> net_plans;
+    std::vector<const fp::NetLayer*> d_net_tables;
+    fp::NetSpec net_spec;
+    uint8_t* d_net_blob = nullptr;
     int input_fused = 0;                   // 1: the first fused run reads the network input directly (no layout conversion launch)
     // head
     int head_src = -1, n_classes = 0, fc_C = 0;
@@ -696,6 +702,11 @@ bool chain_candidate(fp_handle h, const FConv& f) {
 void find_chains(fp_handle h, const std::vector<std::vector<Use>>& uses) {
     h->chains.clear();
     h->op_chain.assign(h->ops.size(), -1);
+    if (h->net_on) {                            // one run from the input to the logits
+        for (size_t i = 1; i + 1 < h->ops.size(); ++i) h->op_chain[i] = 0;
+        h->input_fused = 1;
+        return;
+    }
     const int n_ops = (int)h->ops.size();
     int i = 0;
     while (i < n_ops) {
@@ -765,6 +776,53 @@ void find_chains(fp_handle h, const std::vector<std::vector<Use>>& uses) {
             h->input_fused = 1;
         }
     }
+}
+
+// Can the whole network run as one kernel (resident_net.cu)?  All operators between the input conversion and the head are
+// 3x3 / pad-1 convolutions on square images of 32, 16 or 8 pixels with at most 64 channels, each reading the one before it
+// and adding nothing but the tensor two layers back (as it is, or every second pixel of it behind a strided layer).
+void find_net(fp_handle h, const std::vector<std::vector<Use>>& uses) {
+    h->net_on = 0;
+    h->net_plans.clear();
+    h->d_net_tables.clear();
+    h->net_spec.layers.clear();
+    const int n_ops = (int)h->ops.size();
+    if (h->compute != FP_COMPUTE_BF16_TC || h->keep_outputs || n_ops < 3 || h->in_C > 8 || h->stem_packed || h->stem_fused || uses[0].size() != 1) return;
+    int off = 0;
+    for (int i = 1; i + 1 < n_ops; ++i) {
+        if (h->ops[i].kind != 0) return;
+        const FConv& f = h->convs[h->ops[i].idx];
+        const FConv* prev = i > 1 ? &h->convs[h->ops[i - 1].idx] : nullptr;
+        const Tensor &src = h->tensors[f.src], &out = h->tensors[f.out];
+        if (f.src != (prev ? prev->out : 0) || f.R != 3 || f.S != 3 || f.pad != 1 || f.scatter || f.proj >= 0 || f.absorbed ||
+            !fp::net_layer_supported(src.H, src.W, out.H, out.W, f.C_pad, f.K_rows, f.stride)) return;
+        if (f.res_mode) {
+            if (!prev || f.res_tid != prev->src || f.stride != 1) return;
+            const Tensor& r = h->tensors[f.res_tid];
+            if (f.res_mode == 1 && (f.res_tid == 0 || prev->stride != 1 || r.C_pad != out.C_pad)) return;
+            if (f.res_mode == 2 && (prev->stride != 2 || f.res_stride != 2)) return;
+        }
+        for (const Use& u : uses[f.out]) {
+            const bool next = u.how == 0 && u.op == i + 1, shortcut = u.how == 1 && u.op == i + 2;
+            if (!next && !shortcut) return;
+        }
+        fp::NetSpecLayer l;
+        memset(&l, 0, sizeof(l));
+        l.chunks = f.C_pad / 8; l.n8 = (f.K_rows + 7) / 8; l.stride = f.stride; l.relu = f.relu;
+        l.res_mode = f.res_mode; l.res_pad_lo = f.res_pad_lo; l.res_C = f.res_mode ? h->tensors[f.res_tid].C : 0;
+        l.Hin = src.H; l.Win = src.W;
+        l.blob_off = off; l.blob_bytes = fp::net_blob_bytes(l.chunks, l.n8);
+        off += (l.blob_bytes + 127) / 128 * 128;
+        h->net_spec.layers.push_back(l);
+    }
+    if (h->ops[n_ops - 1].kind != 2 || h->head_src != h->convs[h->ops[n_ops - 2].idx].out) return;
+    const int choices[][2] = {{1, 1}, {2, 1}, {1, 2}, {1, 4}};       // images per CTA, CTAs per image
+    for (const auto& c : choices) {
+        fp::NetPlan p;
+        if (fp::plan_net(h->net_spec, c[0], c[1], &p)) h->net_plans.push_back(p);
+        else if (h->net_plans.empty()) return;             // one image does not fit
+    }
+    h->net_on = 1;
 }
 
 // How a convolution reads a parity-split input tensor: 0 it cannot, 'A' 3x3 / stride 2 / pad 1 (nine taps over the four
@@ -1043,6 +1101,7 @@ fp_status replan(fp_handle h) {
             head_chan = add_idx(chan_src);
         }
     }
+    find_net(h, uses);
     find_chains(h, uses);
 
     // --- packed filters, biases, FC matrix: sizes and jobs, then one region, one upload and one launch ---
@@ -1104,6 +1163,20 @@ fp_status replan(fp_handle h) {
             wants.push_back({(void**)&f.d_bp, (size_t)f.K_pad * sizeof(float)});
             add_job(bias(f), (void**)&f.d_bp, 0);
         }
+        if (h->net_on) {
+            const std::vector<fp::NetSpecLayer>& ls = h->net_spec.layers;
+            wants.push_back({(void**)&h->d_net_blob, (size_t)ls.back().blob_off + ls.back().blob_bytes});
+            for (size_t l = 0; l < ls.size(); ++l) {
+                const FConv& f = h->convs[h->ops[l + 1].idx];
+                fp::PackJob j = filters(f, fp::PACK_CONV);
+                j.rows = j.K_pad = j.n_tile = ls[l].n8 * 8;
+                j.units = j.rows * j.chunks;
+                add_job(j, (void**)&h->d_net_blob, (size_t)ls[l].blob_off);
+                fp::PackJob b = bias(f);
+                b.units = j.rows;
+                add_job(b, (void**)&h->d_net_blob, (size_t)ls[l].blob_off + ls[l].blob_bytes - ls[l].n8 * 32);
+            }
+        }
         for (Chain& ch : h->chains) {
             wants.push_back({(void**)&ch.d_blob, ch.blob_bytes});
             for (size_t l = 0; l < ch.convs.size(); ++l) {
@@ -1134,7 +1207,9 @@ fp_status replan(fp_handle h) {
         int n_blocks = 0;
         for (fp::PackJob& j : jobs) { j.first_block = n_blocks; n_blocks += (j.units + fp::kPackThreads - 1) / fp::kPackThreads; }
         const size_t o_blocks = align256(jobs.size() * sizeof(fp::PackJob)), o_idx = o_blocks + align256((size_t)n_blocks * 4);
-        const size_t meta = o_idx + align256(idx.size() * 4 + 4);
+        size_t meta = o_idx + align256(idx.size() * 4 + 4);
+        std::vector<size_t> o_tables;
+        for (const fp::NetPlan& np : h->net_plans) { o_tables.push_back(meta); meta += align256(np.table.size() * sizeof(fp::NetLayer)); }
         TRY(region_reserve(h, h->meta_region, meta));
         TRY(pinned_reserve(h, meta));
         uint8_t *hm = (uint8_t*)h->pinned, *dm = (uint8_t*)h->meta_region.p;
@@ -1144,6 +1219,10 @@ fp_status replan(fp_handle h) {
             for (int b = 0; b < (jobs[k].units + fp::kPackThreads - 1) / fp::kPackThreads; ++b) *bj++ = (int32_t)k;
         memcpy(hm + o_idx, idx.data(), idx.size() * 4);
         h->d_idx = (const int32_t*)(dm + o_idx);
+        for (size_t k = 0; k < o_tables.size(); ++k) {
+            memcpy(hm + o_tables[k], h->net_plans[k].table.data(), h->net_plans[k].table.size() * sizeof(fp::NetLayer));
+            h->d_net_tables.push_back((const fp::NetLayer*)(dm + o_tables[k]));
+        }
         CK(cudaMemcpyAsync(dm, hm, meta, cudaMemcpyHostToDevice, st));
         fp::launch_pack((const fp::PackJob*)dm, (const int32_t*)(dm + o_blocks), n_blocks, h->d_idx, st);
         CK(cudaGetLastError());
@@ -1167,6 +1246,11 @@ fp_status replan(fp_handle h) {
         for (int i = 0; i < (int)h->ops.size(); ++i) {
             const Op& op = h->ops[i];
             int tid = -1;
+            if (h->net_on) {                                    // no tensor of the network exists in memory
+                if (op.kind == 0) h->tensors[h->convs[op.idx].out].d = nullptr;
+                else if (op.kind == 3) h->tensors[0].d = nullptr;
+                continue;
+            }
             if (op.kind == 0 && h->op_chain[i] >= 0) {
                 // a fused run is one kernel: only its last tensor exists in memory, and it must not share
                 // a buffer with the run's inputs, which other CTAs still read while the first ones finish
@@ -1208,7 +1292,7 @@ fp_status replan(fp_handle h) {
         std::vector<size_t> start(bufs.size());
         size_t total = 0;
         for (size_t b = 0; b < bufs.size(); ++b) { start[b] = total; total += align256(bufs[b].bytes); }
-        TRY(region_reserve(h, h->act_region, total));
+        TRY(region_reserve(h, h->act_region, total ? total : 256));
         CK(cudaMemsetAsync(h->act_region.p, 0, total, st));
         for (const auto& pl : placed)
             h->tensors[pl.first].d = (uint8_t*)h->act_region.p + start[pl.second] + (size_t)fp::kGuardVectors * vec_bytes;
@@ -1270,12 +1354,40 @@ fp_status need_plan(fp_handle h, const char* who) {
 // execution
 // ---------------------------------------------------------------------------------------
 
+// The network as one kernel, given to the CTAs the way that is cheapest for this batch: rounds over the GPU times the cost
+// of a round in units of one image per CTA (measured, ResNet-56: see the figures beside).
+void launch_network(fp_handle h, const void* d_input, int batch, float* d_logits, cudaStream_t st, int dump_layer = -1, void* dump = nullptr) {
+    int best = 0;
+    double best_cost = 0;
+    for (size_t k = 0; k < h->net_plans.size(); ++k) {
+        const fp::NetPlan& np = h->net_plans[k];
+        const int at_once = std::max(1, fp::sm_count() / np.cs);      // CTAs or clusters; the last round may carry one image each
+        const int full = batch / (at_once * np.G), rest = batch - full * at_once * np.G;
+        const double one = np.cs == 4 ? 0.55 : np.cs == 2 ? 0.7 : 1.0, two = 1.5;
+        const double cost = full * (np.G == 2 ? two : one) + (rest == 0 ? 0.0 : rest > at_once ? two : one);
+        if (k == 0 || cost < best_cost) { best = (int)k; best_cost = cost; }
+    }
+    const Tensor& last = h->tensors[h->head_src];
+    fp::NetArgs a;
+    memset(&a, 0, sizeof(a));
+    a.x = d_input; a.logits = d_logits; a.w = h->d_net_blob; a.fcw = h->d_fcw_packed; a.fcb = h->d_fcb;
+    a.N = batch; a.H = h->in_H; a.W = h->in_W; a.in_C = h->in_C; a.in_mode = h->in_dtype == FP_DTYPE_BF16 ? 2 : 1;
+    a.n_classes = h->n_classes; a.fc_pitch = last.C_pad; a.last_H = last.H; a.last_W = last.W;
+    a.last_chunks = h->net_spec.layers.back().n8;
+    a.dump_layer = dump_layer; a.dump = dump;
+    fp::launch_net(h->net_plans[best], a, h->d_net_tables[best], h->d_status, st);
+}
+
 // n0, n_count: the images an input conversion handles (the other operators always run the whole batch)
 void launch_op(fp_handle h, int op_index, const void* d_input, int batch, float* d_logits, cudaStream_t st, int n0 = 0,
                int n_count = -1) {
     if (n_count < 0) n_count = batch;
     const Op& op = h->ops[op_index];
     const int bf16 = h->act_is_bf16();
+    if (h->net_on) {                                    // one kernel, launched by the first convolution
+        if (op_index == 1) launch_network(h, d_input, batch, d_logits, st);
+        return;
+    }
     if (op.kind == 3 && (h->input_fused || h->stem_fused)) return;        // the first kernel reads the network input itself
     if (h->stem_fused && op_index == 2) return;         // pooled inside the first convolution's kernel
     if (h->stem_fused && op_index == 1) {
@@ -1755,7 +1867,7 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             n -= h->input_fused;
             n -= 2 * h->stem_fused;                                          // conversion, convolution and pooling are one
             for (const FConv& c : h->convs) n -= c.absorbed;                 // a projection inside the layer that adds it
-            *(int32_t*)h_out = n;
+            *(int32_t*)h_out = h->net_on ? 1 : n;
             return FP_OK;
         }
         case FP_Q_CONV_K_FUSED: TRY(need(4)); TRY(conv_of(&f)); *(int32_t*)h_out = f ? f->K : 0; return FP_OK;
@@ -1819,6 +1931,26 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             const Op& op = h->ops[index];
             const int tid = op.kind == 0 ? h->convs[op.idx].out : op.kind == 1 ? h->pools[op.idx].out : 0;
             const Tensor& t = h->tensors[tid];
+            if (h->net_on) {
+                // the last layer of every resolution can be read: the network runs again and writes that layer's output out
+                const FConv& f = h->convs[op.idx];
+                if (index + 2 < (int)h->ops.size() && h->convs[h->ops[index + 1].idx].stride == 1)
+                    return fail(FP_ERR_UNSUPPORTED, "fp_query: operator %d runs inside the network's kernel and its output never reaches memory "
+                                "(set keep_outputs to run every layer on its own)", index);
+                const size_t cnt = (size_t)h->last_batch * t.C * t.H * t.W, vecs = (size_t)(t.C_pad / 8) * h->last_batch * (t.H + 2) * (t.W + 2);
+                TRY(need(cnt * sizeof(float)));
+                CK(cudaDeviceSynchronize());
+                float* d_tmp;
+                TRY(dev_alloc_raw(h, (void**)&d_tmp, align256(cnt * sizeof(float)) + vecs * 16));
+                uint8_t* d_planar = (uint8_t*)d_tmp + align256(cnt * sizeof(float));
+                cudaMemsetAsync(d_planar, 0, vecs * 16, 0);
+                launch_network(h, h->last_input, h->last_batch, h->d_logits_stage, 0, index - 1, d_planar);
+                fp::launch_planar_to_nchw_f32(d_planar, 1, d_tmp, h->last_batch, t.H, t.W, t.C_pad, f.K_rows, 0, 0);
+                cudaError_t e = cudaMemcpy(h_out, d_tmp, cnt * sizeof(float), cudaMemcpyDeviceToHost);
+                dev_free(h, d_tmp);
+                if (e != cudaSuccess) return fail(FP_ERR_CUDA, "fp_query: copy failed: %s", cudaGetErrorString(e));
+                return FP_OK;
+            }
             if (!t.d) return fail(FP_ERR_UNSUPPORTED, "fp_query: operator %d runs inside another kernel (a fused run of layers, or the layer "
                                   "that adds this projection shortcut) and its output never reaches memory (set keep_outputs to run "
                                   "every layer on its own)", index);
@@ -1869,7 +2001,7 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
                 // an operator without a launch of its own (a layer inside a fused run, a layout conversion done by the
                 // first run) adds nothing to the prefix
                 const Op& op = h->ops[i];
-                const bool silent = (op.kind == 0 && h->op_chain[i] >= 0 && h->chains[h->op_chain[i]].first_op != i) ||
+                const bool silent = (h->net_on && i != 1) || (!h->net_on && op.kind == 0 && h->op_chain[i] >= 0 && h->chains[h->op_chain[i]].first_op != i) ||
                                     (op.kind == 3 && (h->input_fused || h->stem_fused)) || (h->stem_fused && i == 2) ||
                                     (op.kind == 0 && h->convs[op.idx].absorbed);
                 if (silent) { prefix[i] = i ? prefix[i - 1] : 0.f; continue; }

@@ -19,6 +19,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <vector>
+
 namespace fp {
 
 // Streaming multiprocessors of the current device (asked once per device; 148 on a B200).  Grids are sized from it.
@@ -193,6 +195,45 @@ struct StemPoolPlan { int valid, tiles, tmem_cols; unsigned smem_bytes; };
 bool stem_pool_supported(int C, int H, int W, int K_pad);
 int plan_stem_pool(const StemPoolArgs& a, StemPoolPlan* plan, char* err, size_t err_len);
 void launch_stem_pool(const StemPoolPlan& plan, const StemPoolArgs& a, int* d_status, cudaStream_t st);
+
+// A whole network of 3x3 convolutions on square images of 32, 16 or 8 pixels, from the NCHW input to the logits, as one
+// kernel (resident_net.cu).  How its layers are placed and split depends on how many images a CTA carries (G) or how many
+// CTAs share an image (cs): one plan per choice, the launch takes the cheapest for its batch.
+enum { NET_STRIP = 0, NET_TILE = 1, NET_STRIDED = 2 };
+constexpr int kNetUnits = 32;
+struct NetUnit { uint16_t a_vec, dst_vec; uint8_t n8, nt, row, x; };   // a warp's piece of a layer: where its input and output start (vectors),
+                                                 // first filter / 8, filters / 8, first output row and column
+struct NetLayer {             // one layer as the kernel reads it (offsets and strides in bytes; buffers relative to an image's memory)
+    int w_off, w_src, w_bytes, next;             // filters: place in shared memory, place in `w`, size; next: first layer to request behind this one
+    int requests, req_off, req_src, req_bytes;   // how many to request, the first one's w_off, w_src, w_bytes
+    int form, units, res_mode, zero_bytes;       // form | input channels / 16 << 8 | rows of a piece << 16 | width 8 << 24; clear that much of the output first
+    int in_off, out_off, w_addr, bias_addr;
+    int row_step, k_step, b_k, b_tap;            // input row, 16 input channels, filters of 16 channels, of a tap
+    int out_plane, out_pitch, out_slab, relu;
+    int a_chunk, a_px8, a_px, R;                 // a chunk, pixels 8-15 of a tile, a pixel of the input; output rows per CTA
+    int res_plane, res_pitch, res_pad_lo, res_C;
+    int res_off, W, n8, pad_;
+    NetUnit unit[kNetUnits];
+};
+struct NetSpecLayer { int chunks, n8, stride, relu, res_mode, res_pad_lo, res_C, Hin, Win, blob_off, blob_bytes; };
+struct NetSpec { std::vector<NetSpecLayer> layers; };
+struct NetPlan {
+    int G = 0, cs = 0, img_bytes = 0, act_bytes = 0, head_off = 0, last_off = 0, last_PV = 0, first_requests = 0;
+    unsigned smem_bytes = 0;
+    std::vector<NetLayer> table;
+};
+struct NetArgs {
+    const void* x;            // network input, N x in_C x H x W, NCHW; in_mode 1: fp32, 2: bf16
+    float* logits;
+    const void* w;            // blobs of all layers
+    const float *fcw, *fcb;   // FC matrix [class][fc_pitch] scaled by 1 / (H * W) of the last tensor; fcb may be nullptr
+    void* dump;               // diagnostic: planar-8 tensor with border that layer dump_layer's output is written to
+    int N, H, W, in_C, in_mode, n_classes, fc_pitch, last_H, last_W, last_chunks, dump_layer;
+};
+int net_blob_bytes(int chunks, int n8);
+bool net_layer_supported(int H, int W, int P, int Q, int C_pad, int K, int stride);
+bool plan_net(const NetSpec& spec, int G, int cs, NetPlan* plan);
+void launch_net(const NetPlan& plan, const NetArgs& a, const NetLayer* d_table, int* d_status, cudaStream_t st);
 
 // A run of stride-1 3x3 convolutions executed by one kernel with the activations in shared memory.
 constexpr int kChainMaxLayers = 40;

@@ -1,0 +1,885 @@
+// A whole CIFAR-shaped residual network - every 3x3 convolution, shortcut, the average pooling and the FC layer - as ONE
+// kernel: a CTA (or, for few images, a cluster of two or four CTAs that share an image by rows) carries its images from
+// the NCHW input to the logits with the activations in shared memory.  Only the input, the filters and the logits touch
+// global memory, and there is one launch.
+//
+//   Why mma.sync and not tcgen05 here.  These layers are 8 to 64 channels wide.  A tcgen05.mma of 128 positions x 16
+//   channels needs 39-59 cycles for its operand fetch whatever N <= 48 is, which at N = 16 is 560-840 FMA per cycle and SM,
+//   and its results come back through tensor memory about a thousand cycles after the issue; a run of such layers is bound
+//   by that round trip (chain_tc.cu: 2400 cycles per tile and layer, four tiles in flight).  mma.sync m16n8k16 runs at
+//   1018 FMA per cycle and SM with 20 cycles of latency (measured, 8 warps), takes filters in steps of 8 instead of 16,
+//   and leaves its results in the registers of the warp that finishes them.
+//
+//   Activations   planar-8: [chunk of 8 channels][row][pixel], one 16-byte vector per pixel and chunk, row pitch W + 1 (a
+//                 zero vector before every row is also the one behind the row above), a zero or halo row above and below:
+//                 ldmatrix takes eight pixels' vectors as they lie, at any row and column offset, without conflicts.
+//   GEMM view     M = 16 pixels (half an image row of 32, a row of 16, two rows of 8), N = 8 filters, K = 16 channels of one
+//                 tap.  Filters arrive as [tap][chunk][filter][8] by bulk copies, one or two layers ahead of their use.
+//   Two forms     width >= 16: a warp takes four rows of a column strip and 16 filters, keeps the filters of 16 input
+//                 channels (all nine taps) in registers and reads an input row's fragments once for the three output rows
+//                 they touch.  Width 8: a warp owns 1-2 pairs of rows and 8-32 filters and streams the filters'
+//                 fragments from shared memory, activations still read once for three taps.  A result's order of
+//                 summation depends on the layer alone, so it does not depend on the batch it was computed in.
+//   Clusters      an image's rows are split over the CTAs; a CTA also sends the first and last row of its result into its
+//                 neighbours' halo rows (st.async to distributed shared memory, counted on a barrier there).
+#include "fp_internal.h"
+#include "tc_common.cuh"
+
+#include <algorithm>
+#include <cstdio>
+#include <cstring>
+#include <type_traits>
+#include <vector>
+
+namespace fp {
+
+namespace {
+
+using namespace tc;
+
+constexpr int kWarps = 8;                       // computing warps per image
+constexpr int kThreads = 32 * kWarps;           // threads per image
+constexpr int kMaxG = 2;                        // images a CTA carries at a time, each by eight warps of its own
+struct NetGeom { int kc, n8, W, Win, R, stride, out_PV; };        // what a layer's split depends on
+constexpr int kRing = 4;                        // layers whose descriptor (and filters) can be on the way or in use
+
+struct NetCtrl {
+    uint64_t full[kRing];
+    uint64_t halo[2];                           // clusters: the neighbours' rows of an even / odd layer's result are here
+    NetLayer layer[kRing];
+    int done[kRing];                            // images that are through with a layer
+    int abort_flag;
+    int pad_[3];
+};
+static_assert(sizeof(NetLayer) % 16 == 0 && sizeof(NetCtrl) % 16 == 0, "bulk copies need 16-byte alignment");
+
+struct NetParams {
+    NetArgs a;
+    const NetLayer* table;
+    int G, cs, L, img_bytes, n_clusters;
+    int in_off, in_rows;                        // slab of the network input: rows per CTA
+    int head_off, last_off, last_PV, first_requests;
+    int* status;
+};
+
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void ldm2(uint32_t (&r)[2], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
+}
+__device__ __forceinline__ void ldm_filters(uint32_t (&r)[4], uint32_t addr) { ldm4(r, addr); }     // 16 filters
+__device__ __forceinline__ void ldm_filters(uint32_t (&r)[2], uint32_t addr) { ldm2(r, addr); }     // 8 filters
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ void sts128_zero(uint32_t addr) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0) : "memory");
+}
+__device__ __forceinline__ uint32_t remote(uint32_t addr, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// the same, counted in bytes on a barrier of the CTA it goes to
+__device__ __forceinline__ void st_async32(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_remote32(uint32_t addr, uint32_t v) { asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+// acc + the lower / upper bf16 of a pair: one instruction, one rounding
+__device__ __forceinline__ void add_pair(float& lo, float& hi, uint32_t v) {
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tadd.rn.f32.bf16 %0, l, %0;\n\tadd.rn.f32.bf16 %1, h, %1;\n\t}" : "+f"(lo), "+f"(hi) : "r"(v));
+}
+__device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+
+// ends a layer: all warps of an image in this CTA
+__device__ __forceinline__ void layer_sync(int slot) { asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(kThreads) : "memory"); }
+// all CTAs that share the image
+template <bool CLUSTER>
+__device__ __forceinline__ void image_sync(int slot) {
+    if (CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else layer_sync(slot);
+}
+
+// What a warp needs to know of a layer to finish a tile.
+struct Out {
+    uint32_t plane, pitch;  // bytes per output chunk plane and row
+    uint32_t slab;          // bytes of this CTA's rows of a plane: R * pitch
+    int relu;
+    uint32_t bias;          // address of the fp32 shifts
+    int R, rank, cs, res_mode;
+    uint32_t halo;          // clusters: barrier that this layer's rows for the neighbours are counted on
+    int turn;               // > 0: two images take turns on the tensor pipe; this image's barrier (the other's is 7 - turn)
+    uint32_t res;           // option A: address of the shortcut operand, its plane and row strides, first channel, channels
+    uint32_t res_plane, res_pitch;
+    int res_pad_lo, res_C;
+};
+
+// Finishes M tiles of NT x 8 filters: of tile m, accumulator rows 0-7 are this lane's word `dst` + m * step of the first
+// chunk, rows 8-15 lie `half` bytes further on.  The bias is already in the accumulator.  res_mode 1: the tensor two layers back
+// lies where the result goes - all of its words are read before the first result is written; 2: every second pixel of
+// it, channel k from k - pad_lo.  row: first output row, W8: a tile is two rows (else one), x: column of rows 0-7.
+template <bool CLUSTER, int M, int NT, bool W8>
+__device__ __forceinline__ void finish(const Out& o, float (&acc)[M][NT][4], int n8, uint32_t dst, uint32_t step, uint32_t half, int row, int x, int t) {
+    uint32_t v[M][NT][2];
+    if (o.res_mode) {
+        if (o.res_mode == 1) {
+#pragma unroll
+            for (int m = 0; m < M; ++m)
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh) v[m][j][hh] = lds32(dst + (uint32_t)m * step + (uint32_t)j * o.plane + hh * half);
+        } else {
+#pragma unroll
+            for (int m = 0; m < M; ++m)
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const int c0 = (n8 + j) * 8 + 2 * t - o.res_pad_lo, c1 = c0 + 1;
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh) {
+                        const int rr = W8 ? row + 2 * m + hh : row + m, xx = W8 ? x : x + 8 * hh;
+                        const uint32_t p = o.res + (uint32_t)(2 * rr + 1) * o.res_pitch + (uint32_t)(2 * xx + 1) * 16u;
+                        uint32_t lo = 0u, hi = 0u;
+                        if (c0 >= 0 && c0 < o.res_C) lo = lds32(p + (uint32_t)(c0 >> 3) * o.res_plane + (uint32_t)((c0 & 6) * 2)) >> (16 * (c0 & 1));
+                        if (c1 >= 0 && c1 < o.res_C) hi = lds32(p + (uint32_t)(c1 >> 3) * o.res_plane + (uint32_t)((c1 & 6) * 2)) >> (16 * (c1 & 1));
+                        v[m][j][hh] = (lo & 0xffffu) | (hi << 16);
+                    }
+                }
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) add_pair(acc[m][j][2 * hh], acc[m][j][2 * hh + 1], v[m][j][hh]);
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) v[m][j][hh] = pack_bf16x2_relu(acc[m][j][2 * hh], acc[m][j][2 * hh + 1]);
+    if (!o.relu) {
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) v[m][j][hh] = pack_bf16x2(acc[m][j][2 * hh], acc[m][j][2 * hh + 1]);
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) sts32(dst + (uint32_t)m * step + (uint32_t)j * o.plane + hh * half, v[m][j][hh]);
+    if (CLUSTER) {
+        // the neighbours' halo rows: our first row is row R of the CTA above, our last row is row -1 of the CTA below
+        const bool first = o.halo && row == 0 && o.rank > 0, last = o.halo && row + (W8 ? 2 * M : M) == o.R && o.rank + 1 < o.cs;
+        if (first) {
+            const uint32_t d = remote(dst + o.slab, o.rank - 1), bar = remote(o.halo, o.rank - 1);
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                st_async32(d + (uint32_t)j * o.plane, v[0][j][0], bar);
+                if (!W8) st_async32(d + (uint32_t)j * o.plane + half, v[0][j][1], bar);
+            }
+        }
+        if (last) {
+            const uint32_t d = remote(dst + (uint32_t)(M - 1) * step - o.slab, o.rank + 1), bar = remote(o.halo, o.rank + 1);
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                if (!W8) st_async32(d + (uint32_t)j * o.plane, v[M - 1][j][0], bar);
+                st_async32(d + (uint32_t)j * o.plane + half, v[M - 1][j][1], bar);
+            }
+        }
+    }
+}
+
+// Two images of a CTA, eight warps each, take strict turns: while one issues its MMAs, the other finishes its tile, ends its
+// layer and gets ready for the next.  (Left to themselves both went through the same phases at the same time, and the tensor
+// pipe stood still in the phases without MMAs: ResNet-56's first stage 8000 cycles a layer and pair of images.)  A turn is
+// given away a row of MMAs before its end, so that the other image's loads are on the way when the pipe falls free.
+template <bool CLUSTER>
+__device__ __forceinline__ void take_turn(const Out& o) {
+    if (!CLUSTER && o.turn) asm volatile("bar.sync %0, %1;" ::"r"(o.turn), "n"(2 * kThreads) : "memory");
+}
+template <bool CLUSTER>
+__device__ __forceinline__ void give_turn(const Out& o) {
+    if (!CLUSTER && o.turn) asm volatile("bar.arrive %0, %1;" ::"r"(7 - o.turn), "n"(2 * kThreads) : "memory");
+}
+
+__device__ __forceinline__ float2 lds_bias(uint32_t bias, int n8, int t) {
+    float2 b;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(b.x), "=f"(b.y) : "r"(bias + (uint32_t)(n8 * 8 + 2 * t) * 4u));
+    return b;
+}
+
+// RUN rows of a strip of 16 columns and NT x 8 filters (NT 1 or 2): per 16 input channels the nine taps' filters are read
+// into registers once, and every input row's fragments feed the up to three output rows they touch.  `a0`: this lane's
+// ldmatrix address of (input row `row` - 1, strip's first column), `b0`: of the filters, `dst`: its word of the first output row.
+template <bool CLUSTER, int RUN, int NT>
+__device__ __forceinline__ void conv_strip(const Out& o, uint32_t a0, uint32_t row_step, uint32_t k_step, int kc_n, uint32_t b0, uint32_t b_tap,
+                                           uint32_t b_k, int row, int x, int n8, uint32_t dst, int lane) {
+    const int t = lane & 3;
+    float acc[RUN][NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+        const float2 b = lds_bias(o.bias, n8 + j, t);
+#pragma unroll
+        for (int q = 0; q < RUN; ++q) { acc[q][j][0] = acc[q][j][2] = b.x; acc[q][j][1] = acc[q][j][3] = b.y; }
+    }
+#pragma unroll 1
+    for (int kc = 0; kc < kc_n; ++kc) {
+        uint32_t w[9][2 * NT];
+#pragma unroll
+        for (int i = 0; i < RUN + 2; ++i) {                    // input row `row` - 1 + i
+            uint32_t f[3][4];
+            if (i < 3) {
+#pragma unroll
+                for (int s = 0; s < 3; ++s) ldm_filters(w[3 * i + s], b0 + (uint32_t)(3 * i + s) * b_tap);
+            }
+#pragma unroll
+            for (int s = 0; s < 3; ++s) ldm4(f[s], a0 + (uint32_t)i * row_step + (uint32_t)s * 16u);
+            if (i == 0 && kc == 0) take_turn<CLUSTER>(o);
+            if (i == RUN + 1 && kc == kc_n - 1) give_turn<CLUSTER>(o);
+#pragma unroll
+            for (int s = 0; s < 3; ++s)
+#pragma unroll
+                for (int r = 0; r < 3; ++r)
+                    if (i - r >= 0 && i - r < RUN) {
+#pragma unroll
+                        for (int j = 0; j < NT; ++j)
+                            mma16816(acc[i - r][j], f[s][0], f[s][1], f[s][2], f[s][3], w[3 * r + s][2 * j], w[3 * r + s][2 * j + 1]);
+                    }
+        }
+        a0 += k_step;
+        b0 += b_k;
+    }
+    finish<CLUSTER, RUN, NT, false>(o, acc, n8, dst, o.pitch, 128u, row, x, t);
+}
+
+// Images 8 pixels wide: a tile of MT pairs of rows and NT x 8 filters, filters' fragments streamed.  `a0`: this lane's address of the tile's first input row (output row - 1), `b0`: of its filters.
+template <bool CLUSTER, int MT, int NT>
+__device__ __forceinline__ void conv_tile(const Out& o, uint32_t a0, uint32_t row_step, uint32_t k_step, int kc_n, uint32_t b0, uint32_t b_tap,
+                                          uint32_t b_k, int row, int n8, uint32_t dst, int lane) {
+    const int t = lane & 3;
+    float acc[MT][NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+        const float2 b = lds_bias(o.bias, n8 + j, t);
+#pragma unroll
+        for (int m = 0; m < MT; ++m) { acc[m][j][0] = acc[m][j][2] = b.x; acc[m][j][1] = acc[m][j][3] = b.y; }
+    }
+    constexpr int NF = MT + 1;                        // fragments that cover the tile's input rows
+    constexpr int NB = (NT + 1) / 2;
+    // nine (s, r) steps per 16 channels; a step's filters are fetched during the step before, a column's activations
+    // during the last row of the column before
+    uint32_t f[2][NF][4], b[2][NB][4];
+    auto load_f = [&](uint32_t (&d)[NF][4], uint32_t at) {
+#pragma unroll
+        for (int q = 0; q < NF; ++q) ldm4(d[q], at + (uint32_t)(2 * q) * row_step);
+    };
+    auto load_b = [&](uint32_t (&d)[NB][4], uint32_t at) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) ldm4(d[q], at + (uint32_t)q * 256u);
+    };
+    load_f(f[0], a0);
+    load_b(b[0], b0);
+    take_turn<CLUSTER>(o);
+    auto turn = [&](auto P, bool more) {              // one group of 16 channels; P: the buffer its first step reads (nine steps: it alternates)
+        constexpr int p = decltype(P)::value;
+#pragma unroll
+        for (int s = 0; s < 3; ++s)
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const int k = 3 * s + r;
+                uint32_t (&bc)[NB][4] = b[(k + p) & 1];
+                uint32_t (&fc)[NF][4] = f[(s + p) & 1];
+                if (k < 8) {
+                    const int ns = (k + 1) / 3, nr = (k + 1) % 3;
+                    load_b(b[(k + 1 + p) & 1], b0 + (uint32_t)(3 * nr + ns) * b_tap);
+                    if (r == 1 && s < 2) load_f(f[(s + 1 + p) & 1], a0 + (uint32_t)(s + 1) * 16u);
+                } else if (more) {
+                    load_b(b[(k + 1 + p) & 1], b0 + b_k);
+                }
+                if (k == 7 && more) load_f(f[(3 + p) & 1], a0 + k_step);
+                if (k == 7 && !more) give_turn<CLUSTER>(o);
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    uint32_t x[4];
+                    if (r == 1) {              // rows 2m+1 and 2m+2: the lower half of one fragment, the upper of the next
+                        x[0] = fc[m][1]; x[1] = fc[m + 1][0]; x[2] = fc[m][3]; x[3] = fc[m + 1][2];
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) x[e] = fc[m + r / 2][e];
+                    }
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) mma16816(acc[m][j], x[0], x[1], x[2], x[3], bc[j / 2][2 * (j & 1)], bc[j / 2][2 * (j & 1) + 1]);
+                }
+            }
+        a0 += k_step;
+        b0 += b_k;
+    };
+#pragma unroll 1
+    for (int kc = 0; kc < kc_n; kc += 2) {
+        turn(std::integral_constant<int, 0>(), kc + 1 < kc_n);
+        if (kc + 1 < kc_n) turn(std::integral_constant<int, 1>(), kc + 2 < kc_n);
+    }
+    finish<CLUSTER, MT, NT, true>(o, acc, n8, dst, 2u * o.pitch, o.pitch, row, lane >> 2, t);
+}
+
+// 16 output pixels of a stride-2 layer and NT x 8 filters.
+template <bool CLUSTER, int NT, bool W8>
+__device__ __forceinline__ void conv_strided(const Out& o, uint32_t a0, uint32_t row_step, uint32_t k_step, int kc_n, uint32_t b0,
+                                             uint32_t b_tap, uint32_t b_k, int row, int x, int n8, uint32_t dst, int lane) {
+    const int t = lane & 3;
+    float acc[1][NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+        const float2 b = lds_bias(o.bias, n8 + j, t);
+        acc[0][j][0] = acc[0][j][2] = b.x; acc[0][j][1] = acc[0][j][3] = b.y;
+    }
+    take_turn<CLUSTER>(o);
+#pragma unroll 1
+    for (int kc = 0; kc < kc_n; ++kc) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                uint32_t f[4], b[(NT + 1) / 2][4];
+                ldm4(f, a0 + (uint32_t)r * row_step + (uint32_t)s * 16u);
+#pragma unroll
+                for (int q = 0; q < (NT + 1) / 2; ++q) ldm4(b[q], b0 + (uint32_t)(3 * r + s) * b_tap + (uint32_t)q * 256u);
+#pragma unroll
+                for (int j = 0; j < NT; ++j) mma16816(acc[0][j], f[0], f[1], f[2], f[3], b[j / 2][2 * (j & 1)], b[j / 2][2 * (j & 1) + 1]);
+            }
+        a0 += k_step;
+        b0 += b_k;
+    }
+    give_turn<CLUSTER>(o);
+    finish<CLUSTER, 1, NT, W8>(o, acc, n8, dst, 0u, W8 ? o.pitch : 128u, row, x, t);
+}
+
+// One layer: the warp's units of work, one after the other.  Everything that does not depend on the lane was worked out by
+// the planner: a layer of one image is five thousand cycles, and a division or a chain of address arithmetic in front of
+// every unit was a tenth of that.
+template <bool CLUSTER>
+__device__ __forceinline__ void run_layer(const NetParams& p, const NetLayer& ly, int res_mode, int turn, uint32_t send, uint32_t wait, uint32_t wait_phase, volatile int* abort_flag,
+                                          int form, int units, uint32_t act0, uint32_t img0, int rank, int warp,
+                                          int lane) {
+    const int4 c0 = *reinterpret_cast<const int4*>(&ly.in_off), c1 = *reinterpret_cast<const int4*>(&ly.row_step);
+    const int4 c2 = *reinterpret_cast<const int4*>(&ly.out_plane), c3 = *reinterpret_cast<const int4*>(&ly.a_chunk);
+    Out o;
+    o.plane = (uint32_t)c2.x; o.pitch = (uint32_t)c2.y; o.slab = (uint32_t)c2.z; o.relu = c2.w;
+    o.bias = act0 + (uint32_t)c0.w;
+    o.R = c3.w; o.rank = rank; o.cs = p.cs; o.res_mode = res_mode; o.turn = turn; o.halo = send;
+    if (res_mode == 2) {
+        const int4 c4 = *reinterpret_cast<const int4*>(&ly.res_plane);
+        o.res = img0 + (uint32_t)ly.res_off;
+        o.res_plane = (uint32_t)c4.x; o.res_pitch = (uint32_t)c4.y; o.res_pad_lo = c4.z; o.res_C = c4.w;
+    }
+    const uint32_t row_step = (uint32_t)c1.x, k_step = (uint32_t)c1.y, b_k = (uint32_t)c1.z, b_tap = (uint32_t)c1.w;
+    const int kc = form >> 8 & 255, run_rows = form >> 16 & 255, w8 = form >> 24;
+    // ldmatrix addresses relative to a tile: activations - matrices (pixels 0-7 | 8-15) x (first | second chunk); filters -
+    // matrices (first | second chunk) x (filters 0-7 | 8-15)
+    const int mi = lane >> 3, mr = lane & 7;
+    const uint32_t a_lane = img0 + (uint32_t)c0.x + (uint32_t)((mi >> 1) * c3.x + (mi & 1) * c3.y + mr * c3.z);
+    const uint32_t b_lane = act0 + (uint32_t)c0.z + (mi & 1) * (b_k >> 1) + (uint32_t)((mi >> 1) * 128 + mr * 16);
+    const uint32_t d_lane = img0 + (uint32_t)c0.y + (uint32_t)((lane >> 2) * 16 + (lane & 3) * 4);
+    const int turns = (units + kWarps - 1) / kWarps;
+    for (int k = 0, u = warp; k < turns; ++k, u += kWarps) {
+        if (u >= units) {                        // nothing for this warp, but the turns go on
+            take_turn<CLUSTER>(o);
+            give_turn<CLUSTER>(o);
+            continue;
+        }
+        const uint2 un = *reinterpret_cast<const uint2*>(&ly.unit[u]);
+        const uint32_t a0 = a_lane + (un.x & 0xffffu) * 16u, dst = d_lane + (un.x >> 16) * 16u;
+        const int n8 = (int)(un.y & 255u), nt = (int)(un.y >> 8 & 255u), row = (int)(un.y >> 16 & 255u), x = (int)(un.y >> 24) + (lane >> 2);
+        const uint32_t b0 = b_lane + (uint32_t)n8 * 128u;
+        if (CLUSTER && wait && (row == 0 || row + run_rows == o.R) && !mbar_test_wait(wait, wait_phase)) mbar_wait(wait, wait_phase, abort_flag);
+        switch (form & 255) {
+            case NET_STRIP:
+#define FP_STRIP(RUN, NT) conv_strip<CLUSTER, RUN, NT>(o, a0, row_step, k_step, kc, b0, b_tap, b_k, row, x, n8, dst, lane)
+                if (run_rows == 4) { if (nt == 2) FP_STRIP(4, 2); else FP_STRIP(4, 1); }
+                else { if (nt == 2) FP_STRIP(2, 2); else FP_STRIP(2, 1); }
+#undef FP_STRIP
+                break;
+            case NET_TILE:
+#define FP_TILE(MT, NT) conv_tile<CLUSTER, MT, NT>(o, a0, row_step, k_step, kc, b0, b_tap, b_k, row, n8, dst, lane)
+                if (run_rows == 4) {
+                    switch (nt) { case 4: FP_TILE(2, 4); break; case 3: FP_TILE(2, 3); break; case 2: FP_TILE(2, 2); break; default: FP_TILE(2, 1); }
+                } else {
+                    switch (nt) { case 4: FP_TILE(1, 4); break; case 3: FP_TILE(1, 3); break; case 2: FP_TILE(1, 2); break; default: FP_TILE(1, 1); }
+                }
+#undef FP_TILE
+                break;
+            default:
+#define FP_STRIDED(NT, W8) conv_strided<CLUSTER, NT, W8>(o, a0, row_step, k_step, kc, b0, b_tap, b_k, row, x, n8, dst, lane)
+                    if (w8) { switch (nt) { case 4: FP_STRIDED(4, true); break; case 3: FP_STRIDED(3, true); break; case 2: FP_STRIDED(2, true); break; default: FP_STRIDED(1, true); } }
+                    else { switch (nt) { case 4: FP_STRIDED(4, false); break; case 3: FP_STRIDED(3, false); break; case 2: FP_STRIDED(2, false); break; default: FP_STRIDED(1, false); } }
+#undef FP_STRIDED
+        }
+    }
+}
+
+__device__ __forceinline__ void zero_bytes(uint32_t addr, int bytes, int tid) {
+    for (int i = tid; i < bytes / 16; i += kThreads) sts128_zero(addr + (uint32_t)i * 16u);
+}
+
+template <bool CLUSTER>
+__global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resident_net_kernel(const __grid_constant__ NetParams p) {
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    NetCtrl* ctrl = reinterpret_cast<NetCtrl*>(smem_raw);
+    const uint32_t ctrl_addr = smem_u32(smem_raw);
+    const uint32_t act0 = (ctrl_addr + (uint32_t)sizeof(NetCtrl) + 127u) & ~127u;
+    uint8_t* const act = smem_raw + (act0 - ctrl_addr);
+    volatile int* abort_flag = &ctrl->abort_flag;
+    // every image has eight warps and a memory of its own; the images of a CTA share the filters as they come in
+    const int slot = CLUSTER ? 0 : (int)threadIdx.x / kThreads, tid = (int)threadIdx.x - slot * kThreads, warp = tid >> 5, lane = tid & 31;
+    const uint32_t full0 = ctrl_addr + (uint32_t)offsetof(NetCtrl, full);
+    const int rank = CLUSTER ? (int)(blockIdx.x % (unsigned)p.cs) : 0;
+    const int cluster_id = CLUSTER ? (int)(blockIdx.x / (unsigned)p.cs) : (int)blockIdx.x;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kRing; ++s) { mbar_init(full0 + 8 * s, 1); ctrl->done[s] = 0; }
+        for (int s = 0; s < 2; ++s) mbar_init(ctrl_addr + (uint32_t)offsetof(NetCtrl, halo) + 8 * s, 1);
+        ctrl->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    const int L = p.L, H = p.a.H, W = p.a.W, dump_layer = p.a.dump_layer;
+    const uint32_t img0 = act0 + (uint32_t)(slot * p.img_bytes);
+    uint8_t* const img = act + slot * p.img_bytes;
+    uint32_t it = 0;                   // layers run so far, over all rounds
+    const uint32_t halo0 = ctrl_addr + (uint32_t)offsetof(NetCtrl, halo);
+    uint32_t sent = 0;                 // layers whose border rows went to the neighbours (all but a round's last)
+    const int neighbours = CLUSTER ? (rank > 0) + (rank + 1 < p.cs) : 0;
+    for (int n0 = cluster_id; n0 < p.a.N; n0 += p.n_clusters * p.G) {
+        const int n = n0 + slot * p.n_clusters;            // this image; the last round may have fewer
+        int active = 1;
+        for (int s = 1; s < p.G; ++s) active += n0 + s * p.n_clusters < p.a.N;
+        const uint32_t it0 = it;
+        const int turn = active > 1 ? 3 + slot : 0;
+        // Requests the descriptor and filters of layer `next` (one warp).  What other threads read or wrote in the place they
+        // go to lies behind the barrier just passed.
+        auto request = [&](int next, int off, int src, int bytes) {
+            const uint32_t ring = (it0 + (uint32_t)next) & (kRing - 1), bar = full0 + 8 * ring;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (lane == 0) {
+                mbar_expect_tx(bar, (uint32_t)bytes + (uint32_t)sizeof(NetLayer));
+                bulk_copy(ctrl_addr + (uint32_t)offsetof(NetCtrl, layer) + ring * (uint32_t)sizeof(NetLayer), p.table + next, (uint32_t)sizeof(NetLayer), bar);
+            }
+            __syncwarp();
+            for (int o = lane * 16384; o < bytes; o += 32 * 16384)
+                bulk_copy(act0 + (uint32_t)(off + o), reinterpret_cast<const uint8_t*>(p.a.w) + src + o, (uint32_t)min(16384, bytes - o), bar);
+        };
+        __syncthreads();               // the previous round is over
+        if (threadIdx.x < 32)
+            for (int k = 0; k < p.first_requests; ++k) {
+                const int4 q = __ldg(reinterpret_cast<const int4*>(p.table + k));
+                request(k, q.x, q.y, q.z);
+            }
+        if (n >= p.a.N) continue;
+        if (turn == 4 && it == 0) asm volatile("bar.arrive 3, %0;" ::"n"(2 * kThreads) : "memory");      // the first image begins
+        zero_bytes(img0, p.img_bytes, tid);
+        if (it == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+        image_sync<CLUSTER>(slot);
+        // ---- the network input: NCHW to the first chunk of the input buffer, halo rows included ----
+        {
+            const int rows = p.in_rows + 2, C = p.a.in_C;
+            for (int i = tid; i < rows * W; i += kThreads) {
+                const int w = i % W, rr = i / W, h = rank * p.in_rows + rr - 1;
+                if (h < 0 || h >= H) continue;
+                const size_t e0 = ((size_t)n * C * H + h) * W + w;
+                float v[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    v[c] = 0.0f;
+                    if (c < C) v[c] = p.a.in_mode == 1 ? __ldg(reinterpret_cast<const float*>(p.a.x) + e0 + (size_t)c * H * W)
+                                                      : __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p.a.x)[e0 + (size_t)c * H * W]);
+                }
+                uint4 q;
+                q.x = pack_bf16x2(v[0], v[1]); q.y = pack_bf16x2(v[2], v[3]); q.z = pack_bf16x2(v[4], v[5]); q.w = pack_bf16x2(v[6], v[7]);
+                *reinterpret_cast<uint4*>(img + p.in_off + ((size_t)rr * (W + 1) + w + 1) * 16) = q;
+            }
+        }
+        image_sync<CLUSTER>(slot);
+        // ---- layers ----
+        for (int l = 0; l < L; ++l, ++it) {
+            const uint32_t ring = it & (kRing - 1), bar = full0 + 8 * ring, parity = (it / kRing) & 1;
+            if (!mbar_test_wait(bar, parity) && !mbar_wait(bar, parity, abort_flag) && lane == 0) {
+                atomicExch(&ctrl->abort_flag, 1);
+                atomicExch(p.status, 21);
+            }
+            const NetLayer& ly = ctrl->layer[ring];
+            const int4 q = *reinterpret_cast<const int4*>(&ly.form);         // form, units, res_mode, zero_bytes
+            if (q.w) {                                 // another geometry moves in: its borders have to be zero
+                zero_bytes(img0 + (uint32_t)ly.out_off, q.w, tid);
+                image_sync<CLUSTER>(slot);
+            }
+            uint32_t send = 0, wait = 0, wait_phase = 0;
+            if (CLUSTER) {
+                // A layer's border rows are sent as they are finished and counted in bytes on one of two barriers in turn; the
+                // pieces of the next layer that touch the border wait for them.  (A neighbour that is a layer ahead writes
+                // into a buffer that nobody reads: its rows needed ours of the layer before.)
+                if (l > 0) { wait = halo0 + 8 * ((sent - 1) & 1); wait_phase = ((sent - 1) >> 1) & 1; }
+                if (l + 1 < L) {
+                    send = halo0 + 8 * (sent & 1);
+                    if (tid == 0) mbar_expect_tx(send, (uint32_t)(neighbours * ly.W * ly.n8 * 16));
+                    ++sent;
+                }
+            }
+            run_layer<CLUSTER>(p, ly, q.z, turn, send, wait, wait_phase, abort_flag, q.x, q.y, act0, img0, rank, warp, lane);
+            if (CLUSTER && l + 1 == L) image_sync<CLUSTER>(slot);          // (the head's sums may go where other CTAs still read)
+            else layer_sync(slot);
+            if (l == dump_layer) {                 // diagnostic: this layer's output as a planar-8 tensor with border
+                const int P2 = (ly.R * p.cs + 2) * (ly.W + 2), out_PV = ly.out_plane / 16;
+                uint4* y = reinterpret_cast<uint4*>(p.a.dump);
+                for (int i = tid; i < ly.n8 * ly.R * ly.W; i += kThreads) {
+                    const int w = i % ly.W, r = i / ly.W % ly.R, c = i / (ly.W * ly.R);
+                    y[(size_t)c * p.a.N * P2 + (size_t)n * P2 + (size_t)(rank * ly.R + r + 1) * (ly.W + 2) + w + 1] =
+                        *reinterpret_cast<const uint4*>(img + ly.out_off + ((size_t)c * out_PV + (size_t)(r + 1) * (ly.W + 1) + w + 1) * 16);
+                }
+                layer_sync(slot);
+            }
+            if (warp == (l & (kWarps - 1))) {          // the image that is through with the layer last makes the request
+                const int4 r = *reinterpret_cast<const int4*>(&ly.requests);         // layers to request; the first one's place, source and size
+                if (active > 1) {
+                    int last = 0;
+                    if (lane == 0) {
+                        __threadfence_block();
+                        last = atomicAdd(&ctrl->done[ring], 1) == active - 1;
+                        if (last) { ctrl->done[ring] = 0; __threadfence_block(); }
+                    }
+                    if (!__shfl_sync(0xffffffffu, last, 0)) continue;
+                }
+                const int next = ly.next;
+                for (int k = 0; k < r.x; ++k) {
+                    int4 e = make_int4(r.y, r.z, r.w, 0);
+                    if (k) e = __ldg(reinterpret_cast<const int4*>(p.table + next + k));
+                    request(next + k, e.x, e.y, e.z);
+                }
+            }
+        }
+        // ---- average pooling and FC: sums along the rows into the first CTA, then over rows, then the matrix ----
+        {
+            const int Wl = p.a.last_W, Rl = p.a.last_H / p.cs, C = p.a.last_chunks * 8;
+            const int head = p.head_off + slot * (p.a.last_H + 1) * C * 4;
+            float* rows = reinterpret_cast<float*>(act + head);
+            for (int i = tid; i < Rl * p.a.last_chunks; i += kThreads) {
+                const int c = i % p.a.last_chunks, r = i / p.a.last_chunks;
+                const uint4* v = reinterpret_cast<const uint4*>(img + p.last_off + ((size_t)c * p.last_PV + (size_t)(r + 1) * (Wl + 1) + 1) * 16);
+                float s[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) s[e] = 0.0f;
+                for (int w = 0; w < Wl; ++w) {
+                    const uint4 q = v[w];
+                    s[0] += bf_lo(q.x); s[1] += bf_hi(q.x); s[2] += bf_lo(q.y); s[3] += bf_hi(q.y);
+                    s[4] += bf_lo(q.z); s[5] += bf_hi(q.z); s[6] += bf_lo(q.w); s[7] += bf_hi(q.w);
+                }
+                uint32_t dst = act0 + (uint32_t)(head + ((rank * Rl + r) * C + c * 8) * 4);
+                if (CLUSTER) dst = remote(dst, 0);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    if (CLUSTER) st_remote32(dst + 4 * e, __float_as_uint(s[e]));
+                    else sts32(dst + 4 * e, __float_as_uint(s[e]));
+                }
+            }
+            image_sync<CLUSTER>(slot);
+            float* pooled = rows + p.a.last_H * C;
+            if (rank == 0)
+                for (int c = tid; c < C; c += kThreads) {
+                    float s = 0.0f;
+                    for (int r = 0; r < p.a.last_H; ++r) s += rows[r * C + c];
+                    pooled[c] = s;
+                }
+            image_sync<CLUSTER>(slot);                 // (and no CTA of a cluster leaves while others write to it)
+            if (rank == 0)
+                for (int k = warp; k < p.a.n_classes; k += kWarps) {
+                    float s = 0.0f;
+                    for (int c = lane; c < C; c += 32) s = fmaf(pooled[c], __ldg(p.a.fcw + (size_t)k * p.a.fc_pitch + c), s);
+#pragma unroll
+                    for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+                    if (lane == 0) p.a.logits[(size_t)n * p.a.n_classes + k] = s + (p.a.fcb ? p.a.fcb[k] : 0.0f);
+                }
+        }
+    }
+    if (*abort_flag) {
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);     // let copies in flight land before shared memory is released
+    }
+}
+
+constexpr int kSmemMax = 232448;                // opt-in dynamic shared memory per CTA
+
+int up(int v, int m) { return (v + m - 1) / m * m; }
+
+struct Span { int off, bytes, birth, death; };      // a piece of shared memory in use from layer `birth` to layer `death`
+
+// Form and split of one layer over the eight warps of an image (R: output rows of this CTA).
+bool split_layer(NetLayer* e, const NetGeom& q) {
+    const int kc = q.kc, n8 = q.n8, R = q.R, strips = q.W >= 16 ? q.W / 16 : 1;
+    double best = 0;
+    int form_ = 0, nt_ = 1, run_ = 1;
+    auto offer = [&](int form, int nt, int run) {
+        const int runs = (R + run - 1) / run, groups = (n8 + nt - 1) / nt, units = strips * runs * groups;
+        if (units > kNetUnits) return;
+        double tensor, shared;                              // cycles of a unit: one warp's MMAs, shared-memory reads
+        if (form == NET_STRIP) {
+            tensor = 9.0 * kc * nt * run * 8 + 150;
+            shared = kc * (18.0 * nt + 12.0 * (run + 2)) + 16;
+        } else if (form == NET_TILE) {
+            const int mt = run / 2;
+            tensor = 9.0 * kc * mt * nt * 8 + 150;
+            shared = 3.0 * kc * (4 * (mt + 1) + 3 * (nt == 1 ? 2 : 4 * ((nt + 1) / 2)));
+        } else {
+            tensor = 9.0 * kc * nt * 8 + 150;
+            shared = 9.0 * kc * (4 + 4 * ((nt + 1) / 2));
+        }
+        const int turns = (units + kWarps - 1) / kWarps;
+        // units of one scheduler; a warp alone on it leaves the tensor pipe waiting for its loads
+        const double busy = units >= kWarps ? 2.0 * turns : units > 4 ? 2.0 : 1.4;
+        const double cost = std::max(busy * tensor * (n8 / (double)(groups * nt)), units * shared);
+        if (best == 0 || cost < best * 0.999) { best = cost; form_ = form; nt_ = nt; run_ = run; }
+    };
+    if (q.stride == 2) {
+        for (int nt = std::min(4, n8); nt >= 1; --nt) offer(NET_STRIDED, nt, q.W == 8 ? 2 : 1);
+    } else if (q.W >= 16) {
+        for (int run : {4, 2})
+            for (int nt = std::min(2, n8); nt >= 1; --nt) if (R % run == 0) offer(NET_STRIP, nt, run);
+    } else {
+        for (int run : {4, 2})
+            for (int nt = std::min(4, n8); nt >= 1; --nt) if (R % run == 0) offer(NET_TILE, nt, run);
+    }
+    if (best == 0) return false;                            // more pieces than a layer's table holds
+    const int runs = (R + run_ - 1) / run_, groups = (n8 + nt_ - 1) / nt_;
+    e->form = form_ | kc << 8 | run_ << 16 | (q.W == 8 ? 1 : 0) << 24;
+    e->units = strips * runs * groups;
+    // filter groups outermost: a narrower last group then falls to the schedulers evenly
+    int u = 0;
+    for (int g = 0; g < groups; ++g)
+        for (int s = 0; s < strips; ++s)
+            for (int r = 0; r < runs; ++r, ++u) {
+                const int row = r * run_, x = 16 * s;
+                NetUnit& v = e->unit[u];
+                v.a_vec = (uint16_t)(row * q.stride * (q.Win + 1) + x * q.stride);
+                v.dst_vec = (uint16_t)(g * nt_ * q.out_PV + (row + 1) * (q.W + 1) + x + 1);
+                v.n8 = (uint8_t)(g * nt_); v.nt = (uint8_t)std::min(nt_, n8 - g * nt_);
+                v.row = (uint8_t)row; v.x = (uint8_t)x;
+            }
+    return true;
+}
+
+}  // namespace
+
+// A layer's filters and shifts as they travel: [tap][chunk][filter][8] bf16, then fp32 shifts.
+int net_blob_bytes(int chunks, int n8) { return 9 * chunks * n8 * 128 + n8 * 32; }
+
+bool net_layer_supported(int H, int W, int P, int Q, int C_pad, int K, int stride) {
+    if (H != W || P != Q || !(W == 8 || W == 16 || W == 32) || !(stride == 1 || stride == 2)) return false;
+    if (Q != W / stride || Q < 8) return false;
+    return C_pad % 16 == 0 && C_pad <= 64 && K >= 1 && K <= 64;
+}
+
+// Places the activations and every layer's filters in shared memory for groups of G images over cs CTAs.  Activations:
+// tensors live from the layer that writes them to the last that reads them, a result with an identity shortcut takes the
+// place of that operand; filters go where nothing is alive from the moment they are requested.  Returns false if it does
+// not fit.
+bool plan_net(const NetSpec& spec, int G, int cs, NetPlan* plan) {
+    const int L = (int)spec.layers.size();
+    plan->G = G; plan->cs = cs;
+    plan->table.assign(L, NetLayer());
+    plan->first_requests = 0;
+    struct Buf { int W, R, PV, chunks, birth, death, off; };
+    std::vector<Buf> bufs;
+    std::vector<int> buf_of(L + 1);                        // tensor (0 = network input, l + 1 = layer l's output) -> buffer
+    auto make = [&](int W, int H, int chunks, int birth) -> int {
+        if (H % cs) return -1;
+        Buf b;
+        b.W = W; b.R = H / cs; b.PV = (b.R + 2) * (W + 1) + 1; b.chunks = chunks; b.birth = birth; b.death = birth; b.off = -1;
+        bufs.push_back(b);
+        return (int)bufs.size() - 1;
+    };
+    if ((buf_of[0] = make(spec.layers[0].Win, spec.layers[0].Hin, spec.layers[0].chunks, -1)) < 0) return false;
+    for (int l = 0; l < L; ++l) {
+        const NetSpecLayer& s = spec.layers[l];
+        const int W = s.Win / s.stride, H = s.Hin / s.stride;
+        if (W == 8 && (H / cs) % 2) return false;          // an MMA's 16 pixels are two rows
+        if (s.res_mode == 1) buf_of[l + 1] = buf_of[l - 1];
+        else if ((buf_of[l + 1] = make(W, H, up(s.n8, 2), l)) < 0) return false;
+        Buf& in = bufs[buf_of[l]];
+        in.death = std::max(in.death, l);
+        if (s.res_mode) bufs[buf_of[l - 1]].death = std::max(bufs[buf_of[l - 1]].death, l);
+        bufs[buf_of[l + 1]].death = std::max(bufs[buf_of[l + 1]].death, l);
+    }
+    bufs[buf_of[L]].death = L;
+    // one chunk count per geometry, so that buffers of a stage can follow one another without clearing borders
+    for (Buf& b : bufs)
+        for (const Buf& o : bufs) if (o.W == b.W) b.chunks = std::max(b.chunks, o.chunks);
+    auto bytes_of = [](const Buf& b) { return b.chunks * b.PV * 16; };
+    // first fit, but for the stream of the first stage, which is kept clear of the room that the second stage's two tensors
+    // need: they are written while it is still read
+    int second = 0;
+    for (const Buf& b : bufs) if (b.W == bufs[0].W / 2) second = std::max(second, 2 * bytes_of(b));
+    int img_bytes = 0;
+    for (size_t i = 0; i < bufs.size(); ++i) {
+        int at = i == 1 ? std::max(bytes_of(bufs[0]), second) : 0;
+        for (bool moved = true; moved;) {
+            moved = false;
+            for (size_t j = 0; j < i; ++j)
+                if (bufs[j].birth <= bufs[i].death && bufs[j].death >= bufs[i].birth && at < bufs[j].off + bytes_of(bufs[j]) &&
+                    at + bytes_of(bufs[i]) > bufs[j].off) { at = bufs[j].off + bytes_of(bufs[j]); moved = true; }
+        }
+        bufs[i].off = at;
+        img_bytes = std::max(img_bytes, at + bytes_of(bufs[i]));
+    }
+    plan->img_bytes = img_bytes;
+    plan->act_bytes = G * img_bytes;
+    const int room = kSmemMax - (int)((sizeof(NetCtrl) + 127) & ~127u) - 128;
+    if (plan->act_bytes > room || G > kMaxG) return false;
+    std::vector<Span> spans;
+    for (const Buf& b : bufs)
+        for (int i = 0; i < G; ++i) spans.push_back({i * img_bytes + b.off, bytes_of(b), b.birth, b.death});
+    // the activations' memory is cleared while the first layers' filters already come in
+    spans.push_back({0, plan->act_bytes, -1, 0});
+    // where a piece can go so that it can be requested earliest (behind layer `after`, not before `floor`)
+    auto place = [&](int bytes, int birth_floor, int death, int* off, int* after) {
+        int best_after = 1 << 30, best_off = 0;
+        std::vector<int> cand(1, 0);
+        for (const Span& s : spans) cand.push_back(s.off + s.bytes);
+        cand.push_back(plan->act_bytes);
+        for (int c : cand) {
+            c = up(c, 128);
+            if (c + bytes > room) continue;
+            int a = birth_floor;
+            bool ok = true;
+            for (const Span& s : spans) {
+                if (c >= s.off + s.bytes || c + bytes <= s.off || s.birth > death) continue;
+                if (s.death >= death) { ok = false; break; }
+                a = std::max(a, s.death);
+            }
+            if (!ok) continue;
+            // nothing may move in between the request and the use
+            for (const Span& s : spans)
+                if (c < s.off + s.bytes && c + bytes > s.off && s.birth <= death && s.death > a) ok = false;
+            if (ok && a < best_after) { best_after = a; best_off = c; }
+        }
+        if (best_after >= death) return false;
+        *off = best_off; *after = best_after;
+        return true;
+    };
+    struct Format { int off, bytes, PV; };
+    std::vector<Format> formats;                            // what the borders in memory are zero for
+    int prev_after = -1;
+    for (int l = 0; l < L; ++l) {
+        const NetSpecLayer& s = spec.layers[l];
+        NetLayer& e = plan->table[l];
+        const Buf &in = bufs[buf_of[l]], &out = bufs[buf_of[l + 1]];
+        NetGeom q;
+        q.kc = s.chunks / 2; q.n8 = s.n8; q.stride = s.stride; q.W = out.W; q.Win = in.W; q.R = out.R; q.out_PV = out.PV;
+        if (!split_layer(&e, q)) return false;
+        e.in_off = in.off; e.out_off = out.off; e.R = out.R; e.W = out.W; e.n8 = s.n8; e.res_mode = s.res_mode;
+        e.row_step = (in.W + 1) * 16; e.k_step = 2 * in.PV * 16;
+        e.b_k = 2 * s.n8 * 128; e.b_tap = q.kc * e.b_k;
+        e.out_plane = out.PV * 16; e.out_pitch = (out.W + 1) * 16; e.out_slab = out.R * e.out_pitch; e.relu = s.relu;
+        e.a_chunk = in.PV * 16; e.a_px8 = out.W == 8 ? s.stride * e.row_step : 8 * s.stride * 16; e.a_px = s.stride * 16;
+        e.res_pad_lo = s.res_pad_lo; e.res_C = s.res_C;
+        if (s.res_mode) { const Buf& r = bufs[buf_of[l - 1]]; e.res_off = r.off; e.res_plane = r.PV * 16; e.res_pitch = (r.W + 1) * 16; }
+        if (bytes_of(out) / 16 > 65535 || bytes_of(in) / 16 > 65535) return false;
+        e.w_src = s.blob_off; e.w_bytes = s.blob_bytes;
+        int after;
+        // (a fragment load of an odd last group reaches 128 bytes behind the filters)
+        if (!place(s.blob_bytes + 128, std::max(-1, l - 3), l, &e.w_off, &after)) return false;
+        after = std::max(after, prev_after);                // requests are in order
+        if (after >= l) return false;
+        prev_after = after;
+        e.w_addr = e.w_off; e.bias_addr = e.w_off + s.blob_bytes - s.n8 * 32;
+        if (after < 0) ++plan->first_requests;
+        else {
+            NetLayer& f = plan->table[after];
+            if (f.requests++ == 0) { f.req_off = e.w_off; f.req_src = e.w_src; f.req_bytes = e.w_bytes; f.next = l; }
+        }
+        spans.push_back({e.w_off, s.blob_bytes + 128, after + 1, l});
+        // Borders: everything is cleared before the first layer; a buffer of another geometry than what its place held (or
+        // whose place held filters in between) is cleared by the layer that writes it first.
+        if (s.res_mode != 1) {
+            bool clean = l < 1;
+            for (const Format& f : formats) clean |= f.off == out.off && f.PV == out.PV && f.bytes == bytes_of(out);
+            if (!clean) e.zero_bytes = bytes_of(out);
+            std::vector<Format> left;
+            for (const Format& f : formats)
+                if (f.off + f.bytes <= out.off || out.off + bytes_of(out) <= f.off) left.push_back(f);
+            left.push_back({out.off, bytes_of(out), out.PV});
+            if (l == 0) left.push_back({in.off, bytes_of(in), in.PV});
+            formats = left;
+        }
+        // filters that went over an activation buffer's place unformat it
+        std::vector<Format> left;
+        for (const Format& f : formats) {
+            bool hit = false;
+            for (int i = 0; i < G; ++i)
+                hit |= e.w_off < i * img_bytes + f.off + f.bytes && e.w_off + s.blob_bytes + 128 > i * img_bytes + f.off;
+            if (!hit) left.push_back(f);
+        }
+        formats = left;
+    }
+    {   // the head's sums: rows, then pooled channels
+        const Buf& last = bufs[buf_of[L]];
+        const int H = last.R * cs, C = spec.layers[L - 1].n8 * 8;
+        int after;
+        if (!place(G * (H + 1) * C * 4, L - 2, L, &plan->head_off, &after)) return false;
+        plan->last_off = last.off; plan->last_PV = last.PV;
+    }
+    int top = plan->act_bytes;
+    for (const Span& s : spans) top = std::max(top, s.off + s.bytes);
+    top = std::max(top, plan->head_off + G * (bufs[buf_of[L]].R * cs + 1) * spec.layers[L - 1].n8 * 32);
+    plan->smem_bytes = (unsigned)(((sizeof(NetCtrl) + 127) & ~127u) + 128 + top);
+    for (bool cluster : {false, true}) {
+        const void* fn = cluster ? (const void*)resident_net_kernel<true> : (const void*)resident_net_kernel<false>;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) { cudaGetLastError(); return false; }
+    }
+    return true;
+}
+
+void launch_net(const NetPlan& plan, const NetArgs& a, const NetLayer* d_table, int* d_status, cudaStream_t st) {
+    NetParams p;
+    memset(&p, 0, sizeof(p));
+    p.a = a;
+    p.table = d_table;
+    p.G = plan.G; p.cs = plan.cs; p.L = (int)plan.table.size();
+    p.img_bytes = plan.img_bytes;
+    p.in_off = plan.table[0].in_off; p.in_rows = a.H / plan.cs;
+    p.head_off = plan.head_off; p.last_off = plan.last_off; p.last_PV = plan.last_PV; p.first_requests = plan.first_requests;
+    p.status = d_status;
+    int clusters = sm_count() / plan.cs;
+    if (clusters > a.N) clusters = a.N;
+    p.n_clusters = clusters;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(clusters * plan.cs));
+    cfg.blockDim = dim3((unsigned)(kThreads * plan.G));
+    cfg.dynamicSmemBytes = plan.smem_bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)plan.cs; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = plan.cs > 1 ? 2 : 1;
+    void* args[1] = {(void*)&p};
+    cudaLaunchKernelExC(&cfg, plan.cs > 1 ? (const void*)resident_net_kernel<true> : (const void*)resident_net_kernel<false>, args);
+}
+
+}  // namespace fp

@@ -34,7 +34,7 @@ def test_static_rank_sizes(B, K, per, norm):
     B.fp_rank_filters_static(bank, K, per, norm, q, rank, mask)
     torch.cuda.synchronize()
     scores = fpo.score_filters(w.reshape(K, per, 1, 1), norm)
-    want_rank, want_mask = fpo.rank_mask(scores, q)
+    want_mask, want_rank = fpo.rank_mask(scores, q)
     np.testing.assert_array_equal(rank.cpu().numpy(), want_rank)
     np.testing.assert_array_equal(mask.cpu().numpy(), want_mask)
 

@@ -1,0 +1,58 @@
+"""A whole CIFAR-shaped network as one kernel: every way of giving images to CTAs (four or two CTAs per image, one image per
+CTA, two images taking turns, several rounds), the layer shapes at which its pieces change, and what is left to the other
+kernels.  Against the oracle, and bit for bit between batch sizes: a result must not depend on how the batch was divided."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2010_16165_b200 import workloads as wl
+from test_gpu_parity import Gpu, err, oracle_pruned, TOL_BF16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2010_16165_b200 import binding
+    binding.lib()
+    return binding
+
+
+def test_batches_divided_every_way(B, fpo):
+    w = wl.tiny_cifar(widths=(16, 32, 64), in_hw=32, batch=7, n_per_stage=1, p=0.3)
+    gp, _, _, _ = oracle_pruned(fpo, w)
+    ref = fpo.fused_forward(gp, w.x)
+    g = Gpu(B, w, B.FP_COMPUTE_BF16_TC, max_batch=600)
+    try:
+        B.fp_prune(g.h, w.ratios)
+        assert B.fp_query_int(g.h, B.FP_Q_N_LAUNCHES) == 1
+        one = g.forward(w.x)
+        assert err(one, ref) < TOL_BF16
+        for n in (1, 2, 36, 37, 38, 74, 75, 147, 148, 149, 296, 297, 445, 600):
+            x = np.concatenate([w.x] * (n // 7 + 1))[:n]
+            np.testing.assert_array_equal(g.forward(x), np.concatenate([one] * (n // 7 + 1))[:n])
+        assert B.fp_query_int(g.h, B.FP_Q_DEVICE_STATUS) == 0
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("widths,hw", [((16, 32, 64), 32), ((8, 8, 8), 32), ((9, 17, 33), 32), ((7, 24, 40), 32), ((16, 48, 56), 32),
+                                       ((24, 64), 16), ((33, 50), 16), ((64,), 8), ((12,), 8)])
+@pytest.mark.parametrize("batch", [2, 90, 160])          # four CTAs per image, one image per CTA, two images per CTA
+def test_layer_shapes(B, fpo, widths, hw, batch):
+    net = wl.resnet_cifar(2, widths, in_hw=hw, n_classes=11, pad_lo_centered=True, name="resident_shapes")
+    w = wl.Workload("resident_shapes", net, 2, 31 + hw + sum(widths), True, wl.uniform_ratios(0.25), "uniform 0.25")
+    g = Gpu(B, w, B.FP_COMPUTE_BF16_TC, max_batch=batch)
+    try:
+        B.fp_prune(g.h, w.ratios)
+        x = np.concatenate([w.x] * (batch // 2))
+        got = g.forward(x)
+        gp, _, _, _ = oracle_pruned(fpo, w)
+        ref = fpo.fused_forward(gp, w.x)
+        assert err(got[:2], ref) < TOL_BF16
+        np.testing.assert_array_equal(got, np.concatenate([got[:2]] * (batch // 2)))
+    finally:
+        g.close()

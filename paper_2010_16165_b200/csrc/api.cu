@@ -170,6 +170,8 @@ struct fp_handle_s {
     cudaEvent_t copy_events[kHostPieces + 1] = {};
     double* d_scores = nullptr;            // fp_score
     std::map<GraphKey, cudaGraphExec_t> graphs;
+    struct KnownPlan { fp::ConvArgs geometry; fp::ConvPlanTC plan; };      // geometry: no pointers, padding zeroed
+    std::vector<KnownPlan> known_plans;
     const void* last_input = nullptr; int last_batch = 0;
     int soft_epochs = 0;                   // passes of fp_soft_prune_epoch since fp_fuse
     // selection over all banks at once (fp_prune, fp_soft_prune_epoch): bank table, filter -> bank map, scores, and ranks with
@@ -835,8 +837,8 @@ char split_reader(const FConv& f) {
     return 0;
 }
 
-// Which tensors are stored parity-split (tensor-core path): tensors written by a convolution of their own kernel, with
-// even height and width, that only stride-2 convolutions read - directly, or through 1x1 layers whose output is split
+// Which tensors are stored parity-split (tensor-core path): tensors written by a convolution of their own kernel that only
+// stride-2 convolutions read - directly, or through 1x1 layers whose output is split
 // in turn (the first 1x1 of a strided bottleneck block).  A stride-2 convolution over such a tensor is a stride-1
 // convolution over contiguous runs (bulk copies) instead of a gather.
 void decide_splits(fp_handle h, const std::vector<std::vector<Use>>& uses) {
@@ -846,7 +848,7 @@ void decide_splits(fp_handle h, const std::vector<std::vector<Use>>& uses) {
     std::vector<int> cand(nt, 0);
     for (int t = 1; t < nt; ++t) {
         const Tensor& T = h->tensors[t];
-        if (T.producer < 0 || h->ops[T.producer].kind != 0 || T.H % 2 || T.W % 2 || T.H < 2 || T.W < 2 || uses[t].empty()) continue;
+        if (T.producer < 0 || h->ops[T.producer].kind != 0 || T.H < 2 || T.W < 2 || uses[t].empty()) continue;
         const FConv& pf = h->convs[h->ops[T.producer].idx];
         if (pf.src == 0 && (pf.R == 7 || h->stem_packed)) continue;                    // the first convolution has forms of its own
         cand[t] = 1;
@@ -860,7 +862,10 @@ void decide_splits(fp_handle h, const std::vector<std::vector<Use>>& uses) {
                 if (u.how != 0 || h->ops[u.op].kind != 0) { ok = false; break; }
                 const FConv& f = h->convs[h->ops[u.op].idx];
                 const char kind = split_reader(f);
-                if (!kind || (kind == 'C' && !cand[f.out])) { ok = false; break; }
+                // (an odd height or width: the last row or column of the odd-parity images does not exist and has to stay
+                // zero, which a 1x1 layer over all four images would not leave it)
+                const Tensor& T = h->tensors[t];
+                if (!kind || (kind == 'C' && (!cand[f.out] || T.H % 2 || T.W % 2))) { ok = false; break; }
             }
             if (!ok) { cand[t] = 0; changed = true; }
         }
@@ -880,7 +885,7 @@ void conv_geometry(fp_handle h, const FConv& f, fp::ConvArgs* a) {
     }
     if (src.split) {
         const char kind = split_reader(f);
-        a->H = src.H / 2; a->W = src.W / 2; a->stride = 1;
+        a->H = (src.H + 1) / 2; a->W = (src.W + 1) / 2; a->stride = 1;
         if (kind == 'A') { a->x_s2d = 1; }
         else if (kind == 'B') { a->x_plane_mult = 4; }
         else { a->N = 4 * h->max_batch; a->P = out.H / 2; a->Q = out.W / 2; }        // 'C': 4 N half-size images in, the same out
@@ -1064,11 +1069,21 @@ fp_status replan(fp_handle h) {
                 memset(&ga, 0, sizeof(ga));
                 conv_geometry(h, f, &ga);
                 ga.C_pad = (h->stem_packed && f.src == 0) ? 80 : C_pad_total;
-                ga.K_pad = f.K_pad;
+                ga.K_pad = f.K_pad; ga.res_mode = f.res_mode;
                 ga.scatter = f.scatter; ga.out_C_pad = out.C_pad; ga.n_tile_forced = f.n_tile_forced;
                 char msg[256];
-                if (fp::plan_conv_tc(ga, &f.tc, msg, sizeof(msg)) != 0)
-                    return fail(FP_ERR_UNSUPPORTED, "convolution %d: %s", f.conv_index, msg);
+                // layers of the same geometry share a plan (a network has a third as many geometries as layers, and a plan
+                // is a search of some ten microseconds)
+                const fp_handle_s::KnownPlan* known = nullptr;
+                for (const auto& k : h->known_plans)
+                    if (!memcmp(&k.geometry, &ga, sizeof(ga))) { known = &k; break; }
+                if (known) f.tc = known->plan;
+                else {
+                    if (fp::plan_conv_tc(ga, &f.tc, msg, sizeof(msg)) != 0)
+                        return fail(FP_ERR_UNSUPPORTED, "convolution %d: %s", f.conv_index, msg);
+                    if (h->known_plans.size() >= 256) h->known_plans.clear();
+                    h->known_plans.push_back({ga, f.tc});
+                }
             }
             f.row_off = add_idx(row_src); f.chan_off = add_idx(chan_src);
             if (pj >= 0) { f.proj = pj; f.proj_kind = 1; h->convs[pj].absorbed = 1; }
@@ -1076,7 +1091,7 @@ fp_status replan(fp_handle h) {
             // resolution): the projection becomes extra K groups with a centre tap only, read from its own packed bank.
             if (pj < 0 && h->compute == FP_COMPUTE_BF16_TC && !h->keep_outputs && f.res_mode == 1 && f.R == 3 && f.S == 3 &&
                 f.stride == 1 && f.pad == 1 && !f.scatter && !src.split && !out.split && uses[f.res_tid].size() == 1 && f.tc.valid &&
-                f.tc.flat && !f.tc.b_resident && f.tc.blocked_bank == 0 && !(h->stem_packed && f.src == 0)) {
+                f.tc.flat && !f.tc.b_resident && (f.tc.blocked_bank == 0 || f.tc.split) && !(h->stem_packed && f.src == 0)) {
                 const Tensor& rt = h->tensors[f.res_tid];
                 if (rt.producer >= 0 && h->ops[rt.producer].kind == 0) {
                     const int cand = h->ops[rt.producer].idx;
@@ -1275,7 +1290,7 @@ fp_status replan(fp_handle h) {
             // planar-8 with border, plus guard vectors before and after (halo reads of the first/last tiles)
             t.bytes = ((size_t)(t.C_pad / 8) * h->max_batch * (t.H + 2) * (t.W + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
             if (t.split)
-                t.bytes = ((size_t)(t.C_pad / 8) * 4 * h->max_batch * (t.H / 2 + 2) * (t.W / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
+                t.bytes = ((size_t)(t.C_pad / 8) * 4 * h->max_batch * ((t.H + 1) / 2 + 2) * ((t.W + 1) / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
             if (tid == 0 && h->stem_packed)
                 t.bytes = ((size_t)10 * h->max_batch * (t.H / 2 + 2) * (t.W / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
             int best = -1;
@@ -1733,7 +1748,7 @@ extern "C" fp_status fp_debug_expire_wait(fp_handle h, void* stream) {
         const Op& op = h->ops[i];
         if (op.kind != 0 || h->op_chain[i] >= 0 || (h->stem_fused && i == 1)) continue;
         const FConv& f = h->convs[op.idx];
-        if (!f.tc.valid || !f.tc.flat || f.tc.blocked_bank || h->tensors[f.src].split || h->tensors[f.out].split || f.proj >= 0 || f.absorbed) continue;
+        if (!f.tc.valid || !f.tc.flat || (f.tc.blocked_bank && !f.tc.split) || h->tensors[f.src].split || h->tensors[f.out].split || f.proj >= 0 || f.absorbed) continue;
         // the first round of the activation producer is left out, so the MMA-issuing thread's wait for that stage runs
         // out after a millisecond (two million cycles), raises the status word and takes every role of the CTA with it
         fp::launch_conv_tc(f.tc, f.args, h->d_status, (cudaStream_t)stream, 0, 2000000LL);

@@ -1000,6 +1000,7 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
     const int sms = sm_count();
     if (a.C_pad % 16 || a.K_pad % 16) { snprintf(err, err_len, "channel counts must be padded to 16"); return 1; }
     if (a.W > kMaxWidth || a.Q > kMaxWidth) { snprintf(err, err_len, "images wider than %d are not supported", kMaxWidth); return 1; }
+    if (plan_conv_split(a, plan)) return 0;
     const int cchunks = a.C_pad / 8;
     const int taps = a.R * a.S;
     const int a_par = a.x_s2d ? 4 : 1;       // activation runs per chunk in a stage (parity images)
@@ -1236,6 +1237,7 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
 }
 
 void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cudaStream_t st, int skip_round, long long wait_cycles) {
+    if (plan.split > 0) { launch_conv_split(plan, a, d_status, st, skip_round, wait_cycles); return; }
     TcParams p;
     memset(&p, 0, sizeof(p));
     p.a = a;
@@ -1249,7 +1251,7 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.m_total = p.plane_out;
     p.plane_y = p.plane_out;
     if (a.y_split) {
-        p.y_split = 1; p.y_Wh2 = a.Q / 2 + 2; p.y_P2h = (a.P / 2 + 2) * p.y_Wh2;
+        p.y_split = 1; p.y_Wh2 = (a.Q + 1) / 2 + 2; p.y_P2h = ((a.P + 1) / 2 + 2) * p.y_Wh2;
         p.plane_y = 4ll * a.N * p.y_P2h;
     }
     p.a_par = a.x_s2d ? 4 : 1;

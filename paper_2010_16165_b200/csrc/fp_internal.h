@@ -154,6 +154,7 @@ void launch_conv_simt(const ConvArgs& a, int is_bf16, cudaStream_t st);
 // Tensor-core path: per-layer plan built once per fp_prune.
 struct ConvPlanTC {
     int valid;
+    int split;            // > 0: few positions - conv_split_kernel, the reduction over that many CTAs (conv_split.cu)
     int flat;             // 1: stride-1 "same" convolution, activation tiles fetched as contiguous runs
                           //    of flat positions (bulk copies); 0: gathered by loader threads
     int b_resident;       // flat only: the whole filter bank stays in shared memory
@@ -174,6 +175,9 @@ struct ConvPlanTC {
 };
 // Filters per CTA tile the plan would choose for K_pad filter rows of this geometry (used to lay out scattered banks).
 void conv_tc_filter_tile(const ConvArgs& a, int K_pad, int* n_tile, int* n_tiles);
+// The plan for few output positions, where it applies: false, and nothing changed, where it does not.
+bool plan_conv_split(const ConvArgs& a, ConvPlanTC* plan);
+void launch_conv_split(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cudaStream_t st, int skip_round, long long wait_cycles);
 // Returns 0 on success, otherwise writes a message.
 int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len);
 // skip_round / wait_cycles: diagnostic launch (see fp_debug_expire_wait): the activation producer of a stride-1 layer leaves

@@ -400,7 +400,7 @@ template <bool BF16>
 __global__ void planar_to_nchw_f32_kernel(const void* __restrict__ x, float* __restrict__ out, int N, int H, int W,
                                           int chunks, int C_out, int split) {
     // a parity-split tensor (see ConvArgs) is 4 N images of half the size
-    const int Wp = split ? W / 2 + 2 : W + 2, P2 = split ? (H / 2 + 2) * Wp : (H + 2) * Wp;
+    const int Wp = split ? (W + 1) / 2 + 2 : W + 2, P2 = split ? ((H + 1) / 2 + 2) * Wp : (H + 2) * Wp;
     const size_t plane = (size_t)N * P2 * (split ? 4 : 1);
     const size_t total = (size_t)N * chunks * H * W;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {

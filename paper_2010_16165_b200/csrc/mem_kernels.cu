@@ -4,6 +4,9 @@
 // 32 consecutive vectors of a chunk plane: 512 contiguous bytes of bf16.
 #include "fp_internal.h"
 
+#include <algorithm>
+#include <cstring>
+
 namespace fp {
 
 namespace {
@@ -304,95 +307,115 @@ __global__ void maxpool3s2_bf16_kernel(const Vec8h* __restrict__ x, Vec8h* __res
     }
 }
 
-// Head, step 1: spatial sum per channel in fp32.  One warp per (image, chunk of 8 channels): lanes
-// stride over the interior positions with 16-byte loads, shuffle-reduce, and write 8 sums.
+// Head, step 1: spatial sum per channel in fp32.  One warp per (image, chunk of 8 channels): lanes stride over the interior
+// positions with 16-byte loads, then the lanes' eight sums are added with nine shuffles - every exchange halves the channels
+// a lane still carries - instead of five per channel (ResNet-50 at batch 128, 32768 warps: the shuffles were half of 17 us).
+// (x here and sums below are the previous kernel's: not __restrict__, so that no load of them moves in front of the wait for it.)
 template <bool BF16>
-__global__ void pool_sum_kernel(const void* __restrict__ x, int N, int H, int W, int chunks, float* __restrict__ sums) {
+__global__ void pool_sum_kernel(const void* x, int N, int H, int W, int chunks, float* __restrict__ sums) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int Wp = W + 2, P2 = (H + 2) * Wp, HW = H * W;
     const size_t plane = (size_t)N * P2;
     const int lane = threadIdx.x & 31;
-    const size_t warp = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5;
-    if (warp >= (size_t)N * chunks) return;
-    const int j = (int)(warp % chunks);
-    const size_t n = warp / chunks;
+    const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (warp >= (unsigned)N * (unsigned)chunks) return;
+    const unsigned n = warp / (unsigned)chunks, j = warp - n * (unsigned)chunks;
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
     for (int i = lane; i < HW; i += 32) {
         const int h = i / W, w = i - h * W;
         float v[8];
-        load_vec8<BF16>(x, (size_t)j * plane + n * P2 + (size_t)(h + 1) * Wp + (w + 1), v);
+        load_vec8<BF16>(x, (size_t)j * plane + (size_t)n * P2 + (size_t)(h + 1) * Wp + (w + 1), v);
 #pragma unroll
         for (int e = 0; e < 8; ++e) acc[e] += v[e];
     }
+    int first = 0;                         // of the channels this lane still carries
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
+    for (int d = 16, keep = 4; d >= 4; d >>= 1, keep >>= 1) {
+        const bool up = (lane & d) != 0;   // keeps the upper half, hands the lower one over
 #pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], d);
+        for (int e = 0; e < 4; ++e)
+            if (e < keep) {
+                const float give = up ? acc[e] : acc[e + keep];
+                const float got = __shfl_xor_sync(0xffffffffu, give, d);
+                acc[e] = (up ? acc[e + keep] : acc[e]) + got;
+            }
+        if (up) first += keep;
     }
-    if (lane == 0) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) sums[n * (size_t)chunks * 8 + j * 8 + e] = acc[e];
-    }
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+    if ((lane & 3) == 0) sums[(size_t)n * chunks * 8 + j * 8 + first] = acc[0];
 }
 
-// Head, step 2: logits[n][k] = sum_c sums[n][c] * Wfc[k][c] + b[k]; the 1/(H*W) of the average is
-// already folded into Wfc.  A block handles IMG images x 32 classes, the channels in slabs of 512: the slab of
-// channel sums of its images sits in shared memory and every FC row it reads serves all of them (16 images per
-// block instead of 4 was measured and is slower at batch 64-256: fewer blocks, and L2 is not the bound).
-// A warp owns the classes k0 + warp + 8*t and walks their FC rows together: four independent row loads per
-// step.  Each (image, class) sum has a fixed order: lanes stride over the channels, then a butterfly over the lanes.
-constexpr int kFcClasses = 32, kFcSlab = 512;
-template <int IMG>
-__global__ void fc_kernel(const float* __restrict__ sums, int N, int C_pad, const float* __restrict__ fcw,
-                          const float* __restrict__ fcb, int n_classes, float* __restrict__ logits) {
-    extern __shared__ float sh[];          // IMG * kFcSlab
-    const int n0 = blockIdx.x * IMG, k0 = blockIdx.y * kFcClasses;
+// Head, step 2: logits[n][k] = sum_c sums[n][c] * Wfc[k][c] + b[k]; the 1/(H*W) of the average is already folded into Wfc.
+// A block handles IMAGES images (one, four or eight: the sums of images that do not exist would be computed as well), whose channel sums it holds in shared memory, and 8 * CPW classes: a warp walks the FC
+// rows of its CPW classes with 16-byte loads, all images a time.  The first rows are asked for before the channel sums
+// exist (programmatic dependent launch).  Each (image, class) sum has a fixed order: lanes stride over the channels, then a
+// butterfly.  CPW: every sum read from shared memory serves CPW classes, which bounds large batches (128 images x 1000 classes
+// x 2048 channels: 7 us of FMAs at full rate, four classes a warp bring the shared-memory reads down to that); one class a warp
+// spreads the FC matrix of a single image over 125 SMs instead of 32.
+constexpr int kFcWarps = 8, kFcSlab4 = 512;         // channels / 4 held at a time
+// AHEAD: places of the rows a lane has on the way at a time; a place is asked for again as soon as it has been used.
+template <int IMAGES, int CPW, int AHEAD>
+__global__ void __launch_bounds__(32 * kFcWarps, 2) fc_kernel(const float* sums, int N, int C_pad, const float* __restrict__ fcw,
+                                                           const float* __restrict__ fcb, int n_classes, float* __restrict__ logits) {
+    extern __shared__ float4 sh4[];        // IMAGES x kFcSlab4
+    const int n0 = blockIdx.x * IMAGES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int kWarps = 8, kPerWarp = kFcClasses / kWarps;       // launched with 256 threads
-    const float* wr[kPerWarp];
-    float acc[kPerWarp][IMG];
+    const int k0 = (blockIdx.y * kFcWarps + warp) * CPW, c4 = C_pad >> 2;
+    const float4* wr[CPW];
+    float4 w[CPW][AHEAD];
+    auto rows = [&](int c, int i) {        // 128 channels of the warp's rows, zeros behind the last
 #pragma unroll
-    for (int t = 0; t < kPerWarp; ++t) {
-        const int k = k0 + warp + kWarps * t;
-        wr[t] = fcw + (size_t)(k < n_classes ? k : 0) * C_pad;
+        for (int t = 0; t < CPW; ++t) w[t][i] = c < c4 ? __ldg(wr[t] + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    };
 #pragma unroll
-        for (int i = 0; i < IMG; ++i) acc[t][i] = 0.0f;
-    }
-    for (int c0 = 0; c0 < C_pad; c0 += kFcSlab) {
-        const int cw = C_pad - c0 < kFcSlab ? C_pad - c0 : kFcSlab;
-        __syncthreads();                   // the previous slab has been consumed
-        for (int img = warp; img < IMG; img += kWarps)
-            for (int cc = lane; cc < cw; cc += 32)
-                sh[img * kFcSlab + cc] = (n0 + img < N) ? sums[(size_t)(n0 + img) * C_pad + c0 + cc] : 0.0f;
+    for (int t = 0; t < CPW; ++t) wr[t] = reinterpret_cast<const float4*>(fcw + (size_t)min(k0 + t, n_classes - 1) * C_pad);
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i) rows(lane + 32 * i, i);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int images = min(IMAGES, N - n0);
+    float acc[CPW][IMAGES];
+#pragma unroll
+    for (int t = 0; t < CPW; ++t)
+#pragma unroll
+        for (int i = 0; i < IMAGES; ++i) acc[t][i] = 0.0f;
+    for (int slab = 0; slab < c4; slab += kFcSlab4) {
+        const int n4 = min(kFcSlab4, c4 - slab);
+        if (slab) __syncthreads();         // the previous slab has been consumed
+        for (int img = warp; img < IMAGES; img += kFcWarps) {
+            const float4* from = reinterpret_cast<const float4*>(sums + (size_t)(n0 + min(img, images - 1)) * C_pad) + slab;
+            for (int i = lane; i < n4; i += 32) sh4[img * kFcSlab4 + i] = from[i];
+        }
         __syncthreads();
-#pragma unroll 4
-        for (int c = lane; c < cw; c += 32) {      // unrolled: 16 row loads in flight per lane
-            float wv[kPerWarp];
+        for (int c = lane; c < n4; c += 32 * AHEAD) {                // (a slab that is not the last is a multiple of that)
 #pragma unroll
-            for (int t = 0; t < kPerWarp; ++t) wv[t] = wr[t][c0 + c];
+            for (int i = 0; i < AHEAD; ++i) {
+                const int cc = min(c + 32 * i, n4 - 1);
 #pragma unroll
-            for (int i = 0; i < IMG; ++i) {
-                const float sv = sh[i * kFcSlab + c];
+                for (int img = 0; img < IMAGES; ++img) {
+                    const float4 s = sh4[img * kFcSlab4 + cc];
 #pragma unroll
-                for (int t = 0; t < kPerWarp; ++t) acc[t][i] = fmaf(sv, wv[t], acc[t][i]);
+                    for (int t = 0; t < CPW; ++t)
+                        acc[t][img] = fmaf(s.w, w[t][i].w, fmaf(s.z, w[t][i].z, fmaf(s.y, w[t][i].y, fmaf(s.x, w[t][i].x, acc[t][img]))));
+                }
+                rows(slab + c + 32 * (AHEAD + i), i);
             }
         }
     }
 #pragma unroll
-    for (int t = 0; t < kPerWarp; ++t) {
-        const int k = k0 + warp + kWarps * t;
+    for (int t = 0; t < CPW; ++t) {
+        float mine = 0.0f;                 // lane i ends up with image i's sum
 #pragma unroll
-        for (int i = 0; i < IMG; ++i) {
+        for (int img = 0; img < IMAGES; ++img) {
+            float v = acc[t][img];
 #pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) acc[t][i] += __shfl_xor_sync(0xffffffffu, acc[t][i], d);
+            for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+            if (lane == img) mine = v;
         }
-        if (lane == 0 && k < n_classes) {
-            const float b = fcb ? fcb[k] : 0.0f;
-#pragma unroll
-            for (int i = 0; i < IMG; ++i)
-                if (n0 + i < N) logits[(size_t)(n0 + i) * n_classes + k] = acc[t][i] + b;
-        }
+        if (lane < images && k0 + t < n_classes) logits[(size_t)(n0 + lane) * n_classes + k0 + t] = mine + (fcb ? fcb[k0 + t] : 0.0f);
     }
 }
 
@@ -461,18 +484,34 @@ void launch_maxpool(const void* x, void* y, int is_bf16, int N, int H, int W, in
 
 void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, const float* fcw, const float* fcb,
                  int n_classes, float* logits, float* pool_scratch, cudaStream_t st) {
-    const size_t warps = (size_t)N * (C_pad / 8);
-    const int blocks = (int)((warps * 32 + 255) / 256);
-    if (is_bf16) pool_sum_kernel<true><<<blocks, 256, 0, st>>>(x, N, H, W, C_pad / 8, pool_scratch);
-    else pool_sum_kernel<false><<<blocks, 256, 0, st>>>(x, N, H, W, C_pad / 8, pool_scratch);
-    const int classes = (n_classes + kFcClasses - 1) / kFcClasses;
-    // Every block re-reads the FC rows of its classes: with many channels and images that traffic (through L2) is what
-    // bounds the kernel, so wide heads take 16 images per block (ResNet-50 at batch 128: 2048 channels, 8 MB of FC
-    // weights read 8 times instead of 32); narrow ones keep 4, where more blocks matter more.
-    if (C_pad >= 1024 && N >= 64)
-        fc_kernel<16><<<dim3((N + 15) / 16, classes), 256, 16 * kFcSlab * sizeof(float), st>>>(pool_scratch, N, C_pad, fcw, fcb, n_classes, logits);
-    else
-        fc_kernel<4><<<dim3((N + 3) / 4, classes), 256, 4 * kFcSlab * sizeof(float), st>>>(pool_scratch, N, C_pad, fcw, fcb, n_classes, logits);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.stream = st;
+    cfg.blockDim = dim3(256);
+    cfg.gridDim = dim3((unsigned)(((size_t)N * (C_pad / 8) * 32 + 255) / 256));
+    const int chunks = C_pad / 8;
+    cudaLaunchKernelEx(&cfg, is_bf16 ? pool_sum_kernel<true> : pool_sum_kernel<false>, x, N, H, W, chunks, pool_scratch);
+    // classes per warp: one while that is what fills the GPU, four once there are blocks enough
+    typedef void (*Fc)(const float*, int, int, const float*, const float*, int, float*);
+    const int images = N == 1 ? 1 : N <= 4 ? 4 : 8, groups = (N + images - 1) / images;
+    const int cpw = images < 8 ? 1 : groups * ((n_classes + 31) / 32) >= 2 * sm_count() ? 4 : groups * ((n_classes + 15) / 16) >= sm_count() ? 2 : 1;
+    const Fc fn = cpw == 4 ? (Fc)fc_kernel<8, 4, 2> : cpw == 2 ? (Fc)fc_kernel<8, 2, 4> : images == 8 ? (Fc)fc_kernel<8, 1, 8>
+                : images == 4 ? (Fc)fc_kernel<4, 1, 8> : (Fc)fc_kernel<1, 1, 16>;
+    cfg.gridDim = dim3((unsigned)groups, (unsigned)((n_classes + kFcWarps * cpw - 1) / (kFcWarps * cpw)));
+    cfg.dynamicSmemBytes = (size_t)images * kFcSlab4 * sizeof(float4);
+    static bool raised[64];                // per device, once
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !raised[dev]) {
+        for (Fc f : {(Fc)fc_kernel<8, 1, 8>, (Fc)fc_kernel<8, 2, 4>, (Fc)fc_kernel<8, 4, 2>})
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * kFcSlab4 * sizeof(float4)));
+        if (dev >= 0 && dev < 64) raised[dev] = true;
+    }
+    cudaLaunchKernelEx(&cfg, fn, (const float*)pool_scratch, N, C_pad, fcw, fcb, n_classes, logits);
 }
 
 void launch_planar_to_nchw_f32(const void* x, int is_bf16, float* out, int N, int H, int W, int C_pad, int C_out,

@@ -1,0 +1,42 @@
+"""GPU parity of the average pooling and FC layer: batches at the edges of the image groups (1, 4, 8), classes per warp (1, 2,
+4), channels around the 2048 held at a time, image sizes below and above a warp of positions."""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2010_16165_b200 import workloads as wl
+from test_gpu_parity import Gpu, TOL_BF16, TOL_FP32, err, oracle_pruned
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2010_16165_b200 import binding
+    binding.lib()
+    return binding
+
+
+def one_layer(batch, hw, channels, classes):
+    net = wl.Net(3, hw, hw, "one_layer")
+    x = net.relu(net.bn(net.conv(-1, channels, 3, 1, 1, 0), channels))
+    net.fc(net.gavgpool(x, channels), classes, channels)
+    net.n_blocks = 0
+    return wl.Workload("one_layer", net, batch, 29, False, wl.uniform_ratios(0.0), "none")
+
+
+@pytest.mark.parametrize("batch, hw, channels, classes", [
+    (1, 7, 2048, 1000), (1, 4, 2064, 11), (2, 9, 72, 1003), (4, 3, 4112, 9), (5, 7, 512, 1000), (8, 2, 24, 1),
+    (9, 7, 2032, 130), (24, 5, 136, 1000), (83, 3, 520, 1000), (97, 3, 2080, 801),
+])
+@pytest.mark.parametrize("compute", ["fp32", "tc"])
+def test_head_matches_oracle(B, fpo, batch, hw, channels, classes, compute):
+    w = one_layer(batch, hw, channels, classes)
+    g = Gpu(B, w, B.FP_COMPUTE_FP32 if compute == "fp32" else B.FP_COMPUTE_BF16_TC)
+    try:
+        gp, _, _, _ = oracle_pruned(fpo, w)
+        assert err(g.forward(w.x), fpo.fused_forward(gp, w.x)) < (TOL_FP32 if compute == "fp32" else TOL_BF16)
+    finally:
+        g.close()

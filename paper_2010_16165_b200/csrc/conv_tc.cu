@@ -86,7 +86,7 @@ struct TcParams {
 // descriptors differ only in their low words: one address unit is one 16-byte row, so a tap's
 // activation operand is `a_lo + r*Wp + s` and a K step advances both operands by two planes.
 template <int R, int S, int KSTEPS>
-__device__ __forceinline__ void issue_flat_resident(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t Wp,
+__device__ __forceinline__ void issue_flat_resident(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t Wp,
                                                     uint32_t a_ks, uint32_t b_ks, uint32_t b_tap, uint32_t idesc,
                                                     uint32_t accumulate) {
 #pragma unroll
@@ -95,7 +95,7 @@ __device__ __forceinline__ void issue_flat_resident(uint32_t d_tmem, uint32_t a_
         for (int sx = 0; sx < S; ++sx) {
 #pragma unroll
             for (int ks = 0; ks < KSTEPS; ++ks) {
-                umma_bf16_lo(d_tmem, a_lo + (uint32_t)r * Wp + (uint32_t)sx + (uint32_t)ks * a_ks,
+                umma_bf16_lo_if(leader, d_tmem, a_lo + (uint32_t)r * Wp + (uint32_t)sx + (uint32_t)ks * a_ks,
                              b_lo + (uint32_t)(r * S + sx) * b_tap + (uint32_t)ks * b_ks, idesc,
                              (r | sx | ks) ? 1u : accumulate);
             }
@@ -104,31 +104,31 @@ __device__ __forceinline__ void issue_flat_resident(uint32_t d_tmem, uint32_t a_
 }
 
 template <int R, int S>
-__device__ __forceinline__ void issue_flat_resident_k(int ksteps, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo,
+__device__ __forceinline__ void issue_flat_resident_k(uint32_t leader, int ksteps, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo,
                                                       uint32_t Wp, uint32_t a_ks, uint32_t b_ks, uint32_t b_tap,
                                                       uint32_t idesc, uint32_t accumulate) {
     switch (ksteps) {
-        case 1: issue_flat_resident<R, S, 1>(d_tmem, a_lo, b_lo, Wp, a_ks, b_ks, b_tap, idesc, accumulate); break;
-        case 2: issue_flat_resident<R, S, 2>(d_tmem, a_lo, b_lo, Wp, a_ks, b_ks, b_tap, idesc, accumulate); break;
-        case 3: issue_flat_resident<R, S, 3>(d_tmem, a_lo, b_lo, Wp, a_ks, b_ks, b_tap, idesc, accumulate); break;
-        default: issue_flat_resident<R, S, 4>(d_tmem, a_lo, b_lo, Wp, a_ks, b_ks, b_tap, idesc, accumulate); break;
+        case 1: issue_flat_resident<R, S, 1>(leader, d_tmem, a_lo, b_lo, Wp, a_ks, b_ks, b_tap, idesc, accumulate); break;
+        case 2: issue_flat_resident<R, S, 2>(leader, d_tmem, a_lo, b_lo, Wp, a_ks, b_ks, b_tap, idesc, accumulate); break;
+        case 3: issue_flat_resident<R, S, 3>(leader, d_tmem, a_lo, b_lo, Wp, a_ks, b_ks, b_tap, idesc, accumulate); break;
+        default: issue_flat_resident<R, S, 4>(leader, d_tmem, a_lo, b_lo, Wp, a_ks, b_ks, b_tap, idesc, accumulate); break;
     }
 }
 
 // The K=16 steps of one (tap, K group) block for one accumulator, unrolled.
 template <int KSTEPS>
-__device__ __forceinline__ void issue_ksteps_n(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t a_ks, uint32_t b_ks,
+__device__ __forceinline__ void issue_ksteps_n(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t a_ks, uint32_t b_ks,
                                                uint32_t idesc, uint32_t accumulate) {
 #pragma unroll
     for (int ks = 0; ks < KSTEPS; ++ks)
-        umma_bf16_lo(d_tmem, a_lo + (uint32_t)ks * a_ks, b_lo + (uint32_t)ks * b_ks, idesc, ks ? 1u : accumulate);
+        umma_bf16_lo_if(leader, d_tmem, a_lo + (uint32_t)ks * a_ks, b_lo + (uint32_t)ks * b_ks, idesc, ks ? 1u : accumulate);
 }
-__device__ __forceinline__ void issue_ksteps(int ksteps, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t a_ks,
+__device__ __forceinline__ void issue_ksteps(uint32_t leader, int ksteps, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t a_ks,
                                              uint32_t b_ks, uint32_t idesc, uint32_t accumulate) {
     // (a plain counted loop: a switch over unrolled bodies measured the same)
 #pragma unroll 1
     for (int ks = 0; ks < ksteps; ++ks) {
-        umma_bf16_lo(d_tmem, a_lo, b_lo, idesc, ks ? 1u : accumulate);
+        umma_bf16_lo_if(leader, d_tmem, a_lo, b_lo, idesc, ks ? 1u : accumulate);
         a_lo += a_ks;
         b_lo += b_ks;
     }
@@ -139,11 +139,11 @@ __device__ __forceinline__ void issue_ksteps(int ksteps, uint32_t d_tmem, uint32
 // that looked its offset up by a computed index, each tap cost the issuing thread about 350 cycles - ResNet-50's
 // three strided 3x3 layers at batch 128: 51 / 48 / 47 us so, 33 / 28 / 27 us unrolled.)
 template <int KSTEPS>
-__device__ __forceinline__ void issue_taps9(uint32_t d_tmem, uint32_t a_row0, const int (&tap_off)[9], uint32_t b_lo, uint32_t b_tap,
+__device__ __forceinline__ void issue_taps9(uint32_t leader, uint32_t d_tmem, uint32_t a_row0, const int (&tap_off)[9], uint32_t b_lo, uint32_t b_tap,
                                             uint32_t a_ks, uint32_t b_ks, uint32_t idesc, uint32_t accumulate) {
 #pragma unroll
     for (int t = 0; t < 9; ++t)
-        issue_ksteps_n<KSTEPS>(d_tmem, a_row0 + (uint32_t)tap_off[t], b_lo + (uint32_t)t * b_tap, a_ks, b_ks, idesc, t ? 1u : accumulate);
+        issue_ksteps_n<KSTEPS>(leader, d_tmem, a_row0 + (uint32_t)tap_off[t], b_lo + (uint32_t)t * b_tap, a_ks, b_ks, idesc, t ? 1u : accumulate);
 }
 
 // Shared-memory control block at the start of dynamic shared memory.
@@ -402,18 +402,21 @@ conv_tc_kernel(const TcParams p) {
         }
     } else if (issuer >= 0) {
         // ------------------------------ MMA issuer --------------------------------
-        if (lane == 0 && issuer < (int)n_issuers) {
+        // the whole warp goes through the loops, one elected lane issues: see umma_bf16_lo_if
+        if (issuer < (int)n_issuers) {
+            const uint32_t leader = elect_one();
+            auto wait_for = [&](uint32_t bar, uint32_t ph) { return __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_flag, wait_limit)); };
             // instruction descriptor: D = f32, A = B = bf16, both K-major, N = n_tile, M = 128
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.n_tile >> 3) << 17) | ((128u >> 4) << 24);
             uint32_t a_stage = 0, a_phase = 0, b_stage = 0, b_phase = 0;
             uint32_t acc_phase0 = 0, acc_phase1 = 0;
             int local = 0;
             bool ok = true;
-            if (MODE == MODE_FLAT_RESIDENT) ok = mbar_wait(b_full0, 0, abort_flag, wait_limit);
+            if (MODE == MODE_FLAT_RESIDENT) ok = wait_for(b_full0, 0);
             for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x, ++local) {
                 const int acc = local & 1;
                 const uint32_t ph = acc ? acc_phase1 : acc_phase0;
-                if (!mbar_wait(tempty0 + 8 * acc, ph ^ 1, abort_flag, wait_limit)) { ok = false; break; }
+                if (!wait_for(tempty0 + 8 * acc, ph ^ 1)) { ok = false; break; }
                 if (acc) acc_phase1 ^= 1; else acc_phase0 ^= 1;
                 tc_fence_after();
                 const int nt = tile - (int)fdiv((uint32_t)tile, p.div_ntiles) * p.n_tiles;
@@ -425,7 +428,7 @@ conv_tc_kernel(const TcParams p) {
                     const uint32_t a_ks = 2u * (uint32_t)(p.a_par * p.rows_a), b_ks = 2u * (uint32_t)p.n_tile;
                     const uint32_t d_acc = d_tmem + (uint32_t)(issuer * p.n_tile);
                     for (int g = 0; g < p.groups && ok; ++g) {
-                        if (!mbar_wait(a_full0 + 8 * a_stage, a_phase, abort_flag, wait_limit)) { ok = false; break; }
+                        if (!wait_for(a_full0 + 8 * a_stage, a_phase)) { ok = false; break; }
                         tc_fence_after();
                         int cgg = p.cchunks - g * p.cg;
                         if (cgg > p.cg) cgg = p.cg;
@@ -436,26 +439,26 @@ conv_tc_kernel(const TcParams p) {
                         uint32_t b_lo = ((sa + (uint32_t)p.a_stage_bytes) >> 4) | ((uint32_t)p.n_tile << 16);
                         const uint32_t b_tap = (uint32_t)(cgg * p.n_tile);
                         if (p.a.x_s2d) {
-                            if (ksteps == 1) issue_taps9<1>(d_acc, a_row0, p.tap_off, b_lo, b_tap, a_ks, b_ks, idesc, accumulate);
-                            else issue_taps9<2>(d_acc, a_row0, p.tap_off, b_lo, b_tap, a_ks, b_ks, idesc, accumulate);
+                            if (ksteps == 1) issue_taps9<1>(leader, d_acc, a_row0, p.tap_off, b_lo, b_tap, a_ks, b_ks, idesc, accumulate);
+                            else issue_taps9<2>(leader, d_acc, a_row0, p.tap_off, b_lo, b_tap, a_ks, b_ks, idesc, accumulate);
                             accumulate = 1;
                         } else
                         for (int r = 0; r < p.a.R; ++r) {
                             for (int sx = 0; sx < p.a.S; ++sx) {
-                                issue_ksteps(ksteps, d_acc, a_row + (uint32_t)sx, b_lo, a_ks, b_ks, idesc, accumulate);
+                                issue_ksteps(leader, ksteps, d_acc, a_row + (uint32_t)sx, b_lo, a_ks, b_ks, idesc, accumulate);
                                 accumulate = 1;
                                 b_lo += b_tap;
                             }
                             a_row += (uint32_t)p.Wp_in;
                         }
-                        umma_commit(a_empty0 + 8 * a_stage);     // releases the stage once these MMAs have read it
+                        if (leader) umma_commit(a_empty0 + 8 * a_stage);     // releases the stage once these MMAs have read it
                         if (++a_stage == (uint32_t)p.a_stages) { a_stage = 0; a_phase ^= 1; }
                     }
                 } else if (MODE != MODE_GATHER) {
                     // Descriptors differ only in their 16-byte start-address field, so the inner loops
                     // just add row counts to the low word (rows are 16 bytes: one row = one address unit).
                     for (int g = 0; g < p.groups && ok; ++g) {
-                        if (!mbar_wait(a_full0 + 8 * a_stage, a_phase, abort_flag, wait_limit)) { ok = false; break; }
+                        if (!wait_for(a_full0 + 8 * a_stage, a_phase)) { ok = false; break; }
                         tc_fence_after();
                         int cgg = p.cchunks - g * p.cg;
                         if (cgg > p.cg) cgg = p.cg;
@@ -472,61 +475,61 @@ conv_tc_kernel(const TcParams p) {
                             // (unrolled: an index into the parameters that is not a constant costs some 300 cycles per use)
 #pragma unroll
                             for (int tap = 0; tap < 9; ++tap)
-                                issue_ksteps(ksteps, d_tmem, a_row + (uint32_t)p.tap_off[tap], b_tap + (uint32_t)tap * b_tap_step, a_ks, b_ks,
+                                issue_ksteps(leader, ksteps, d_tmem, a_row + (uint32_t)p.tap_off[tap], b_tap + (uint32_t)tap * b_tap_step, a_ks, b_ks,
                                              idesc, tap ? 1u : accumulate);
                             accumulate = 1;
                         } else if (MODE == MODE_FLAT_RESIDENT) {
                             if (p.a.R == 3 && p.a.S == 3)
-                                issue_flat_resident_k<3, 3>(ksteps, d_tmem, a_row, b_tap, (uint32_t)p.Wp_in, a_ks, b_ks, b_tap_step, idesc, accumulate);
+                                issue_flat_resident_k<3, 3>(leader, ksteps, d_tmem, a_row, b_tap, (uint32_t)p.Wp_in, a_ks, b_ks, b_tap_step, idesc, accumulate);
                             else if (p.a.R == 3)
-                                issue_flat_resident_k<3, 1>(ksteps, d_tmem, a_row, b_tap, (uint32_t)p.Wp_in, a_ks, b_ks, b_tap_step, idesc, accumulate);
+                                issue_flat_resident_k<3, 1>(leader, ksteps, d_tmem, a_row, b_tap, (uint32_t)p.Wp_in, a_ks, b_ks, b_tap_step, idesc, accumulate);
                             else
-                                issue_flat_resident_k<1, 1>(ksteps, d_tmem, a_row, b_tap, (uint32_t)p.Wp_in, a_ks, b_ks, b_tap_step, idesc, accumulate);
+                                issue_flat_resident_k<1, 1>(leader, ksteps, d_tmem, a_row, b_tap, (uint32_t)p.Wp_in, a_ks, b_ks, b_tap_step, idesc, accumulate);
                             accumulate = 1;
                         } else {
                         for (int r = 0; r < p.a.R && ok; ++r) {
                             // streamed filters: one block per (K group, filter row).  Every 128-position tile of the step
                             // uses it: its own accumulator and issuing warp, its activation rows 128 further on
-                            if (!mbar_wait(b_full0 + 8 * b_stage, b_phase, abort_flag, wait_limit)) { ok = false; break; }
+                            if (!wait_for(b_full0 + 8 * b_stage, b_phase)) { ok = false; break; }
                             tc_fence_after();
                             uint32_t b_lo = ((b_base + b_stage * p.b_stage_bytes) >> 4) | ((uint32_t)p.n_tile << 16);
                             for (int sx = 0; sx < p.a.S; ++sx) {
-                                issue_ksteps(ksteps, d_tmem + (uint32_t)(issuer * p.n_tile), a_row + (uint32_t)sx + (uint32_t)(issuer * 128),
+                                issue_ksteps(leader, ksteps, d_tmem + (uint32_t)(issuer * p.n_tile), a_row + (uint32_t)sx + (uint32_t)(issuer * 128),
                                              b_lo, a_ks, b_ks, idesc, accumulate);
                                 accumulate = 1;
                                 b_lo += (uint32_t)(cgg * p.n_tile);
                             }
-                            umma_commit(b_empty0 + 8 * b_stage);
+                            if (leader) umma_commit(b_empty0 + 8 * b_stage);
                             if (++b_stage == (uint32_t)p.b_stages) { b_stage = 0; b_phase ^= 1; }
                             a_row += (uint32_t)p.Wp_in;
                         }
                         }
                         if (!ok) break;
-                        umma_commit(a_empty0 + 8 * a_stage);     // releases the stage once these MMAs have read it
+                        if (leader) umma_commit(a_empty0 + 8 * a_stage);     // releases the stage once these MMAs have read it
                         if (++a_stage == (uint32_t)p.a_stages) { a_stage = 0; a_phase ^= 1; }
                     }
                     // streamed 3x3 layer with a projection shortcut taken in: the K groups of the second input, centre tap only
                     for (int g2 = 0; MODE == MODE_FLAT_STREAM && g2 < p.groups2 && ok; ++g2) {
-                        if (!mbar_wait(a_full0 + 8 * a_stage, a_phase, abort_flag, wait_limit)) { ok = false; break; }
-                        if (!mbar_wait(b_full0 + 8 * b_stage, b_phase, abort_flag, wait_limit)) { ok = false; break; }
+                        if (!wait_for(a_full0 + 8 * a_stage, a_phase)) { ok = false; break; }
+                        if (!wait_for(b_full0 + 8 * b_stage, b_phase)) { ok = false; break; }
                         tc_fence_after();
                         int cgg = p.cchunks2 - g2 * p.cg;
                         if (cgg > p.cg) cgg = p.cg;
                         const uint32_t a_row = (((a_base + a_stage * p.a_stage_bytes) >> 4) + (uint32_t)p.halo + (uint32_t)(issuer * 128)) |
                                                ((uint32_t)p.rows_a << 16);
                         const uint32_t b_lo = ((b_base + b_stage * p.b_stage_bytes) >> 4) | ((uint32_t)p.n_tile << 16);
-                        issue_ksteps(cgg >> 1, d_tmem + (uint32_t)(issuer * p.n_tile), a_row, b_lo, 2u * (uint32_t)p.rows_a,
+                        issue_ksteps(leader, cgg >> 1, d_tmem + (uint32_t)(issuer * p.n_tile), a_row, b_lo, 2u * (uint32_t)p.rows_a,
                                      2u * (uint32_t)p.n_tile, idesc, accumulate);
                         accumulate = 1;
-                        umma_commit(b_empty0 + 8 * b_stage);
+                        if (leader) umma_commit(b_empty0 + 8 * b_stage);
                         if (++b_stage == (uint32_t)p.b_stages) { b_stage = 0; b_phase ^= 1; }
-                        umma_commit(a_empty0 + 8 * a_stage);
+                        if (leader) umma_commit(a_empty0 + 8 * a_stage);
                         if (++a_stage == (uint32_t)p.a_stages) { a_stage = 0; a_phase ^= 1; }
                     }
                 } else {
                     const int stage_bytes = p.a_stage_bytes + p.b_stage_bytes;
                     for (int kb = 0; kb < p.kblocks; ++kb) {
-                        if (!mbar_wait(a_full0 + 8 * a_stage, a_phase, abort_flag, wait_limit)) { ok = false; break; }
+                        if (!wait_for(a_full0 + 8 * a_stage, a_phase)) { ok = false; break; }
                         tc_fence_after();
                         int planes;
                         if (p.groups > 1) { const int g = kb % p.groups; planes = p.cchunks - g * p.cg; if (planes > p.cg) planes = p.cg; }
@@ -536,18 +539,18 @@ conv_tc_kernel(const TcParams p) {
                         uint32_t a_lo = (sa >> 4) | (128u << 16);
                         uint32_t b_lo = (sb >> 4) | ((uint32_t)p.n_tile << 16);
                         for (int ks = 0; ks < planes / 2; ++ks) {
-                            umma_bf16_lo(d_tmem, a_lo, b_lo, idesc, accumulate);
+                            umma_bf16_lo_if(leader, d_tmem, a_lo, b_lo, idesc, accumulate);
                             accumulate = 1;
                             a_lo += 256u;
                             b_lo += 2u * (uint32_t)p.n_tile;
                         }
-                        umma_commit(a_empty0 + 8 * a_stage);
+                        if (leader) umma_commit(a_empty0 + 8 * a_stage);
                         if (++a_stage == (uint32_t)p.a_stages) { a_stage = 0; a_phase ^= 1; }
                     }
                 }
-                if (ok) umma_commit(tfull0 + 8 * acc);   // accumulator complete
+                if (ok && leader) umma_commit(tfull0 + 8 * acc);   // accumulator complete
             }
-            if (!ok) raise(ctrl, p.status, 2);
+            if (!ok && leader) raise(ctrl, p.status, 2);
         }
     } else if (warp < 2 + EPI) {
         // ------------------------------ epilogue ----------------------------------

@@ -919,25 +919,27 @@ fp_status replan(fp_handle h) {
     // A 7x7 / stride-2 / pad-3 first convolution on <= 3 channels runs as a 3x1 convolution over a packed
     // copy of the input (tensor-core path only; the validation paths keep the plain form).
     h->stem_packed = 0;
+    bool stem7 = false;
     for (const FConv& f : h->convs)
         if (f.src == 0 && h->compute == FP_COMPUTE_BF16_TC && uses[0].size() == 1 && f.R == 7 && f.S == 7 &&
-            f.stride == 2 && f.pad == 3 && f.C <= 3 && h->in_H % 2 == 0 && h->in_W % 2 == 0)
-            h->stem_packed = 1;
+            f.stride == 2 && f.pad == 3 && f.C <= 3)
+            stem7 = true;
+    h->stem_packed = stem7 && h->in_H % 2 == 0 && h->in_W % 2 == 0;
     decide_splits(h, uses);
     for (FConv& f : h->convs) {
         f.n_mult = (h->tensors[f.src].split && split_reader(f) == 'C') ? 4 : 1;
         f.proj = -1; f.proj_kind = 0; f.absorbed = 0; f.plain_bank = 0;
     }
-    // ... and, where a 3x3 / stride-2 max pooling is the only reader of that convolution and the input is bf16, input
-    // conversion, convolution and pooling run as one kernel (decided below, once the filter count is known).
+    // ... and, where a 3x3 / stride-2 max pooling is the only reader of that convolution, input conversion, convolution and
+    // pooling run as one kernel (decided below, once the filter count is known).
     h->stem_fused = 0;
     bool stem_candidate = false;
-    if (h->stem_packed && !h->keep_outputs && h->in_dtype == FP_DTYPE_BF16 && h->ops.size() >= 3 && h->ops[1].kind == 0 &&
+    if (stem7 && !h->keep_outputs && h->ops.size() >= 3 && h->ops[1].kind == 0 &&
         h->ops[2].kind == 1) {
         const FConv& f = h->convs[h->ops[1].idx];
         const Pool& pl = h->pools[h->ops[2].idx];
         stem_candidate = f.src == 0 && f.relu && f.res_mode == 0 && pl.src == f.out && uses[f.out].size() == 1 &&
-                         pl.R == 3 && pl.stride == 2 && pl.pad == 1 && h->in_H % 4 == 0 && h->in_W % 8 == 0;
+                         pl.R == 3 && pl.stride == 2 && pl.pad == 1;
     }
     for (const Op& op : h->ops) {
         if (op.kind == 0) {
@@ -1350,7 +1352,7 @@ fp_status replan(fp_handle h) {
         fp::StemPoolArgs& a = h->stem_args;
         memset(&a, 0, sizeof(a));
         a.y = h->tensors[h->pools[h->ops[2].idx].out].d; a.w = f.d_wp; a.bias = f.d_bp;
-        a.N = h->max_batch; a.C = f.C; a.H = h->in_H; a.W = h->in_W; a.K_pad = f.K_pad; a.n0 = 0; a.n_count = h->max_batch;
+        a.N = h->max_batch; a.C = f.C; a.H = h->in_H; a.W = h->in_W; a.K_pad = f.K_pad; a.in_f32 = h->in_dtype != FP_DTYPE_BF16; a.n0 = 0; a.n_count = h->max_batch;
         char msg[256];
         if (fp::plan_stem_pool(a, &h->stem_plan, msg, sizeof(msg)) != 0) return fail(FP_ERR_UNSUPPORTED, "%s", msg);
     }

@@ -1154,7 +1154,7 @@ fp_status replan(fp_handle h) {
             fp::PackJob j = filters(f, fp::PACK_CONV);
             size_t vecs;
             if (h->stem_fused && i == 1) {
-                j.kind = fp::PACK_STEM_DIRECT;
+                j.kind = fp::PACK_STEM_DIRECT; j.w2 = f.d_b32;
                 j.units = 32 * f.K_pad; vecs = (size_t)j.units;
             } else if (h->stem_packed && f.src == 0) {
                 j.kind = fp::PACK_STEM;
@@ -1351,7 +1351,7 @@ fp_status replan(fp_handle h) {
         const FConv& f = h->convs[h->ops[1].idx];
         fp::StemPoolArgs& a = h->stem_args;
         memset(&a, 0, sizeof(a));
-        a.y = h->tensors[h->pools[h->ops[2].idx].out].d; a.w = f.d_wp; a.bias = f.d_bp;
+        a.y = h->tensors[h->pools[h->ops[2].idx].out].d; a.w = f.d_wp;
         a.N = h->max_batch; a.C = f.C; a.H = h->in_H; a.W = h->in_W; a.K_pad = f.K_pad; a.in_f32 = h->in_dtype != FP_DTYPE_BF16; a.n0 = 0; a.n_count = h->max_batch;
         char msg[256];
         if (fp::plan_stem_pool(a, &h->stem_plan, msg, sizeof(msg)) != 0) return fail(FP_ERR_UNSUPPORTED, "%s", msg);

@@ -190,12 +190,12 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
 struct StemPoolArgs {
     const void* x;        // network input, N x C x H x W, NCHW, bf16 or fp32 (rounded to bf16 on load)
     void* y;              // pooled tensor, planar-8 with border, K_pad channels, N images
-    const void* w;        // filters [16 taps (ta, tb)][2 chunks of 8][K_pad rows][8] bf16 over the parity channels (PACK_STEM_DIRECT)
-    const float* bias;    // [K_pad]
+    const void* w;        // filters [16 taps (ta, tb)][2 chunks of 8][K_pad rows][8] bf16 over the parity channels, shifts included
+                          // (PACK_STEM_DIRECT)
     int N, C, H, W, K_pad, in_f32;
     int n0, n_count;      // the images this launch handles (the tensor's plane pitch is that of all N)
 };
-struct StemPoolPlan { int valid, acc_rows, tmem_cols; unsigned smem_bytes; };
+struct StemPoolPlan { int valid, tmem_cols; unsigned smem_bytes; };
 bool stem_pool_supported(int C, int H, int W, int K_pad);
 int plan_stem_pool(const StemPoolArgs& a, StemPoolPlan* plan, char* err, size_t err_len);
 void launch_stem_pool(const StemPoolPlan& plan, const StemPoolArgs& a, int* d_status, cudaStream_t st);

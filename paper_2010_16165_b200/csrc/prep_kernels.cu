@@ -272,7 +272,8 @@ __device__ __forceinline__ void pack_stem_vec(const PackJob& j, const int32_t* _
 
 // A 7x7 first convolution for the kernel that fuses it with the pooling: the 7x7 / stride-2 window over C channels as a
 // 4x4 window over the 4 C parity channels of the half-resolution input - tap (ta, tb), channel (2a + b) C + c takes
-// w[k][c][2 ta + a - 1][2 tb + b - 1] (zero where an index is -1) - as [tap][chunk of 8][filter][8].
+// w[k][c][2 ta + a - 1][2 tb + b - 1] (zero where an index is -1) - as [tap][chunk of 8][filter][8].  Channels 4 C .. 4 C + 2,
+// which the kernel feeds with ones, hold the filter's shift at tap 0, as three bf16 that add up to the fp32 value.
 __device__ __forceinline__ void pack_stem_direct_vec(const PackJob& j, const int32_t* __restrict__ idx, int u) {
     const int k = u % j.K_pad, chunk = u / j.K_pad % 2, tap = u / (2 * j.K_pad);
     const int ta = tap >> 2, tb = tap & 3;
@@ -282,6 +283,11 @@ __device__ __forceinline__ void pack_stem_direct_vec(const PackJob& j, const int
     for (int e = 0; e < 8; ++e) {
         const int ch = chunk * 8 + e;
         v[e] = 0.0f;
+        if (ks >= 0 && tap == 0 && ch >= 4 * j.C && ch < 4 * j.C + 3) {
+            float b = j.w2[ks];
+            for (int i = 4 * j.C; i < ch; ++i) b -= __bfloat162float(__float2bfloat16(b));
+            v[e] = b;
+        }
         if (ks < 0 || ch >= 4 * j.C) continue;
         const int par = ch / j.C, c = ch - par * j.C;
         const int r = 2 * ta + (par >> 1) - 1, s = 2 * tb + (par & 1) - 1;

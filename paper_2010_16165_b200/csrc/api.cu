@@ -818,12 +818,19 @@ void find_net(fp_handle h, const std::vector<std::vector<Use>>& uses) {
         h->net_spec.layers.push_back(l);
     }
     if (h->ops[n_ops - 1].kind != 2 || h->head_src != h->convs[h->ops[n_ops - 2].idx].out) return;
-    const int choices[][2] = {{1, 1}, {2, 1}, {1, 2}, {1, 4}};       // images per CTA, CTAs per image
+    // images per CTA, CTAs per image, warps per image; a choice that no batch of this handle takes is not planned (a plan is 50 us for
+    // 109 layers): clusters of four while all images find one, then of two, then a CTA each, then pairs
+    const int choices[][3] = {{1, 4, 8}, {1, 2, 8}, {1, 1, 16}, {2, 1, 8}};
     for (const auto& c : choices) {
         fp::NetPlan p;
-        if (fp::plan_net(h->net_spec, c[0], c[1], &p)) h->net_plans.push_back(p);
-        else if (h->net_plans.empty()) return;             // one image does not fit
+        if (fp::plan_net(h->net_spec, c[0], c[1], c[2], &p)) {
+            h->net_plans.push_back(p);
+            if (c[0] == 1 && h->max_batch <= fp::net_at_once(c[1])) break;
+        } else if (c[1] == 1 && h->net_plans.empty()) {
+            return;                                        // one image does not fit
+        }
     }
+    if (h->net_plans.empty()) return;
     h->net_on = 1;
 }
 
@@ -1371,28 +1378,53 @@ fp_status need_plan(fp_handle h, const char* who) {
 // execution
 // ---------------------------------------------------------------------------------------
 
-// The network as one kernel, given to the CTAs the way that is cheapest for this batch: rounds over the GPU times the cost
-// of a round in units of one image per CTA (measured, ResNet-56: see the figures beside).
-void launch_network(fp_handle h, const void* d_input, int batch, float* d_logits, cudaStream_t st, int dump_layer = -1, void* dump = nullptr) {
-    int best = 0;
-    double best_cost = 0;
-    for (size_t k = 0; k < h->net_plans.size(); ++k) {
-        const fp::NetPlan& np = h->net_plans[k];
-        const int at_once = std::max(1, fp::sm_count() / np.cs);      // CTAs or clusters; the last round may carry one image each
-        const int full = batch / (at_once * np.G), rest = batch - full * at_once * np.G;
-        const double one = np.cs == 4 ? 0.55 : np.cs == 2 ? 0.7 : 1.0, two = 1.5;
-        const double cost = full * (np.G == 2 ? two : one) + (rest == 0 ? 0.0 : rest > at_once ? two : one);
-        if (k == 0 || cost < best_cost) { best = (int)k; best_cost = cost; }
+// The network as one kernel, given to the CTAs the way that is cheapest for this batch: rounds over the GPU times the cost of a
+// round (ResNet-56: clusters of four 84 us, of two 104 us, a CTA of sixteen warps per image 137 us, pairs of images 221 us).
+// What full rounds of pairs leave over goes the way that is cheapest for it, in a launch of its own.
+struct NetPart { int plan, images; };
+std::vector<NetPart> network_parts(fp_handle h, int batch) {
+    auto cheapest = [&](int n) {
+        int best = 0;
+        double best_cost = 0;
+        for (size_t k = 0; k < h->net_plans.size(); ++k) {
+            const fp::NetPlan& np = h->net_plans[k];
+            const int per_round = fp::net_at_once(np.cs) * np.G;
+            const double cost = (n + per_round - 1) / per_round * (np.G == 2 ? 2.21 : np.cs == 4 ? 0.84 : np.cs == 2 ? 1.04 : 1.37);
+            if (k == 0 || cost < best_cost) { best = (int)k; best_cost = cost; }
+        }
+        return best;
+    };
+    std::vector<NetPart> parts;
+    const fp::NetPlan& last = h->net_plans.back();
+    const int pairs = last.G == 2 ? batch / (2 * fp::net_at_once(1)) * 2 * fp::net_at_once(1) : 0, rest = batch - pairs;
+    if (pairs > 0) parts.push_back({(int)h->net_plans.size() - 1, pairs});
+    if (rest > 0) {
+        const int k = cheapest(rest);
+        if (!parts.empty() && k == parts[0].plan) parts[0].images += rest;
+        else parts.push_back({k, rest});
     }
+    return parts;
+}
+
+void launch_network(fp_handle h, const void* d_input, int batch, float* d_logits, cudaStream_t st, int dump_layer = -1, void* dump = nullptr) {
     const Tensor& last = h->tensors[h->head_src];
     fp::NetArgs a;
     memset(&a, 0, sizeof(a));
-    a.x = d_input; a.logits = d_logits; a.w = h->d_net_blob; a.fcw = h->d_fcw_packed; a.fcb = h->d_fcb;
-    a.N = batch; a.H = h->in_H; a.W = h->in_W; a.in_C = h->in_C; a.in_mode = h->in_dtype == FP_DTYPE_BF16 ? 2 : 1;
+    a.w = h->d_net_blob; a.fcw = h->d_fcw_packed; a.fcb = h->d_fcb;
+    a.H = h->in_H; a.W = h->in_W; a.in_C = h->in_C; a.in_mode = h->in_dtype == FP_DTYPE_BF16 ? 2 : 1;
     a.n_classes = h->n_classes; a.fc_pitch = last.C_pad; a.last_H = last.H; a.last_W = last.W;
     a.last_chunks = h->net_spec.layers.back().n8;
     a.dump_layer = dump_layer; a.dump = dump;
-    fp::launch_net(h->net_plans[best], a, h->d_net_tables[best], h->d_status, st);
+    std::vector<NetPart> parts = network_parts(h, batch);
+    if (dump) parts.assign(1, {parts[0].plan, batch});                // (the dumped tensor is the whole batch's)
+    int done = 0;
+    for (const NetPart& part : parts) {
+        a.x = (const uint8_t*)d_input + (size_t)done * h->in_C * h->in_H * h->in_W * h->in_elem();
+        a.logits = d_logits + (size_t)done * h->n_classes;
+        a.N = part.images;
+        fp::launch_net(h->net_plans[part.plan], a, h->d_net_tables[part.plan], h->d_status, st);
+        done += part.images;
+    }
 }
 
 // n0, n_count: the images an input conversion handles (the other operators always run the whole batch)
@@ -1702,7 +1734,8 @@ extern "C" fp_status fp_soft_prune_finish(fp_handle h) {
 
 // Operators first .. last of the forward on `st`, as a replayed CUDA graph where the handle asks for one.
 static fp_status forward_from(fp_handle h, const void* d_input, int32_t batch, float* d_logits, cudaStream_t st, int first) {
-    const bool graphable = h->use_graph && st != 0 && st != cudaStreamLegacy && st != cudaStreamPerThread;
+    // (a forward of one or two launches is launched: as a graph of one node it took 3 us more of the caller's time)
+    const bool graphable = h->use_graph && !h->net_on && st != 0 && st != cudaStreamLegacy && st != cudaStreamPerThread;
     if (!graphable) {
         launch_all(h, d_input, batch, d_logits, st, first);
         CK(cudaGetLastError());
@@ -1884,7 +1917,7 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             n -= h->input_fused;
             n -= 2 * h->stem_fused;                                          // conversion, convolution and pooling are one
             for (const FConv& c : h->convs) n -= c.absorbed;                 // a projection inside the layer that adds it
-            *(int32_t*)h_out = h->net_on ? 1 : n;
+            *(int32_t*)h_out = h->net_on ? (int)network_parts(h, h->last_batch > 0 ? h->last_batch : h->max_batch).size() : n;
             return FP_OK;
         }
         case FP_Q_CONV_K_FUSED: TRY(need(4)); TRY(conv_of(&f)); *(int32_t*)h_out = f ? f->K : 0; return FP_OK;

@@ -222,7 +222,7 @@ struct NetLayer {             // one layer as the kernel reads it (offsets and s
 struct NetSpecLayer { int chunks, n8, stride, relu, res_mode, res_pad_lo, res_C, Hin, Win, blob_off, blob_bytes; };
 struct NetSpec { std::vector<NetSpecLayer> layers; };
 struct NetPlan {
-    int G = 0, cs = 0, img_bytes = 0, act_bytes = 0, head_off = 0, last_off = 0, last_PV = 0, first_requests = 0;
+    int G = 0, cs = 0, warps = 8, img_bytes = 0, act_bytes = 0, head_off = 0, last_off = 0, last_PV = 0, first_requests = 0;
     unsigned smem_bytes = 0;
     std::vector<NetLayer> table;
 };
@@ -236,7 +236,8 @@ struct NetArgs {
 };
 int net_blob_bytes(int chunks, int n8);
 bool net_layer_supported(int H, int W, int P, int Q, int C_pad, int K, int stride);
-bool plan_net(const NetSpec& spec, int G, int cs, NetPlan* plan);
+bool plan_net(const NetSpec& spec, int G, int cs, int warps, NetPlan* plan);
+int net_at_once(int cs);
 void launch_net(const NetPlan& plan, const NetArgs& a, const NetLayer* d_table, int* d_status, cudaStream_t st);
 
 // A run of stride-1 3x3 convolutions executed by one kernel with the activations in shared memory.

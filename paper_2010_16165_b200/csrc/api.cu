@@ -835,7 +835,7 @@ void find_net(fp_handle h, const std::vector<std::vector<Use>>& uses) {
             return;                                        // one image does not fit
         }
     }
-    if (h->net_plans.empty()) return;
+    if (h->net_plans.empty() || !fp::prepare_net()) return;
     h->net_on = 1;
 }
 

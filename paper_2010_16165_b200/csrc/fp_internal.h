@@ -219,6 +219,9 @@ void launch_stem_pool(const StemPoolPlan& plan, const StemPoolArgs& a, int* d_st
 // CTAs share an image (cs): one plan per choice, the launch takes the cheapest for its batch.
 enum { NET_STRIP = 0, NET_TILE = 1, NET_STRIDED = 2 };
 constexpr int kNetUnits = 32;
+constexpr int kNetMaxG = 2;                      // images a CTA carries at a time
+constexpr int kNetSmemMax = 232448;              // opt-in dynamic shared memory per CTA,
+constexpr int kNetCtrlBytes = 1920;              // of which the kernel's barriers and descriptors take this much, alignment included
 struct NetUnit { uint16_t a_vec, dst_vec; uint8_t n8, nt, row, x; };   // a warp's piece of a layer: where its input and output start (vectors),
                                                  // first filter / 8, filters / 8, first output row and column
 struct NetLayer {             // one layer as the kernel reads it (offsets and strides in bytes; buffers relative to an image's memory)
@@ -251,6 +254,7 @@ struct NetArgs {
 int net_blob_bytes(int chunks, int n8);
 bool net_layer_supported(int H, int W, int P, int Q, int C_pad, int K, int stride);
 bool plan_net(const NetSpec& spec, int G, int cs, int warps, NetPlan* plan);
+bool prepare_net();              // lets the kernel have that much shared memory; false where the device refuses
 int net_at_once(int cs);
 void launch_net(const NetPlan& plan, const NetArgs& a, const NetLayer* d_table, int* d_status, cudaStream_t st);
 

@@ -227,7 +227,7 @@ struct NetUnit { uint16_t a_vec, dst_vec; uint8_t n8, nt, row, x; };   // a warp
 struct NetLayer {             // one layer as the kernel reads it (offsets and strides in bytes; buffers relative to an image's memory)
     int w_off, w_src, w_bytes, next;             // filters: place in shared memory, place in `w`, size; next: first layer to request behind this one
     int requests, req_off, req_src, req_bytes;   // how many to request, the first one's w_off, w_src, w_bytes
-    int form, units, res_mode, zero_bytes;       // form | input channels / 16 << 8 | rows of a piece << 16 | width 8 << 24; clear that much of the output first
+    int form, units, res_mode, zero_bytes;       // form | input channels / 16 << 8 | rows of a piece << 16 | width 8 << 24; clear that much of the output first (bit 0: begin together)
     int in_off, out_off, w_addr, bias_addr;
     int row_step, k_step, b_k, b_tap;            // input row, 16 input channels, filters of 16 channels, of a tap
     int out_plane, out_pitch, out_slab, relu;

@@ -84,6 +84,12 @@ bool net_layer_supported(int H, int W, int P, int Q, int C_pad, int K, int strid
 // tensors live from the layer that writes them to the last that reads them, a result with an identity shortcut takes the
 // place of that operand; filters go where nothing is alive from the moment they are requested.  Returns false if it does
 // not fit.
+//
+// Two images in a CTA (G = 2) are not at the same point.  Taking turns at the tensor pipe orders an image's results behind the
+// other's reads of the layer before (a turn is given away behind the last of them), and filters are requested when both are through
+// with a layer; but an image that has finished layer l goes on to clear the place of its next result, or to write the head's sums,
+// while the other may not have begun to read layer l's filters.  So a layer that may write where the filters of the layer before
+// lie begins when both images have ended that layer (bit 0 of zero_bytes), and the head's sums go over nothing that the last layer reads.
 bool plan_net(const NetSpec& spec, int G, int cs, int warps, NetPlan* plan) {
     const int L = (int)spec.layers.size();
     plan->G = G; plan->cs = cs; plan->warps = warps;
@@ -224,6 +230,14 @@ bool plan_net(const NetSpec& spec, int G, int cs, int warps, NetPlan* plan) {
             if (l == 0) left.push_back({in.off, bytes_of(in), in.PV});
             formats = left;
         }
+        if (G > 1 && l > 0) {
+            const NetLayer& before = plan->table[l - 1];
+            const int bytes = std::max(e.zero_bytes, s.n8 * e.out_plane);
+            for (int i = 0; i < G; ++i) {
+                const int at = i * img_bytes + out.off;
+                if (at < before.w_off + before.w_bytes + 128 && at + bytes > before.w_off) e.zero_bytes |= 1;
+            }
+        }
         // filters that went over an activation buffer's place unformat it
         std::vector<Format> left;
         for (const Format& f : formats) {
@@ -238,7 +252,7 @@ bool plan_net(const NetSpec& spec, int G, int cs, int warps, NetPlan* plan) {
         const Buf& last = bufs[buf_of[L]];
         const int H = last.R * cs, C = spec.layers[L - 1].n8 * 8;
         int after;
-        if (!place(G * (H + 1) * C * 4, L - 2, L, &plan->head_off, &after)) return false;
+        if (!place(G * (H + 1) * C * 4, L - 2, L, &plan->head_off, &after) || (G > 1 && after > L - 2)) return false;
         plan->last_off = last.off; plan->last_PV = last.PV;
     }
     int top = plan->act_bytes;

@@ -530,6 +530,8 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
             const NetLayer& ly = ctrl->layer[ring];
             const int4 q = *reinterpret_cast<const int4*>(&ly.form);         // form, units, res_mode, zero_bytes
             if (q.w) {                                 // another geometry moves in: its borders have to be zero
+                // bit 0: the other image may still read filters from that place (plan_net)
+                if (!CLUSTER && (q.w & 1) && active > 1) asm volatile("bar.sync 5, %0;" ::"n"(2 * kThreads) : "memory");
                 zero_bytes(img0 + (uint32_t)ly.out_off, q.w, tid, threads);
                 image_sync<CLUSTER, WARPS>(slot);
             }

@@ -56,3 +56,20 @@ def test_layer_shapes(B, fpo, widths, hw, batch):
         np.testing.assert_array_equal(got, np.concatenate([got[:2]] * (batch // 2)))
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("p", [0.2, 0.55])
+def test_second_image_of_a_pair_keeps_its_filters(B, p):
+    """ResNet-32 at ratios where filters lie in the place of the next layer's result: the first image of a pair must not clear it
+    before the second one has read them."""
+    net = wl.resnet_cifar(5)
+    w = wl.Workload("resident_pairs", net, 8, 53, True, wl.uniform_ratios(p), "uniform")
+    g = Gpu(B, w, B.FP_COMPUTE_BF16_TC, max_batch=296)
+    try:
+        B.fp_prune(g.h, w.ratios)
+        one = np.concatenate([g.forward(w.x[i:i + 1]) for i in range(8)])
+        x = np.concatenate([w.x] * 37)
+        for _ in range(5):
+            np.testing.assert_array_equal(g.forward(x), np.concatenate([one] * 37))
+    finally:
+        g.close()

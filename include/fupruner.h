@@ -311,7 +311,8 @@ fp_status fp_rank_filters_static(const float* d_filters, int32_t K, int32_t per_
  * the tensor cores, for the other warps) has a time limit; when one runs out the CTA raises the handle's status word,
  * all of its roles leave their loops, tensor memory is released and the kernel returns.  This call launches the first
  * stride-1 convolution of the graph that runs as a kernel of its own with the first round of its activation copies
- * left out and a limit of one millisecond, so exactly that happens; nothing faults and nothing hangs.  The
+ * left out and a limit of one millisecond, so exactly that happens; nothing faults and nothing hangs.  (Where the whole network
+ * is one kernel: that kernel for one image, one of the CTAs that share it announcing its border rows on the wrong barrier.)  The
  * activations of the handle are garbage afterwards (run fp_forward again), and the next
  * fp_query(FP_Q_DEVICE_STATUS) reports FP_ERR_TIMEOUT, once.  Asynchronous on `stream`.
  * Errors: FP_ERR_ARG, FP_ERR_UNSUPPORTED (no such convolution in the graph), FP_ERR_CUDA.

@@ -1436,7 +1436,7 @@ std::vector<NetPart> network_parts(fp_handle h, int batch) {
     return parts;
 }
 
-void launch_network(fp_handle h, const void* d_input, int batch, float* d_logits, cudaStream_t st, int dump_layer = -1, void* dump = nullptr) {
+fp::NetArgs network_args(fp_handle h) {
     const Tensor& last = h->tensors[h->head_src];
     fp::NetArgs a;
     memset(&a, 0, sizeof(a));
@@ -1444,6 +1444,12 @@ void launch_network(fp_handle h, const void* d_input, int batch, float* d_logits
     a.H = h->in_H; a.W = h->in_W; a.in_C = h->in_C; a.in_mode = h->in_dtype == FP_DTYPE_BF16 ? 2 : 1;
     a.n_classes = h->n_classes; a.fc_pitch = last.C_pad; a.last_H = last.H; a.last_W = last.W;
     a.last_chunks = h->net_spec.layers.back().n8;
+    a.dump_layer = -1;
+    return a;
+}
+
+void launch_network(fp_handle h, const void* d_input, int batch, float* d_logits, cudaStream_t st, int dump_layer = -1, void* dump = nullptr) {
+    fp::NetArgs a = network_args(h);
     a.dump_layer = dump_layer; a.dump = dump;
     std::vector<NetPart> parts = network_parts(h, batch);
     if (dump) parts.assign(1, {parts[0].plan, batch});                // (the dumped tensor is the whole batch's)
@@ -1809,6 +1815,18 @@ extern "C" fp_status fp_forward(fp_handle h, const void* d_input, int32_t batch,
 extern "C" fp_status fp_debug_expire_wait(fp_handle h, void* stream) {
     if (!h) return fail(FP_ERR_ARG, "fp_debug_expire_wait: NULL handle");
     TRY(need_plan(h, "fp_debug_expire_wait"));
+    if (h->net_on) {
+        // one image shared by the CTAs of a cluster, the second of which counts border rows on the barrier of the next layer: the first
+        // CTA's wait for them runs out
+        for (size_t k = 0; k < h->net_plans.size(); ++k) {
+            if (h->net_plans[k].cs == 1) continue;
+            fp::NetArgs a = network_args(h);
+            a.x = h->d_in_stage; a.logits = h->d_logits_stage; a.N = 1; a.other_barrier = 1; a.wait_cycles = 2000000LL;
+            fp::launch_net(h->net_plans[k], a, h->d_net_tables[k], h->d_status, (cudaStream_t)stream);
+            CK(cudaGetLastError());
+            return FP_OK;
+        }
+    }
     for (int i = 0; i < (int)h->ops.size(); ++i) {
         const Op& op = h->ops[i];
         if (op.kind != 0 || h->op_chain[i] >= 0 || (h->stem_fused && i == 1)) continue;

@@ -250,6 +250,8 @@ struct NetArgs {
     const float *fcw, *fcb;   // FC matrix [class][fc_pitch] scaled by 1 / (H * W) of the last tensor; fcb may be nullptr
     void* dump;               // diagnostic: planar-8 tensor with border that layer dump_layer's output is written to
     int N, H, W, in_C, in_mode, n_classes, fc_pitch, last_H, last_W, last_chunks, dump_layer;
+    int other_barrier;        // diagnostic (fp_debug_expire_wait): 1: CTA 1 of a cluster counts border rows on the wrong one of the two barriers, and
+    long long wait_cycles;    // every wait gives up after this many SM clock cycles; 0: a normal launch
 };
 int net_blob_bytes(int chunks, int n8);
 bool net_layer_supported(int H, int W, int P, int Q, int C_pad, int K, int stride);

@@ -73,3 +73,23 @@ def test_second_image_of_a_pair_keeps_its_filters(B, p):
             np.testing.assert_array_equal(g.forward(x), np.concatenate([one] * 37))
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("hw, widths", [(32, (16, 32, 64)), (8, (24,))])
+def test_rows_that_never_come_are_reported(B, hw, widths):
+    """CTAs that share an image wait for each other's border rows: with one of them announcing its rows on the wrong barrier, the wait runs
+    out after a millisecond, the status says so - once - and the next forward is as before."""
+    net = wl.resnet_cifar(2, widths, in_hw=hw)
+    w = wl.Workload("resident_expiry", net, 3, 59, True, wl.uniform_ratios(0.3), "uniform")
+    g = Gpu(B, w, B.FP_COMPUTE_BF16_TC)
+    try:
+        B.fp_prune(g.h, w.ratios)
+        assert B.fp_query_int(g.h, B.FP_Q_N_LAUNCHES) == 1
+        before = g.forward(w.x)
+        B.fp_debug_expire_wait(g.h)
+        torch.cuda.synchronize()
+        assert B.fp_query_int(g.h, B.FP_Q_DEVICE_STATUS) == B.FP_ERR_TIMEOUT
+        assert B.fp_query_int(g.h, B.FP_Q_DEVICE_STATUS) == 0
+        np.testing.assert_array_equal(g.forward(w.x), before)
+    finally:
+        g.close()

@@ -839,6 +839,69 @@ void find_net(fp_handle h, const std::vector<std::vector<Use>>& uses) {
     h->net_on = 1;
 }
 
+// The network as one kernel, given to the CTAs the way that is cheapest for this batch: rounds over the GPU times the cost of a
+// round (ResNet-56: clusters of four 84 us, of two 104 us, a CTA of sixteen warps per image 137 us, pairs of images 221 us).
+// What full rounds of pairs leave over goes the way that is cheapest for it, in a launch of its own.
+struct NetPart { int plan, images; };
+std::vector<NetPart> network_parts(fp_handle h, int batch) {
+    auto cheapest = [&](int n) {
+        int best = 0;
+        double best_cost = 0;
+        for (size_t k = 0; k < h->net_plans.size(); ++k) {
+            const fp::NetPlan& np = h->net_plans[k];
+            const int per_round = fp::net_at_once(np.cs) * np.G;
+            const double cost = (n + per_round - 1) / per_round * (np.G == 2 ? 2.21 : np.cs == 4 ? 0.84 : np.cs == 2 ? 1.04 : 1.37);
+            if (k == 0 || cost < best_cost) { best = (int)k; best_cost = cost; }
+        }
+        return best;
+    };
+    std::vector<NetPart> parts;
+    const fp::NetPlan& last = h->net_plans.back();
+    const int pairs = last.G == 2 ? batch / (2 * fp::net_at_once(1)) * 2 * fp::net_at_once(1) : 0, rest = batch - pairs;
+    if (pairs > 0) parts.push_back({(int)h->net_plans.size() - 1, pairs});
+    if (rest > 0) {
+        const int k = cheapest(rest);
+        if (!parts.empty() && k == parts[0].plan) parts[0].images += rest;
+        else parts.push_back({k, rest});
+    }
+    return parts;
+}
+
+// Microseconds of a forward of the largest batch, as one kernel and layer by layer (runs of layers where there are any): fitted to 524
+// timings of networks of 7 to 109 layers, 8 to 64 filters wide, pruned at 0 to 0.6, batches from 148 (4 % rms each).  One kernel: every
+// round over the GPU costs the planner's cycles and the ends of the layers.  Layer by layer: a launch, and per run the rounds of its
+// groups times the tiles' chains; single layers by their MMAs, strided ones by the gathered positions.
+double network_cost(fp_handle h) {
+    double us = 6.1;
+    for (const NetPart& part : network_parts(h, h->max_batch)) {
+        const fp::NetPlan& np = h->net_plans[part.plan];
+        const int per_round = fp::net_at_once(np.cs) * np.G, rounds = (part.images + per_round - 1) / per_round;
+        const double per_cycle = np.G == 2 ? 1.26e-3 : np.cs == 4 ? 6.6e-4 : np.cs == 2 ? 4.4e-4 : 6.2e-4;
+        const double per_layer = np.G == 2 ? 0.76 : np.cs == 4 ? 1.12 : np.cs == 2 ? 1.38 : 0.81;
+        us += rounds * (per_cycle * np.cycles + per_layer * (double)np.table.size());
+    }
+    return us;
+}
+double layers_cost(fp_handle h) {
+    const double sms = fp::sm_count(), N = h->max_batch;
+    double us = 0;
+    for (const Chain& ch : h->chains) {
+        const int groups = (h->max_batch + ch.plan.G - 1) / ch.plan.G, rounds = (groups + (int)sms - 1) / (int)sms;
+        for (int l = 0; l < ch.args.n_layers; ++l)
+            us += rounds * ((ch.plan.tiles + 1.5) * (0.194 * ch.args.layers[l].K_pad / 16 + 0.003) + 0.6);
+    }
+    for (int i = 0; i < (int)h->ops.size(); ++i) {
+        if (h->ops[i].kind != 0 || h->op_chain[i] >= 0) continue;
+        const FConv& f = h->convs[h->ops[i].idx];
+        const Tensor& out = h->tensors[f.out];
+        us += 5.7;
+        if (f.stride == 1) us += 1.17 * std::ceil((out.H + 2) * (out.W + 2) * N / 128) * 9 * (f.C_pad / 16) * std::max(f.K_pad / 2.0, 32 + f.K_pad / 4.0) / (sms * 1900);
+        else us += 2.5e-4 * N * out.H * out.W * (f.C_pad / 16);
+    }
+    const Tensor& last = h->tensors[h->head_src];
+    return us + 2 * 5.7 + 2.6e-5 * N * last.H * last.W * (last.C_pad / 16);
+}
+
 // How a convolution reads a parity-split input tensor: 0 it cannot, 'A' 3x3 / stride 2 / pad 1 (nine taps over the four
 // parity images), 'B' 1x1 / stride 2 (the parity-00 image), 'C' 1x1 / stride 1 without shortcut (position by position:
 // its output is then split the same way).
@@ -1136,8 +1199,20 @@ fp_status replan(fp_handle h) {
             std::copy(src.keep.begin(), src.keep.begin() + src.C, idx.begin() + head_chan);
         }
     }
+    // One kernel or layer by layer, by the batch that the handle is made for - not by each call's, so that a result does not depend on
+    // the batch it was computed in.  Many layers on many images go layer by layer (unpruned ResNet-110: batch 444 514 us against 705,
+    // 1024 1461 against 1593; ResNet-56 at 0.3: batch 592 393 against 430), few layers or few images as one kernel (ResNet-20: 300
+    // against 355 at batch 1024; ResNet-56 at 0.3, batch 256: 216 against 229).
     find_net(h, uses);
+    const bool one_kernel = h->net_on;
+    h->net_on = 0;
     find_chains(h, uses);
+    if (one_kernel && network_cost(h) <= layers_cost(h)) {
+        h->net_on = 1;
+        find_chains(h, uses);
+    } else {
+        h->net_plans.clear();
+    }
 
     // --- packed filters, biases, FC matrix: sizes and jobs, then one region, one upload and one launch ---
     {
@@ -1407,34 +1482,6 @@ fp_status need_plan(fp_handle h, const char* who) {
 // ---------------------------------------------------------------------------------------
 // execution
 // ---------------------------------------------------------------------------------------
-
-// The network as one kernel, given to the CTAs the way that is cheapest for this batch: rounds over the GPU times the cost of a
-// round (ResNet-56: clusters of four 84 us, of two 104 us, a CTA of sixteen warps per image 137 us, pairs of images 221 us).
-// What full rounds of pairs leave over goes the way that is cheapest for it, in a launch of its own.
-struct NetPart { int plan, images; };
-std::vector<NetPart> network_parts(fp_handle h, int batch) {
-    auto cheapest = [&](int n) {
-        int best = 0;
-        double best_cost = 0;
-        for (size_t k = 0; k < h->net_plans.size(); ++k) {
-            const fp::NetPlan& np = h->net_plans[k];
-            const int per_round = fp::net_at_once(np.cs) * np.G;
-            const double cost = (n + per_round - 1) / per_round * (np.G == 2 ? 2.21 : np.cs == 4 ? 0.84 : np.cs == 2 ? 1.04 : 1.37);
-            if (k == 0 || cost < best_cost) { best = (int)k; best_cost = cost; }
-        }
-        return best;
-    };
-    std::vector<NetPart> parts;
-    const fp::NetPlan& last = h->net_plans.back();
-    const int pairs = last.G == 2 ? batch / (2 * fp::net_at_once(1)) * 2 * fp::net_at_once(1) : 0, rest = batch - pairs;
-    if (pairs > 0) parts.push_back({(int)h->net_plans.size() - 1, pairs});
-    if (rest > 0) {
-        const int k = cheapest(rest);
-        if (!parts.empty() && k == parts[0].plan) parts[0].images += rest;
-        else parts.push_back({k, rest});
-    }
-    return parts;
-}
 
 fp::NetArgs network_args(fp_handle h) {
     const Tensor& last = h->tensors[h->head_src];

@@ -241,6 +241,7 @@ struct NetSpec { std::vector<NetSpecLayer> layers; };
 struct NetPlan {
     int G = 0, cs = 0, warps = 8, img_bytes = 0, act_bytes = 0, head_off = 0, last_off = 0, last_PV = 0, first_requests = 0;
     unsigned smem_bytes = 0;
+    double cycles = 0;        // what the layers of one image take by the planner's estimate of each
     std::vector<NetLayer> table;
 };
 struct NetArgs {

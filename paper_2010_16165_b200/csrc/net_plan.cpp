@@ -16,7 +16,7 @@ int up(int v, int m) { return (v + m - 1) / m * m; }
 struct Span { int off, bytes, birth, death; };      // a piece of shared memory in use from layer `birth` to layer `death`
 
 // Form and split of one layer over the warps of an image (eight; sixteen where an image has a CTA of that many to itself) (R: output rows of this CTA).
-bool split_layer(NetLayer* e, const NetGeom& q, int warps) {
+bool split_layer(NetLayer* e, const NetGeom& q, int warps, double* cycles) {
     const int kc = q.kc, n8 = q.n8, R = q.R, strips = q.W >= 16 ? q.W / 16 : 1;
     double best = 0;
     int form_ = 0, nt_ = 1, run_ = 1;
@@ -50,6 +50,7 @@ bool split_layer(NetLayer* e, const NetGeom& q, int warps) {
         for (int run : {4, 2})
             for (int nt = std::min(4, n8); nt >= 1; --nt) if (R % run == 0) offer(NET_TILE, nt, run);
     }
+    *cycles += best;
     if (best == 0) return false;                            // more pieces than a layer's table holds
     const int runs = (R + run_ - 1) / run_, groups = (n8 + nt_ - 1) / nt_;
     e->form = form_ | kc << 8 | run_ << 16 | (q.W == 8 ? 1 : 0) << 24;
@@ -95,6 +96,7 @@ bool plan_net(const NetSpec& spec, int G, int cs, int warps, NetPlan* plan) {
     plan->G = G; plan->cs = cs; plan->warps = warps;
     plan->table.assign(L, NetLayer());
     plan->first_requests = 0;
+    plan->cycles = 0;
     struct Buf { int W, R, PV, chunks, birth, death, off; };
     std::vector<Buf> bufs;
     std::vector<int> buf_of(L + 1);                        // tensor (0 = network input, l + 1 = layer l's output) -> buffer
@@ -193,7 +195,7 @@ bool plan_net(const NetSpec& spec, int G, int cs, int warps, NetPlan* plan) {
         const Buf &in = bufs[buf_of[l]], &out = bufs[buf_of[l + 1]];
         NetGeom q;
         q.kc = s.chunks / 2; q.n8 = s.n8; q.stride = s.stride; q.W = out.W; q.Win = in.W; q.R = out.R; q.out_PV = out.PV;
-        if (!split_layer(&e, q, warps)) return false;
+        if (!split_layer(&e, q, warps, &plan->cycles)) return false;
         e.in_off = in.off; e.out_off = out.off; e.R = out.R; e.W = out.W; e.n8 = s.n8; e.res_mode = s.res_mode;
         e.row_step = (in.W + 1) * 16; e.k_step = 2 * in.PV * 16;
         e.b_k = 2 * s.n8 * 128; e.b_tap = q.kc * e.b_k;

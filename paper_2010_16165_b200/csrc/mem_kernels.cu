@@ -383,20 +383,20 @@ __global__ void __launch_bounds__(32 * kFcWarps, 2) fc_kernel(const float* sums,
 #pragma unroll
         for (int i = 0; i < IMAGES; ++i) acc[t][i] = 0.0f;
     for (int slab = 0; slab < c4; slab += kFcSlab4) {
-        const int n4 = min(kFcSlab4, c4 - slab);
+        // (zeros behind the last channel, where the rows' are zeros too: a sum that is infinite there would make them NaN)
+        const int n4 = min(kFcSlab4, c4 - slab), padded = (n4 + 32 * AHEAD - 1) / (32 * AHEAD) * (32 * AHEAD);
         if (slab) __syncthreads();         // the previous slab has been consumed
         for (int img = warp; img < IMAGES; img += kFcWarps) {
             const float4* from = reinterpret_cast<const float4*>(sums + (size_t)(n0 + min(img, images - 1)) * C_pad) + slab;
-            for (int i = lane; i < n4; i += 32) sh4[img * kFcSlab4 + i] = from[i];
+            for (int i = lane; i < padded; i += 32) sh4[img * kFcSlab4 + i] = i < n4 ? from[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
         __syncthreads();
         for (int c = lane; c < n4; c += 32 * AHEAD) {                // (a slab that is not the last is a multiple of that)
 #pragma unroll
             for (int i = 0; i < AHEAD; ++i) {
-                const int cc = min(c + 32 * i, n4 - 1);
 #pragma unroll
                 for (int img = 0; img < IMAGES; ++img) {
-                    const float4 s = sh4[img * kFcSlab4 + cc];
+                    const float4 s = sh4[img * kFcSlab4 + c + 32 * i];
 #pragma unroll
                     for (int t = 0; t < CPW; ++t)
                         acc[t][img] = fmaf(s.w, w[t][i].w, fmaf(s.z, w[t][i].z, fmaf(s.y, w[t][i].y, fmaf(s.x, w[t][i].x, acc[t][img]))));

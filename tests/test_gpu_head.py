@@ -1,5 +1,6 @@
 """GPU parity of the average pooling and FC layer: batches at the edges of the image groups (1, 4, 8), classes per warp (1, 2,
 4), channels around the 2048 held at a time, image sizes below and above a warp of positions."""
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -38,5 +39,22 @@ def test_head_matches_oracle(B, fpo, batch, hw, channels, classes, compute):
     try:
         gp, _, _, _ = oracle_pruned(fpo, w)
         assert err(g.forward(w.x), fpo.fused_forward(gp, w.x)) < (TOL_FP32 if compute == "fp32" else TOL_BF16)
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("batch, channels, classes", [(1, 32, 11), (3, 32, 11), (9, 528, 9), (24, 528, 1000), (83, 528, 1000)])
+@pytest.mark.parametrize("compute", ["fp32", "tc"])
+def test_an_infinite_average_stays_infinite(B, batch, channels, classes, compute):
+    """Every logit is plus or minus infinity by the sign of its weight for the last channel, whose average is infinite; none is NaN."""
+    w = one_layer(batch, 5, channels, classes)
+    w.x[:] = 1e20
+    bank = w.weights[:channels * 3].reshape(channels, 3)
+    bank[:-1] = 1e-3
+    bank[-1] = 1e20
+    fc = w.weights[channels * 3:channels * 3 + classes * channels].reshape(classes, channels)
+    g = Gpu(B, w, B.FP_COMPUTE_FP32 if compute == "fp32" else B.FP_COMPUTE_BF16_TC)
+    try:
+        np.testing.assert_array_equal(g.forward(w.x), np.broadcast_to(np.sign(fc[:, -1]) * np.inf, (batch, classes)))
     finally:
         g.close()

@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(32 * kFcWarps, 2) fc_kernel(const float* sums,
     extern __shared__ float4 sh4[];        // IMAGES x kFcSlab4
     const int n0 = blockIdx.x * IMAGES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int k0 = (blockIdx.y * kFcWarps + warp) * CPW, c4 = C_pad >> 2;
+    const int k0 = ((int)(blockIdx.z * gridDim.y + blockIdx.y) * kFcWarps + warp) * CPW, c4 = C_pad >> 2;
     const float4* wr[CPW];
     float4 w[CPW][AHEAD];
     auto rows = [&](int c, int i) {        // 128 channels of the warp's rows, zeros behind the last
@@ -502,7 +502,9 @@ void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, con
     const int cpw = images < 8 ? 1 : groups * ((n_classes + 31) / 32) >= 2 * sm_count() ? 4 : groups * ((n_classes + 15) / 16) >= sm_count() ? 2 : 1;
     const Fc fn = cpw == 4 ? (Fc)fc_kernel<8, 4, 2> : cpw == 2 ? (Fc)fc_kernel<8, 2, 4> : images == 8 ? (Fc)fc_kernel<8, 1, 8>
                 : images == 4 ? (Fc)fc_kernel<4, 1, 8> : (Fc)fc_kernel<1, 1, 16>;
-    cfg.gridDim = dim3((unsigned)groups, (unsigned)((n_classes + kFcWarps * cpw - 1) / (kFcWarps * cpw)));
+    // (65535 blocks are the most along y; a matrix of more classes goes on along z)
+    const unsigned class_blocks = (unsigned)((n_classes + kFcWarps * cpw - 1) / (kFcWarps * cpw)), along_y = std::min(class_blocks, 65535u);
+    cfg.gridDim = dim3((unsigned)groups, along_y, (class_blocks + along_y - 1) / along_y);
     cfg.dynamicSmemBytes = (size_t)images * kFcSlab4 * sizeof(float4);
     static bool raised[64];                // per device, once
     int dev = 0;

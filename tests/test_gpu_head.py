@@ -58,3 +58,13 @@ def test_an_infinite_average_stays_infinite(B, batch, channels, classes, compute
         np.testing.assert_array_equal(g.forward(w.x), np.broadcast_to(np.sign(fc[:, -1]) * np.inf, (batch, classes)))
     finally:
         g.close()
+
+
+def test_more_classes_than_one_grid_dimension_holds(B, fpo):
+    w = one_layer(2, 3, 16, 540_001)
+    g = Gpu(B, w, B.FP_COMPUTE_BF16_TC)
+    try:
+        gp, _, _, _ = oracle_pruned(fpo, w)
+        assert err(g.forward(w.x), fpo.fused_forward(gp, w.x)) < TOL_BF16
+    finally:
+        g.close()

@@ -19,13 +19,14 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <atomic>
 #include <vector>
 
 namespace fp {
 
 // Streaming multiprocessors of the current device (asked once per device; 148 on a B200).  Grids are sized from it.
 inline int sm_count() {
-    static int cached[64] = {0};
+    static std::atomic<int> cached[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return 148; }
     if (cached[dev] == 0) {

@@ -5,6 +5,7 @@
 #include "fp_internal.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 
 namespace fp {
@@ -506,7 +507,7 @@ void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, con
     const unsigned class_blocks = (unsigned)((n_classes + kFcWarps * cpw - 1) / (kFcWarps * cpw)), along_y = std::min(class_blocks, 65535u);
     cfg.gridDim = dim3((unsigned)groups, along_y, (class_blocks + along_y - 1) / along_y);
     cfg.dynamicSmemBytes = (size_t)images * kFcSlab4 * sizeof(float4);
-    static bool raised[64];                // per device, once
+    static std::atomic<bool> raised[64];   // per device, once (threads may all be the first)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !raised[dev]) {
         for (Fc f : {(Fc)fc_kernel<8, 1, 8>, (Fc)fc_kernel<8, 2, 4>, (Fc)fc_kernel<8, 4, 2>})

@@ -26,6 +26,7 @@
 #include "tc_common.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <type_traits>
@@ -707,7 +708,7 @@ bool prepare_net() {
 // of four on a B200, not 37 (ResNet-56, 36 images: 165 us as two waves of clusters of four, 104 us in clusters of two).
 int net_at_once(int cs) {
     if (cs == 1) return sm_count();
-    static int known[64][9];
+    static std::atomic<int> known[64][9];              // (threads may all be the first: each finds the same)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || cs > 8) { cudaGetLastError(); return std::max(1, sm_count() / cs); }
     if (!known[dev][cs]) {

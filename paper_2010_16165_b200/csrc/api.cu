@@ -973,7 +973,7 @@ void conv_geometry(fp_handle h, const FConv& f, fp::ConvArgs* a) {
 // Rebuilds everything that depends on the masks.  The old buffers are released first, so while this runs - and
 // after it failed half-way (out of memory, a layer left without filters) - the handle has no plan: `planned` stays
 // 0 and every call that would launch kernels refuses until a later fp_prune succeeds.
-fp_status replan(fp_handle h) {
+fp_status build_plan(fp_handle h) {
     h->planned = 0;
     drop_graphs(h);
     CK(cudaDeviceSynchronize());
@@ -1471,6 +1471,14 @@ fp_status replan(fp_handle h) {
     CK(cudaDeviceSynchronize());
     h->planned = 1;
     return FP_OK;
+}
+
+// A plan that failed half-way may have left its upload and the packing launch on their way: the pinned memory they read, and the regions
+// they write, are the next call's.
+fp_status replan(fp_handle h) {
+    const fp_status s = build_plan(h);
+    if (s != FP_OK) cudaDeviceSynchronize();
+    return s;
 }
 
 fp_status need_plan(fp_handle h, const char* who) {

@@ -75,3 +75,56 @@ def test_another_plan_right_behind_one_that_failed(B, refuse_after):
     finally:
         B.fp_destroy(h)
     assert not pool.live
+
+
+def straight_net(hw):
+    """Convolutions in a row, most of the activations in the first two, most of the weights in the last."""
+    net = wl.Net(3, hw, hw, "straight")
+    x, C = -1, 3
+    for K, stride in ((64, 1), (64, 1), (16, 2), (16, 2), (16, 2), (512, 1), (512, 1)):
+        x = net.relu(net.bn(net.conv(x, K, C, 3, stride, 1), K))
+        C = K
+    net.fc(net.gavgpool(x, C), 10, C)
+    net.n_blocks = 0
+    return net
+
+
+def test_a_plan_takes_no_more_than_the_larger_of_two(B):
+    """From few filters where the weights are to few filters where the activations are: with a caller's allocator the old plan's memory is
+    back before the new plan's is taken, so room for either is room for the change."""
+    w = wl.Workload("straight", straight_net(24), 64, 67, True, wl.uniform_ratios(0.0), "none")
+    wide, narrow = np.array([0.0, 0, 0, 0, 0, 0.9, 0.9]), np.array([0.75, 0.75, 0, 0, 0, 0, 0])
+    pool = Pool(B)
+    dw, dbn = to_dev(w.weights), to_dev(w.bn)
+    h = B.fp_fuse(w.net, dw, dbn, w.batch, B.FP_COMPUTE_BF16_TC, B.FP_DTYPE_BF16, 0, 0, 0, pool)
+    try:
+        B.fp_prune(h, narrow)
+        few_activations, want = pool.bytes, forward(B, h, w)
+        B.fp_prune(h, wide)
+        pool.limit = max(pool.bytes, few_activations)
+        B.fp_prune(h, narrow)
+        np.testing.assert_array_equal(forward(B, h, w), want)
+        B.fp_prune(h, wide)
+    finally:
+        B.fp_destroy(h)
+    assert not pool.live
+
+
+def test_pruning_gives_memory_back(B):
+    w = wl.Workload("straight", straight_net(24), 2, 67, True, wl.uniform_ratios(0.0), "none")
+    dw, dbn = to_dev(w.weights), to_dev(w.bn)
+    h = B.fp_fuse(w.net, dw, dbn, 8192, B.FP_COMPUTE_BF16_TC, B.FP_DTYPE_BF16, 0, 1)
+    try:
+        free = lambda: torch.cuda.mem_get_info()[0]                  # noqa: E731
+        before = free()
+        B.fp_prune(h, np.array([0.75, 0.75, 0, 0, 0, 0, 0]))
+        # the first two layers' outputs, 64 -> 16 channels of 26 x 26 positions, less a quarter of what is left of all layers'
+        freed, kept = 2 * 8192 * 26 * 26 * 48 * 2, free() - before
+        assert kept > freed // 2
+        small = forward(B, h, w)
+        B.fp_prune(h, np.zeros(7))
+        forward(B, h, w)
+        B.fp_prune(h, np.array([0.75, 0.75, 0, 0, 0, 0, 0]))
+        np.testing.assert_array_equal(forward(B, h, w), small)
+    finally:
+        B.fp_destroy(h)

@@ -212,7 +212,10 @@ typedef enum {
                                 Without keep_outputs the launches up to that operator are run again first (the
                                 last input must still be alive), and a layer inside a fused run, whose output
                                 never reaches memory, is refused with FP_ERR_UNSUPPORTED - the run's last
-                                layer can be read */
+                                layer can be read, and every strided one.  A first convolution that is pooled in
+                                its own kernel, and a projection computed inside the layer that adds it, are
+                                planned apart for the query and the graph is planned again behind it, which takes
+                                memory as fp_prune does */
     FP_Q_DEVICE_STATUS = 12, /* int32: 0, or FP_ERR_TIMEOUT if a bounded device wait ran out since the last query
                                 (the flag is cleared by the query that reports it); synchronises with the device's
                                 earlier work through the copy that reads it                             */

@@ -191,6 +191,7 @@ struct fp_handle_s {
     fp::StemPoolArgs stem_args;
     fp::StemPoolPlan stem_plan;
     int scatter_policy = 0;                // fp_model_desc::scatter
+    int apart = -1;                        // operator that FP_Q_OP_OUTPUT asks for: planned as a launch of its own
     int planned = 0;                       // 1: buffers, packed banks and launch plans match the masks (set by replan)
     int act_is_bf16() const { return compute != FP_COMPUTE_FP32; }
     size_t act_elem() const { return act_is_bf16() ? 2 : 4; }
@@ -801,7 +802,7 @@ void find_net(fp_handle h, const std::vector<std::vector<Use>>& uses) {
     h->d_net_tables.clear();
     h->net_spec.layers.clear();
     const int n_ops = (int)h->ops.size();
-    if (h->compute != FP_COMPUTE_BF16_TC || h->keep_outputs || n_ops < 3 || h->in_C > 8 || h->stem_packed || h->stem_fused || uses[0].size() != 1) return;
+    if (h->compute != FP_COMPUTE_BF16_TC || h->keep_outputs || n_ops < 3 || h->apart == 0 || h->in_C > 8 || h->stem_packed || h->stem_fused || uses[0].size() != 1) return;
     int off = 0;
     for (int i = 1; i + 1 < n_ops; ++i) {
         if (h->ops[i].kind != 0) return;
@@ -1021,7 +1022,7 @@ fp_status build_plan(fp_handle h) {
     // pooling run as one kernel (decided below, once the filter count is known).
     h->stem_fused = 0;
     bool stem_candidate = false;
-    if (stem7 && !h->keep_outputs && h->ops.size() >= 3 && h->ops[1].kind == 0 &&
+    if (stem7 && !h->keep_outputs && h->apart != 0 && h->apart != 1 && h->ops.size() >= 3 && h->ops[1].kind == 0 &&
         h->ops[2].kind == 1) {
         const FConv& f = h->convs[h->ops[1].idx];
         const Pool& pl = h->pools[h->ops[2].idx];
@@ -1143,7 +1144,7 @@ fp_status build_plan(fp_handle h) {
             if (h->compute == FP_COMPUTE_BF16_TC && !h->keep_outputs && f.res_mode == 1 && f.R == 1 && f.S == 1 && f.stride == 1 &&
                 f.pad == 0 && !f.scatter && !src.split && !out.split && uses[f.res_tid].size() == 1) {
                 const Tensor& rt = h->tensors[f.res_tid];
-                if (rt.producer >= 0 && h->ops[rt.producer].kind == 0) {
+                if (rt.producer >= 0 && rt.producer != h->apart && h->ops[rt.producer].kind == 0) {
                     const int cand = h->ops[rt.producer].idx;
                     const FConv& q = h->convs[cand];
                     const Tensor& X = h->tensors[q.src];
@@ -1184,7 +1185,7 @@ fp_status build_plan(fp_handle h) {
                 f.stride == 1 && f.pad == 1 && !f.scatter && !src.split && !out.split && uses[f.res_tid].size() == 1 && f.tc.valid &&
                 f.tc.flat && !f.tc.b_resident && (f.tc.blocked_bank == 0 || f.tc.split) && !(h->stem_packed && f.src == 0)) {
                 const Tensor& rt = h->tensors[f.res_tid];
-                if (rt.producer >= 0 && h->ops[rt.producer].kind == 0) {
+                if (rt.producer >= 0 && rt.producer != h->apart && h->ops[rt.producer].kind == 0) {
                     const int cand = h->ops[rt.producer].idx;
                     FConv& q = h->convs[cand];
                     const Tensor& X = h->tensors[q.src];
@@ -2085,6 +2086,21 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
                 return fail(FP_ERR_ARG, "fp_query: operator %d has no activation output", index);
             if (h->last_batch <= 0) return fail(FP_ERR_ARG, "fp_query: no forward has run yet");
             TRY(need_plan(h, "fp_query"));
+            // What is computed inside another launch, but on the operator's own terms - the first convolution behind which the pooling
+            // follows, a projection inside the layer that adds it, the input's conversion where it has a plain form - is planned as
+            // a launch of its own for this query, and the graph planned again behind it.
+            if (h->apart < 0 && ((h->stem_fused && (index == 1 || (index == 0 && (h->in_H % 2 || h->in_W % 2)))) ||
+                                 (h->ops[index].kind == 0 && h->convs[h->ops[index].idx].absorbed) ||
+                                 (h->net_on && index == 0 && h->convs[h->ops[1].idx].stride == 2))) {
+                h->apart = index;
+                fp_status s = replan(h);
+                if (s == FP_OK) s = fp_query(h, what, index, h_out, bytes);
+                const std::string message = g_err;
+                h->apart = -1;
+                TRY(replan(h));
+                if (s != FP_OK) g_err = message;
+                return s;
+            }
             if (h->ops[index].kind == 3 && h->stem_packed) return fail(FP_ERR_UNSUPPORTED, "fp_query: the network input is stored in packed form");
             if (h->ops[index].kind == 3 && (h->input_fused || h->stem_fused)) return fail(FP_ERR_UNSUPPORTED, "fp_query: the network input is converted inside the first fused run "
                                                                         "and never stored (set keep_outputs to run every layer on its own)");
@@ -2092,9 +2108,10 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             const int tid = op.kind == 0 ? h->convs[op.idx].out : op.kind == 1 ? h->pools[op.idx].out : 0;
             const Tensor& t = h->tensors[tid];
             if (h->net_on) {
-                // the last layer of every resolution can be read: the network runs again and writes that layer's output out
+                // the last layer of every resolution and the strided ones can be read, as where only the layers between them run as one:
+                // the network runs again and writes that layer's output out
                 const FConv& f = h->convs[op.idx];
-                if (index + 2 < (int)h->ops.size() && h->convs[h->ops[index + 1].idx].stride == 1)
+                if (index + 2 < (int)h->ops.size() && f.stride == 1 && h->convs[h->ops[index + 1].idx].stride == 1)
                     return fail(FP_ERR_UNSUPPORTED, "fp_query: operator %d runs inside the network's kernel and its output never reaches memory "
                                 "(set keep_outputs to run every layer on its own)", index);
                 const size_t cnt = (size_t)h->last_batch * t.C * t.H * t.W, vecs = (size_t)(t.C_pad / 8) * h->last_batch * (t.H + 2) * (t.W + 2);

@@ -201,7 +201,7 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
                     long long wait_cycles = 0);
 
 // First convolution (7x7 / stride 2 / pad 3, at most 3 input channels, ReLU) and the 3x3 / stride 2 / pad 1 max pooling
-// behind it as one kernel that reads the NCHW network input (images up to 256 wide) and writes the pooled tensor.
+// behind it as one kernel that reads the NCHW network input  and writes the pooled tensor.
 struct StemPoolArgs {
     const void* x;        // network input, N x C x H x W, NCHW, bf16 or fp32 (rounded to bf16 on load)
     void* y;              // pooled tensor, planar-8 with border, K_pad channels, N images

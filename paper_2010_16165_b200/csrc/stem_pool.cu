@@ -18,6 +18,9 @@
 //                  shared memory, each made once; convolution rows through a ring of accumulators, each computed once (the
 //                  row that two pooled rows share is carried over in registers); a run starts with one extra row, an
 //                  image with none.  Two CTAs share an SM.
+//   Parts          Where a row has more than 128 convolution columns, or there are more than 64 filters, a CTA takes a strip of the
+//                  pooled columns (its tile begins one convolution column to the left of them) and a part of the filters; strips and
+//                  parts are the grid's other dimensions.  Every part makes the half-resolution rows it reads itself.
 //   Roles          five warps turn input rows into half-resolution rows (a thread per pixel: one load per channel and row
 //                  parity gives both column parities; the next row's are asked for before this one's place is waited
 //                  for), one warp issues the MMAs, eight warps pool.
@@ -51,9 +54,10 @@ constexpr int kBlocks = 7;                 // filter blocks of a column tap: ta 
 struct SpParams {
     StemPoolArgs a;
     int Hc, Wc, Hp, Wp;            // convolution and pooled sizes
-    int pitch;                     // half-resolution pixels per row: Wc + 3 (columns -2 .. Wc)
+    int strip, k_tile;             // pooled columns of a strip and filters of a part (the last ones may have fewer); Wp and K_pad where there is one
+    int pitch;                     // half-resolution pixels per row of a strip: its convolution columns and 3 more (-2 .. +1)
     int plane;                     // 16-byte rows per chunk of the ring (kRing * pitch, plus what the last row's taps reach)
-    int b_bytes;                   // filters: 4 column taps * 2 chunks * 7 blocks * K_pad * 16
+    int b_bytes;                   // filters: 4 column taps * 2 chunks * 7 blocks * k_tile * 16
     int tmem_cols;
     int rows;                      // pooled rows of all images
     int* status;
@@ -114,12 +118,15 @@ __device__ __forceinline__ void load_pixel(const uint8_t* at, int row_bytes, siz
     }
 }
 
-template <bool F32, int C>
+// PARTS: there are several strips or parts of the filters (W > 256 or K_pad > 64).
+template <bool F32, int C, bool PARTS>
 __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p, const int paired) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     SpCtrl* ctrl = reinterpret_cast<SpCtrl*>(smem_raw);
     const uint32_t base = smem_u32(smem_raw);
-    const int K_pad = p.a.K_pad;
+    const int k_base = PARTS ? (int)blockIdx.z * p.k_tile : 0, K_pad = PARTS ? min(p.k_tile, p.a.K_pad - k_base) : p.a.K_pad;
+    const int x0 = PARTS ? (int)blockIdx.y * p.strip : 0, Wp = PARTS ? min(p.strip, p.Wp - x0) : p.Wp;       // this CTA's pooled columns
+    const int left = x0 > 0, c0 = 2 * x0 - left, Wc = PARTS ? min(p.Wc - c0, 2 * Wp + left) : p.Wc;         // and convolution columns
     const uint32_t b_addr = (base + (uint32_t)sizeof(SpCtrl) + 127u) & ~127u;
     const uint32_t x_addr = b_addr + (uint32_t)p.b_bytes;
     uint4* ring = reinterpret_cast<uint4*>(smem_raw + (x_addr - base));
@@ -139,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
     }
     // the places of the columns left and right of the row: zero, and never written
     for (int i = threadIdx.x; i < 4 * (K_pad >> 3); i += kThreads)
-        (ring + 2 * p.plane)[(size_t)(i >> 1) * (2 * p.Wp + 1) + p.Wp + (i & 1) * p.Wp] = make_uint4(0, 0, 0, 0);
+        (ring + 2 * p.plane)[(size_t)(i >> 1) * (2 * Wp + 1) + Wp + (i & 1) * Wp] = make_uint4(0, 0, 0, 0);
     if (warp == kRowWarps) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(base + (uint32_t)offsetof(SpCtrl, tmem_base)), "r"((uint32_t)p.tmem_cols) : "memory");
@@ -152,11 +159,11 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
     // filters: resident for the whole kernel (they are not written by the previous kernel in the stream)
     if (warp == 0) {
         const uint32_t block = (uint32_t)K_pad * 16u;
-        if (lane == 0) mbar_expect_tx(b_full, (uint32_t)p.b_bytes);
+        if (lane == 0) mbar_expect_tx(b_full, 8u * kBlocks * block);
         __syncwarp();
         for (int i = lane; i < 8 * kBlocks; i += 32) {
             const int plane = i / kBlocks, blk = i - plane * kBlocks, tb = plane >> 1, ta = 3 - (blk & 3);
-            bulk_copy(b_addr + (uint32_t)i * block, reinterpret_cast<const uint8_t*>(p.a.w) + (size_t)((ta * 4 + tb) * 2 + (plane & 1)) * block, block, b_full);
+            bulk_copy(b_addr + (uint32_t)i * block, reinterpret_cast<const uint8_t*>(p.a.w) + (size_t)((ta * 4 + tb) * 2 + (plane & 1)) * (size_t)(p.a.K_pad * 16) + k_base * 16, block, b_full);
         }
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -166,10 +173,10 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
     bool ok = true;
     if (warp < kRowWarps) {
         // ------------------------------ half-resolution rows ------------------------------
-        const int jx = threadIdx.x;                      // pixel of the row: half-resolution column jx - 2
+        const int jx = threadIdx.x;                      // pixel of the row: half-resolution column c0 + jx - 2
         const bool mine = jx < p.pitch;
         constexpr int elem = F32 ? 4 : 2;
-        const int col = 2 * (jx - 2), row_bytes = p.a.W * elem;
+        const int col = 2 * (c0 + jx - 2), row_bytes = p.a.W * elem;
         const size_t plane_bytes = (size_t)p.a.H * row_bytes;
         const bool in = (unsigned)col < (unsigned)p.a.W, second = col + 1 < p.a.W;
         uint32_t slot = 0, phase = 0;
@@ -269,13 +276,13 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
         const int pw = warp - (kRowWarps + 1), quarter = warp & 3, half = pw >> 2;
         const int col = quarter * 32 + lane;             // convolution column; the lower or the upper half of the filter groups
         const int first_group = half ? ((K_pad >> 4) + 1) >> 1 : 0, groups = half ? (K_pad >> 4) - first_group : ((K_pad >> 4) + 1) >> 1;
-        const bool live = col < p.Wc;
+        const bool live = col < Wc;
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + 16u * (uint32_t)min(first_group, (K_pad >> 4) - 1);
-        const int Wq = p.Wp + 2, P2o = (p.Hp + 2) * Wq, pitch = 2 * p.Wp + 1;
+        const int Wq = p.Wp + 2, P2o = (p.Hp + 2) * Wq, pitch = 2 * Wp + 1;
         const long long plane_out = (long long)p.a.N * P2o;
         uint4* yout = reinterpret_cast<uint4*>(p.a.y);
         uint4* cols_s = reinterpret_cast<uint4*>(smem_raw + (x_addr - base)) + 2 * p.plane;      // [row parity][chunk]: even columns, then odd ones from -1 on
-        const int place = col & 1 ? p.Wp + ((col + 1) >> 1) : col >> 1;
+        const int off = col - left, place = off & 1 ? Wp + ((off + 1) >> 1) : off >> 1;      // off: from the strip's first even column
         uint32_t acc = 0, acc_phase = 0;
         uint32_t m[2][8];                                // the convolution row above the pooled row's two, then the maxima with them: bf16 pairs
         // The next convolution row, ReLU and bf16 (the filters' shifts are in the sums): use(group, row, carried row or maxima so far).
@@ -338,20 +345,21 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
                 for (int ch = quarter; ch < 2 * groups; ch += 4) {
                     const int chunk = 2 * first_group + ch;
                     const uint4* from = cols_s + (size_t)(parity * (K_pad >> 3) + chunk) * pitch;
-                    uint4* to = yout + (long long)chunk * plane_out + (long long)s.n * P2o + (long long)(q + 1) * Wq;
-                    for (int k0 = lane; k0 < Wq; k0 += 64) {
+                    uint4* to = yout + (long long)((k_base >> 3) + chunk) * plane_out + (long long)s.n * P2o + (long long)(q + 1) * Wq + x0;
+                    for (int k0 = lane; k0 < Wp + 2; k0 += 64) {
                         uint4 l[2], c[2], r[2];          // two positions' loads in flight
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {    // columns 2k - 3 .. 2k - 1
-                            const int k = max(1, min(k0 + 32 * i, p.Wp));
-                            l[i] = from[p.Wp + k - 1]; c[i] = from[k - 1]; r[i] = from[p.Wp + k];
+                            const int k = max(1, min(k0 + 32 * i, Wp));
+                            l[i] = from[Wp + k - 1]; c[i] = from[k - 1]; r[i] = from[Wp + k];
                         }
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
                             const int k = k0 + 32 * i;
-                            if (k >= Wq) break;
+                            if (k >= Wp + 2) break;
+                            if (PARTS && ((k == 0 && x0 > 0) || (k == Wp + 1 && x0 + Wp < p.Wp))) continue;      // another strip's column
                             uint4 o = make_uint4(0, 0, 0, 0);
-                            if (k >= 1 && k <= p.Wp)
+                            if (k >= 1 && k <= Wp)
                                 o = make_uint4(max3(l[i].x, c[i].x, r[i].x), max3(l[i].y, c[i].y, r[i].y), max3(l[i].z, c[i].z, r[i].z), max3(l[i].w, c[i].w, r[i].w));
                             to[k] = o;
                             if (q == 0) to[k - Wq] = make_uint4(0, 0, 0, 0);
@@ -380,28 +388,36 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
 
 constexpr unsigned kSmemMax = 233472u / 2 - 1024u;       // two CTAs on an SM
 
-struct Shape { int Hc, Wc, Hp, Wp, pitch, plane, b_bytes; unsigned smem; };
+struct Shape { int Hc, Wc, Hp, Wp, strips, strip, parts, k_tile, pitch, plane, b_bytes; unsigned smem; };
 Shape shape_of(int H, int W, int K_pad) {
     Shape s;
     s.Hc = (H - 1) / 2 + 1; s.Wc = (W - 1) / 2 + 1; s.Hp = (s.Hc - 1) / 2 + 1; s.Wp = (s.Wc - 1) / 2 + 1;
-    s.pitch = s.Wc + 3;
+    // a strip's convolution columns - two for a pooled one, and one to the left - are a tile of 128
+    s.strips = s.Wc <= 128 ? 1 : (s.Wp + 62) / 63;
+    s.strip = (s.Wp + s.strips - 1) / s.strips;
+    s.parts = (kAcc * K_pad + 255) / 256;
+    s.k_tile = (K_pad / 16 + s.parts - 1) / s.parts * 16;
+    s.pitch = std::min(s.Wc, s.strips == 1 ? s.Wc : 2 * s.strip + 1) + 3;
     s.plane = (kRing * s.pitch + 128 + 7) & ~7;
-    s.b_bytes = 8 * kBlocks * K_pad * 16;
+    s.b_bytes = 8 * kBlocks * s.k_tile * 16;
     s.smem = (unsigned)sizeof(SpCtrl) + 128u + (unsigned)s.b_bytes + 2u * (unsigned)s.plane * 16u +
-             2u * (unsigned)(K_pad / 8) * (unsigned)(2 * s.Wp + 1) * 16u;
+             2u * (unsigned)(s.k_tile / 8) * (unsigned)(2 * s.strip + 1) * 16u;
     return s;
 }
 
 typedef void (*StemKernel)(const SpParams, const int);
-template <bool F32>
-StemKernel kernel_of(int C) { return C == 3 ? stem_pool_kernel<F32, 3> : C == 2 ? stem_pool_kernel<F32, 2> : stem_pool_kernel<F32, 1>; }
-StemKernel kernel_of(const StemPoolArgs& a) { return a.in_f32 ? kernel_of<true>(a.C) : kernel_of<false>(a.C); }
+template <bool F32, bool PARTS>
+StemKernel kernel_of(int C) { return C == 3 ? stem_pool_kernel<F32, 3, PARTS> : C == 2 ? stem_pool_kernel<F32, 2, PARTS> : stem_pool_kernel<F32, 1, PARTS>; }
+StemKernel kernel_of(const StemPoolArgs& a) {
+    const Shape s = shape_of(a.H, a.W, a.K_pad);
+    if (s.strips * s.parts > 1) return a.in_f32 ? kernel_of<true, true>(a.C) : kernel_of<false, true>(a.C);
+    return a.in_f32 ? kernel_of<true, false>(a.C) : kernel_of<false, false>(a.C);
+}
 
 }  // namespace
 
-// A convolution row is one tile of 128 positions, so images up to 256 wide; four rows' filters are one MMA's, so up to 64.
 bool stem_pool_supported(int C, int H, int W, int K_pad) {
-    if (C < 1 || C > 3 || H < 8 || W < 8 || W > 256 || K_pad % 16 || K_pad < 16 || kAcc * K_pad > 256) return false;
+    if (C < 1 || C > 3 || H < 8 || W < 8 || W > kMaxWidth || K_pad % 16 || K_pad < 16 || K_pad > 128) return false;
     return shape_of(H, W, K_pad).smem <= kSmemMax;
 }
 
@@ -410,7 +426,7 @@ int plan_stem_pool(const StemPoolArgs& a, StemPoolPlan* plan, char* err, size_t 
     if (!stem_pool_supported(a.C, a.H, a.W, a.K_pad)) { snprintf(err, err_len, "first convolution + pooling: shape not supported"); return 1; }
     plan->smem_bytes = shape_of(a.H, a.W, a.K_pad).smem;
     plan->tmem_cols = 64;
-    while (plan->tmem_cols < kAcc * a.K_pad) plan->tmem_cols *= 2;           // at most half of an SM's, for two CTAs
+    while (plan->tmem_cols < kAcc * shape_of(a.H, a.W, a.K_pad).k_tile) plan->tmem_cols *= 2;           // at most half of an SM's, for two CTAs
     if (cudaFuncSetAttribute(kernel_of(a), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
         snprintf(err, err_len, "cannot raise the dynamic shared memory limit");
         cudaGetLastError();
@@ -425,7 +441,7 @@ void launch_stem_pool(const StemPoolPlan& plan, const StemPoolArgs& a, int* d_st
     memset(&p, 0, sizeof(p));
     const Shape s = shape_of(a.H, a.W, a.K_pad);
     p.a = a;
-    p.Hc = s.Hc; p.Wc = s.Wc; p.Hp = s.Hp; p.Wp = s.Wp; p.pitch = s.pitch; p.plane = s.plane; p.b_bytes = s.b_bytes;
+    p.Hc = s.Hc; p.Wc = s.Wc; p.Hp = s.Hp; p.Wp = s.Wp; p.strip = s.strip; p.k_tile = s.k_tile; p.pitch = s.pitch; p.plane = s.plane; p.b_bytes = s.b_bytes;
     p.tmem_cols = plan.tmem_cols;
     p.rows = a.n_count * s.Hp;
     p.status = d_status;
@@ -433,7 +449,7 @@ void launch_stem_pool(const StemPoolPlan& plan, const StemPoolArgs& a, int* d_st
     const int paired = a.W % 2 == 0 && (uintptr_t)a.x % (a.in_f32 ? 8 : 4) == 0;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)std::max(1, std::min(2 * sm_count(), p.rows)));
+    cfg.gridDim = dim3((unsigned)std::max(1, std::min(2 * sm_count() / (s.strips * s.parts), p.rows)), (unsigned)s.strips, (unsigned)s.parts);
     cfg.blockDim = dim3((unsigned)kThreads);
     cfg.dynamicSmemBytes = plan.smem_bytes;
     cfg.stream = st;

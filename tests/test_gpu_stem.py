@@ -48,3 +48,13 @@ def test_stem_sizes(B, fpo, H, W, K, C, batch, bf16):
         np.testing.assert_array_equal(out.cpu().numpy().astype(np.float64), got)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("H, W, K, C, batch", [
+    (13, 257, 48, 3, 2), (21, 258, 16, 3, 3), (32, 288, 64, 3, 2), (17, 399, 24, 2, 2), (12, 504, 40, 1, 3), (9, 511, 64, 3, 1), (24, 512, 64, 3, 2),
+    (30, 40, 65, 3, 9), (23, 100, 80, 3, 40), (16, 184, 96, 3, 5), (11, 256, 112, 1, 2), (40, 33, 128, 3, 7), (18, 290, 128, 3, 2), (26, 381, 100, 2, 1),
+])
+@pytest.mark.parametrize("bf16", [True, False])
+def test_rows_in_strips_and_filters_in_parts(B, fpo, H, W, K, C, batch, bf16):
+    """More than 128 convolution columns, more than 64 filters: at the edges of the strips and parts, with one and several CTAs each."""
+    test_stem_sizes(B, fpo, H, W, K, C, batch, bf16)

@@ -850,8 +850,15 @@ void find_net(fp_handle h, const std::vector<std::vector<Use>>& uses) {
 // The network as one kernel, given to the CTAs the way that is cheapest for this batch: rounds over the GPU times the cost of a
 // round (ResNet-56: clusters of four 84 us, of two 104 us, a CTA of sixteen warps per image 137 us, pairs of images 221 us).
 // What full rounds of pairs leave over goes the way that is cheapest for it, in a launch of its own.
+// (A fixed array: a forward allocates nothing that could throw.)
 struct NetPart { int plan, images; };
-std::vector<NetPart> network_parts(fp_handle h, int batch) {
+struct NetParts {
+    NetPart part[2];
+    int n = 0;
+    const NetPart* begin() const { return part; }
+    const NetPart* end() const { return part + n; }
+};
+NetParts network_parts(fp_handle h, int batch) {
     auto cheapest = [&](int n) {
         int best = 0;
         double best_cost = 0;
@@ -863,14 +870,14 @@ std::vector<NetPart> network_parts(fp_handle h, int batch) {
         }
         return best;
     };
-    std::vector<NetPart> parts;
+    NetParts parts;
     const fp::NetPlan& last = h->net_plans.back();
     const int pairs = last.G == 2 ? batch / (2 * fp::net_at_once(1)) * 2 * fp::net_at_once(1) : 0, rest = batch - pairs;
-    if (pairs > 0) parts.push_back({(int)h->net_plans.size() - 1, pairs});
+    if (pairs > 0) parts.part[parts.n++] = {(int)h->net_plans.size() - 1, pairs};
     if (rest > 0) {
         const int k = cheapest(rest);
-        if (!parts.empty() && k == parts[0].plan) parts[0].images += rest;
-        else parts.push_back({k, rest});
+        if (parts.n && k == parts.part[0].plan) parts.part[0].images += rest;
+        else parts.part[parts.n++] = {k, rest};
     }
     return parts;
 }
@@ -1514,8 +1521,8 @@ fp::NetArgs network_args(fp_handle h) {
 void launch_network(fp_handle h, const void* d_input, int batch, float* d_logits, cudaStream_t st, int dump_layer = -1, void* dump = nullptr) {
     fp::NetArgs a = network_args(h);
     a.dump_layer = dump_layer; a.dump = dump;
-    std::vector<NetPart> parts = network_parts(h, batch);
-    if (dump) parts.assign(1, {parts[0].plan, batch});                // (the dumped tensor is the whole batch's)
+    NetParts parts = network_parts(h, batch);
+    if (dump) { parts.part[0].images = batch; parts.n = 1; }                // (the dumped tensor is the whole batch's)
     int done = 0;
     for (const NetPart& part : parts) {
         a.x = (const uint8_t*)d_input + (size_t)done * h->in_C * h->in_H * h->in_W * h->in_elem();
@@ -2028,7 +2035,7 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             n -= h->input_fused;
             n -= 2 * h->stem_fused;                                          // conversion, convolution and pooling are one
             for (const FConv& c : h->convs) n -= c.absorbed;                 // a projection inside the layer that adds it
-            *(int32_t*)h_out = h->net_on ? (int)network_parts(h, h->last_batch > 0 ? h->last_batch : h->max_batch).size() : n;
+            *(int32_t*)h_out = h->net_on ? network_parts(h, h->last_batch > 0 ? h->last_batch : h->max_batch).n : n;
             return FP_OK;
         }
         case FP_Q_CONV_K_FUSED: TRY(need(4)); TRY(conv_of(&f)); *(int32_t*)h_out = f ? f->K : 0; return FP_OK;

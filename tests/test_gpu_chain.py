@@ -3,6 +3,11 @@ shared memory): against the CPU oracle, and against the library's own layer-by-l
 
 The fused kernel is chosen by the library when `keep_outputs` is 0 and a run of stride-1 3x3 convolutions
 works on images 8, 16 or 32 pixels wide; with `keep_outputs` = 1 every layer runs on its own.
+
+A network that is made of such layers alone may be ONE launch (resident_net.cu, test_gpu_resident_net.py): the "cifar32" cases, the
+600-image test, the operator times and the pruned half of the aggressive test run there, and what they assert holds for both kernels.
+The runs of layers have "cifar16", "cifar8_one_stage", "imagenet_projection", the non-square images, the unpruned aggressive network,
+and the large batches at the end of this file.
 """
 import numpy as np
 import pytest
@@ -156,5 +161,26 @@ def test_operator_times_add_up(B):
                 if o.chain in seen:
                     assert t == 0
                 seen.add(o.chain)
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("widths, per_stage, runs", [((16, 48, 72), 2, 2), ((32, 72), 3, 1)])
+def test_runs_of_layers_at_large_batches(B, fpo, widths, per_stage, runs):
+    """More filters in the last stage than the one-kernel form takes: several images per group, several groups per CTA, a last group that
+    is not full."""
+    net = wl.resnet_cifar(per_stage, widths, in_hw=32, n_classes=9, name="wide_cifar")
+    w = wl.Workload("wide_cifar", net, 11, 73, True, wl.uniform_ratios(0.1), "uniform 0.1")
+    gp, _, _, _ = oracle_pruned(fpo, w)
+    g = Gpu(B, w, B.FP_COMPUTE_BF16_TC, max_batch=701)
+    try:
+        B.fp_prune(g.h, w.ratios)
+        assert len(_runs(B, g.h)) == runs
+        full = g.forward(w.x)
+        assert B.fp_query_int(g.h, B.FP_Q_N_LAUNCHES) >= 5           # runs, strided layers, the last stage's layers, two head kernels
+        assert err(full, fpo.fused_forward(gp, w.x)) < TOL_BF16
+        for n in (1, 148, 149, 297, 445, 600, 701):
+            x = np.concatenate([w.x] * 64)[:n]
+            np.testing.assert_array_equal(g.forward(x), np.concatenate([full] * 64)[:n])
     finally:
         g.close()

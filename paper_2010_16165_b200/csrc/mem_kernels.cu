@@ -357,12 +357,12 @@ __global__ void pool_sum_kernel(const void* x, int N, int H, int W, int chunks, 
 // butterfly.  CPW: every sum read from shared memory serves CPW classes, which bounds large batches (128 images x 1000 classes
 // x 2048 channels: 7 us of FMAs at full rate, four classes a warp bring the shared-memory reads down to that); one class a warp
 // spreads the FC matrix of a single image over 125 SMs instead of 32.
-constexpr int kFcWarps = 8, kFcSlab4 = 512;         // channels / 4 held at a time
+constexpr int kFcWarps = 8, kFcSlab4 = 512, kFcPitch4 = kFcSlab4 + 1;       // channels / 4 held at a time, and a zero behind them
 // AHEAD: places of the rows a lane has on the way at a time; a place is asked for again as soon as it has been used.
 template <int IMAGES, int CPW, int AHEAD>
 __global__ void __launch_bounds__(32 * kFcWarps, 2) fc_kernel(const float* sums, int N, int C_pad, const float* __restrict__ fcw,
                                                            const float* __restrict__ fcb, int n_classes, float* __restrict__ logits) {
-    extern __shared__ float4 sh4[];        // IMAGES x kFcSlab4
+    extern __shared__ float4 sh4[];        // IMAGES x kFcPitch4
     const int n0 = blockIdx.x * IMAGES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k0 = ((int)(blockIdx.z * gridDim.y + blockIdx.y) * kFcWarps + warp) * CPW, c4 = C_pad >> 2;
@@ -384,20 +384,21 @@ __global__ void __launch_bounds__(32 * kFcWarps, 2) fc_kernel(const float* sums,
 #pragma unroll
         for (int i = 0; i < IMAGES; ++i) acc[t][i] = 0.0f;
     for (int slab = 0; slab < c4; slab += kFcSlab4) {
-        // (zeros behind the last channel, where the rows' are zeros too: a sum that is infinite there would make them NaN)
-        const int n4 = min(kFcSlab4, c4 - slab), padded = (n4 + 32 * AHEAD - 1) / (32 * AHEAD) * (32 * AHEAD);
+        const int n4 = min(kFcSlab4, c4 - slab);
         if (slab) __syncthreads();         // the previous slab has been consumed
         for (int img = warp; img < IMAGES; img += kFcWarps) {
             const float4* from = reinterpret_cast<const float4*>(sums + (size_t)(n0 + min(img, images - 1)) * C_pad) + slab;
-            for (int i = lane; i < padded; i += 32) sh4[img * kFcSlab4 + i] = i < n4 ? from[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int i = lane; i < n4; i += 32) sh4[img * kFcPitch4 + i] = from[i];
+            if (lane == 0) sh4[img * kFcPitch4 + n4] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
         __syncthreads();
         for (int c = lane; c < n4; c += 32 * AHEAD) {                // (a slab that is not the last is a multiple of that)
 #pragma unroll
             for (int i = 0; i < AHEAD; ++i) {
+                const int cc = min(c + 32 * i, n4);      // behind the last channel a zero, as the rows' are: a sum that is infinite would make them NaN
 #pragma unroll
                 for (int img = 0; img < IMAGES; ++img) {
-                    const float4 s = sh4[img * kFcSlab4 + c + 32 * i];
+                    const float4 s = sh4[img * kFcPitch4 + cc];
 #pragma unroll
                     for (int t = 0; t < CPW; ++t)
                         acc[t][img] = fmaf(s.w, w[t][i].w, fmaf(s.z, w[t][i].z, fmaf(s.y, w[t][i].y, fmaf(s.x, w[t][i].x, acc[t][img]))));
@@ -506,12 +507,12 @@ void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, con
     // (65535 blocks are the most along y; a matrix of more classes goes on along z)
     const unsigned class_blocks = (unsigned)((n_classes + kFcWarps * cpw - 1) / (kFcWarps * cpw)), along_y = std::min(class_blocks, 65535u);
     cfg.gridDim = dim3((unsigned)groups, along_y, (class_blocks + along_y - 1) / along_y);
-    cfg.dynamicSmemBytes = (size_t)images * kFcSlab4 * sizeof(float4);
+    cfg.dynamicSmemBytes = (size_t)images * kFcPitch4 * sizeof(float4);
     static std::atomic<bool> raised[64];   // per device, once (threads may all be the first)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !raised[dev]) {
         for (Fc f : {(Fc)fc_kernel<8, 1, 8>, (Fc)fc_kernel<8, 2, 4>, (Fc)fc_kernel<8, 4, 2>})
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * kFcSlab4 * sizeof(float4)));
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * kFcPitch4 * sizeof(float4)));
         if (dev >= 0 && dev < 64) raised[dev] = true;
     }
     cudaLaunchKernelEx(&cfg, fn, (const float*)pool_scratch, N, C_pad, fcw, fcb, n_classes, logits);

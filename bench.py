@@ -272,18 +272,14 @@ def percentile(v, q):
 
 
 def kernel_report(B, m, peaks, peak_kind, reps):
-    """Per-kernel-class figures of one forward from the library's per-operator times: the convolution class that
-    takes more of the step (the `roofline` object), and the memory-bound side kernels."""
+    """Per-kernel figures of one forward from the library's per-operator times: the convolution kernel that
+    takes most of the step (the `roofline` object), and the memory-bound side kernels."""
     w = m.w
     ops = B.op_infos(m.h)
     op_ms = B.fp_query_array(m.h, B.FP_Q_OP_TIMES, reps, np.float32, len(ops))
-    # Convolution launches fall in two classes: fused runs of layers (one chain_tc_kernel launch per run, or
-    # resident_net_kernel where the whole network is one run; its time reported at the run's first layer) and
-    # single layers (conv_tc_kernel, conv_split_kernel).  Algorithmic bytes and flops are the per-layer figures
-    # summed over the layers a launch executes.
-    whole = all(o.chain == 0 for o in ops if o.kind == 0) and B.fp_query_int(m.h, B.FP_Q_N_LAUNCHES) <= 2
-    runs = "resident_net_kernel" if whole else "chain_tc_kernel"
-    classes = {runs: [0, 0.0, 0.0, 0.0], "conv_tc_kernel": [0, 0.0, 0.0, 0.0]}
+    # Convolution launches by the kernel that computes them; a run's or a whole network's time is reported at its first layer.
+    # Algorithmic bytes and flops are the per-layer figures summed over the layers a launch executes.
+    classes = {}
     side = {}
     seen_runs = set()
     for o, t in zip(ops, op_ms):
@@ -294,7 +290,7 @@ def kernel_report(B, m, peaks, peak_kind, reps):
             s[1] += float(t)
             s[2] += o.bytes_per_image * w.batch + o.bytes_fixed
             continue
-        c = classes[runs if o.chain >= 0 else "conv_tc_kernel"]
+        c = classes.setdefault(B.CONV_KERNELS[o.kernel], [0, 0.0, 0.0, 0.0])
         if o.chain < 0 and t <= 0 and o.flops_per_image == 0:
             continue                   # a projection shortcut computed inside the layer that adds it: no launch of its own
         if o.chain < 0 or o.chain not in seen_runs:

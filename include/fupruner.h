@@ -231,6 +231,9 @@ typedef enum {
     FP_Q_CONV_BANK_ELEMS = 15 /* int64: weights in the fused fp32 bank of conv `index` (K_fused*C_fused*R*S), 0 if absorbed */
 } fp_query_what;
 
+enum { FP_KERNEL_CONV_TC = 1, FP_KERNEL_CONV_SPLIT = 2, FP_KERNEL_STEM_POOL = 3, FP_KERNEL_CHAIN_TC = 4, FP_KERNEL_RESIDENT_NET = 5,
+       FP_KERNEL_CONV_SIMT = 6 };   /* fp_op_info::kernel */
+
 typedef struct {
     int32_t kind;            /* 0 conv, 1 maxpool, 2 avgpool+fc head, 3 input layout conversion     */
     int32_t conv_index;      /* description conv number, -1 for non-conv operators                  */
@@ -245,7 +248,7 @@ typedef struct {
     int32_t chain;           /* >= 0: the operator is a layer of fused run number `chain` (one kernel for the
                                 whole run, activations in shared memory; FP_Q_OP_TIMES reports the run's time
                                 at its first layer and 0 at the others); -1: launched on its own          */
-    int32_t reserved;
+    int32_t kernel;          /* convolutions: the kernel that computes it (FP_KERNEL_*); 0 for other operators    */
 } fp_op_info;
 
 fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_out, size_t bytes);

@@ -28,6 +28,7 @@ EXPORTS = ["fp_fuse", "fp_prune", "fp_forward", "fp_forward_host", "fp_forward_h
            "fp_last_error", "fp_rank_filters_static", "fp_soft_prune_epoch", "fp_soft_prune_finish",
            "fp_debug_expire_wait", "fp_fuse_with_allocator"]
 FP_STATIC_RANK_MAX_FILTERS = 4096
+CONV_KERNELS = ("", "conv_tc_kernel", "conv_split_kernel", "stem_pool_kernel", "chain_tc_kernel", "resident_net_kernel", "conv_simt_kernel")
 
 
 class fp_node(ctypes.Structure):
@@ -49,7 +50,7 @@ class fp_op_info(ctypes.Structure):
                 ("kind", "conv_index", "K", "C", "R", "S", "stride", "pad", "K_pad", "C_pad", "H", "W", "P", "Q",
                  "res_mode", "relu")] + \
                [("flops_per_image", ctypes.c_double), ("bytes_per_image", ctypes.c_double),
-                ("bytes_fixed", ctypes.c_double), ("chain", ctypes.c_int32), ("reserved", ctypes.c_int32)]
+                ("bytes_fixed", ctypes.c_double), ("chain", ctypes.c_int32), ("kernel", ctypes.c_int32)]
 
 
 ALLOC_FN = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p)

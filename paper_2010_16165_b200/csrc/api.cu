@@ -1991,6 +1991,8 @@ static void fill_op_info(fp_handle h, int i, fp_op_info* o) {
             o->bytes_fixed += (double)q.K_kept * q.C_kept * e + 4.0 * q.K_kept;
             o->flops_per_image += 2.0 * t.H * t.W * (double)q.K_kept * q.C_kept;
         }
+        o->kernel = h->net_on ? FP_KERNEL_RESIDENT_NET : h->op_chain[i] >= 0 ? FP_KERNEL_CHAIN_TC : h->stem_fused && i == 1 ? FP_KERNEL_STEM_POOL
+                  : !f.tc.valid ? FP_KERNEL_CONV_SIMT : f.tc.split ? FP_KERNEL_CONV_SPLIT : FP_KERNEL_CONV_TC;
         if (f.absorbed) { o->flops_per_image = 0.0; o->bytes_per_image = 0.0; o->bytes_fixed = 0.0; }
     } else if (op.kind == 1) {
         const Pool& p = h->pools[op.idx];

@@ -106,7 +106,7 @@ struct Chain {
     size_t blob_bytes = 0;
 };
 
-// One device allocation that is kept from one planning to the next while its size suits (reserve_regions).
+// One device allocation that is kept from one planning to the next while its size suits (region_reserve).
 struct Region { void* p = nullptr; size_t cap = 0; };
 
 struct Op { int kind; int idx; };
@@ -246,26 +246,22 @@ fp_status dev_alloc(fp_handle h, std::vector<void*>& owner, void** out, size_t b
     return FP_OK;
 }
 
-// Room for a plan: what the regions hold is given up.  An earlier plan's allocation is used again where it is large enough - cudaMalloc
+void give_back(fp_handle h, Region& r) {
+    dev_free(h, r.p);
+    r = Region();
+    if (&r == &h->act_region) h->act_base = nullptr;           // whatever comes there next has not been cleared
+}
+
+// Room for `bytes`: what the region holds is given up.  An earlier plan's allocation is used again where it is large enough - cudaMalloc
 // and cudaFree of every packed array cost fp_prune of ResNet-50 more than 20 ms - and not much too large: what pruning saves goes back to
-// the device but for a quarter or 64 MB, which a search over ratios goes up and down in.  Where memory runs out, and with a caller's
-// allocator always, everything goes back before anything is taken: a plan fits wherever it would fit alone.
-fp_status reserve_regions(fp_handle h, size_t pack, size_t meta, size_t act) {
-    struct { Region* r; size_t bytes; } const wants[] = {{&h->pack_region, pack}, {&h->meta_region, meta}, {&h->act_region, act}};
-    auto give_back = [&](Region* r) {
-        dev_free(h, r->p);
-        *r = Region();
-        if (r == &h->act_region) h->act_base = nullptr;        // whatever comes there next has not been cleared
-    };
-    for (const auto& w : wants)
-        if (h->dealloc || w.r->cap < w.bytes || w.r->cap - w.bytes > std::max(w.bytes / 4, (size_t)64 << 20)) give_back(w.r);
-    for (int again = h->dealloc ? 1 : 0;; ++again) {
-        fp_status s = FP_OK;
-        for (const auto& w : wants)
-            if (s == FP_OK && !w.r->p && (s = dev_alloc_raw(h, &w.r->p, w.bytes)) == FP_OK) w.r->cap = w.bytes;
-        if (s == FP_OK || again) return s;
-        for (const auto& w : wants) give_back(w.r);
+// the device but for a quarter or 64 MB, which a search over ratios goes up and down in.
+fp_status region_reserve(fp_handle h, Region& r, size_t bytes) {
+    if (r.cap < bytes || r.cap - bytes > std::max(bytes / 4, (size_t)64 << 20)) give_back(h, r);
+    if (!r.p) {
+        TRY(dev_alloc_raw(h, &r.p, bytes));
+        r.cap = bytes;
     }
+    return FP_OK;
 }
 
 fp_status pinned_reserve(fp_handle h, size_t bytes) {
@@ -1229,72 +1225,6 @@ fp_status build_plan(fp_handle h) {
         h->net_plans.clear();
     }
 
-    // --- activation memory: buffers are reused once their last reader has run ---
-    std::vector<std::pair<int, int>> placed;             // (tensor, buffer)
-    std::vector<size_t> start;                           // of every buffer
-    size_t act_bytes = 0;
-    const size_t vec_bytes = 8 * h->act_elem();
-    {
-        const int nt = (int)h->tensors.size();
-        std::vector<int> last_use(nt, -1);
-        for (int t = 0; t < nt; ++t)
-            for (const Use& u : uses[t]) last_use[t] = std::max(last_use[t], u.op);
-        for (int i = 0; i < (int)h->ops.size(); ++i)           // a layer that took a projection in also reads the projection's input
-            if (h->ops[i].kind == 0 && h->convs[h->ops[i].idx].proj >= 0) {
-                const int x = h->convs[h->convs[h->ops[i].idx].proj].src;
-                last_use[x] = std::max(last_use[x], i);
-            }
-        struct Buf { size_t bytes; int free_after; };
-        std::vector<Buf> bufs;
-        for (int i = 0; i < (int)h->ops.size(); ++i) {
-            const Op& op = h->ops[i];
-            int tid = -1;
-            if (h->net_on) {                                    // no tensor of the network exists in memory
-                if (op.kind == 0) h->tensors[h->convs[op.idx].out].d = nullptr;
-                else if (op.kind == 3) h->tensors[0].d = nullptr;
-                continue;
-            }
-            if (op.kind == 0 && h->op_chain[i] >= 0) {
-                // a fused run is one kernel: only its last tensor exists in memory, and it must not share
-                // a buffer with the run's inputs, which other CTAs still read while the first ones finish
-                const Chain& ch = h->chains[h->op_chain[i]];
-                if (i != ch.last_op) h->tensors[h->convs[op.idx].out].d = nullptr;
-                if (i != ch.first_op) continue;
-                tid = h->convs[ch.convs.back()].out;
-            }
-            else if (op.kind == 0) tid = h->convs[op.idx].out;
-            else if (op.kind == 1) tid = h->pools[op.idx].out;
-            else if (op.kind == 3) tid = 0;
-            if (h->stem_fused && (i == 0 || i == 1)) {          // neither the converted input nor the first convolution's output exists
-                h->tensors[tid].d = nullptr;
-                continue;
-            }
-            if (op.kind == 0 && h->convs[op.idx].absorbed) {    // a projection computed inside the layer that adds it
-                h->tensors[tid].d = nullptr;
-                continue;
-            }
-            if (tid < 0) continue;
-            Tensor& t = h->tensors[tid];
-            // planar-8 with border, plus guard vectors before and after (halo reads of the first/last tiles)
-            t.bytes = ((size_t)(t.C_pad / 8) * h->max_batch * (t.H + 2) * (t.W + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
-            if (t.split)
-                t.bytes = ((size_t)(t.C_pad / 8) * 4 * h->max_batch * ((t.H + 1) / 2 + 2) * ((t.W + 1) / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
-            if (tid == 0 && h->stem_packed)
-                t.bytes = ((size_t)10 * h->max_batch * (t.H / 2 + 2) * (t.W / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
-            int best = -1;
-            if (!h->keep_outputs)
-                for (int b = 0; b < (int)bufs.size(); ++b)
-                    if (bufs[b].free_after < i && bufs[b].bytes >= t.bytes && (best < 0 || bufs[b].bytes < bufs[best].bytes)) best = b;
-            if (best < 0) {
-                bufs.push_back({t.bytes, 0});
-                best = (int)bufs.size() - 1;
-            }
-            placed.push_back({tid, best});
-            bufs[best].free_after = std::max(last_use[tid], i);
-        }
-        for (const Buf& b : bufs) { start.push_back(act_bytes); act_bytes += align256(b.bytes); }
-    }
-
     // --- packed filters, biases, FC matrix: sizes and jobs, then one region, one upload and one launch ---
     {
         struct Want { void** slot; size_t bytes; };
@@ -1397,7 +1327,8 @@ fp_status build_plan(fp_handle h) {
         size_t meta = o_idx + align256(idx.size() * 4 + 4);
         std::vector<size_t> o_tables;
         for (const fp::NetPlan& np : h->net_plans) { o_tables.push_back(meta); meta += align256(np.table.size() * sizeof(fp::NetLayer)); }
-        TRY(reserve_regions(h, total, meta, act_bytes ? act_bytes : 256));
+        TRY(region_reserve(h, h->pack_region, total));
+        TRY(region_reserve(h, h->meta_region, meta));
         TRY(pinned_reserve(h, meta));
         size_t at = 0;
         for (const Want& w : wants) { *w.slot = (uint8_t*)h->pack_region.p + at; at += align256(w.bytes ? w.bytes : 16); }
@@ -1418,6 +1349,72 @@ fp_status build_plan(fp_handle h) {
         CK(cudaGetLastError());
     }
 
+    // --- activation memory: buffers are reused once their last reader has run ---
+    std::vector<std::pair<int, int>> placed;             // (tensor, buffer)
+    std::vector<size_t> start;                           // of every buffer
+    size_t act_bytes = 0;
+    const size_t vec_bytes = 8 * h->act_elem();
+    {
+        const int nt = (int)h->tensors.size();
+        std::vector<int> last_use(nt, -1);
+        for (int t = 0; t < nt; ++t)
+            for (const Use& u : uses[t]) last_use[t] = std::max(last_use[t], u.op);
+        for (int i = 0; i < (int)h->ops.size(); ++i)           // a layer that took a projection in also reads the projection's input
+            if (h->ops[i].kind == 0 && h->convs[h->ops[i].idx].proj >= 0) {
+                const int x = h->convs[h->convs[h->ops[i].idx].proj].src;
+                last_use[x] = std::max(last_use[x], i);
+            }
+        struct Buf { size_t bytes; int free_after; };
+        std::vector<Buf> bufs;
+        for (int i = 0; i < (int)h->ops.size(); ++i) {
+            const Op& op = h->ops[i];
+            int tid = -1;
+            if (h->net_on) {                                    // no tensor of the network exists in memory
+                if (op.kind == 0) h->tensors[h->convs[op.idx].out].d = nullptr;
+                else if (op.kind == 3) h->tensors[0].d = nullptr;
+                continue;
+            }
+            if (op.kind == 0 && h->op_chain[i] >= 0) {
+                // a fused run is one kernel: only its last tensor exists in memory, and it must not share
+                // a buffer with the run's inputs, which other CTAs still read while the first ones finish
+                const Chain& ch = h->chains[h->op_chain[i]];
+                if (i != ch.last_op) h->tensors[h->convs[op.idx].out].d = nullptr;
+                if (i != ch.first_op) continue;
+                tid = h->convs[ch.convs.back()].out;
+            }
+            else if (op.kind == 0) tid = h->convs[op.idx].out;
+            else if (op.kind == 1) tid = h->pools[op.idx].out;
+            else if (op.kind == 3) tid = 0;
+            if (h->stem_fused && (i == 0 || i == 1)) {          // neither the converted input nor the first convolution's output exists
+                h->tensors[tid].d = nullptr;
+                continue;
+            }
+            if (op.kind == 0 && h->convs[op.idx].absorbed) {    // a projection computed inside the layer that adds it
+                h->tensors[tid].d = nullptr;
+                continue;
+            }
+            if (tid < 0) continue;
+            Tensor& t = h->tensors[tid];
+            // planar-8 with border, plus guard vectors before and after (halo reads of the first/last tiles)
+            t.bytes = ((size_t)(t.C_pad / 8) * h->max_batch * (t.H + 2) * (t.W + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
+            if (t.split)
+                t.bytes = ((size_t)(t.C_pad / 8) * 4 * h->max_batch * ((t.H + 1) / 2 + 2) * ((t.W + 1) / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
+            if (tid == 0 && h->stem_packed)
+                t.bytes = ((size_t)10 * h->max_batch * (t.H / 2 + 2) * (t.W / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
+            int best = -1;
+            if (!h->keep_outputs)
+                for (int b = 0; b < (int)bufs.size(); ++b)
+                    if (bufs[b].free_after < i && bufs[b].bytes >= t.bytes && (best < 0 || bufs[b].bytes < bufs[best].bytes)) best = b;
+            if (best < 0) {
+                bufs.push_back({t.bytes, 0});
+                best = (int)bufs.size() - 1;
+            }
+            placed.push_back({tid, best});
+            bufs[best].free_after = std::max(last_use[tid], i);
+        }
+        for (const Buf& b : bufs) { start.push_back(act_bytes); act_bytes += align256(b.bytes); }
+    }
+    TRY(region_reserve(h, h->act_region, act_bytes ? act_bytes : 256));
     {
         // the activations' memory: zeros in the borders and guards; where every tensor lies as in the last plan, a forward leaves them as the next needs them
         std::vector<fp_handle_s::Placed> layout;
@@ -1489,11 +1486,19 @@ fp_status build_plan(fp_handle h) {
 }
 
 // A plan that failed half-way may have left its upload and the packing launch on their way: the pinned memory they read, and the regions
-// they write, are the next call's.
+// they write, are the next call's.  Where memory ran out everything goes back and is taken anew, and with a caller's allocator everything
+// goes back before anything is taken: a plan fits wherever it would fit alone.
 fp_status replan(fp_handle h) {
-    const fp_status s = build_plan(h);
-    if (s != FP_OK) cudaDeviceSynchronize();
-    return s;
+    for (int again = 0;; ++again) {
+        if (again || h->dealloc) {
+            cudaDeviceSynchronize();
+            for (Region* r : {&h->pack_region, &h->meta_region, &h->act_region}) give_back(h, *r);
+        }
+        const fp_status s = build_plan(h);
+        if (s == FP_OK) return s;
+        cudaDeviceSynchronize();
+        if (s != FP_ERR_NOMEM || again || h->dealloc) return s;
+    }
 }
 
 fp_status need_plan(fp_handle h, const char* who) {

@@ -84,6 +84,8 @@ struct FConv {
     int proj = -1;             // >= 0: the projection shortcut (index into convs) that this layer computes itself
     int proj_kind = 0;         // 1: filters stacked along the channels (1x1 layer); 2: extra centre-tap K groups (streamed 3x3 layer)
     int absorbed = 0;          // 1: this projection runs inside the layer that adds its result; its operator launches nothing
+    int pair = -1;             // >= 0: the narrow layer (index into convs) that reads this one's output and runs in its kernel
+    int paired = 0;            // 1: this layer runs in the kernel of the one it reads; its operator launches nothing
     int plain_bank = 0;        // 1: an absorbed projection whose bank is read as [chunk][K_pad][8] (proj_kind 2)
     int K_kept = 0, K_rows = 0, K_pad = 0, C_kept = 0, C_pad = 0;
     void* d_wp = nullptr;      // packed filters in the compute type, in the order the plan reads them (fp::PackJob)
@@ -92,6 +94,8 @@ struct FConv {
     int chan_off = -1;         // packed input channel -> fused input channel (-1 = zero channel), in the index array
     fp::ConvArgs args;
     fp::ConvPlanTC tc;
+    fp::PairArgs pair_args;
+    fp::PairPlan pair_plan;
 };
 
 struct Pool { int src, out, R, stride, pad; };
@@ -981,6 +985,37 @@ void conv_geometry(fp_handle h, const FConv& f, fp::ConvArgs* a) {
     }
 }
 
+// A 1x1 layer and a 1x1 layer that reads its output run as one kernel where that is the shorter way (plan_pair): the wide tensor between
+// the two is written, for its other readers, but not read again.
+void find_pairs(fp_handle h, const std::vector<std::vector<Use>>& uses) {
+    if (h->compute != FP_COMPUTE_BF16_TC || h->keep_outputs || h->net_on) return;
+    auto pointwise = [&](int op) {
+        if (h->ops[op].kind != 0 || h->op_chain[op] >= 0) return false;
+        const FConv& f = h->convs[h->ops[op].idx];
+        return f.R == 1 && f.S == 1 && f.stride == 1 && f.pad == 0 && !f.scatter && !f.absorbed && f.tc.valid && f.src != 0;
+    };
+    for (int i = 0; i < (int)h->ops.size(); ++i) {
+        if (!pointwise(i)) continue;
+        FConv& f = h->convs[h->ops[i].idx];
+        if (f.paired || h->tensors[f.src].split || f.res_mode == 2) continue;
+        for (const Use& u : uses[f.out]) {
+            if (u.how != 0 || !pointwise(u.op)) continue;
+            FConv& g = h->convs[h->ops[u.op].idx];
+            if (g.res_mode || g.proj >= 0 || h->tensors[f.out].split != h->tensors[g.out].split) continue;
+            fp::PairArgs& a = f.pair_args;
+            memset(&a, 0, sizeof(a));
+            const Tensor& out = h->tensors[f.out];
+            a.N = h->max_batch; a.P = out.H; a.Q = out.W; a.K = f.K_pad; a.K2 = g.K_pad;
+            a.C_pad = f.C_pad + (f.proj >= 0 ? h->convs[f.proj].C_pad : 0);
+            a.y_split = out.split; a.relu1 = f.relu; a.relu2 = g.relu;
+            if (!fp::plan_pair(a, &f.pair_plan)) continue;
+            f.pair = h->ops[u.op].idx;
+            g.paired = 1;
+            break;
+        }
+    }
+}
+
 // Rebuilds everything that depends on the masks.  The old buffers are released first, so while this runs - and
 // after it failed half-way (out of memory, a layer left without filters) - the handle has no plan: `planned` stays
 // 0 and every call that would launch kernels refuses until a later fp_prune succeeds.
@@ -1019,7 +1054,7 @@ fp_status build_plan(fp_handle h) {
     decide_splits(h, uses);
     for (FConv& f : h->convs) {
         f.n_mult = (h->tensors[f.src].split && split_reader(f) == 'C') ? 4 : 1;
-        f.proj = -1; f.proj_kind = 0; f.absorbed = 0; f.plain_bank = 0;
+        f.proj = -1; f.proj_kind = 0; f.absorbed = 0; f.plain_bank = 0; f.pair = -1; f.paired = 0;
     }
     // ... and, where a 3x3 / stride-2 max pooling is the only reader of that convolution, input conversion, convolution and
     // pooling run as one kernel (decided below, once the filter count is known).
@@ -1225,6 +1260,8 @@ fp_status build_plan(fp_handle h) {
         h->net_plans.clear();
     }
 
+    find_pairs(h, uses);
+
     // --- packed filters, biases, FC matrix: sizes and jobs, then one region, one upload and one launch ---
     {
         struct Want { void** slot; size_t bytes; };
@@ -1270,7 +1307,9 @@ fp_status build_plan(fp_handle h) {
                     j.chunks += q.C_pad / 8;
                     j.cg = j.chunks;
                 }
-                if (f.tc.valid && f.tc.blocked_bank && !f.plain_bank) {
+                if (f.pair >= 0) {
+                    j.n_tile = f.pair_plan.G; j.rows = round_up(f.K_pad, f.pair_plan.G);
+                } else if (f.tc.valid && f.tc.blocked_bank && !f.plain_bank && !f.paired) {
                     // the streamed form of the kernel reads its bank block by block, one copy per pipeline stage; gathered and
                     // resident layers with several filter tiles read it tile by tile
                     j.n_tile = f.tc.n_tile; j.rows = f.tc.n_tile * f.tc.n_tiles;
@@ -1366,6 +1405,25 @@ fp_status build_plan(fp_handle h) {
             }
         struct Buf { size_t bytes; int free_after; };
         std::vector<Buf> bufs;
+        auto place = [&](int tid, int i) {                      // a buffer for a tensor that operator i writes
+            Tensor& t = h->tensors[tid];
+            // planar-8 with border, plus guard vectors before and after (halo reads of the first/last tiles)
+            t.bytes = ((size_t)(t.C_pad / 8) * h->max_batch * (t.H + 2) * (t.W + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
+            if (t.split)
+                t.bytes = ((size_t)(t.C_pad / 8) * 4 * h->max_batch * ((t.H + 1) / 2 + 2) * ((t.W + 1) / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
+            if (tid == 0 && h->stem_packed)
+                t.bytes = ((size_t)10 * h->max_batch * (t.H / 2 + 2) * (t.W / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
+            int best = -1;
+            if (!h->keep_outputs)
+                for (int b = 0; b < (int)bufs.size(); ++b)
+                    if (bufs[b].free_after < i && bufs[b].bytes >= t.bytes && (best < 0 || bufs[b].bytes < bufs[best].bytes)) best = b;
+            if (best < 0) {
+                bufs.push_back({t.bytes, 0});
+                best = (int)bufs.size() - 1;
+            }
+            placed.push_back({tid, best});
+            bufs[best].free_after = std::max(last_use[tid], i);
+        };
         for (int i = 0; i < (int)h->ops.size(); ++i) {
             const Op& op = h->ops[i];
             int tid = -1;
@@ -1393,24 +1451,9 @@ fp_status build_plan(fp_handle h) {
                 h->tensors[tid].d = nullptr;
                 continue;
             }
-            if (tid < 0) continue;
-            Tensor& t = h->tensors[tid];
-            // planar-8 with border, plus guard vectors before and after (halo reads of the first/last tiles)
-            t.bytes = ((size_t)(t.C_pad / 8) * h->max_batch * (t.H + 2) * (t.W + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
-            if (t.split)
-                t.bytes = ((size_t)(t.C_pad / 8) * 4 * h->max_batch * ((t.H + 1) / 2 + 2) * ((t.W + 1) / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
-            if (tid == 0 && h->stem_packed)
-                t.bytes = ((size_t)10 * h->max_batch * (t.H / 2 + 2) * (t.W / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
-            int best = -1;
-            if (!h->keep_outputs)
-                for (int b = 0; b < (int)bufs.size(); ++b)
-                    if (bufs[b].free_after < i && bufs[b].bytes >= t.bytes && (best < 0 || bufs[b].bytes < bufs[best].bytes)) best = b;
-            if (best < 0) {
-                bufs.push_back({t.bytes, 0});
-                best = (int)bufs.size() - 1;
-            }
-            placed.push_back({tid, best});
-            bufs[best].free_after = std::max(last_use[tid], i);
+            if (tid < 0 || (op.kind == 0 && h->convs[op.idx].paired)) continue;     // (placed with the layer it runs with)
+            place(tid, i);
+            if (op.kind == 0 && h->convs[op.idx].pair >= 0) place(h->convs[h->convs[op.idx].pair].out, i);
         }
         for (const Buf& b : bufs) { start.push_back(act_bytes); act_bytes += align256(b.bytes); }
     }
@@ -1460,11 +1503,19 @@ fp_status build_plan(fp_handle h) {
     for (const Op& op : h->ops) {
         if (op.kind != 0) continue;
         FConv& f = h->convs[op.idx];
-        if (f.absorbed && !f.plain_bank) continue;
+        if ((f.absorbed && !f.plain_bank) || f.paired) continue;
         const int second = f.proj >= 0 ? h->convs[f.proj].src : f.res_mode ? f.res_tid : f.src;
         const int largest = h->tensors[second].bytes > h->tensors[f.src].bytes ? second : f.src;
-        f.args.reverse = f.tc.valid && !f.tc.split && !walked[largest];
+        f.args.reverse = f.tc.valid && (!f.tc.split || f.pair >= 0) && !walked[largest];
         walked[f.src] = walked[second] = walked[f.out] = f.args.reverse;
+        if (f.pair >= 0) {
+            const FConv& g = h->convs[f.pair];
+            fp::PairArgs& a = f.pair_args;
+            a.x = f.args.x; a.x2 = f.args.x2; a.res = f.args.res; a.w1 = f.d_wp; a.w2 = g.d_wp; a.bias1 = f.d_bp; a.bias2 = g.d_bp;
+            a.y = f.args.y; a.z = g.args.y;
+            a.x2_chunk0 = f.args.x2_chunk0; a.x2_plane_mult = f.args.x2_plane_mult; a.reverse = f.args.reverse;
+            walked[g.out] = f.args.reverse;
+        }
     }
     for (Chain& ch : h->chains) {
         const FConv& f0 = h->convs[ch.convs.front()];
@@ -1556,7 +1607,14 @@ void launch_op(fp_handle h, int op_index, const void* d_input, int batch, float*
         fp::launch_stem_pool(h->stem_plan, a, h->d_status, st);
         return;
     }
-    if (op.kind == 0 && h->convs[op.idx].absorbed) return;        // runs inside the layer that adds its result
+    if (op.kind == 0 && (h->convs[op.idx].absorbed || h->convs[op.idx].paired)) return;        // runs inside another layer's kernel
+    if (op.kind == 0 && h->convs[op.idx].pair >= 0) {
+        const FConv& f = h->convs[op.idx];
+        fp::PairArgs a = f.pair_args;
+        a.N = batch;
+        fp::launch_pair(f.pair_plan, a, h->d_status, st);
+        return;
+    }
     if (op.kind == 0 && h->op_chain[op_index] >= 0) {
         const Chain& ch = h->chains[h->op_chain[op_index]];
         if (op_index != ch.first_op) return;       // the run's first operator launches all of it
@@ -1906,7 +1964,7 @@ extern "C" fp_status fp_debug_expire_wait(fp_handle h, void* stream) {
         const Op& op = h->ops[i];
         if (op.kind != 0 || h->op_chain[i] >= 0 || (h->stem_fused && i == 1)) continue;
         const FConv& f = h->convs[op.idx];
-        if (!f.tc.valid || !f.tc.flat || (f.tc.blocked_bank && !f.tc.split) || h->tensors[f.src].split || h->tensors[f.out].split || f.proj >= 0 || f.absorbed) continue;
+        if (!f.tc.valid || !f.tc.flat || (f.tc.blocked_bank && !f.tc.split) || h->tensors[f.src].split || h->tensors[f.out].split || f.proj >= 0 || f.absorbed || f.pair >= 0 || f.paired) continue;
         // the first round of the activation producer is left out, so the MMA-issuing thread's wait for that stage runs
         // out after a millisecond (two million cycles), raises the status word and takes every role of the CTA with it
         fp::launch_conv_tc(f.tc, f.args, h->d_status, (cudaStream_t)stream, 0, 2000000LL);
@@ -1996,9 +2054,17 @@ static void fill_op_info(fp_handle h, int i, fp_op_info* o) {
             o->bytes_fixed += (double)q.K_kept * q.C_kept * e + 4.0 * q.K_kept;
             o->flops_per_image += 2.0 * t.H * t.W * (double)q.K_kept * q.C_kept;
         }
+        if (f.pair >= 0) {
+            // the narrow layer computed by the same kernel: its figures, as of a layer of its own
+            const FConv& g = h->convs[f.pair];
+            const Tensor& z = h->tensors[g.out];
+            o->bytes_per_image += (double)t.H * t.W * (t.C + z.C) * e;
+            o->bytes_fixed += (double)g.K_kept * g.C_kept * e + 4.0 * g.K_kept;
+            o->flops_per_image += 2.0 * t.H * t.W * (double)g.K_kept * g.C_kept;
+        }
         o->kernel = h->net_on ? FP_KERNEL_RESIDENT_NET : h->op_chain[i] >= 0 ? FP_KERNEL_CHAIN_TC : h->stem_fused && i == 1 ? FP_KERNEL_STEM_POOL
-                  : !f.tc.valid ? FP_KERNEL_CONV_SIMT : f.tc.split ? FP_KERNEL_CONV_SPLIT : FP_KERNEL_CONV_TC;
-        if (f.absorbed) { o->flops_per_image = 0.0; o->bytes_per_image = 0.0; o->bytes_fixed = 0.0; }
+                  : !f.tc.valid ? FP_KERNEL_CONV_SIMT : f.pair >= 0 || f.paired ? FP_KERNEL_CONV_PAIR : f.tc.split ? FP_KERNEL_CONV_SPLIT : FP_KERNEL_CONV_TC;
+        if (f.absorbed || f.paired) { o->flops_per_image = 0.0; o->bytes_per_image = 0.0; o->bytes_fixed = 0.0; }
     } else if (op.kind == 1) {
         const Pool& p = h->pools[op.idx];
         const Tensor& s = h->tensors[p.src];
@@ -2041,7 +2107,7 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             for (const Chain& ch : h->chains) n -= (int)ch.convs.size() - 1; // a fused run is one
             n -= h->input_fused;
             n -= 2 * h->stem_fused;                                          // conversion, convolution and pooling are one
-            for (const FConv& c : h->convs) n -= c.absorbed;                 // a projection inside the layer that adds it
+            for (const FConv& c : h->convs) n -= c.absorbed + c.paired;      // a projection inside the layer that adds it, a layer inside the one it reads
             *(int32_t*)h_out = h->net_on ? network_parts(h, h->last_batch > 0 ? h->last_batch : h->max_batch).n : n;
             return FP_OK;
         }
@@ -2194,7 +2260,7 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
                 const Op& op = h->ops[i];
                 const bool silent = (h->net_on && i != 1) || (!h->net_on && op.kind == 0 && h->op_chain[i] >= 0 && h->chains[h->op_chain[i]].first_op != i) ||
                                     (op.kind == 3 && (h->input_fused || h->stem_fused)) || (h->stem_fused && i == 2) ||
-                                    (op.kind == 0 && h->convs[op.idx].absorbed);
+                                    (op.kind == 0 && (h->convs[op.idx].absorbed || h->convs[op.idx].paired));
                 if (silent) { prefix[i] = i ? prefix[i - 1] : 0.f; continue; }
                 cudaGraph_t g = nullptr;
                 cudaGraphExec_t ge = nullptr;

@@ -200,6 +200,21 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
 void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cudaStream_t st, int skip_round = -1,
                     long long wait_cycles = 0);
 
+// Two 1x1 / stride-1 convolutions as one kernel, the second reading the first's output (pair_tc.cu): the layer that writes a bottleneck
+// network's residual stream, and the narrow layer that reads it.
+struct PairArgs {
+    const void *x, *x2;   // input of the first layer; chunks >= x2_chunk0 (0: none) come from x2, as in ConvArgs
+    const void* res;      // its shortcut operand, on its output's grid, or nullptr
+    const void *w1, *w2;  // filters: [group of G][C_pad / 8][G rows][8] and [K / 8][K2][8]
+    const float *bias1, *bias2;
+    void *y, *z;          // the two outputs, y_split: both parity-split
+    int N, P, Q, C_pad, K, K2;          // K, K2: padded filters of the two
+    int x2_chunk0, x2_plane_mult, y_split, relu1, relu2, reverse;
+};
+struct PairPlan { int valid, G, x_stages, slots, slot_bytes, tmem_cols; unsigned smem_bytes; };
+bool plan_pair(const PairArgs& a, PairPlan* plan);       // false where the two do better, or only run, as kernels of their own
+void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStream_t st);
+
 // First convolution (7x7 / stride 2 / pad 3, at most 3 input channels, ReLU) and the 3x3 / stride 2 / pad 1 max pooling
 // behind it as one kernel that reads the NCHW network input  and writes the pooled tensor.
 struct StemPoolArgs {

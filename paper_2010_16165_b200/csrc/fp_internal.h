@@ -211,7 +211,7 @@ struct PairArgs {
     int N, P, Q, C_pad, K, K2;          // K, K2: padded filters of the two
     int x2_chunk0, x2_plane_mult, y_split, relu1, relu2, reverse;
 };
-struct PairPlan { int valid, G, x_stages, slots, slot_bytes, tmem_cols; unsigned smem_bytes; };
+struct PairPlan { int valid, G, x_stages, sum2_stages, slots, slot_bytes, tmem_cols; unsigned smem_bytes; };
 bool plan_pair(const PairArgs& a, PairPlan* plan);       // false where the two do better, or only run, as kernels of their own
 void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStream_t st);
 

@@ -12,16 +12,18 @@
 //                 that adds a vector of 8 channels writes the sum where it read it.  From there the second convolution's MMAs and
 //                 the bulk copies to memory both take it; the slot is free when both have read it.  Filters come with every tile
 //                 again: they are in L2, and shared memory holds several slots so, which is what keeps enough reads in flight.
-//   Tensor memory the second convolution's sums (K2 columns, over all groups of a tile) and four stages of G columns of the first's.
+//   Tensor memory the second convolution's sums (K2 columns, over all groups of a tile; two tiles' where they fit) and four stages of
+//                 G columns of the first's.
 //   Latency       A group's way - slot filled, MMAs, commit, accumulator read, sum written, MMAs, copies out - is some 3000 cycles
 //                 of barriers and round trips for a few hundred of work.  So no role waits for another's group before it starts
 //                 its next: each convolution has its issuing warp, and two teams of eight finishing warps take the groups in turn.
+//                 A warp's bulk copies go out one after the other, some 110 cycles each, so four warps share a group's dozen copies
+//                 in and two its copies out (one warp for the former alone took 1100-1500 cycles a group, and that was the kernel's time).
 //                 z of a tile is finished behind the first groups of the next, so that nobody waits for its last MMAs.
 //   Turns         the numbers of slots and stages are multiples of the number of teams, so a slot, a stage and the barriers of both always
-//                 meet the same team and the same copying warp: a warp that skips the others' uses of a barrier could take the parity
-//                 of an older phase for its own.
-//   Warp roles    warp 0 copies in, warp 1 issues the first convolution's MMAs, sixteen warps finish both convolutions, one warp
-//                 issues the second convolution's MMAs, two warps take turns at copying y out.
+//                 meet the same team: a warp that skips the others' uses of a barrier could take the parity of an older phase for its own.
+//   Warp roles    warps 0-3 copy in, sixteen warps finish both convolutions, one warp each issues the MMAs of the first and of
+//                 the second, two copy y out.
 //   Sums          in the order of the two kernels this stands for (conv_tc.cu), so the results are theirs bit by bit.
 //   Waits         bounded as in conv_tc.cu.
 #include "fp_internal.h"
@@ -36,18 +38,19 @@ namespace {
 using namespace tc;
 
 constexpr int kMaxSlots = 8, kSums = 4;
-constexpr int kTeams = 2, kTeamWarps = 8, kStoreWarps = 2;
-constexpr int kEpiWarps = kTeams * kTeamWarps;
-constexpr int kThreads = 32 * (2 + kEpiWarps + 1 + kStoreWarps);
+constexpr int kInWarps = 4, kTeams = 2, kTeamWarps = 8, kOutWarps = 2;
+constexpr int kEpi0 = kInWarps, kFirst = kEpi0 + kTeams * kTeamWarps, kSecond = kFirst + 1, kOut0 = kSecond + 1;      // warps
+constexpr int kThreads = 32 * (kOut0 + kOutWarps);
 constexpr unsigned kSmemMax = 232448u - 1024u;
 
 struct PairCtrl {
     uint64_t slot_full[kMaxSlots], slot_empty[kMaxSlots], y_ready[kMaxSlots];
     uint64_t sum1_full[kSums], sum1_empty[kSums];
     uint64_t x_full[2], x_empty[2];
-    uint64_t sum2_full[kTeams], sum2_empty;
+    uint64_t sum2_full[2], sum2_empty[2];      // by the parity of the tile's number, which is its team and, with two stages, its stage
     uint32_t tmem_base;
     int abort_flag;
+    int pad_[2];
 };
 static_assert(sizeof(PairCtrl) % 16 == 0, "the tables of shifts behind it are read as 16-byte vectors");
 
@@ -57,7 +60,7 @@ struct PairParams {
     int Qp, P2, m_total, m_tiles, m_first, m_sign;
     long long plane_x, plane_x2, plane_y;      // vectors per chunk plane (the shortcut's planes are m_total apart)
     int chunks1, chunks, groups;               // channel chunks of x, of y; groups of y
-    int x_stages, slots, slot_bytes, tmem_cols;
+    int x_stages, sum2_stages, slots, slot_bytes, tmem_cols;
     int y_P2h, y_Wh2;                          // parity-split output: half-resolution grid
     long long wait_cycles;
     int* status;
@@ -92,7 +95,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
     const uint32_t y_ready0 = base + (uint32_t)offsetof(PairCtrl, y_ready);
     const uint32_t x_full0 = base + (uint32_t)offsetof(PairCtrl, x_full), x_empty0 = base + (uint32_t)offsetof(PairCtrl, x_empty);
     const uint32_t sum1_full0 = base + (uint32_t)offsetof(PairCtrl, sum1_full), sum1_empty0 = base + (uint32_t)offsetof(PairCtrl, sum1_empty);
-    const uint32_t sum2_full0 = base + (uint32_t)offsetof(PairCtrl, sum2_full), sum2_empty = base + (uint32_t)offsetof(PairCtrl, sum2_empty);
+    const uint32_t sum2_full0 = base + (uint32_t)offsetof(PairCtrl, sum2_full), sum2_empty0 = base + (uint32_t)offsetof(PairCtrl, sum2_empty);
     volatile int* abort_flag = &ctrl->abort_flag;
     const long long limit = p.wait_cycles > 0 ? p.wait_cycles : kWaitCycles;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -100,7 +103,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxSlots; ++s) {
             mbar_init(slot_full0 + 8 * s, 1);
-            mbar_init(slot_empty0 + 8 * s, 2);                      // the second convolution's MMAs, the copies to memory
+            mbar_init(slot_empty0 + 8 * s, 1 + kOutWarps);          // the second convolution's MMAs, the copies to memory
             mbar_init(y_ready0 + 8 * s, 32 * kTeamWarps);
         }
         for (int s = 0; s < kSums; ++s) {
@@ -111,15 +114,17 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
             mbar_init(x_full0 + 8 * s, 1);
             mbar_init(x_empty0 + 8 * s, 1);
         }
-        for (int t = 0; t < kTeams; ++t) mbar_init(sum2_full0 + 8 * t, 1);
-        mbar_init(sum2_empty, 32 * kTeamWarps);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(sum2_full0 + 8 * s, 1);
+            mbar_init(sum2_empty0 + 8 * s, 32 * kTeamWarps);
+        }
         ctrl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     for (int i = threadIdx.x; i < p.a.K; i += kThreads) bias1[i] = p.a.bias1[i];
     for (int i = threadIdx.x; i < p.a.K2; i += kThreads) bias2[i] = p.a.bias2[i];
-    if (warp == 1) {
+    if (warp == kFirst) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(base + (uint32_t)offsetof(PairCtrl, tmem_base)), "r"((uint32_t)p.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -128,7 +133,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&ctrl->tmem_base);
-    const uint32_t tmem_sum1 = tmem + (uint32_t)p.a.K2;             // the first convolution's stages behind the second's sums
+    const uint32_t tmem_sum1 = tmem + (uint32_t)(p.sum2_stages * p.a.K2);             // the first convolution's stages behind the second's sums
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -137,20 +142,19 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
     const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);      // see conv_tc.cu
     bool ok = true;
     Ring slot, sum, xs;
-    if (warp == 0) {
-        // ------------------------------ copies in ------------------------------
+    if (warp < kInWarps) {
+        // ------------------------------ copies in: each warp a quarter of the runs and half of one of the filters ------------------------------
         const uint4* xv = reinterpret_cast<const uint4*>(p.a.x);
         const uint4* x2v = reinterpret_cast<const uint4*>(p.a.x2);
         const uint4* rv = reinterpret_cast<const uint4*>(p.a.res);
-        const uint4* w1v = reinterpret_cast<const uint4*>(p.a.w1);
-        const uint4* w2v = reinterpret_cast<const uint4*>(p.a.w2);
         const int chunk2 = p.a.x2_chunk0 > 0 ? p.a.x2_chunk0 : p.chunks1;
+        const uint32_t w1_bytes = (uint32_t)(p.chunks1 * G) * 16u, w2_step = (uint32_t)(GC * p.a.K2) * 16u;
         for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x) {
             const long long f0 = (long long)(p.m_first + p.m_sign * tile) * 128;
             if (!(ok = wait_all(x_empty0 + 8 * xs.at, xs.phase ^ 1))) break;
-            if (lane == 0) mbar_expect_tx(x_full0 + 8 * xs.at, x_bytes);
+            if (warp == 0 && lane == 0) mbar_expect_tx(x_full0 + 8 * xs.at, x_bytes);
             __syncwarp();
-            for (int c = lane; c < p.chunks1; c += 32)
+            for (int c = warp + kInWarps * lane; c < p.chunks1; c += 32 * kInWarps)
                 bulk_copy(x0 + xs.at * x_bytes + (uint32_t)c * 2048u,
                           (c < chunk2 ? xv + (long long)c * p.plane_x : x2v + (long long)(c - chunk2) * p.plane_x2) + f0, 2048u, x_full0 + 8 * xs.at);
             xs.next(p.x_stages);
@@ -158,24 +162,23 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                 if (!(ok = wait_all(slot_empty0 + 8 * slot.at, slot.phase ^ 1))) break;
                 const int cg = chunks_of(g);
                 const uint32_t dst = slot0 + slot.at * (uint32_t)p.slot_bytes, bar = slot_full0 + 8 * slot.at;
-                const uint32_t w1_bytes = (uint32_t)(p.chunks1 * G) * 16u, w2_bytes = (uint32_t)(cg * p.a.K2) * 16u;
-                if (lane == 0) mbar_expect_tx(bar, (rv ? (uint32_t)cg * 2048u : 0u) + w1_bytes + w2_bytes);
+                const uint32_t w2_bytes = (uint32_t)(cg * p.a.K2) * 16u;
+                // (the others' bytes may be counted before they are expected: the barrier's phase ends no earlier than with this arrival)
+                if (warp == 0 && lane == 0) mbar_expect_tx(bar, (rv ? (uint32_t)cg * 2048u : 0u) + w1_bytes + w2_bytes);
                 __syncwarp();
-                if (lane < 16) {
-                    if (rv && lane < cg) bulk_copy(dst + (uint32_t)lane * 2048u, rv + (long long)(g * GC + lane) * p.m_total + f0, 2048u, bar);
-                } else {                                            // filters in pieces of 8 KB
-                    const bool first = lane < 24;
-                    const uint32_t bytes = first ? w1_bytes : w2_bytes;
-                    const uint8_t* src = reinterpret_cast<const uint8_t*>(first ? w1v + (long long)g * p.chunks1 * G : w2v + (long long)(g * GC) * p.a.K2);
-                    for (uint32_t off = (uint32_t)(lane & 7) * 8192u; off < bytes; off += 65536u)
-                        bulk_copy(dst + (first ? w1_off : w2_off) + off, src + off, min(8192u, bytes - off), bar);
+                if (lane == 0) {
+                    const uint32_t bytes = warp < 2 ? w1_bytes : w2_bytes, half = bytes / 32u * 16u, off = warp & 1 ? half : 0u;
+                    const uint8_t* src = reinterpret_cast<const uint8_t*>(warp < 2 ? p.a.w1 : p.a.w2) + (long long)g * (warp < 2 ? w1_bytes : w2_step);
+                    bulk_copy(dst + (warp < 2 ? w1_off : w2_off) + off, src + off, warp & 1 ? bytes - half : half, bar);
+                } else if (const int c = warp + kInWarps * (lane - 1); rv && c < cg) {
+                    bulk_copy(dst + (uint32_t)c * 2048u, rv + (long long)(g * GC + c) * p.m_total + f0, 2048u, bar);
                 }
                 __syncwarp();
                 slot.next(p.slots);
             }
         }
         if (!ok && lane == 0) { atomicExch(&ctrl->abort_flag, 1); atomicExch(p.status, 1); }
-    } else if (warp == 1) {
+    } else if (warp == kFirst) {
         // ------------------------------ first convolution's MMAs ------------------------------
         const uint32_t leader = elect_one();
         for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x) {
@@ -202,10 +205,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
             xs.next(p.x_stages);
         }
         if (!ok && leader) { atomicExch(&ctrl->abort_flag, 1); atomicExch(p.status, 2); }
-    } else if (warp < 2 + kEpiWarps) {
+    } else if (warp < kFirst) {
         // ------------------------------ finish ------------------------------
         constexpr int HC = G / 16;                                  // chunks of a group that a warp finishes: half of them
-        const int team = (warp - 2) / kTeamWarps, quarter = warp & 3, half = ((warp - 2) >> 2) & 1, row = quarter * 32 + lane;
+        const int team = (warp - kEpi0) / kTeamWarps, quarter = warp & 3, half = ((warp - kEpi0) >> 2) & 1, row = quarter * 32 + lane;
         const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
         struct Place { bool exists, interior; long long f; };
         auto place_of = [&](int tile) {                             // this thread's position; f: its vector in y's and z's planes
@@ -234,10 +237,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
         auto finish_z = [&](const Place& o, int local) -> bool {
             if (!wait_all(sum2_full0 + 8 * team, (uint32_t)(local / kTeams) & 1u)) return false;
             tc_fence_after();
+            const uint32_t sums = tmem + lanes + (uint32_t)((local & (p.sum2_stages - 1)) * p.a.K2);
 #pragma unroll 1
             for (int u = half ? first2 : 0; u < (half ? cols2 : first2); ++u) {
                 uint32_t v[16];
-                tmem_ld16(tmem + lanes + (uint32_t)(16 * u), v);
+                tmem_ld16(sums + (uint32_t)(16 * u), v);
                 tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
@@ -251,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                 }
             }
             tc_fence_before();
-            mbar_arrive(sum2_empty);
+            mbar_arrive(sum2_empty0 + 8 * team);
             return true;
         };
         Place before;
@@ -307,54 +311,52 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
         }
         if (ok && local > 0 && ((local - 1) & 1) == team) ok = finish_z(before, local - 1);
         if (!ok && lane == 0) { atomicExch(&ctrl->abort_flag, 1); atomicExch(p.status, 3); }
-    } else if (warp == 2 + kEpiWarps) {
+    } else if (warp == kSecond) {
         // ------------------------------ second convolution's MMAs ------------------------------
         const uint32_t leader = elect_one();
         const uint32_t idesc = idesc0 | ((uint32_t)(p.a.K2 >> 3) << 17);
-        uint32_t phase = 0, turn = 0;                               // turn: the team that finishes the tile's z
-        for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x, turn = (turn + 1) % kTeams) {
+        int local = 0;
+        for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x, ++local) {
+            const uint32_t d = tmem + (uint32_t)((local & (p.sum2_stages - 1)) * p.a.K2);
             for (int g = 0; g < p.groups; ++g) {
                 if (!(ok = wait_all(y_ready0 + 8 * slot.at, slot.phase))) break;
-                if (g == 0) {
-                    if (!(ok = wait_all(sum2_empty, phase ^ 1))) break;
-                    phase ^= 1;
-                }
+                // the stage's columns were last used sum2_stages tiles ago: z of that tile has been read
+                const int read = local - p.sum2_stages;
+                if (g == 0 && read >= 0 && !(ok = wait_all(sum2_empty0 + 8 * (read & 1), (uint32_t)(read >> 1) & 1u))) break;
                 tc_fence_after();
                 const uint32_t at = slot0 + slot.at * (uint32_t)p.slot_bytes;
                 uint32_t a_lo = (at >> 4) | (128u << 16), b_lo = ((at + w2_off) >> 4) | ((uint32_t)p.a.K2 << 16);
                 const int ks = chunks_of(g) >> 1;
 #pragma unroll 1
                 for (int i = 0; i < ks; ++i) {
-                    umma_bf16_lo_if(leader, tmem, a_lo, b_lo, idesc, (g | i) ? 1u : 0u);
+                    umma_bf16_lo_if(leader, d, a_lo, b_lo, idesc, (g | i) ? 1u : 0u);
                     a_lo += 256u;
                     b_lo += 2u * (uint32_t)p.a.K2;
                 }
                 if (leader) umma_commit(slot_empty0 + 8 * slot.at);
-                if (leader && g == p.groups - 1) umma_commit(sum2_full0 + 8 * turn);
+                if (leader && g == p.groups - 1) umma_commit(sum2_full0 + 8 * (local & 1));
                 __syncwarp();
                 slot.next(p.slots);
             }
         }
         if (!ok && leader) { atomicExch(&ctrl->abort_flag, 1); atomicExch(p.status, 4); }
     } else {
-        // ------------------------------ copies out: every other group each ------------------------------
-        const int turn = warp - (3 + kEpiWarps);
+        // ------------------------------ copies out: half of the chunks each ------------------------------
+        const int turn = warp - kOut0;
         uint4* yv = reinterpret_cast<uint4*>(p.a.y);
-        int q = 0;
         for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x) {
             const long long f0 = (long long)(p.m_first + p.m_sign * tile) * 128;
             const uint32_t bytes = (uint32_t)min(128LL, p.m_total - f0) * 16u;
-            for (int g = 0; g < p.groups; ++g, ++q) {
-                if (q % kStoreWarps == turn) {
-                    if (!(ok = wait_all(y_ready0 + 8 * slot.at, slot.phase))) break;
-                    if (!p.a.y_split && lane < chunks_of(g)) {
-                        bulk_store(yv + (long long)(g * GC + lane) * p.plane_y + f0, slot0 + slot.at * (uint32_t)p.slot_bytes + (uint32_t)lane * 2048u, bytes);
-                        bulk_store_commit();
-                        bulk_store_wait_read();
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(slot_empty0 + 8 * slot.at);
+            for (int g = 0; g < p.groups; ++g) {
+                if (!(ok = wait_all(y_ready0 + 8 * slot.at, slot.phase))) break;
+                const int c = turn + kOutWarps * lane;
+                if (!p.a.y_split && c < chunks_of(g)) {
+                    bulk_store(yv + (long long)(g * GC + c) * p.plane_y + f0, slot0 + slot.at * (uint32_t)p.slot_bytes + (uint32_t)c * 2048u, bytes);
+                    bulk_store_commit();
+                    bulk_store_wait_read();
                 }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(slot_empty0 + 8 * slot.at);
                 slot.next(p.slots);
             }
         }
@@ -368,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == kFirst) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)p.tmem_cols) : "memory");
     }
@@ -381,15 +383,16 @@ bool plan_pair(const PairArgs& a, PairPlan* plan) {
     const int m_tiles = (int)(((long long)a.N * (a.P + 2) * (a.Q + 2) + 127) / 128);
     if (m_tiles < sm_count() || a.K2 > 256) return false;
     for (int G = 64; G >= 32; G -= 32) {
+        const int sum2_stages = 2 * a.K2 + kSums * G <= 512 ? 2 : 1;
         int cols = 32;
-        while (cols < a.K2 + kSums * G) cols *= 2;
+        while (cols < sum2_stages * a.K2 + kSums * G) cols *= 2;
         const unsigned fixed = (unsigned)sizeof(PairCtrl) + (unsigned)(a.K + a.K2) * 4u + 128u, x_bytes = (unsigned)(a.C_pad / 8) * 2048u;
         const unsigned slot = (unsigned)(G / 8) * 2048u + (unsigned)(a.C_pad / 8 * G) * 16u + (unsigned)(G / 8 * a.K2) * 16u;
         for (int xs = 2; xs >= 1; --xs) {
             if (fixed + (unsigned)xs * x_bytes >= kSmemMax) continue;
             const int slots = (int)((kSmemMax - fixed - (unsigned)xs * x_bytes) / slot) & ~1;
             if (slots < 4) continue;
-            plan->G = G; plan->x_stages = xs; plan->slots = slots < kMaxSlots ? slots : kMaxSlots;
+            plan->G = G; plan->x_stages = xs; plan->sum2_stages = sum2_stages; plan->slots = slots < kMaxSlots ? slots : kMaxSlots;
             plan->slot_bytes = (int)slot; plan->tmem_cols = cols;
             plan->smem_bytes = fixed + (unsigned)xs * x_bytes + (unsigned)plan->slots * slot;
             if (cudaFuncSetAttribute(G == 64 ? conv_pair_kernel<64> : conv_pair_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
@@ -417,7 +420,7 @@ void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStr
         p.plane_y = 4LL * a.N * p.y_P2h;
     }
     p.chunks1 = a.C_pad / 8; p.chunks = a.K / 8; p.groups = (a.K + plan.G - 1) / plan.G;
-    p.x_stages = plan.x_stages; p.slots = plan.slots; p.slot_bytes = plan.slot_bytes; p.tmem_cols = plan.tmem_cols;
+    p.x_stages = plan.x_stages; p.sum2_stages = plan.sum2_stages; p.slots = plan.slots; p.slot_bytes = plan.slot_bytes; p.tmem_cols = plan.tmem_cols;
     p.status = d_status;
     p.div_p2out = make_fastdiv((uint32_t)p.P2);
     p.div_qp = make_fastdiv((uint32_t)p.Qp);

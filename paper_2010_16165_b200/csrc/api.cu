@@ -195,6 +195,7 @@ struct fp_handle_s {
     fp::StemPoolArgs stem_args;
     fp::StemPoolPlan stem_plan;
     int scatter_policy = 0;                // fp_model_desc::scatter
+    int whole_outputs = 0;                 // 1 while FP_Q_OP_OUTPUT runs the forward again: tensors are written whole, read or not
     int apart = -1;                        // operator that FP_Q_OP_OUTPUT asks for: planned as a launch of its own
     int planned = 0;                       // 1: buffers, packed banks and launch plans match the masks (set by replan)
     int act_is_bf16() const { return compute != FP_COMPUTE_FP32; }
@@ -1009,6 +1010,9 @@ void find_pairs(fp_handle h, const std::vector<std::vector<Use>>& uses) {
             a.C_pad = f.C_pad + (f.proj >= 0 ? h->convs[f.proj].C_pad : 0);
             a.y_split = out.split; a.relu1 = f.relu; a.relu2 = g.relu;
             if (!fp::plan_pair(a, &f.pair_plan)) continue;
+            a.y_quarter = out.split;
+            for (const Use& other : uses[f.out])
+                if (other.op != u.op && (h->ops[other.op].kind != 0 || split_reader(h->convs[h->ops[other.op].idx]) != 'B')) a.y_quarter = 0;
             f.pair = h->ops[u.op].idx;
             g.paired = 1;
             break;
@@ -1612,6 +1616,7 @@ void launch_op(fp_handle h, int op_index, const void* d_input, int batch, float*
         const FConv& f = h->convs[op.idx];
         fp::PairArgs a = f.pair_args;
         a.N = batch;
+        if (h->whole_outputs) a.y_quarter = 0;
         fp::launch_pair(f.pair_plan, a, h->d_status, st);
         return;
     }
@@ -2219,7 +2224,9 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
                 // Buffers are reused once their last reader has run, so the tensor may have been overwritten since:
                 // run the forward's launches up to this operator again (same input, same kernels) and stop there.
                 if (!h->last_input) return fail(FP_ERR_ARG, "fp_query: no forward has run yet");
+                h->whole_outputs = 1;
                 for (int j = 0; j <= index; ++j) launch_op(h, j, h->last_input, h->last_batch, h->d_logits_stage, 0);
+                h->whole_outputs = 0;
                 CK(cudaDeviceSynchronize());
             }
             TRY(dev_alloc_raw(h, (void**)&d_tmp, cnt * sizeof(float)));

@@ -210,8 +210,9 @@ struct PairArgs {
     void *y, *z;          // the two outputs, y_split: both parity-split
     int N, P, Q, C_pad, K, K2;          // K, K2: padded filters of the two
     int x2_chunk0, x2_plane_mult, y_split, relu1, relu2, reverse;
+    int y_quarter;                      // y_split: only the parity-00 images of y are written - nobody but 1x1 / stride-2 convolutions reads the rest
 };
-struct PairPlan { int valid, G, x_stages, sum2_stages, slots, slot_bytes, tmem_cols; unsigned smem_bytes; };
+struct PairPlan { int valid, G, x_stages, sum2_stages, slots, w_stages, w_stays, tmem_cols; unsigned smem_bytes; };
 bool plan_pair(const PairArgs& a, PairPlan* plan);       // false where the two do better, or only run, as kernels of their own
 void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStream_t st);
 

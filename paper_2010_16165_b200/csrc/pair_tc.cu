@@ -8,22 +8,23 @@
 //   Here a tile of y stays in shared memory, where it is the second convolution's operand as it lies.
 //   CTA tile      128 consecutive flat positions, all channels; one persistent CTA per SM.
 //   Groups        y is made G channels at a time.  A slot of a ring in shared memory holds a group's shortcut (bulk copies, one run
-//                 of 2 KB per 8 channels), its rows of W1 and its columns of W2.  y takes the shortcut's place: the thread
-//                 that adds a vector of 8 channels writes the sum where it read it.  From there the second convolution's MMAs and
-//                 the bulk copies to memory both take it; the slot is free when both have read it.  Filters come with every tile
-//                 again: they are in L2, and shared memory holds several slots so, which is what keeps enough reads in flight.
+//                 of 2 KB per 8 channels) and then, in its place, y: the thread that adds a vector of 8 channels writes the sum where it
+//                 read it.  From there the second convolution's MMAs and the bulk copies to memory both take it; the slot is free
+//                 when both have read it.
+//   Filters       a group's rows of W1 and its columns of W2 have rings of their own, since either is in use for a short part of a slot's
+//                 time; where both banks fit they are brought once and stay.  Coming with every tile again they come from L2.
 //   Tensor memory the second convolution's sums (K2 columns, over all groups of a tile; two tiles' where they fit) and four stages of
 //                 G columns of the first's.
 //   Latency       A group's way - slot filled, MMAs, commit, accumulator read, sum written, MMAs, copies out - is some 3000 cycles
 //                 of barriers and round trips for a few hundred of work.  So no role waits for another's group before it starts
 //                 its next: each convolution has its issuing warp, and two teams of eight finishing warps take the groups in turn.
-//                 A warp's bulk copies go out one after the other, some 110 cycles each, so four warps share a group's dozen copies
-//                 in and two its copies out (one warp for the former alone took 1100-1500 cycles a group, and that was the kernel's time).
+//                 A warp's bulk copies go out one after the other, some 110 cycles each, so several warps share them (one warp for
+//                 a group's dozen took 1100-1500 cycles a group, and that was the kernel's time).
 //                 z of a tile is finished behind the first groups of the next, so that nobody waits for its last MMAs.
 //   Turns         the numbers of slots and stages are multiples of the number of teams, so a slot, a stage and the barriers of both always
 //                 meet the same team: a warp that skips the others' uses of a barrier could take the parity of an older phase for its own.
-//   Warp roles    warps 0-3 copy in, sixteen warps finish both convolutions, one warp each issues the MMAs of the first and of
-//                 the second, two copy y out.
+//   Warp roles    warps 0 and 1 bring x and shortcuts, 2 and 3 the filters of the two convolutions, sixteen warps finish both, one
+//                 warp each issues the MMAs of the first and of the second, two copy y out.
 //   Sums          in the order of the two kernels this stands for (conv_tc.cu), so the results are theirs bit by bit.
 //   Waits         bounded as in conv_tc.cu.
 #include "fp_internal.h"
@@ -37,8 +38,8 @@ namespace {
 
 using namespace tc;
 
-constexpr int kMaxSlots = 8, kSums = 4;
-constexpr int kInWarps = 4, kTeams = 2, kTeamWarps = 8, kOutWarps = 2;
+constexpr int kMaxSlots = 8, kSums = 4, kMaxFilters = 8;
+constexpr int kRunWarps = 2, kInWarps = kRunWarps + 2, kTeams = 2, kTeamWarps = 8, kOutWarps = 2;
 constexpr int kEpi0 = kInWarps, kFirst = kEpi0 + kTeams * kTeamWarps, kSecond = kFirst + 1, kOut0 = kSecond + 1;      // warps
 constexpr int kThreads = 32 * (kOut0 + kOutWarps);
 constexpr unsigned kSmemMax = 232448u - 1024u;
@@ -46,6 +47,7 @@ constexpr unsigned kSmemMax = 232448u - 1024u;
 struct PairCtrl {
     uint64_t slot_full[kMaxSlots], slot_empty[kMaxSlots], y_ready[kMaxSlots];
     uint64_t sum1_full[kSums], sum1_empty[kSums];
+    uint64_t w_full[2][kMaxFilters], w_empty[2][kMaxFilters];
     uint64_t x_full[2], x_empty[2];
     uint64_t sum2_full[2], sum2_empty[2];      // by the parity of the tile's number, which is its team and, with two stages, its stage
     uint32_t tmem_base;
@@ -60,7 +62,7 @@ struct PairParams {
     int Qp, P2, m_total, m_tiles, m_first, m_sign;
     long long plane_x, plane_x2, plane_y;      // vectors per chunk plane (the shortcut's planes are m_total apart)
     int chunks1, chunks, groups;               // channel chunks of x, of y; groups of y
-    int x_stages, sum2_stages, slots, slot_bytes, tmem_cols;
+    int x_stages, sum2_stages, slots, w_stages, w_stays, tmem_cols;      // w_stays: all groups' filters have a stage of their own
     int y_P2h, y_Wh2;                          // parity-split output: half-resolution grid
     long long wait_cycles;
     int* status;
@@ -90,11 +92,14 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
     const uint32_t x0 = (base + (uint32_t)sizeof(PairCtrl) + (uint32_t)(p.a.K + p.a.K2) * 4u + 127u) & ~127u;
     const uint32_t x_bytes = (uint32_t)p.chunks1 * 2048u;
     const uint32_t slot0 = x0 + (uint32_t)p.x_stages * x_bytes;
-    const uint32_t w1_off = GC * 2048u, w2_off = w1_off + (uint32_t)(p.chunks1 * G) * 16u;      // within a slot
+    constexpr uint32_t slot_bytes = GC * 2048u;
+    const uint32_t w1_bytes = (uint32_t)(p.chunks1 * G) * 16u, w2_bytes = (uint32_t)(GC * p.a.K2) * 16u;
+    const uint32_t w1_at = slot0 + (uint32_t)p.slots * slot_bytes, w2_at = w1_at + (uint32_t)p.w_stages * w1_bytes;
     const uint32_t slot_full0 = base + (uint32_t)offsetof(PairCtrl, slot_full), slot_empty0 = base + (uint32_t)offsetof(PairCtrl, slot_empty);
     const uint32_t y_ready0 = base + (uint32_t)offsetof(PairCtrl, y_ready);
     const uint32_t x_full0 = base + (uint32_t)offsetof(PairCtrl, x_full), x_empty0 = base + (uint32_t)offsetof(PairCtrl, x_empty);
     const uint32_t sum1_full0 = base + (uint32_t)offsetof(PairCtrl, sum1_full), sum1_empty0 = base + (uint32_t)offsetof(PairCtrl, sum1_empty);
+    const uint32_t w_full0 = base + (uint32_t)offsetof(PairCtrl, w_full), w_empty0 = base + (uint32_t)offsetof(PairCtrl, w_empty);
     const uint32_t sum2_full0 = base + (uint32_t)offsetof(PairCtrl, sum2_full), sum2_empty0 = base + (uint32_t)offsetof(PairCtrl, sum2_empty);
     volatile int* abort_flag = &ctrl->abort_flag;
     const long long limit = p.wait_cycles > 0 ? p.wait_cycles : kWaitCycles;
@@ -102,7 +107,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxSlots; ++s) {
-            mbar_init(slot_full0 + 8 * s, 1);
+            mbar_init(slot_full0 + 8 * s, kRunWarps);
             mbar_init(slot_empty0 + 8 * s, 1 + kOutWarps);          // the second convolution's MMAs, the copies to memory
             mbar_init(y_ready0 + 8 * s, 32 * kTeamWarps);
         }
@@ -110,8 +115,12 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
             mbar_init(sum1_full0 + 8 * s, 1);
             mbar_init(sum1_empty0 + 8 * s, 32 * kTeamWarps);
         }
+        for (int s = 0; s < 2 * kMaxFilters; ++s) {
+            mbar_init(w_full0 + 8 * s, 1);
+            mbar_init(w_empty0 + 8 * s, 1);
+        }
         for (int s = 0; s < 2; ++s) {
-            mbar_init(x_full0 + 8 * s, 1);
+            mbar_init(x_full0 + 8 * s, kRunWarps);
             mbar_init(x_empty0 + 8 * s, 1);
         }
         for (int s = 0; s < 2; ++s) {
@@ -135,47 +144,66 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&ctrl->tmem_base);
     const uint32_t tmem_sum1 = tmem + (uint32_t)(p.sum2_stages * p.a.K2);             // the first convolution's stages behind the second's sums
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (warp < kRunWarps || warp >= kInWarps) asm volatile("griddepcontrol.wait;" ::: "memory");      // (filters: not the previous kernel's)
 
     auto wait_all = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit)) != 0; };
     auto chunks_of = [&](int g) { return min(GC, p.chunks - g * GC); };
     const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);      // see conv_tc.cu
     bool ok = true;
-    Ring slot, sum, xs;
-    if (warp < kInWarps) {
-        // ------------------------------ copies in: each warp a quarter of the runs and half of one of the filters ------------------------------
+    Ring slot, sum, xs, filters;
+    // the next group's filters: their stage is another, or - where all stay - the group's own, filled once
+    auto next_filters = [&](int g) {
+        if (!p.w_stays) filters.next(p.w_stages);
+        else filters.at = g + 1 < p.groups ? (uint32_t)g + 1u : 0u;
+    };
+    if (warp < kRunWarps) {
+        // ------------------------------ x and the shortcut: each warp half of the runs ------------------------------
         const uint4* xv = reinterpret_cast<const uint4*>(p.a.x);
         const uint4* x2v = reinterpret_cast<const uint4*>(p.a.x2);
         const uint4* rv = reinterpret_cast<const uint4*>(p.a.res);
         const int chunk2 = p.a.x2_chunk0 > 0 ? p.a.x2_chunk0 : p.chunks1;
-        const uint32_t w1_bytes = (uint32_t)(p.chunks1 * G) * 16u, w2_step = (uint32_t)(GC * p.a.K2) * 16u;
+        auto share = [&](int n) { return (uint32_t)((n + kRunWarps - 1 - warp) / kRunWarps) * 2048u; };
         for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x) {
             const long long f0 = (long long)(p.m_first + p.m_sign * tile) * 128;
             if (!(ok = wait_all(x_empty0 + 8 * xs.at, xs.phase ^ 1))) break;
-            if (warp == 0 && lane == 0) mbar_expect_tx(x_full0 + 8 * xs.at, x_bytes);
+            if (lane == 0) mbar_expect_tx(x_full0 + 8 * xs.at, share(p.chunks1));
             __syncwarp();
-            for (int c = warp + kInWarps * lane; c < p.chunks1; c += 32 * kInWarps)
+            for (int c = warp + kRunWarps * lane; c < p.chunks1; c += 32 * kRunWarps)
                 bulk_copy(x0 + xs.at * x_bytes + (uint32_t)c * 2048u,
                           (c < chunk2 ? xv + (long long)c * p.plane_x : x2v + (long long)(c - chunk2) * p.plane_x2) + f0, 2048u, x_full0 + 8 * xs.at);
             xs.next(p.x_stages);
             for (int g = 0; g < p.groups; ++g) {
                 if (!(ok = wait_all(slot_empty0 + 8 * slot.at, slot.phase ^ 1))) break;
-                const int cg = chunks_of(g);
-                const uint32_t dst = slot0 + slot.at * (uint32_t)p.slot_bytes, bar = slot_full0 + 8 * slot.at;
-                const uint32_t w2_bytes = (uint32_t)(cg * p.a.K2) * 16u;
-                // (the others' bytes may be counted before they are expected: the barrier's phase ends no earlier than with this arrival)
-                if (warp == 0 && lane == 0) mbar_expect_tx(bar, (rv ? (uint32_t)cg * 2048u : 0u) + w1_bytes + w2_bytes);
+                const int cg = rv ? chunks_of(g) : 0, c = warp + kRunWarps * lane;
+                if (lane == 0) mbar_expect_tx(slot_full0 + 8 * slot.at, share(cg));
                 __syncwarp();
-                if (lane == 0) {
-                    const uint32_t bytes = warp < 2 ? w1_bytes : w2_bytes, half = bytes / 32u * 16u, off = warp & 1 ? half : 0u;
-                    const uint8_t* src = reinterpret_cast<const uint8_t*>(warp < 2 ? p.a.w1 : p.a.w2) + (long long)g * (warp < 2 ? w1_bytes : w2_step);
-                    bulk_copy(dst + (warp < 2 ? w1_off : w2_off) + off, src + off, warp & 1 ? bytes - half : half, bar);
-                } else if (const int c = warp + kInWarps * (lane - 1); rv && c < cg) {
-                    bulk_copy(dst + (uint32_t)c * 2048u, rv + (long long)(g * GC + c) * p.m_total + f0, 2048u, bar);
-                }
+                if (c < cg)
+                    bulk_copy(slot0 + slot.at * slot_bytes + (uint32_t)c * 2048u, rv + (long long)(g * GC + c) * p.m_total + f0, 2048u, slot_full0 + 8 * slot.at);
                 __syncwarp();
                 slot.next(p.slots);
             }
+        }
+        if (!ok && lane == 0) { atomicExch(&ctrl->abort_flag, 1); atomicExch(p.status, 1); }
+    } else if (warp < kInWarps) {
+        // ------------------------------ filters of one convolution ------------------------------
+        const int which = warp - kRunWarps;
+        const uint8_t* src = reinterpret_cast<const uint8_t*>(which ? p.a.w2 : p.a.w1);
+        const uint32_t stage_bytes = which ? w2_bytes : w1_bytes, at = which ? w2_at : w1_at;
+        const uint32_t full = w_full0 + (uint32_t)which * 8u * kMaxFilters, empty = w_empty0 + (uint32_t)which * 8u * kMaxFilters;
+        for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x) {
+            for (int g = 0; g < p.groups; ++g) {
+                if (!p.w_stays && !(ok = wait_all(empty + 8 * filters.at, filters.phase ^ 1))) break;
+                const uint32_t bytes = which ? (uint32_t)(chunks_of(g) * p.a.K2) * 16u : w1_bytes, half = bytes / 32u * 16u;
+                if (lane == 0) mbar_expect_tx(full + 8 * filters.at, bytes);
+                __syncwarp();
+                if (lane < 2) {
+                    const uint32_t off = lane ? half : 0u;
+                    bulk_copy(at + filters.at * stage_bytes + off, src + (long long)g * stage_bytes + off, lane ? bytes - half : half, full + 8 * filters.at);
+                }
+                __syncwarp();
+                next_filters(g);
+            }
+            if (p.w_stays) break;
         }
         if (!ok && lane == 0) { atomicExch(&ctrl->abort_flag, 1); atomicExch(p.status, 1); }
     } else if (warp == kFirst) {
@@ -184,11 +212,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
         for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x) {
             if (!(ok = wait_all(x_full0 + 8 * xs.at, xs.phase))) break;
             for (int g = 0; g < p.groups; ++g) {
-                if (!(ok = wait_all(slot_full0 + 8 * slot.at, slot.phase) && wait_all(sum1_empty0 + 8 * sum.at, sum.phase ^ 1))) break;
+                if (!(ok = wait_all(w_full0 + 8 * filters.at, filters.phase) && wait_all(sum1_empty0 + 8 * sum.at, sum.phase ^ 1))) break;
                 tc_fence_after();
                 const uint32_t idesc = idesc0 | ((uint32_t)chunks_of(g) << 17);
                 uint32_t a_lo = ((x0 + xs.at * x_bytes) >> 4) | (128u << 16);
-                uint32_t b_lo = ((slot0 + slot.at * (uint32_t)p.slot_bytes + w1_off) >> 4) | ((uint32_t)G << 16);
+                uint32_t b_lo = ((w1_at + filters.at * w1_bytes) >> 4) | ((uint32_t)G << 16);
                 const uint32_t d = tmem_sum1 + sum.at * (uint32_t)G;
 #pragma unroll 1
                 for (int i = 0; i < p.chunks1 >> 1; ++i) {
@@ -197,9 +225,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                     b_lo += 2u * (uint32_t)G;
                 }
                 if (leader) umma_commit(sum1_full0 + 8 * sum.at);
+                if (leader && !p.w_stays) umma_commit(w_empty0 + 8 * filters.at);
                 if (leader && g == p.groups - 1) umma_commit(x_empty0 + 8 * xs.at);
                 __syncwarp();
-                slot.next(p.slots);
+                next_filters(g);
                 sum.next(kSums);
             }
             xs.next(p.x_stages);
@@ -210,7 +239,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
         constexpr int HC = G / 16;                                  // chunks of a group that a warp finishes: half of them
         const int team = (warp - kEpi0) / kTeamWarps, quarter = warp & 3, half = ((warp - kEpi0) >> 2) & 1, row = quarter * 32 + lane;
         const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
-        struct Place { bool exists, interior; long long f; };
+        struct Place { bool exists, interior, y_kept; long long f; };
         auto place_of = [&](int tile) {                             // this thread's position; f: its vector in y's and z's planes
             Place o;
             const int f = (p.m_first + p.m_sign * tile) * 128 + row;
@@ -219,9 +248,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
             o.exists = f < p.m_total;
             o.interior = o.exists && hp >= 1 && hp <= p.a.P && wq >= 1 && wq <= p.a.Q;
             o.f = f;
+            o.y_kept = o.exists;
             if (p.a.y_split) {                                      // see conv_tc.cu: the pixel's place in its parity image
                 const int h = hp - 1, w = wq - 1;
                 const int pp = (h & 1) ? ((w & 1) ? 2 : 1) : ((w & 1) ? 3 : 0);
+                if (p.a.y_quarter && pp) o.y_kept = false;
                 o.f = ((long long)pp * p.a.N + n) * p.y_P2h + ((h >> 1) + 1) * p.y_Wh2 + ((w >> 1) + 1);
             }
             return o;
@@ -271,7 +302,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                     if (G == 64) tmem_ld32(tmem_sum1 + lanes + sum.at * (uint32_t)G + (uint32_t)(half * (G / 2)), reinterpret_cast<uint32_t (&)[32]>(v));
                     else tmem_ld16(tmem_sum1 + lanes + sum.at * (uint32_t)G + (uint32_t)(half * (G / 2)), reinterpret_cast<uint32_t (&)[16]>(v));
                     const int c0 = g * GC + half * HC;
-                    uint8_t* at = smem_raw + (slot0 - base) + slot.at * (uint32_t)p.slot_bytes + (uint32_t)(half * HC) * 2048u + (uint32_t)row * 16u;
+                    uint8_t* at = smem_raw + (slot0 - base) + slot.at * slot_bytes + (uint32_t)(half * HC) * 2048u + (uint32_t)row * 16u;
                     uint4 r[HC];
 #pragma unroll
                     for (int c = 0; c < HC; ++c) r[c] = p.a.res ? *reinterpret_cast<const uint4*>(at + c * 2048) : make_uint4(0, 0, 0, 0);
@@ -294,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                         uint4 out = pack(s, p.a.relu1);
                         if (!o.interior) out = make_uint4(0, 0, 0, 0);
                         *reinterpret_cast<uint4*>(at + c * 2048) = out;
-                        if (p.a.y_split && o.exists) yv[(long long)(c0 + c) * p.plane_y + o.f] = out;
+                        if (p.a.y_split && o.y_kept) yv[(long long)(c0 + c) * p.plane_y + o.f] = out;
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // for the MMAs and the copies out
                     mbar_arrive(y_ready0 + 8 * slot.at);
@@ -319,13 +350,12 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
         for (int tile = blockIdx.x; tile < p.m_tiles && ok; tile += gridDim.x, ++local) {
             const uint32_t d = tmem + (uint32_t)((local & (p.sum2_stages - 1)) * p.a.K2);
             for (int g = 0; g < p.groups; ++g) {
-                if (!(ok = wait_all(y_ready0 + 8 * slot.at, slot.phase))) break;
+                if (!(ok = wait_all(w_full0 + 8 * (kMaxFilters + filters.at), filters.phase) && wait_all(y_ready0 + 8 * slot.at, slot.phase))) break;
                 // the stage's columns were last used sum2_stages tiles ago: z of that tile has been read
                 const int read = local - p.sum2_stages;
                 if (g == 0 && read >= 0 && !(ok = wait_all(sum2_empty0 + 8 * (read & 1), (uint32_t)(read >> 1) & 1u))) break;
                 tc_fence_after();
-                const uint32_t at = slot0 + slot.at * (uint32_t)p.slot_bytes;
-                uint32_t a_lo = (at >> 4) | (128u << 16), b_lo = ((at + w2_off) >> 4) | ((uint32_t)p.a.K2 << 16);
+                uint32_t a_lo = ((slot0 + slot.at * slot_bytes) >> 4) | (128u << 16), b_lo = ((w2_at + filters.at * w2_bytes) >> 4) | ((uint32_t)p.a.K2 << 16);
                 const int ks = chunks_of(g) >> 1;
 #pragma unroll 1
                 for (int i = 0; i < ks; ++i) {
@@ -334,9 +364,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                     b_lo += 2u * (uint32_t)p.a.K2;
                 }
                 if (leader) umma_commit(slot_empty0 + 8 * slot.at);
+                if (leader && !p.w_stays) umma_commit(w_empty0 + 8 * (kMaxFilters + filters.at));
                 if (leader && g == p.groups - 1) umma_commit(sum2_full0 + 8 * (local & 1));
                 __syncwarp();
                 slot.next(p.slots);
+                next_filters(g);
             }
         }
         if (!ok && leader) { atomicExch(&ctrl->abort_flag, 1); atomicExch(p.status, 4); }
@@ -351,7 +383,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                 if (!(ok = wait_all(y_ready0 + 8 * slot.at, slot.phase))) break;
                 const int c = turn + kOutWarps * lane;
                 if (!p.a.y_split && c < chunks_of(g)) {
-                    bulk_store(yv + (long long)(g * GC + c) * p.plane_y + f0, slot0 + slot.at * (uint32_t)p.slot_bytes + (uint32_t)c * 2048u, bytes);
+                    bulk_store(yv + (long long)(g * GC + c) * p.plane_y + f0, slot0 + slot.at * slot_bytes + (uint32_t)c * 2048u, bytes);
                     bulk_store_commit();
                     bulk_store_wait_read();
                 }
@@ -386,15 +418,22 @@ bool plan_pair(const PairArgs& a, PairPlan* plan) {
         const int sum2_stages = 2 * a.K2 + kSums * G <= 512 ? 2 : 1;
         int cols = 32;
         while (cols < sum2_stages * a.K2 + kSums * G) cols *= 2;
-        const unsigned fixed = (unsigned)sizeof(PairCtrl) + (unsigned)(a.K + a.K2) * 4u + 128u, x_bytes = (unsigned)(a.C_pad / 8) * 2048u;
-        const unsigned slot = (unsigned)(G / 8) * 2048u + (unsigned)(a.C_pad / 8 * G) * 16u + (unsigned)(G / 8 * a.K2) * 16u;
+        const unsigned x_bytes = (unsigned)(a.C_pad / 8) * 2048u, slot = (unsigned)(G / 8) * 2048u;
+        const unsigned filters = (unsigned)(a.C_pad / 8 * G) * 16u + (unsigned)(G / 8 * a.K2) * 16u;
+        const unsigned fixed = (unsigned)sizeof(PairCtrl) + (unsigned)(a.K + a.K2) * 4u + 128u;
+        const int groups = (a.K + G - 1) / G;
+        auto slots_with = [&](int xs, int ws) {
+            const unsigned used = fixed + (unsigned)xs * x_bytes + (unsigned)ws * filters;
+            return used < kSmemMax ? (int)((kSmemMax - used) / slot) & ~1 : 0;
+        };
+        const bool stays = groups <= kMaxFilters && slots_with(2, groups) >= 4;
+        const int ws = stays ? groups : 2;
         for (int xs = 2; xs >= 1; --xs) {
-            if (fixed + (unsigned)xs * x_bytes >= kSmemMax) continue;
-            const int slots = (int)((kSmemMax - fixed - (unsigned)xs * x_bytes) / slot) & ~1;
+            const int slots = slots_with(xs, ws);
             if (slots < 4) continue;
             plan->G = G; plan->x_stages = xs; plan->sum2_stages = sum2_stages; plan->slots = slots < kMaxSlots ? slots : kMaxSlots;
-            plan->slot_bytes = (int)slot; plan->tmem_cols = cols;
-            plan->smem_bytes = fixed + (unsigned)xs * x_bytes + (unsigned)plan->slots * slot;
+            plan->w_stages = ws; plan->w_stays = stays; plan->tmem_cols = cols;
+            plan->smem_bytes = fixed + (unsigned)xs * x_bytes + (unsigned)ws * filters + (unsigned)plan->slots * slot;
             if (cudaFuncSetAttribute(G == 64 ? conv_pair_kernel<64> : conv_pair_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
                 cudaGetLastError();
                 return false;
@@ -420,7 +459,7 @@ void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStr
         p.plane_y = 4LL * a.N * p.y_P2h;
     }
     p.chunks1 = a.C_pad / 8; p.chunks = a.K / 8; p.groups = (a.K + plan.G - 1) / plan.G;
-    p.x_stages = plan.x_stages; p.sum2_stages = plan.sum2_stages; p.slots = plan.slots; p.slot_bytes = plan.slot_bytes; p.tmem_cols = plan.tmem_cols;
+    p.x_stages = plan.x_stages; p.sum2_stages = plan.sum2_stages; p.slots = plan.slots; p.w_stages = plan.w_stages; p.w_stays = plan.w_stays; p.tmem_cols = plan.tmem_cols;
     p.status = d_status;
     p.div_p2out = make_fastdiv((uint32_t)p.P2);
     p.div_qp = make_fastdiv((uint32_t)p.Qp);

@@ -421,6 +421,104 @@ __global__ void __launch_bounds__(32 * kFcWarps, 2) fc_kernel(const float* sums,
     }
 }
 
+// Head, step 2, many images: a block takes 8 * IPL images times 32 classes.  Slabs of 256 channels of the sums and of the FC rows go through
+// shared memory (two on the way behind the one in use), a warp takes 32 channels of each, a lane IPL images times 8 classes of the tile: a
+// vector of 4 channels of an image serves 8 classes and one of a class IPL images, so that 12 shared-memory reads feed 64 pairs of
+// FMAs.  (In the kernel above every lane reads its own channels of every image, four wavefronts for 4 classes: both that and the L2
+// reads of the FC matrix, once for every 8 images, took longer than the FMAs.)  Channels are added in pairs (one instruction
+// for two), each warp's in order, then the pair, then the warps' sums in order.
+constexpr int kTileClasses = 32, kTileSlab4 = 64, kTilePitch4 = kTileSlab4 + 1;      // (rows 16 bytes off a multiple of 128: no bank twice)
+constexpr int kTileStages = 3;
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+constexpr int fc_tile_smem(int ipl) { return kTileStages * (kTileClasses + 8 * ipl) * kTilePitch4 * (int)sizeof(float4); }
+template <int IPL>
+__global__ void __launch_bounds__(256, 1) fc_tile_kernel(const float* sums, int N, int C_pad, const float* __restrict__ fcw,
+                                                         const float* __restrict__ fcb, int n_classes, float* __restrict__ logits) {
+    extern __shared__ float4 sh4[];        // stages: FC rows, then the images' sums
+    constexpr int kImages = 8 * IPL, kStage4 = (kTileClasses + kImages) * kTilePitch4;
+    const int n0 = blockIdx.x * kImages, k0 = (int)(blockIdx.z * gridDim.y + blockIdx.y) * kTileClasses, c4 = C_pad >> 2;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int slabs = (c4 + kTileSlab4 - 1) / kTileSlab4;
+    // A thread brings the same channel vector of every fourth row.  Rows of the tile that do not exist repeat the last one (nobody reads
+    // what they give); channels behind the last are zeros.
+    const int col = threadIdx.x & (kTileSlab4 - 1), row = threadIdx.x / kTileSlab4;
+    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(sh4) + (uint32_t)(row * kTilePitch4 + col) * 16u;
+    auto fetch_rows = [&](int slab, uint32_t stage, bool images) {
+        const int at = slab * kTileSlab4 + col;
+        const float* from = (images ? sums : fcw) + 4 * (size_t)min(at, c4 - 1);
+        const int first = (images ? n0 : k0) + row, last = (images ? N : n_classes) - 1;
+        const uint32_t to = mine + (stage * kStage4 + (images ? kTileClasses * kTilePitch4 : 0)) * 16u;
+#pragma unroll
+        for (int j = 0; j < (images ? kImages : kTileClasses) / 4; ++j)
+            cp_async16(to + (uint32_t)(4 * j * kTilePitch4) * 16u, from + (size_t)min(first + 4 * j, last) * C_pad, at < c4);
+    };
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    fetch_rows(0, 0, false);               // the FC matrix does not wait for the kernel before
+    if (slabs > 1) fetch_rows(1, 1, false);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    fetch_rows(0, 0, true);
+    commit();
+    if (slabs > 1) fetch_rows(1, 1, true);
+    commit();
+    unsigned long long acc[IPL][8];
+#pragma unroll
+    for (int i = 0; i < IPL; ++i)
+#pragma unroll
+        for (int t = 0; t < 8; ++t) acc[i][t] = 0ull;
+    const int li = lane & 7, lc = lane >> 3;      // image li + 8 i, class lc + 4 t
+    uint32_t stage = 0;
+    for (int slab = 0; slab < slabs; ++slab) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();                   // this slab is there, and the one before has been used
+        if (slab + 2 < slabs) {
+            const uint32_t to = stage == 0 ? 2 : stage - 1;
+            fetch_rows(slab + 2, to, false);
+            fetch_rows(slab + 2, to, true);
+        }
+        commit();
+        const ulonglong2* w = reinterpret_cast<const ulonglong2*>(sh4 + stage * kStage4 + lc * kTilePitch4 + warp * (kTileSlab4 / 8));
+        const ulonglong2* s = reinterpret_cast<const ulonglong2*>(sh4 + stage * kStage4 + (kTileClasses + li) * kTilePitch4 + warp * (kTileSlab4 / 8));
+#pragma unroll
+        for (int c = 0; c < kTileSlab4 / 8; ++c) {
+            ulonglong2 sv[IPL];
+#pragma unroll
+            for (int i = 0; i < IPL; ++i) sv[i] = s[8 * i * kTilePitch4 + c];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const ulonglong2 wv = w[4 * t * kTilePitch4 + c];
+#pragma unroll
+                for (int i = 0; i < IPL; ++i) {
+                    fma2(acc[i][t], sv[i].x, wv.x);
+                    fma2(acc[i][t], sv[i].y, wv.y);
+                }
+            }
+        }
+        if (++stage == kTileStages) stage = 0;
+    }
+    __syncthreads();
+    float* part = reinterpret_cast<float*>(sh4);                 // [warp][image][class], a float behind every row
+#pragma unroll
+    for (int i = 0; i < IPL; ++i)
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const float2 v = *reinterpret_cast<const float2*>(&acc[i][t]);
+            part[(warp * kImages + li + 8 * i) * (kTileClasses + 1) + lc + 4 * t] = v.x + v.y;
+        }
+    __syncthreads();
+    for (int o = threadIdx.x; o < kImages * kTileClasses; o += 256) {
+        const int i = o / kTileClasses, t = o - i * kTileClasses;
+        float v = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v += part[(k * kImages + i) * (kTileClasses + 1) + t];
+        if (n0 + i < N && k0 + t < n_classes) logits[(size_t)(n0 + i) * n_classes + k0 + t] = v + (fcb ? fcb[k0 + t] : 0.0f);
+    }
+}
+
 template <bool BF16>
 __global__ void planar_to_nchw_f32_kernel(const void* __restrict__ x, float* __restrict__ out, int N, int H, int W,
                                           int chunks, int C_out, int split) {
@@ -500,19 +598,28 @@ void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, con
     cudaLaunchKernelEx(&cfg, is_bf16 ? pool_sum_kernel<true> : pool_sum_kernel<false>, x, N, H, W, chunks, pool_scratch);
     // classes per warp: one while that is what fills the GPU, four once there are blocks enough
     typedef void (*Fc)(const float*, int, int, const float*, const float*, int, float*);
-    const int images = N == 1 ? 1 : N <= 4 ? 4 : 8, groups = (N + images - 1) / images;
+    // many images: tiles of 32, 16 or 8 images times 32 classes, the widest that gives most SMs one
+    const int tile_blocks = (n_classes + kTileClasses - 1) / kTileClasses;
+    int ipl = 4;
+    while (ipl > 1 && (N + 8 * ipl - 1) / (8 * ipl) * tile_blocks < sm_count() * 2 / 3) ipl >>= 1;
+    const bool tiled = N >= 16 && n_classes >= kTileClasses;
+    const int images = tiled ? 8 * ipl : N == 1 ? 1 : N <= 4 ? 4 : 8, groups = (N + images - 1) / images;
     const int cpw = images < 8 ? 1 : groups * ((n_classes + 31) / 32) >= 2 * sm_count() ? 4 : groups * ((n_classes + 15) / 16) >= sm_count() ? 2 : 1;
-    const Fc fn = cpw == 4 ? (Fc)fc_kernel<8, 4, 2> : cpw == 2 ? (Fc)fc_kernel<8, 2, 4> : images == 8 ? (Fc)fc_kernel<8, 1, 8>
+    const Fc fn = tiled ? (ipl == 4 ? (Fc)fc_tile_kernel<4> : ipl == 2 ? (Fc)fc_tile_kernel<2> : (Fc)fc_tile_kernel<1>)
+                : cpw == 4 ? (Fc)fc_kernel<8, 4, 2> : cpw == 2 ? (Fc)fc_kernel<8, 2, 4> : images == 8 ? (Fc)fc_kernel<8, 1, 8>
                 : images == 4 ? (Fc)fc_kernel<4, 1, 8> : (Fc)fc_kernel<1, 1, 16>;
     // (65535 blocks are the most along y; a matrix of more classes goes on along z)
-    const unsigned class_blocks = (unsigned)((n_classes + kFcWarps * cpw - 1) / (kFcWarps * cpw)), along_y = std::min(class_blocks, 65535u);
+    const unsigned class_blocks = tiled ? (unsigned)tile_blocks : (unsigned)((n_classes + kFcWarps * cpw - 1) / (kFcWarps * cpw)), along_y = std::min(class_blocks, 65535u);
     cfg.gridDim = dim3((unsigned)groups, along_y, (class_blocks + along_y - 1) / along_y);
-    cfg.dynamicSmemBytes = (size_t)images * kFcPitch4 * sizeof(float4);
+    cfg.dynamicSmemBytes = tiled ? (size_t)fc_tile_smem(ipl) : (size_t)images * kFcPitch4 * sizeof(float4);
     static std::atomic<bool> raised[64];   // per device, once (threads may all be the first)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !raised[dev]) {
         for (Fc f : {(Fc)fc_kernel<8, 1, 8>, (Fc)fc_kernel<8, 2, 4>, (Fc)fc_kernel<8, 4, 2>})
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * kFcPitch4 * sizeof(float4)));
+        cudaFuncSetAttribute(fc_tile_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(4));
+        cudaFuncSetAttribute(fc_tile_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(2));
+        cudaFuncSetAttribute(fc_tile_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(1));
         if (dev >= 0 && dev < 64) raised[dev] = true;
     }
     cudaLaunchKernelEx(&cfg, fn, (const float*)pool_scratch, N, C_pad, fcw, fcb, n_classes, logits);

@@ -1312,7 +1312,7 @@ fp_status build_plan(fp_handle h) {
                     j.cg = j.chunks;
                 }
                 if (f.pair >= 0) {
-                    j.n_tile = f.pair_plan.G; j.rows = round_up(f.K_pad, f.pair_plan.G);
+                    j.n_tile = fp::kPairGroup; j.rows = round_up(f.K_pad, fp::kPairGroup);
                 } else if (f.tc.valid && f.tc.blocked_bank && !f.plain_bank && !f.paired) {
                     // the streamed form of the kernel reads its bank block by block, one copy per pipeline stage; gathered and
                     // resident layers with several filter tiles read it tile by tile

@@ -205,14 +205,15 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
 struct PairArgs {
     const void *x, *x2;   // input of the first layer; chunks >= x2_chunk0 (0: none) come from x2, as in ConvArgs
     const void* res;      // its shortcut operand, on its output's grid, or nullptr
-    const void *w1, *w2;  // filters: [group of G][C_pad / 8][G rows][8] and [K / 8][K2][8]
+    const void *w1, *w2;  // filters: [group of kPairGroup][C_pad / 8][kPairGroup rows][8] and [K / 8][K2][8]
     const float *bias1, *bias2;
     void *y, *z;          // the two outputs, y_split: both parity-split
     int N, P, Q, C_pad, K, K2;          // K, K2: padded filters of the two
     int x2_chunk0, x2_plane_mult, y_split, relu1, relu2, reverse;
     int y_quarter;                      // y_split: only the parity-00 images of y are written - nobody but 1x1 / stride-2 convolutions reads the rest
 };
-struct PairPlan { int valid, G, x_stages, sum2_stages, slots, w_stages, w_stays, tmem_cols; unsigned smem_bytes; };
+constexpr int kPairGroup = 64;          // channels of y made at a time
+struct PairPlan { int valid, x_stages, sum2_stages, slots, w_stages, w_stays, tmem_cols; unsigned smem_bytes; };
 bool plan_pair(const PairArgs& a, PairPlan* plan);       // false where the two do better, or only run, as kernels of their own
 void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStream_t st);
 

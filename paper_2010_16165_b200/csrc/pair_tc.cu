@@ -7,14 +7,14 @@
 //   little arithmetic on it (48 -> 256 -> 48 channels): as kernels of their own they write it and read it again at the copy rate.
 //   Here a tile of y stays in shared memory, where it is the second convolution's operand as it lies.
 //   CTA tile      128 consecutive flat positions, all channels; one persistent CTA per SM.
-//   Groups        y is made G channels at a time.  A slot of a ring in shared memory holds a group's shortcut (bulk copies, one run
+//   Groups        y is made 64 channels at a time.  A slot of a ring in shared memory holds a group's shortcut (bulk copies, one run
 //                 of 2 KB per 8 channels) and then, in its place, y: the thread that adds a vector of 8 channels writes the sum where it
 //                 read it.  From there the second convolution's MMAs and the bulk copies to memory both take it; the slot is free
 //                 when both have read it.
 //   Filters       a group's rows of W1 and its columns of W2 have rings of their own, since either is in use for a short part of a slot's
 //                 time; where both banks fit they are brought once and stay.  Coming with every tile again they come from L2.
 //   Tensor memory the second convolution's sums (K2 columns, over all groups of a tile; two tiles' where they fit) and four stages of
-//                 G columns of the first's.
+//                 64 columns of the first's.
 //   Latency       A group's way - slot filled, MMAs, commit, accumulator read, sum written, MMAs, copies out - is some 3000 cycles
 //                 of barriers and round trips for a few hundred of work.  So no role waits for another's group before it starts
 //                 its next: each convolution has its issuing warp, and two teams of eight finishing warps take the groups in turn.
@@ -38,6 +38,7 @@ namespace {
 
 using namespace tc;
 
+constexpr int G = kPairGroup, GC = G / 8;      // channels and chunks of a group
 constexpr int kMaxSlots = 8, kSums = 4, kMaxFilters = 8;
 constexpr int kRunWarps = 2, kInWarps = kRunWarps + 2, kTeams = 2, kTeamWarps = 8, kOutWarps = 2;
 constexpr int kEpi0 = kInWarps, kFirst = kEpi0 + kTeams * kTeamWarps, kSecond = kFirst + 1, kOut0 = kSecond + 1;      // warps
@@ -81,10 +82,8 @@ struct Ring {
     __device__ __forceinline__ void next(int n) { if (++at == (uint32_t)n) { at = 0; phase ^= 1; } }
 };
 
-template <int G>
 __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams p) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
-    constexpr int GC = G / 8;                                       // chunks per group
     PairCtrl* ctrl = reinterpret_cast<PairCtrl*>(smem_raw);
     const uint32_t base = smem_u32(smem_raw);
     float* bias1 = reinterpret_cast<float*>(smem_raw + sizeof(PairCtrl));
@@ -299,8 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                     if (!(ok = wait_all(sum1_full0 + 8 * sum.at, sum.phase) && wait_all(slot_full0 + 8 * slot.at, slot.phase))) break;
                     tc_fence_after();
                     uint32_t v[8 * HC];
-                    if (G == 64) tmem_ld32(tmem_sum1 + lanes + sum.at * (uint32_t)G + (uint32_t)(half * (G / 2)), reinterpret_cast<uint32_t (&)[32]>(v));
-                    else tmem_ld16(tmem_sum1 + lanes + sum.at * (uint32_t)G + (uint32_t)(half * (G / 2)), reinterpret_cast<uint32_t (&)[16]>(v));
+                    tmem_ld32(tmem_sum1 + lanes + sum.at * (uint32_t)G + (uint32_t)(half * (G / 2)), v);
                     const int c0 = g * GC + half * HC;
                     uint8_t* at = smem_raw + (slot0 - base) + slot.at * slot_bytes + (uint32_t)(half * HC) * 2048u + (uint32_t)row * 16u;
                     uint4 r[HC];
@@ -410,39 +408,39 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
 
 }  // namespace
 
+// One CTA per SM takes a tile of 128 positions at a time: below that many tiles the layers of their own spread over more SMs.  And the ring
+// needs four slots: a layer with a projection's channels behind its own (336 -> 512 -> 80 at 28x28, batch 128) leaves room for one; with
+// groups of 32 channels, which would fit, it took 121 us against 87 of the two kernels.  Where it fits it was the shorter
+// way at every size measured, ResNet-50, us of the two kernels -> of this one: batch 128, 56x56 48 -> 256 -> 48 136 -> 84, 28x28
+// 80 -> 512 -> 80 83 -> 50, 14x14 160 -> 1024 -> 160 46 -> 34; batch 32, 56x56 34 -> 23; batch 8, 56x56 13.5 -> 10.2.
 bool plan_pair(const PairArgs& a, PairPlan* plan) {
     plan->valid = 0;
     const int m_tiles = (int)(((long long)a.N * (a.P + 2) * (a.Q + 2) + 127) / 128);
     if (m_tiles < sm_count() || a.K2 > 256) return false;
-    for (int G = 64; G >= 32; G -= 32) {
-        const int sum2_stages = 2 * a.K2 + kSums * G <= 512 ? 2 : 1;
-        int cols = 32;
-        while (cols < sum2_stages * a.K2 + kSums * G) cols *= 2;
-        const unsigned x_bytes = (unsigned)(a.C_pad / 8) * 2048u, slot = (unsigned)(G / 8) * 2048u;
-        const unsigned filters = (unsigned)(a.C_pad / 8 * G) * 16u + (unsigned)(G / 8 * a.K2) * 16u;
-        const unsigned fixed = (unsigned)sizeof(PairCtrl) + (unsigned)(a.K + a.K2) * 4u + 128u;
-        const int groups = (a.K + G - 1) / G;
-        auto slots_with = [&](int xs, int ws) {
-            const unsigned used = fixed + (unsigned)xs * x_bytes + (unsigned)ws * filters;
-            return used < kSmemMax ? (int)((kSmemMax - used) / slot) & ~1 : 0;
-        };
-        const bool stays = groups <= kMaxFilters && slots_with(2, groups) >= 4;
-        const int ws = stays ? groups : 2;
-        for (int xs = 2; xs >= 1; --xs) {
-            const int slots = slots_with(xs, ws);
-            if (slots < 4) continue;
-            plan->G = G; plan->x_stages = xs; plan->sum2_stages = sum2_stages; plan->slots = slots < kMaxSlots ? slots : kMaxSlots;
-            plan->w_stages = ws; plan->w_stays = stays; plan->tmem_cols = cols;
-            plan->smem_bytes = fixed + (unsigned)xs * x_bytes + (unsigned)ws * filters + (unsigned)plan->slots * slot;
-            if (cudaFuncSetAttribute(G == 64 ? conv_pair_kernel<64> : conv_pair_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
-                cudaGetLastError();
-                return false;
-            }
-            plan->valid = 1;
-            return true;
-        }
+    const int sum2_stages = 2 * a.K2 + kSums * G <= 512 ? 2 : 1, groups = (a.K + G - 1) / G;
+    int cols = 32;
+    while (cols < sum2_stages * a.K2 + kSums * G) cols *= 2;
+    const unsigned x_bytes = (unsigned)(a.C_pad / 8) * 2048u, slot = (unsigned)GC * 2048u;
+    const unsigned filters = (unsigned)(a.C_pad / 8 * G) * 16u + (unsigned)(GC * a.K2) * 16u;
+    const unsigned fixed = (unsigned)sizeof(PairCtrl) + (unsigned)(a.K + a.K2) * 4u + 128u;
+    auto slots_with = [&](int xs, int ws) {
+        const unsigned used = fixed + (unsigned)xs * x_bytes + (unsigned)ws * filters;
+        return used < kSmemMax ? (int)((kSmemMax - used) / slot) / kTeams * kTeams : 0;
+    };
+    const bool stays = groups <= kMaxFilters && slots_with(2, groups) >= 4;
+    const int ws = stays ? groups : 2;
+    int xs = 2, slots = slots_with(xs, ws);
+    if (slots < 4) slots = slots_with(--xs, ws);
+    if (slots < 4) return false;
+    if (cudaFuncSetAttribute(conv_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
     }
-    return false;
+    plan->x_stages = xs; plan->sum2_stages = sum2_stages; plan->slots = slots < kMaxSlots ? slots : kMaxSlots;
+    plan->w_stages = ws; plan->w_stays = stays; plan->tmem_cols = cols;
+    plan->smem_bytes = fixed + (unsigned)xs * x_bytes + (unsigned)ws * filters + (unsigned)plan->slots * slot;
+    plan->valid = 1;
+    return true;
 }
 
 void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStream_t st) {
@@ -458,7 +456,7 @@ void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStr
         p.y_Wh2 = (a.Q + 1) / 2 + 2; p.y_P2h = ((a.P + 1) / 2 + 2) * p.y_Wh2;
         p.plane_y = 4LL * a.N * p.y_P2h;
     }
-    p.chunks1 = a.C_pad / 8; p.chunks = a.K / 8; p.groups = (a.K + plan.G - 1) / plan.G;
+    p.chunks1 = a.C_pad / 8; p.chunks = a.K / 8; p.groups = (a.K + G - 1) / G;
     p.x_stages = plan.x_stages; p.sum2_stages = plan.sum2_stages; p.slots = plan.slots; p.w_stages = plan.w_stages; p.w_stays = plan.w_stays; p.tmem_cols = plan.tmem_cols;
     p.status = d_status;
     p.div_p2out = make_fastdiv((uint32_t)p.P2);
@@ -475,7 +473,7 @@ void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStr
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     void* args[1] = {(void*)&p};
-    cudaLaunchKernelExC(&cfg, plan.G == 64 ? (const void*)conv_pair_kernel<64> : (const void*)conv_pair_kernel<32>, args);
+    cudaLaunchKernelExC(&cfg, (const void*)conv_pair_kernel, args);
 }
 
 }  // namespace fp

@@ -1,5 +1,5 @@
 """GPU parity of the average pooling and FC layer: batches at the edges of the image groups (1, 4, 8), classes per warp (1, 2,
-4), channels around the 2048 held at a time, image sizes below and above a warp of positions."""
+4), tiles of 8, 16 and 32 images times 32 classes, channels around the 2048 and the 256 held at a time, image sizes below and above a warp of positions."""
 import numpy as np
 import pytest
 
@@ -31,6 +31,7 @@ def one_layer(batch, hw, channels, classes):
 @pytest.mark.parametrize("batch, hw, channels, classes", [
     (1, 7, 2048, 1000), (1, 4, 2064, 11), (2, 9, 72, 1003), (4, 3, 4112, 9), (5, 7, 512, 1000), (8, 2, 24, 1),
     (9, 7, 2032, 130), (24, 5, 136, 1000), (83, 3, 520, 1000), (97, 3, 2080, 801),
+    (16, 2, 1024, 32), (33, 2, 272, 70), (64, 2, 16, 1000), (129, 2, 784, 1001),      # tiles of 8 (32 and less classes), 16 and 32 images
 ])
 @pytest.mark.parametrize("compute", ["fp32", "tc"])
 def test_head_matches_oracle(B, fpo, batch, hw, channels, classes, compute):

@@ -911,7 +911,7 @@ double layers_cost(fp_handle h) {
         const FConv& f = h->convs[h->ops[i].idx];
         const Tensor& out = h->tensors[f.out];
         us += 5.7;
-        if (f.stride == 1) us += 1.17 * std::ceil((out.H + 2) * (out.W + 2) * N / 128) * 9 * (f.C_pad / 16) * std::max(f.K_pad / 2.0, 32 + f.K_pad / 4.0) / (sms * 1900);
+        if (f.stride == 1) us += 1.17 * std::ceil((double)fp::used_vecs((int)N, out.H, out.W) / 128) * 9 * (f.C_pad / 16) * std::max(f.K_pad / 2.0, 32 + f.K_pad / 4.0) / (sms * 1900);
         else us += 2.5e-4 * N * out.H * out.W * (f.C_pad / 16);
     }
     const Tensor& last = h->tensors[h->head_src];
@@ -1110,7 +1110,7 @@ fp_status build_plan(fp_handle h) {
                 // 41 position tiles; 28 us with zero rows on 84 CTAs, 41 us scattered on 63).
                 int nt_s = 0, nts_s = 0;
                 fp::conv_tc_filter_tile(ga, round_up(f.K_kept, 16), &nt_s, &nts_s);
-                const long long m_tiles = ((long long)ga.N * (ga.P + 2) * (ga.Q + 2) + 127) / 128;
+                const long long m_tiles = (fp::used_vecs(ga.N, ga.P, ga.Q) + 127) / 128;
                 const bool pays = 5 * pipe_cost(round_up(f.K_kept, 16)) <= 4 * pipe_cost(round_up(f.K, 16)) &&
                                   ga.R * ga.S * ga.C_pad >= 1024 && m_tiles * nts_s >= 2 * fp::sm_count();
                 if (!runs_fused && h->scatter_policy >= 0 && (pays || h->scatter_policy > 0)) f.scatter = 1;
@@ -1412,11 +1412,10 @@ fp_status build_plan(fp_handle h) {
         auto place = [&](int tid, int i) {                      // a buffer for a tensor that operator i writes
             Tensor& t = h->tensors[tid];
             // planar-8 with border, plus guard vectors before and after (halo reads of the first/last tiles)
-            t.bytes = ((size_t)(t.C_pad / 8) * h->max_batch * (t.H + 2) * (t.W + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
-            if (t.split)
-                t.bytes = ((size_t)(t.C_pad / 8) * 4 * h->max_batch * ((t.H + 1) / 2 + 2) * ((t.W + 1) / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
-            if (tid == 0 && h->stem_packed)
-                t.bytes = ((size_t)10 * h->max_batch * (t.H / 2 + 2) * (t.W / 2 + 2) + 2 * (size_t)fp::kGuardVectors) * vec_bytes;
+            const int H2 = (t.H + 1) / 2, W2 = (t.W + 1) / 2;
+            const long long vecs = tid == 0 && h->stem_packed ? 10 * fp::plane_vecs(h->max_batch, t.H / 2, t.W / 2)
+                                 : t.C_pad / 8 * (t.split ? fp::plane_vecs(4 * h->max_batch, H2, W2) : fp::plane_vecs(h->max_batch, t.H, t.W));
+            t.bytes = (size_t)(vecs + 2 * fp::kGuardVectors) * vec_bytes;
             int best = -1;
             if (!h->keep_outputs)
                 for (int b = 0; b < (int)bufs.size(); ++b)
@@ -2199,7 +2198,7 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
                 if (index + 2 < (int)h->ops.size() && f.stride == 1 && h->convs[h->ops[index + 1].idx].stride == 1)
                     return fail(FP_ERR_UNSUPPORTED, "fp_query: operator %d runs inside the network's kernel and its output never reaches memory "
                                 "(set keep_outputs to run every layer on its own)", index);
-                const size_t cnt = (size_t)h->last_batch * t.C * t.H * t.W, vecs = (size_t)(t.C_pad / 8) * h->last_batch * (t.H + 2) * (t.W + 2);
+                const size_t cnt = (size_t)h->last_batch * t.C * t.H * t.W, vecs = (size_t)(t.C_pad / 8) * fp::plane_vecs(h->last_batch, t.H, t.W);
                 TRY(need(cnt * sizeof(float)));
                 CK(cudaDeviceSynchronize());
                 float* d_tmp;

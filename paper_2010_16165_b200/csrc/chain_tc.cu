@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
             // ---- zero border of the group's output images in global memory ----
             {
                 const int out_chunks = s_layers[L - 1].K_pad >> 3;
-                const int border = 2 * p.Wp + 2 * H;
+                const int border = 2 * p.Wp + 1 + H;         // the row above, the left column, behind the last image W + 2 more
                 const int total = p.G * border * out_chunks;
                 for (int i = etid; i < total; i += kEpiThreads) {
                     const int c = i / (p.G * border);
@@ -504,8 +504,9 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                     if (n >= p.a.N) continue;
                     int row, col;
                     if (b < p.Wp) { row = 0; col = b; }
-                    else if (b < 2 * p.Wp) { row = H + 1; col = b - p.Wp; }
-                    else { const int s2 = b - 2 * p.Wp; row = 1 + (s2 >> 1); col = (s2 & 1) ? W + 1 : 0; }
+                    else if (b < p.Wp + H) { row = 1 + b - p.Wp; col = 0; }
+                    else if (n == p.a.N - 1) { row = H + 1; col = b - p.Wp - H; }
+                    else continue;
                     yv[(long long)c * p.plane_out + (long long)n * p.P2 + (long long)row * p.Wp + col] = make_uint4(0, 0, 0, 0);
                 }
             }
@@ -608,12 +609,12 @@ void launch_chain_tc(const ChainPlan& plan, const ChainArgs& a, int* d_status, c
     p.n_groups = (a.N + plan.G - 1) / plan.G;
     p.img_pos = (a.H + 1) * a.W;
     p.w_shift = a.W == 8 ? 3 : a.W == 16 ? 4 : 5;
-    p.Wp = a.W + 2; p.P2 = (a.H + 2) * (a.W + 2);
+    p.Wp = row_vecs(a.W); p.P2 = image_vecs(a.H, a.W);
     p.div_rows = make_fastdiv((uint32_t)(a.H + 1));
-    p.plane_in = (long long)a.N * p.P2;
+    p.plane_in = plane_vecs(a.N, a.H, a.W);
     p.plane_out = p.plane_in;
-    p.rWp = a.res_W + 2; p.rP2 = (a.res_H + 2) * (a.res_W + 2);
-    p.plane_res = (long long)a.N * p.rP2;
+    p.rWp = row_vecs(a.res_W); p.rP2 = image_vecs(a.res_H, a.res_W);
+    p.plane_res = plane_vecs(a.N, a.res_H, a.res_W);
     p.status = d_status;
     const int sms = sm_count();
     int grid = p.n_groups < sms ? p.n_groups : sms;

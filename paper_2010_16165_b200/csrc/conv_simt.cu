@@ -22,8 +22,8 @@ __global__ void conv_simt_kernel(ConvArgs a) {
     const T* __restrict__ w = (const T*)a.w;
     const T* __restrict__ res = (const T*)a.res;
     T* __restrict__ y = (T*)a.y;
-    const int Wp = a.W + 2, P2i = (a.H + 2) * Wp, Qp = a.Q + 2, P2o = (a.P + 2) * Qp;
-    const size_t plane_i = (size_t)a.N * P2i, plane_o = (size_t)a.N * P2o;
+    const int Wp = row_vecs(a.W), P2i = image_vecs(a.H, a.W), Qp = row_vecs(a.Q), P2o = image_vecs(a.P, a.Q);
+    const size_t plane_i = (size_t)plane_vecs(a.N, a.H, a.W), plane_o = (size_t)plane_vecs(a.N, a.P, a.Q);
     const int kchunks = a.K_pad / 8, cchunks = a.C_pad / 8;
     const size_t total = plane_o * kchunks;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -35,7 +35,7 @@ __global__ void conv_simt_kernel(ConvArgs a) {
         float acc[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
-        const bool inside = p >= 0 && p < a.P && q >= 0 && q < a.Q;
+        const bool inside = n < (size_t)a.N && p >= 0 && p < a.P && q >= 0 && q < a.Q;
         if (inside) {
             for (int r = 0; r < a.R; ++r) {
                 const int ih = p * a.stride + r - a.pad;
@@ -66,8 +66,8 @@ __global__ void conv_simt_kernel(ConvArgs a) {
                 } else if (a.res_mode == 2) {
                     const int c = k - a.res_pad_lo;
                     if (c >= 0 && c < a.res_C) {
-                        const int rWp = a.res_W + 2, rP2 = (a.res_H + 2) * rWp;
-                        const size_t rv = (size_t)(c / 8) * a.N * rP2 + n * rP2 + (size_t)(p * a.res_stride + 1) * rWp +
+                        const int rWp = row_vecs(a.res_W), rP2 = image_vecs(a.res_H, a.res_W);
+                        const size_t rv = (size_t)(c / 8) * plane_vecs(a.N, a.res_H, a.res_W) + n * rP2 + (size_t)(p * a.res_stride + 1) * rWp +
                                           (q * a.res_stride + 1);
                         v += to_f<T>(res[rv * 8 + (c & 7)]);
                     }
@@ -83,7 +83,7 @@ __global__ void conv_simt_kernel(ConvArgs a) {
 }  // namespace
 
 void launch_conv_simt(const ConvArgs& a, int is_bf16, cudaStream_t st) {
-    const size_t total = (size_t)a.N * (a.P + 2) * (a.Q + 2) * (a.K_pad / 8);
+    const size_t total = (size_t)plane_vecs(a.N, a.P, a.Q) * (a.K_pad / 8);
     size_t blocks = (total + 255) / 256;
     const size_t cap = (size_t)sm_count() * 32;
     if (blocks > cap) blocks = cap;

@@ -62,7 +62,7 @@ struct SplitParams {
     int n_tile, n_tiles, tmem_cols, a_stage_bytes, stage_bytes, red_bytes, slots;   // slots: chunks a CTA finishes at most
     int bank_tile_vecs;
     int tap_off[9];
-    int y_P2h, y_Wh2;
+    int y_P2h, y_Wh2, y_edges;
     int skip_round;
     long long wait_cycles;
     int* status;
@@ -432,6 +432,20 @@ __global__ void __launch_bounds__(kThreads, 3) conv_split_kernel(const SplitPara
             }
         }
     }
+    if (p.y_edges && finisher && half == 0 && rank == 0)
+        for (int t = 0; t < p.tps; ++t) {                // see conv_tc.cu: the row and column behind an odd image's last
+            const int f = f0 + t * 128 + row, n = (int)fdiv((uint32_t)f, p.div_p2out), rem = f - n * p.P2_out;
+            const int hp = (int)fdiv((uint32_t)rem, p.div_qp), wq = rem - hp * p.Qp;
+            auto zeros = [&](int h, int w) {
+                const int pp = (h & 1) ? ((w & 1) ? 2 : 1) : ((w & 1) ? 3 : 0);
+                uint4* y = reinterpret_cast<uint4*>(p.a.y) + (long long)(k_base >> 3) * p.plane_y + (pp * p.a.N + n) * p.y_P2h + ((h >> 1) + 1) * p.y_Wh2 + ((w >> 1) + 1);
+                for (int q = 0; q < nch; ++q) y[(long long)q * p.plane_y] = make_uint4(0, 0, 0, 0);
+            };
+            const bool below = f < p.m_total && (p.a.P & 1) && hp == p.a.P, right = f < p.m_total && (p.a.Q & 1) && wq == p.a.Q;
+            if (below) zeros(hp, wq - 1);
+            if (right) zeros(hp - 1, wq);
+            if (below && right) zeros(hp, wq);
+        }
     if (!ok && lane == 0) { atomicExch(&ctrl->abort_flag, 1); atomicExch(p.status, 3); }
 
     if (*abort_flag)
@@ -498,10 +512,10 @@ namespace {
 // per K group.  False where it does not fit; else the launch figures and the time expected.
 bool candidate(const ConvArgs& a, const Room& room, int tps, int n_tile, int splits, int cg, ConvPlanTC* c, double* cost) {
     const int taps = a.R * a.S, cchunks = a.C_pad / 8, a_par = a.x_s2d ? 4 : 1;
-    const int halo = taps == 1 ? 0 : a.W + 3;
+    const int halo = taps == 1 ? 0 : row_vecs(a.W) + 1;
     const int rows_a = round_up_i(128 * tps + (a_par > 1 ? 1 : 2) * halo, 8);
     if (rows_a + 8 > kGuardVectors || tps * n_tile > 256) return false;
-    const int m_tiles = (a.N * (a.P + 2) * (a.Q + 2) + 127) / 128, steps = (m_tiles + tps - 1) / tps;
+    const int m_tiles = (int)((used_vecs(a.N, a.P, a.Q) + 127) / 128), steps = (m_tiles + tps - 1) / tps;
     const int n_tiles = (a.K_pad + n_tile - 1) / n_tile, groups = (cchunks + cg - 1) / cg;
     const int units = steps * n_tiles * splits;
     if (groups < splits || units > room.ctas[1][splits]) return false;
@@ -538,7 +552,7 @@ bool plan_conv_split(const ConvArgs& a, ConvPlanTC* plan) {
     const int taps = a.R * a.S;
     const bool flat = a.stride == 1 && a.P == a.H && a.Q == a.W && ((taps == 1 && a.pad == 0) || (a.R == 3 && a.S == 3 && a.pad == 1));
     if (!flat || a.scatter || a.n_tile_forced > 0 || a.res_mode == 2) return false;
-    if (((long long)a.N * (a.P + 2) * (a.Q + 2) + 127) / 128 > 2 * sm_count()) return false;
+    if ((used_vecs(a.N, a.P, a.Q) + 127) / 128 > 2 * sm_count()) return false;
     for (int k = 0; k < 4; ++k)
         if (cudaFuncSetAttribute(kernel_of(k & 1 ? 9 : 1, 1 + (k >> 1)), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemOne) != cudaSuccess) {
             cudaGetLastError();
@@ -579,15 +593,17 @@ void launch_conv_split(const ConvPlanTC& plan, const ConvArgs& a, int* d_status,
     SplitParams p;
     memset(&p, 0, sizeof(p));
     p.a = a;
-    const int P2_in = (a.H + 2) * (a.W + 2);
-    p.Wp_in = a.W + 2; p.Qp = a.Q + 2; p.P2_out = (a.P + 2) * (a.Q + 2);
-    p.plane_in = a.N * P2_in * (a.x_plane_mult > 1 || a.x_s2d ? 4 : 1);
-    p.plane_in2 = a.N * P2_in * (a.x2_plane_mult > 1 ? 4 : 1);
-    p.par_stride = a.N * P2_in;
-    p.m_total = p.plane_out = p.plane_y = a.N * p.P2_out;
+    p.Wp_in = row_vecs(a.W); p.Qp = row_vecs(a.Q); p.P2_out = image_vecs(a.P, a.Q);
+    p.plane_in = (int)plane_vecs(a.x_plane_mult > 1 || a.x_s2d ? 4 * a.N : a.N, a.H, a.W);
+    p.plane_in2 = (int)plane_vecs(a.x2_plane_mult > 1 ? 4 * a.N : a.N, a.H, a.W);
+    p.par_stride = a.N * image_vecs(a.H, a.W);
+    p.plane_out = p.plane_y = (int)plane_vecs(a.N, a.P, a.Q);
+    p.m_total = (int)used_vecs(a.N, a.P, a.Q);
     if (a.y_split) {
-        p.y_Wh2 = (a.Q + 1) / 2 + 2; p.y_P2h = ((a.P + 1) / 2 + 2) * p.y_Wh2;
-        p.plane_y = 4 * a.N * p.y_P2h;
+        p.y_Wh2 = row_vecs((a.Q + 1) / 2); p.y_P2h = image_vecs((a.P + 1) / 2, (a.Q + 1) / 2);
+        p.plane_y = (int)plane_vecs(4 * a.N, (a.P + 1) / 2, (a.Q + 1) / 2);
+        p.y_edges = (a.P & 1) || (a.Q & 1);
+        p.m_total = a.N * p.P2_out;                      // (nobody reads behind the last image of a split tensor)
     }
     p.taps = a.R * a.S; p.cchunks = a.C_pad / 8; p.cg = plan.cg; p.groups = plan.groups;
     p.cchunks2 = a.x2_C_pad / 8; p.groups2 = (p.cchunks2 + plan.cg - 1) / plan.cg;

@@ -11,9 +11,9 @@
 //                 two such stacks ("planes"), `LBO` apart.
 //   FLAT modes    stride-1 "same" convolutions (3x3 pad 1, 3x1 pad 1x0, 1x1 pad 0).  Because every chunk plane
 //                 is contiguous over flat positions, the activations a tile needs - its 128
-//                 positions plus a halo of (W+3) before and after (3x3) - are ONE contiguous run per
+//                 positions plus a halo of (W+2) before and after (3x3) - are ONE contiguous run per
 //                 chunk, fetched with one bulk copy.  The operand of filter tap (r,s) is the same
-//                 shared-memory block read from a start address shifted by (r-1)*(W+2)+(s-1) rows,
+//                 shared-memory block read from a start address shifted by (r-1)*(W+1)+(s-1) rows,
 //                 so each activation is fetched once per tile, not once per tap.  The zero border
 //                 in memory is the convolution's padding.  Filters either stay resident in shared
 //                 memory for the whole kernel (small banks), are streamed per (filter row, K block) into a ring of
@@ -58,7 +58,7 @@ struct TcParams {
     ConvArgs a;
     FastDiv div_ntiles, div_p2out, div_qp;
     int Wp_in, P2_in, Qp, P2_out;
-    long long plane_in, plane_out;      // vectors per chunk plane (N * P2)
+    long long plane_in, plane_out;      // vectors per chunk plane (fp_internal.h)
     long long m_total;                  // flat output positions
     int taps, cchunks, cg, groups, halo, rows_a, a_stages, b_stages;
     int n_tile, n_tiles, tmem_cols, total_tiles;
@@ -76,6 +76,7 @@ struct TcParams {
     long long par_stride;               // x_s2d: vectors between the parity images of one chunk (N * P2)
     int tap_off[9];                     // x_s2d: start row of each tap's operand within a chunk's part of the stage
     int y_split, y_P2h, y_Wh2;          // split output: half-resolution grid
+    int y_edges;                        // split output of an odd height or width: the odd-parity images' row or column that does not exist
     long long plane_y;                  // vectors per chunk plane of the output tensor
     long long wait_cycles;              // limit of every barrier wait in SM clock cycles (0: about a second)
     int skip_round;                     // diagnostic: the activation producer leaves out this round's copies (-1: none)
@@ -615,7 +616,7 @@ conv_tc_kernel(const TcParams p) {
             }
             long long res_vec = 0;
             if (p.a.res_mode == 2) {
-                const int rWp = p.a.res_W + 2, rP2 = (p.a.res_H + 2) * rWp;
+                const int rWp = row_vecs(p.a.res_W), rP2 = image_vecs(p.a.res_H, p.a.res_W);
                 res_vec = (long long)n * rP2 + (long long)((hp - 1) * p.a.res_stride + 1) * rWp + ((wq - 1) * p.a.res_stride + 1);
             }
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((acc * p.tps + t) * p.n_tile);
@@ -631,7 +632,7 @@ conv_tc_kernel(const TcParams p) {
                     if (half) q_begin = mid; else q_end = mid;
                 }
                 float* strip = sstrip + ((warp - 2) * 32 + lane) * 33;
-                const long long rplane = (long long)p.a.N * (p.a.res_H + 2) * (p.a.res_W + 2);
+                const long long rplane = plane_vecs(p.a.N, p.a.res_H, p.a.res_W);
                 uint4 rnext = make_uint4(0, 0, 0, 0);
                 if (res1 && q_begin < q_end) rnext = __ldg(res + (long long)q_begin * p.plane_out + f);
                 int loaded = -1;                 // accumulator columns [.., loaded) of this tile are in the strip
@@ -788,7 +789,7 @@ conv_tc_kernel(const TcParams p) {
                         }
                     } else if (p.a.res_mode == 2) {
                         // shortcut by subsampling: output channel k takes input channel k - pad_lo
-                        const long long rplane = (long long)p.a.N * (p.a.res_H + 2) * (p.a.res_W + 2);
+                        const long long rplane = plane_vecs(p.a.N, p.a.res_H, p.a.res_W);
 #pragma unroll
                         for (int hh = 0; hh < 2; ++hh) {
                             const int cs = k_base + c0 + 8 * hh - p.a.res_pad_lo;
@@ -830,6 +831,19 @@ conv_tc_kernel(const TcParams p) {
                     rq[6] = __ldg(res + vn);
                     rq[7] = __ldg(res + vn + p.plane_out);
                 }
+            }
+            if (p.y_edges && exists && half == 0) {
+                // a pixel in the last row or column writes zeros where the odd-parity images have a place for the row or column behind it
+                const int first = p.a.scatter ? schunk0[nt] : k_base >> 3, last = p.a.scatter ? schunk0[nt + 1] : (k_base + cols) >> 3;
+                auto zeros = [&](int h, int w) {
+                    const int pp = (h & 1) ? ((w & 1) ? 2 : 1) : ((w & 1) ? 3 : 0);
+                    const long long e = ((long long)pp * p.a.N + n) * p.y_P2h + ((h >> 1) + 1) * p.y_Wh2 + ((w >> 1) + 1);
+                    for (int c = first; c < last; ++c) y[(long long)c * p.plane_y + e] = make_uint4(0, 0, 0, 0);
+                };
+                const bool below = (p.a.P & 1) && hp == p.a.P, right = (p.a.Q & 1) && wq == p.a.Q;
+                if (below) zeros(hp, wq - 1);
+                if (right) zeros(hp - 1, wq);
+                if (below && right) zeros(hp, wq);
             }
             }   // tiles of the step
             if (!ok) break;
@@ -972,7 +986,7 @@ void choose_filter_tile(const ConvArgs& a, int K_pad, int* n_tile_out, int* n_ti
     const int taps = a.R * a.S;
     const bool flat = a.stride == 1 && a.P == a.H && a.Q == a.W &&
                       ((a.R == 1 && a.S == 1 && a.pad == 0) || (a.R == 3 && (a.S == 3 || a.S == 1) && a.pad == 1));
-    const long long m_total = (long long)a.N * (a.P + 2) * (a.Q + 2);
+    const long long m_total = used_vecs(a.N, a.P, a.Q);
     const long long m_tiles = (m_total + 127) / 128;
     int n_tiles = (K_pad + 127) / 128;
     int n_tile = round_up_i((K_pad + n_tiles - 1) / n_tiles, 16);
@@ -1012,7 +1026,7 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
                   ((a.R == 1 && a.S == 1 && a.pad == 0) || (a.R == 3 && (a.S == 3 || a.S == 1) && a.pad == 1))) ? 1 : 0;
     plan->cg = cchunks < 8 ? cchunks : 8;
     plan->groups = (cchunks + plan->cg - 1) / plan->cg;
-    const long long m_total = (long long)a.N * (a.P + 2) * (a.Q + 2);
+    const long long m_total = used_vecs(a.N, a.P, a.Q);
     const long long m_tiles = (m_total + 127) / 128;
     if (m_total + 128 >= (1ll << 31)) { snprintf(err, err_len, "more than 2^31 output positions"); return 1; }
 
@@ -1040,7 +1054,7 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
     smem += scatter_smem;
     int want_ctas = 1;
     if (plan->flat) {
-        plan->halo = ((a.R - 1) / 2) * (a.W + 2) + (a.S - 1) / 2;      // rows above + columns to the left
+        plan->halo = ((a.R - 1) / 2) * row_vecs(a.W) + (a.S - 1) / 2;      // rows above + columns to the left
         plan->tps = 1;
         // A 128-position tile is fetched with `halo` rows on either side.  On wide images (the 112-wide stem: 114
         // rows each side of 128) that is most of the traffic into shared memory, so such a layer takes the
@@ -1183,7 +1197,7 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
         if (plan->tpk < 1) plan->tpk = 1;
         const int planes = plan->groups > 1 ? plan->cg : plan->tpk * cchunks;
         const unsigned stage = (unsigned)(planes * 128 * 16 + planes * n_tile * 16);
-        if ((long long)a.N * (a.H + 2) * (a.W + 2) * cchunks >= (1ll << 31)) { snprintf(err, err_len, "input of more than 2^31 vectors"); return 1; }
+        if (plane_vecs(a.N, a.H, a.W) * cchunks >= (1ll << 31)) { snprintf(err, err_len, "input of more than 2^31 vectors"); return 1; }
         const int kblocks = plan->groups > 1 ? taps * plan->groups : (taps + plan->tpk - 1) / plan->tpk;
         smem += (unsigned)kblocks * 64u;                 // the plane-offset table
         // The loader threads wait out one load latency per K block, so co-resident CTAs are what hides it:
@@ -1245,18 +1259,20 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     TcParams p;
     memset(&p, 0, sizeof(p));
     p.a = a;
-    p.Wp_in = a.W + 2; p.P2_in = (a.H + 2) * (a.W + 2);
-    p.Qp = a.Q + 2; p.P2_out = (a.P + 2) * (a.Q + 2);
-    p.plane_in = (long long)a.N * p.P2_in * (a.x_plane_mult > 1 || a.x_s2d ? 4 : 1);
-    p.plane_in2 = (long long)a.N * p.P2_in * (a.x2_plane_mult > 1 ? 4 : 1);
+    p.Wp_in = row_vecs(a.W); p.P2_in = image_vecs(a.H, a.W);
+    p.Qp = row_vecs(a.Q); p.P2_out = image_vecs(a.P, a.Q);
+    p.plane_in = plane_vecs(a.x_plane_mult > 1 || a.x_s2d ? 4 * a.N : a.N, a.H, a.W);
+    p.plane_in2 = plane_vecs(a.x2_plane_mult > 1 ? 4 * a.N : a.N, a.H, a.W);
     p.cchunks2 = a.x2_C_pad / 8;
     p.groups2 = a.x2_C_pad > 0 ? (p.cchunks2 + plan.cg - 1) / plan.cg : 0;
-    p.plane_out = (long long)a.N * p.P2_out;
-    p.m_total = p.plane_out;
+    p.plane_out = plane_vecs(a.N, a.P, a.Q);
+    p.m_total = used_vecs(a.N, a.P, a.Q);
     p.plane_y = p.plane_out;
     if (a.y_split) {
-        p.y_split = 1; p.y_Wh2 = (a.Q + 1) / 2 + 2; p.y_P2h = ((a.P + 1) / 2 + 2) * p.y_Wh2;
-        p.plane_y = 4ll * a.N * p.y_P2h;
+        p.y_split = 1; p.y_Wh2 = row_vecs((a.Q + 1) / 2); p.y_P2h = image_vecs((a.P + 1) / 2, (a.Q + 1) / 2);
+        p.plane_y = plane_vecs(4 * a.N, (a.P + 1) / 2, (a.Q + 1) / 2);
+        p.y_edges = (a.P & 1) || (a.Q & 1);
+        p.m_total = (long long)a.N * p.P2_out;       // (nobody reads behind the last image of a split tensor)
     }
     p.a_par = a.x_s2d ? 4 : 1;
     p.par_stride = (long long)a.N * p.P2_in;
@@ -1266,7 +1282,7 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
         const int r = t / 3, sx = t % 3;
         const int pa = r == 1 ? 0 : 1, pb = sx == 1 ? 0 : 1;
         const int pp = pa ? (pb ? 2 : 1) : (pb ? 3 : 0);
-        p.tap_off[t] = pp * plan.rows_a + plan.halo + (r == 0 ? -(a.W + 2) : 0) + (sx == 0 ? -1 : 0);
+        p.tap_off[t] = pp * plan.rows_a + plan.halo + (r == 0 ? -p.Wp_in : 0) + (sx == 0 ? -1 : 0);
     }
     p.taps = a.R * a.S; p.cchunks = a.C_pad / 8; p.cg = plan.cg; p.groups = plan.groups;
     p.halo = plan.halo; p.rows_a = plan.rows_a; p.a_stages = plan.a_stages; p.b_stages = plan.b_stages;

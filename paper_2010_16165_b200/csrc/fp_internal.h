@@ -1,14 +1,19 @@
 // Internal declarations shared by the host graph builder and the kernel launchers.
 //
 // Activation layout ("planar-8 with border"): channels are grouped in chunks of 8 (one 16-byte
-// vector of bf16, or 32 bytes of fp32); every image carries a one-pixel border of zeros.
+// vector of bf16, or 32 bytes of fp32); every image has a row of zeros above it and a column of
+// zeros to its left.  The row below an image is the next image's upper one, the column to the
+// right of a row the next row's left one; behind the last image of a plane come W + 2 zeros.
 // For a batch of N images of H x W pixels and C_pad channels the vector of chunk j, image n,
 // pixel (h, w) sits at vector index
-//       j * (N * P2)  +  n * P2  +  (h + 1) * (W + 2)  +  (w + 1),      P2 = (H + 2) * (W + 2).
+//       j * plane  +  n * P2  +  (h + 1) * (W + 1)  +  (w + 1),      P2 = (H + 1) * (W + 1),
+// plane = N * P2 + W + 2 rounded up to whole cache lines.
 // So each chunk is one contiguous plane over the whole batch; a run of consecutive "flat
-// positions" f = n*P2 + (h+1)*(W+2) + (w+1) is contiguous in memory for every chunk, and the
-// 3x3 neighbourhood of position f is f + dr*(W+2) + ds.  Every kernel that writes a tensor
+// positions" f = n*P2 + (h+1)*(W+1) + (w+1) is contiguous in memory for every chunk, and the
+// 3x3 neighbourhood of position f is f + dr*(W+1) + ds.  Every kernel that writes a tensor
 // writes all of its positions, zeros on the border, so the border never has to be cleared.
+// (With a border on all four sides, which was the layout before, 7x7 pixels took 81 positions instead
+// of 64, 14x14 256 instead of 225, 28x28 900 instead of 841: work of every convolution and bytes of every tensor.)
 // Buffers carry `kGuardVectors` vectors of slack before and after the data, because tiles of
 // flat positions read a halo that may start before the first plane or end after the last.
 #pragma once
@@ -39,6 +44,12 @@ inline int sm_count() {
 
 constexpr int kGuardVectors = 1024;   // >= 128 + (W + 3) + 8 for every supported width (W <= 512)
 constexpr int kMaxWidth = 512;
+// Vectors of a row, of an image, of N images with the zeros behind them, and from a chunk's plane to the next one's: whole lines of
+// 128 bytes (without, a warp's 512 bytes lay across 17 sectors: ResNet-50 batch 1 190 -> 195 us).
+__host__ __device__ constexpr int row_vecs(int W) { return W + 1; }
+__host__ __device__ constexpr int image_vecs(int H, int W) { return (H + 1) * (W + 1); }
+__host__ __device__ constexpr long long used_vecs(int N, int H, int W) { return (long long)N * image_vecs(H, W) + W + 2; }
+__host__ __device__ constexpr long long plane_vecs(int N, int H, int W) { return (used_vecs(N, H, W) + 7) / 8 * 8; }
 
 // ---------------------------------------------------------------------------------------
 // Convolution launch description (one fused operator: conv + bias + residual + ReLU)

@@ -50,9 +50,9 @@ __device__ __forceinline__ void store_vec8(void* base, size_t vec, const float (
 template <bool OUT_BF16>
 __global__ void input_to_planar_kernel(const void* __restrict__ in, int in_is_bf16, void* __restrict__ out, int N, int C,
                                        int H, int W, int chunks, int n0, int n_count) {
-    const int Wp = W + 2, P2 = (H + 2) * Wp;
-    const size_t plane = (size_t)N * P2;
-    const size_t part = (size_t)n_count * P2;
+    const int Wp = row_vecs(W), P2 = image_vecs(H, W);
+    const size_t plane = (size_t)plane_vecs(N, H, W);
+    const size_t part = (size_t)n_count * P2 + (n0 + n_count == N ? W + 2 : 0);      // the last images' part: with the zeros behind them
     const size_t total = part * chunks;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int j = (int)(i / part);
@@ -86,19 +86,21 @@ __global__ void input_to_planar_kernel(const void* __restrict__ in, int in_is_bf
 //     O (chunks 6-8):  O [p][q][j] = x[c][2p + 1][2q + s - 3]
 // (chunk 9 is zero padding to an even chunk count).  Output row p needs input rows 2p-3 .. 2p+3, which
 // are O'(p-1), E(p-1), O'(p), E(p), O(p), E(p+1), O(p+1): vertical offsets -1, 0, +1 only.
-// One block per (image, output row incl. the two border rows): the three input rows the output row needs are
+// One block per (image, output row incl. the border row): the three input rows the output row needs are
 // staged in shared memory (coalesced reads, each input element read once per block), then every thread builds
 // packed vectors from them.  32-bit index arithmetic only.
 __global__ void input_to_stem_planar_kernel(const void* __restrict__ in, int in_is_bf16, __nv_bfloat16* __restrict__ out,
                                             int N, int C, int H, int W, int n0) {
     extern __shared__ float rows[];                  // [3 rows: 2p-1, 2p, 2p+1][C][W + 6], zero where outside the image
     __shared__ int tap_off[24];                      // packed channel j = s*C + c -> c*(W+6) + s, or -1 (padding)
-    const int P = H / 2, Q = W / 2, Qp = Q + 2, P2 = (P + 2) * Qp;
-    const int n = n0 + blockIdx.x / (P + 2), pp = blockIdx.x % (P + 2);
+    const int P = H / 2, Q = W / 2, Qp = row_vecs(Q), P2 = image_vecs(P, Q);
+    const int n = n0 + blockIdx.x / (P + 1), pp = blockIdx.x % (P + 1);
     const int p = pp - 1;
-    const size_t plane = (size_t)N * P2;
+    const size_t plane = (size_t)plane_vecs(N, P, Q);
     uint4* outv = reinterpret_cast<uint4*>(out) + (size_t)n * P2 + (size_t)pp * Qp;
-    if (p < 0 || p >= P) {                           // border row: zeros in every chunk
+    if (n == N - 1 && p == P - 1)                    // the zeros behind the last image
+        for (int i = threadIdx.x; i < 10 * (Q + 2); i += blockDim.x) outv[(size_t)(i / (Q + 2)) * plane + Qp + i % (Q + 2)] = make_uint4(0, 0, 0, 0);
+    if (p < 0) {                                     // border row: zeros in every chunk
         for (int i = threadIdx.x; i < 10 * Qp; i += blockDim.x) {
             const int j8 = i / Qp, qq = i - j8 * Qp;
             outv[(size_t)j8 * plane + qq] = make_uint4(0, 0, 0, 0);
@@ -152,15 +154,17 @@ __global__ void input_to_stem_planar_rgb_kernel(const void* __restrict__ in, int
                                                 int N, int H, int W, int n0) {
     constexpr int C = 3;
     extern __shared__ float rows[];                  // [3 rows: 2p-1, 2p, 2p+1][C][W + 6], zero where outside the image
-    const int P = H / 2, Q = W / 2, Qp = Q + 2, P2 = (P + 2) * Qp;
-    const int n = n0 + blockIdx.x / (P + 2), pp = blockIdx.x % (P + 2);
+    const int P = H / 2, Q = W / 2, Qp = row_vecs(Q), P2 = image_vecs(P, Q);
+    const int n = n0 + blockIdx.x / (P + 1), pp = blockIdx.x % (P + 1);
     const int p = pp - 1;
-    const size_t plane = (size_t)N * P2;
+    const size_t plane = (size_t)plane_vecs(N, P, Q);
     Vec8h* outv = reinterpret_cast<Vec8h*>(out) + (size_t)n * P2 + (size_t)pp * Qp;
     Vec8h zero;
 #pragma unroll
     for (int e = 0; e < 4; ++e) zero.v[e] = __floats2bfloat162_rn(0.0f, 0.0f);
-    if (p < 0 || p >= P) {                           // border row: zeros in every chunk
+    if (n == N - 1 && p == P - 1)                    // the zeros behind the last image
+        for (int i = threadIdx.x; i < 10 * (Q + 2); i += blockDim.x) outv[(size_t)(i / (Q + 2)) * plane + Qp + i % (Q + 2)] = zero;
+    if (p < 0) {                                     // border row: zeros in every chunk
         for (int j8 = 0; j8 < 10; ++j8)
             for (int qq = threadIdx.x; qq < Qp; qq += blockDim.x) outv[(size_t)j8 * plane + qq] = zero;
         return;
@@ -211,13 +215,14 @@ __global__ void input_to_stem_planar_rgb_kernel(const void* __restrict__ in, int
 template <bool BF16>
 __global__ void maxpool_kernel(const void* __restrict__ x, void* __restrict__ y, int N, int H, int W, int chunks, int P,
                                int Q, int R, int stride, int pad) {
-    const int Wp = W + 2, P2i = (H + 2) * Wp, Qp = Q + 2, P2o = (P + 2) * Qp;
-    const int rows_per_image = P + 2;
+    const int Wp = row_vecs(W), Qp = row_vecs(Q);
+    const int rows_per_image = P + 1;
     const int row = blockIdx.x * blockDim.y + threadIdx.y;
     if (row >= chunks * N * rows_per_image) return;
     const int jn = row / rows_per_image, pp = row - jn * rows_per_image;     // jn = chunk * N + image
-    const int p = pp - 1;
-    const size_t in_base = (size_t)jn * P2i, out_base = (size_t)jn * P2o + (size_t)pp * Qp;
+    const int p = pp - 1, j = jn / N, n = jn - j * N;
+    const size_t in_base = (size_t)j * plane_vecs(N, H, W) + (size_t)n * image_vecs(H, W);
+    const size_t out_base = (size_t)j * plane_vecs(N, P, Q) + (size_t)n * image_vecs(P, Q) + (size_t)pp * Qp;
     for (int qq = threadIdx.x; qq < Qp; qq += blockDim.x) {
         const int q = qq - 1;
         float m[8];
@@ -240,6 +245,10 @@ __global__ void maxpool_kernel(const void* __restrict__ x, void* __restrict__ y,
             }
         }
         store_vec8<BF16>(y, out_base + qq, m);
+    }
+    if (n == N - 1 && p == P - 1) {                  // the zeros behind the last image
+        const float zeros[8] = {};
+        for (int i = threadIdx.x; i < Q + 2; i += blockDim.x) store_vec8<BF16>(y, out_base + Qp + i, zeros);
     }
 }
 
@@ -267,20 +276,21 @@ __device__ __forceinline__ Vec8h vshfl(const Vec8h& a, int src_lane) {
 }
 __global__ void maxpool3s2_bf16_kernel(const Vec8h* __restrict__ x, Vec8h* __restrict__ y, int N, int H, int W, int chunks,
                                        int P, int Q) {
-    const int Wp = W + 2, P2i = (H + 2) * Wp, Qp = Q + 2, P2o = (P + 2) * Qp;
-    const int rows_per_image = P + 2;
+    const int Wp = row_vecs(W), Qp = row_vecs(Q);
+    const int rows_per_image = P + 1;
     const int row = blockIdx.x * blockDim.y + threadIdx.y;
     if (row >= chunks * N * rows_per_image) return;                           // the same for a whole warp
     const int jn = row / rows_per_image, pp = row - jn * rows_per_image;     // jn = chunk * N + image
-    const int p = pp - 1;
-    const size_t in_base = (size_t)jn * P2i, out_base = (size_t)jn * P2o + (size_t)pp * Qp;
+    const int p = pp - 1, j = jn / N, n = jn - j * N;
+    const size_t in_base = (size_t)j * plane_vecs(N, H, W) + (size_t)n * image_vecs(H, W);
+    const size_t out_base = (size_t)j * plane_vecs(N, P, Q) + (size_t)n * image_vecs(P, Q) + (size_t)pp * Qp;
     const int lane = threadIdx.x & 31;
     Vec8h ninf, zero;
 #pragma unroll
     for (int i = 0; i < 4; ++i) { ninf.v[i] = __floats2bfloat162_rn(-INFINITY, -INFINITY); zero.v[i] = __floats2bfloat162_rn(0.0f, 0.0f); }
     for (int qq0 = threadIdx.x - lane; qq0 < Qp; qq0 += blockDim.x) {         // warp-uniform: all 32 lanes take part
         const int qq = qq0 + lane, q = qq - 1;
-        if (p < 0 || p >= P) {                                                // border row: zeros
+        if (p < 0) {                                                          // border row: zeros
             if (qq < Qp) y[out_base + qq] = zero;
             continue;
         }
@@ -306,6 +316,8 @@ __global__ void maxpool3s2_bf16_kernel(const Vec8h* __restrict__ x, Vec8h* __res
         const Vec8h fa = vshfl(WA, (2 * lane) & 31), fb = vshfl(WB, (2 * lane) & 31);
         if (qq < Qp) y[out_base + qq] = (q >= 0 && q < Q) ? (lane < 16 ? fa : fb) : zero;
     }
+    if (n == N - 1 && p == P - 1)                                             // the zeros behind the last image
+        for (int i = threadIdx.x; i < Q + 2; i += blockDim.x) y[out_base + Qp + i] = zero;
 }
 
 // Head, step 1: spatial sum per channel in fp32.  One warp per (image, chunk of 8 channels): lanes stride over the interior
@@ -315,8 +327,8 @@ __global__ void maxpool3s2_bf16_kernel(const Vec8h* __restrict__ x, Vec8h* __res
 template <bool BF16>
 __global__ void pool_sum_kernel(const void* x, int N, int H, int W, int chunks, float* __restrict__ sums) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int Wp = W + 2, P2 = (H + 2) * Wp, HW = H * W;
-    const size_t plane = (size_t)N * P2;
+    const int Wp = row_vecs(W), P2 = image_vecs(H, W), HW = H * W;
+    const size_t plane = (size_t)plane_vecs(N, H, W);
     const int lane = threadIdx.x & 31;
     const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -523,8 +535,8 @@ template <bool BF16>
 __global__ void planar_to_nchw_f32_kernel(const void* __restrict__ x, float* __restrict__ out, int N, int H, int W,
                                           int chunks, int C_out, int split) {
     // a parity-split tensor (see ConvArgs) is 4 N images of half the size
-    const int Wp = split ? (W + 1) / 2 + 2 : W + 2, P2 = split ? ((H + 1) / 2 + 2) * Wp : (H + 2) * Wp;
-    const size_t plane = (size_t)N * P2 * (split ? 4 : 1);
+    const int Hs = split ? (H + 1) / 2 : H, Ws = split ? (W + 1) / 2 : W, Wp = row_vecs(Ws), P2 = image_vecs(Hs, Ws);
+    const size_t plane = (size_t)plane_vecs(split ? 4 * N : N, Hs, Ws);
     const size_t total = (size_t)N * chunks * H * W;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int w = (int)(i % W);
@@ -558,7 +570,7 @@ inline int grid_for(size_t n, int threads) {
 
 void launch_input_to_planar(const void* in, int in_is_bf16, void* out, int out_is_bf16, int N, int C, int H, int W,
                             int C_pad, int n0, int n_count, cudaStream_t st) {
-    const size_t n = (size_t)n_count * (H + 2) * (W + 2) * (C_pad / 8);
+    const size_t n = (size_t)used_vecs(n_count, H, W) * (C_pad / 8);
     if (out_is_bf16) input_to_planar_kernel<true><<<grid_for(n, 256), 256, 0, st>>>(in, in_is_bf16, out, N, C, H, W, C_pad / 8, n0, n_count);
     else input_to_planar_kernel<false><<<grid_for(n, 256), 256, 0, st>>>(in, in_is_bf16, out, N, C, H, W, C_pad / 8, n0, n_count);
 }
@@ -566,15 +578,15 @@ void launch_input_to_planar(const void* in, int in_is_bf16, void* out, int out_i
 void launch_input_to_stem_planar(const void* in, int in_is_bf16, void* out, int N, int C, int H, int W, int n0, int n_count,
                                  cudaStream_t st) {
     const size_t smem = (size_t)3 * C * (W + 6) * sizeof(float);      // <= 36 KB for the supported widths
-    if (C == 3) input_to_stem_planar_rgb_kernel<<<n_count * (H / 2 + 2), 128, smem, st>>>(in, in_is_bf16, (__nv_bfloat16*)out, N, H, W, n0);
-    else input_to_stem_planar_kernel<<<n_count * (H / 2 + 2), 256, smem, st>>>(in, in_is_bf16, (__nv_bfloat16*)out, N, C, H, W, n0);
+    if (C == 3) input_to_stem_planar_rgb_kernel<<<n_count * (H / 2 + 1), 128, smem, st>>>(in, in_is_bf16, (__nv_bfloat16*)out, N, H, W, n0);
+    else input_to_stem_planar_kernel<<<n_count * (H / 2 + 1), 256, smem, st>>>(in, in_is_bf16, (__nv_bfloat16*)out, N, C, H, W, n0);
 }
 
 void launch_maxpool(const void* x, void* y, int is_bf16, int N, int H, int W, int C_pad, int P, int Q, int R,
                     int stride, int pad, cudaStream_t st) {
     // the chunk planes are contiguous over the batch: (chunk, image) pairs are numbered jn = chunk * N + image
-    const int tx = Q + 2 <= 32 ? 32 : Q + 2 <= 64 ? 64 : 128, ty = 256 / tx;
-    const int rows = (C_pad / 8) * N * (P + 2);
+    const int tx = Q + 1 <= 32 ? 32 : Q + 1 <= 64 ? 64 : 128, ty = 256 / tx;
+    const int rows = (C_pad / 8) * N * (P + 1);
     const dim3 block(tx, ty), grid((rows + ty - 1) / ty);
     if (is_bf16 && R == 3 && stride == 2 && pad == 1)
         maxpool3s2_bf16_kernel<<<grid, block, 0, st>>>((const Vec8h*)x, (Vec8h*)y, N, H, W, C_pad / 8, P, Q);

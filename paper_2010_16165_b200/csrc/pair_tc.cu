@@ -61,7 +61,7 @@ struct PairParams {
     PairArgs a;
     FastDiv div_p2out, div_qp;
     int Qp, P2, m_total, m_tiles, m_first, m_sign;
-    long long plane_x, plane_x2, plane_y;      // vectors per chunk plane (the shortcut's planes are m_total apart)
+    long long plane_x, plane_x2, plane_res, plane_y;      // vectors per chunk plane
     int chunks1, chunks, groups;               // channel chunks of x, of y; groups of y
     int x_stages, sum2_stages, slots, w_stages, w_stays, tmem_cols;      // w_stays: all groups' filters have a stage of their own
     int y_P2h, y_Wh2;                          // parity-split output: half-resolution grid
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
                 if (lane == 0) mbar_expect_tx(slot_full0 + 8 * slot.at, share(cg));
                 __syncwarp();
                 if (c < cg)
-                    bulk_copy(slot0 + slot.at * slot_bytes + (uint32_t)c * 2048u, rv + (long long)(g * GC + c) * p.m_total + f0, 2048u, slot_full0 + 8 * slot.at);
+                    bulk_copy(slot0 + slot.at * slot_bytes + (uint32_t)c * 2048u, rv + (long long)(g * GC + c) * p.plane_res + f0, 2048u, slot_full0 + 8 * slot.at);
                 __syncwarp();
                 slot.next(p.slots);
             }
@@ -415,8 +415,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_pair_kernel(const PairParams
 // 80 -> 512 -> 80 83 -> 50, 14x14 160 -> 1024 -> 160 46 -> 34; batch 32, 56x56 34 -> 23; batch 8, 56x56 13.5 -> 10.2.
 bool plan_pair(const PairArgs& a, PairPlan* plan) {
     plan->valid = 0;
-    const int m_tiles = (int)(((long long)a.N * (a.P + 2) * (a.Q + 2) + 127) / 128);
-    if (m_tiles < sm_count() || a.K2 > 256) return false;
+    const int m_tiles = (int)((used_vecs(a.N, a.P, a.Q) + 127) / 128);
+    if (m_tiles < sm_count() || a.K2 > 256 || (a.y_split && (a.P % 2 || a.Q % 2))) return false;
     const int sum2_stages = 2 * a.K2 + kSums * G <= 512 ? 2 : 1, groups = (a.K + G - 1) / G;
     int cols = 32;
     while (cols < sum2_stages * a.K2 + kSums * G) cols *= 2;
@@ -447,14 +447,15 @@ void launch_pair(const PairPlan& plan, const PairArgs& a, int* d_status, cudaStr
     PairParams p;
     memset(&p, 0, sizeof(p));
     p.a = a;
-    p.Qp = a.Q + 2; p.P2 = (a.P + 2) * (a.Q + 2);
-    p.m_total = a.N * p.P2; p.m_tiles = (p.m_total + 127) / 128;
+    p.Qp = row_vecs(a.Q); p.P2 = image_vecs(a.P, a.Q);
+    const long long plane = plane_vecs(a.N, a.P, a.Q);
+    p.m_total = a.y_split ? a.N * p.P2 : (int)used_vecs(a.N, a.P, a.Q); p.m_tiles = (p.m_total + 127) / 128;
     p.m_first = a.reverse ? p.m_tiles - 1 : 0; p.m_sign = a.reverse ? -1 : 1;
-    p.plane_x = p.plane_y = p.m_total;
-    p.plane_x2 = (long long)p.m_total * (a.x2_plane_mult > 1 ? 4 : 1);
+    p.plane_x = p.plane_res = p.plane_y = plane;
+    p.plane_x2 = a.x2_plane_mult > 1 ? plane_vecs(4 * a.N, a.P, a.Q) : plane;
     if (a.y_split) {
-        p.y_Wh2 = (a.Q + 1) / 2 + 2; p.y_P2h = ((a.P + 1) / 2 + 2) * p.y_Wh2;
-        p.plane_y = 4LL * a.N * p.y_P2h;
+        p.y_Wh2 = row_vecs((a.Q + 1) / 2); p.y_P2h = image_vecs((a.P + 1) / 2, (a.Q + 1) / 2);
+        p.plane_y = plane_vecs(4 * a.N, (a.P + 1) / 2, (a.Q + 1) / 2);
     }
     p.chunks1 = a.C_pad / 8; p.chunks = a.K / 8; p.groups = (a.K + G - 1) / G;
     p.x_stages = plan.x_stages; p.sum2_stages = plan.sum2_stages; p.slots = plan.slots; p.w_stages = plan.w_stages; p.w_stays = plan.w_stays; p.tmem_cols = plan.tmem_cols;

@@ -619,11 +619,11 @@ __global__ void __launch_bounds__(CLUSTER ? kThreads : kMaxG * kThreads, 1) resi
             if (CLUSTER && l + 1 == L) image_sync<CLUSTER, WARPS>(slot);          // (the head's sums may go where other CTAs still read)
             else layer_sync<WARPS>(slot);
             if (l == dump_layer) {                 // diagnostic: this layer's output as a planar-8 tensor with border
-                const int P2 = (ly.R * p.cs + 2) * (ly.W + 2), out_PV = ly.out_plane / 16;
+                const int H = ly.R * p.cs, out_PV = ly.out_plane / 16;
                 uint4* y = reinterpret_cast<uint4*>(p.a.dump);
                 for (int i = tid; i < ly.n8 * ly.R * ly.W; i += threads) {
                     const int w = i % ly.W, r = i / ly.W % ly.R, c = i / (ly.W * ly.R);
-                    y[(size_t)c * p.a.N * P2 + (size_t)n * P2 + (size_t)(rank * ly.R + r + 1) * (ly.W + 2) + w + 1] =
+                    y[(size_t)c * plane_vecs(p.a.N, H, ly.W) + (size_t)n * image_vecs(H, ly.W) + (size_t)(rank * ly.R + r + 1) * row_vecs(ly.W) + w + 1] =
                         *reinterpret_cast<const uint4*>(img + ly.out_off + ((size_t)c * out_PV + (size_t)(r + 1) * (ly.W + 1) + w + 1) * 16);
                 }
                 layer_sync<WARPS>(slot);

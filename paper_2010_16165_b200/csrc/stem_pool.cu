@@ -278,8 +278,8 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
         const int first_group = half ? ((K_pad >> 4) + 1) >> 1 : 0, groups = half ? (K_pad >> 4) - first_group : ((K_pad >> 4) + 1) >> 1;
         const bool live = col < Wc;
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + 16u * (uint32_t)min(first_group, (K_pad >> 4) - 1);
-        const int Wq = p.Wp + 2, P2o = (p.Hp + 2) * Wq, pitch = 2 * Wp + 1;
-        const long long plane_out = (long long)p.a.N * P2o;
+        const int Wq = row_vecs(p.Wp), P2o = image_vecs(p.Hp, p.Wp), pitch = 2 * Wp + 1;
+        const long long plane_out = plane_vecs(p.a.N, p.Hp, p.Wp);
         uint4* yout = reinterpret_cast<uint4*>(p.a.y);
         uint4* cols_s = reinterpret_cast<uint4*>(smem_raw + (x_addr - base)) + 2 * p.plane;      // [row parity][chunk]: even columns, then odd ones from -1 on
         const int off = col - left, place = off & 1 ? Wp + ((off + 1) >> 1) : off >> 1;      // off: from the strip's first even column
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
                     const int chunk = 2 * first_group + ch;
                     const uint4* from = cols_s + (size_t)(parity * (K_pad >> 3) + chunk) * pitch;
                     uint4* to = yout + (long long)((k_base >> 3) + chunk) * plane_out + (long long)s.n * P2o + (long long)(q + 1) * Wq + x0;
-                    for (int k0 = lane; k0 < Wp + 2; k0 += 64) {
+                    for (int k0 = lane; k0 < Wp + 1; k0 += 64) {
                         uint4 l[2], c[2], r[2];          // two positions' loads in flight
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {    // columns 2k - 3 .. 2k - 1
@@ -356,14 +356,17 @@ __global__ void __launch_bounds__(kThreads, 2) stem_pool_kernel(const SpParams p
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
                             const int k = k0 + 32 * i;
-                            if (k >= Wp + 2) break;
-                            if (PARTS && ((k == 0 && x0 > 0) || (k == Wp + 1 && x0 + Wp < p.Wp))) continue;      // another strip's column
+                            if (k >= Wp + 1) break;
+                            if (PARTS && k == 0 && x0 > 0) continue;                      // another strip's column
                             uint4 o = make_uint4(0, 0, 0, 0);
-                            if (k >= 1 && k <= Wp)
+                            if (k >= 1)
                                 o = make_uint4(max3(l[i].x, c[i].x, r[i].x), max3(l[i].y, c[i].y, r[i].y), max3(l[i].z, c[i].z, r[i].z), max3(l[i].w, c[i].w, r[i].w));
                             to[k] = o;
                             if (q == 0) to[k - Wq] = make_uint4(0, 0, 0, 0);
-                            if (q == p.Hp - 1) to[k + Wq] = make_uint4(0, 0, 0, 0);
+                            if (q == p.Hp - 1 && s.n == p.a.N - 1) {                      // the zeros behind the last image
+                                to[k + Wq] = make_uint4(0, 0, 0, 0);
+                                if (k == 0) to[2 * Wq] = make_uint4(0, 0, 0, 0);
+                            }
                         }
                     }
                 }

@@ -28,11 +28,11 @@ def bottleneck(layers, widths, hw, batch, ratios):
 
 
 @pytest.mark.parametrize("layers, widths, hw, batch, ratios, pairs", [
-    ((2, 1), (16, 24), 64, 61, wl.inner_bottleneck_ratios(0.3), 2),      # one group a tile; the second stream parity-split, a quarter written
-    ((1, 2), (20, 40), 56, 85, wl.uniform_ratios(0.3), 1),               # a last group of 16 and of 32 channels
-    ((3,), (64,), 36, 163, wl.uniform_ratios(0.0), 2),                   # 9 x 9 pixels, filters stay
-    ((2, 2), (128, 128), 52, 90, wl.inner_bottleneck_ratios(0.2), 1),    # odd images (no parity split), filters with every tile
-    ((3,), (160,), 20, 390, wl.uniform_ratios(0.0), 1),                  # one stage of x and of the second sums
+    ((2, 1), (16, 24), 64, 66, wl.inner_bottleneck_ratios(0.3), 2),      # one group a tile; the second stream parity-split, a quarter written
+    ((1, 2), (20, 40), 56, 87, wl.uniform_ratios(0.3), 1),               # a last group of 16 and of 32 channels
+    ((3,), (64,), 36, 191, wl.uniform_ratios(0.0), 2),                   # 9 x 9 pixels, filters stay
+    ((2, 2), (128, 128), 52, 99, wl.inner_bottleneck_ratios(0.2), 1),    # odd images (no parity split), filters with every tile
+    ((3,), (160,), 20, 531, wl.uniform_ratios(0.0), 1),                  # one stage of x and of the second sums
     ((2,), (48,), 112, 23, wl.inner_bottleneck_ratios(0.5), 1),          # a few tiles a CTA, the last one partial
 ])
 def test_layers_that_run_as_pairs(B, layers, widths, hw, batch, ratios, pairs):

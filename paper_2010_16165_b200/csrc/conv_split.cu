@@ -62,7 +62,7 @@ struct SplitParams {
     int n_tile, n_tiles, tmem_cols, a_stage_bytes, stage_bytes, red_bytes, slots;   // slots: chunks a CTA finishes at most
     int bank_tile_vecs;
     int tap_off[9];
-    int y_P2h, y_Wh2, y_edges;
+    int y_P2h, y_Wh2;
     int skip_round;
     long long wait_cycles;
     int* status;
@@ -100,9 +100,9 @@ __device__ __forceinline__ uint2 ld_global8(const uint2* p) {
 }
 
 // (At least two CTAs on an SM: the next layer's start while this layer's work.  The code is kept short - an instance per kind
-// of layer, loops instead of unrolled bodies - because a launch meets it cold: the same kernel with everything unrolled,
+// of layer (EDGES: a parity-split output of an odd height or width), loops instead of unrolled bodies - because a launch meets it cold: the same kernel with everything unrolled,
 // 106 instead of 64 registers, took 3.9 us instead of 3.0 for a 48 -> 256 layer of one image.)
-template <int TAPS, bool SPLIT>
+template <int TAPS, bool SPLIT, bool EDGES>
 __global__ void __launch_bounds__(kThreads, 3) conv_split_kernel(const SplitParams p) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     SplitCtrl* ctrl = reinterpret_cast<SplitCtrl*>(smem_raw);
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kThreads, 3) conv_split_kernel(const SplitPara
             }
         }
     }
-    if (p.y_edges && finisher && half == 0 && rank == 0)
+    if (EDGES && finisher && half == 0 && rank == 0)
         for (int t = 0; t < p.tps; ++t) {                // see conv_tc.cu: the row and column behind an odd image's last
             const int f = f0 + t * 128 + row, n = (int)fdiv((uint32_t)f, p.div_p2out), rem = f - n * p.P2_out;
             const int hp = (int)fdiv((uint32_t)rem, p.div_qp), wq = rem - hp * p.Qp;
@@ -466,9 +466,12 @@ constexpr unsigned kSmemOne = 232448u - 1024u;
 constexpr unsigned kSmemTwo = 233472u / 2 - 1024u;       // two CTAs on an SM
 
 typedef void (*SplitKernel)(const SplitParams);
-SplitKernel kernel_of(int taps, int splits) {
-    return taps == 9 ? (splits > 1 ? conv_split_kernel<9, true> : conv_split_kernel<9, false>)
-                     : (splits > 1 ? conv_split_kernel<1, true> : conv_split_kernel<1, false>);
+SplitKernel kernel_of(int taps, int splits, bool edges) {
+    if (edges)
+        return taps == 9 ? (splits > 1 ? conv_split_kernel<9, true, true> : conv_split_kernel<9, false, true>)
+                         : (splits > 1 ? conv_split_kernel<1, true, true> : conv_split_kernel<1, false, true>);
+    return taps == 9 ? (splits > 1 ? conv_split_kernel<9, true, false> : conv_split_kernel<9, false, false>)
+                     : (splits > 1 ? conv_split_kernel<1, true, false> : conv_split_kernel<1, false, false>);
 }
 
 // CTAs that run at once in clusters of a size, with one ([0]) or two ([1]) of them on an SM: a cluster lies within a group of
@@ -496,7 +499,7 @@ const Room& cluster_room() {
                 cfg.attrs = &attr;
                 cfg.numAttrs = 1;
                 int n = 0;
-                if (cudaOccupancyMaxActiveClusters(&n, conv_split_kernel<9, true>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+                if (cudaOccupancyMaxActiveClusters(&n, conv_split_kernel<9, true, false>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
                 known[dev].ctas[two][c] = std::min(n * c, (two + 1) * sm_count());
             }
         asked[dev] = true;
@@ -512,7 +515,7 @@ namespace {
 // per K group.  False where it does not fit; else the launch figures and the time expected.
 bool candidate(const ConvArgs& a, const Room& room, int tps, int n_tile, int splits, int cg, ConvPlanTC* c, double* cost) {
     const int taps = a.R * a.S, cchunks = a.C_pad / 8, a_par = a.x_s2d ? 4 : 1;
-    const int halo = taps == 1 ? 0 : row_vecs(a.W) + 1;
+    const int halo = taps == 1 ? 0 : round_up_i(row_vecs(a.W) + 1, 2);      // (copies begin at a 32-byte sector)
     const int rows_a = round_up_i(128 * tps + (a_par > 1 ? 1 : 2) * halo, 8);
     if (rows_a + 8 > kGuardVectors || tps * n_tile > 256) return false;
     const int m_tiles = (int)((used_vecs(a.N, a.P, a.Q) + 127) / 128), steps = (m_tiles + tps - 1) / tps;
@@ -553,8 +556,8 @@ bool plan_conv_split(const ConvArgs& a, ConvPlanTC* plan) {
     const bool flat = a.stride == 1 && a.P == a.H && a.Q == a.W && ((taps == 1 && a.pad == 0) || (a.R == 3 && a.S == 3 && a.pad == 1));
     if (!flat || a.scatter || a.n_tile_forced > 0 || a.res_mode == 2) return false;
     if ((used_vecs(a.N, a.P, a.Q) + 127) / 128 > 2 * sm_count()) return false;
-    for (int k = 0; k < 4; ++k)
-        if (cudaFuncSetAttribute(kernel_of(k & 1 ? 9 : 1, 1 + (k >> 1)), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemOne) != cudaSuccess) {
+    for (int k = 0; k < 8; ++k)
+        if (cudaFuncSetAttribute(kernel_of(k & 1 ? 9 : 1, 1 + (k >> 1 & 1), k >> 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemOne) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
@@ -602,7 +605,6 @@ void launch_conv_split(const ConvPlanTC& plan, const ConvArgs& a, int* d_status,
     if (a.y_split) {
         p.y_Wh2 = row_vecs((a.Q + 1) / 2); p.y_P2h = image_vecs((a.P + 1) / 2, (a.Q + 1) / 2);
         p.plane_y = (int)plane_vecs(4 * a.N, (a.P + 1) / 2, (a.Q + 1) / 2);
-        p.y_edges = (a.P & 1) || (a.Q & 1);
         p.m_total = a.N * p.P2_out;                      // (nobody reads behind the last image of a split tensor)
     }
     p.taps = a.R * a.S; p.cchunks = a.C_pad / 8; p.cg = plan.cg; p.groups = plan.groups;
@@ -620,7 +622,7 @@ void launch_conv_split(const ConvPlanTC& plan, const ConvArgs& a, int* d_status,
             const int pa = r == 1 ? 0 : 1, pb = s == 1 ? 0 : 1;
             p.tap_off[t] = (pa ? (pb ? 2 : 1) : (pb ? 3 : 0)) * plan.rows_a + plan.halo + (r == 0 ? -p.Wp_in : 0) + (s == 0 ? -1 : 0);
         } else {
-            p.tap_off[t] = r * p.Wp_in + s;
+            p.tap_off[t] = plan.halo - (p.Wp_in + 1) + r * p.Wp_in + s;
         }
     }
     p.skip_round = skip_round; p.wait_cycles = wait_cycles; p.status = d_status;
@@ -643,7 +645,7 @@ void launch_conv_split(const ConvPlanTC& plan, const ConvArgs& a, int* d_status,
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     void* args[1] = {(void*)&p};
-    cudaLaunchKernelExC(&cfg, (const void*)kernel_of(p.taps, plan.split), args);
+    cudaLaunchKernelExC(&cfg, (const void*)kernel_of(p.taps, plan.split, a.y_split && (a.P % 2 || a.Q % 2)), args);
 }
 
 }  // namespace fp

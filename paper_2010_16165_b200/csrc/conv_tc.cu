@@ -74,6 +74,7 @@ struct TcParams {
     int cchunks2, groups2;              // streamed 3x3 layer: chunks / extra K groups of the second input (centre tap only)
     int a_par;                          // activation runs per channel chunk in a stage: 1, or 4 parity images (x_s2d)
     long long par_stride;               // x_s2d: vectors between the parity images of one chunk (N * P2)
+    int tap0;                           // rows of the halo before the first tap's operand
     int tap_off[9];                     // x_s2d: start row of each tap's operand within a chunk's part of the stage
     int y_split, y_P2h, y_Wh2;          // split output: half-resolution grid
     int y_edges;                        // split output of an odd height or width: the odd-parity images' row or column that does not exist
@@ -465,7 +466,7 @@ conv_tc_kernel(const TcParams p) {
                         int cgg = p.cchunks - g * p.cg;
                         if (cgg > p.cg) cgg = p.cg;
                         const int ksteps = cgg >> 1;
-                        uint32_t a_row = ((a_base + a_stage * p.a_stage_bytes) >> 4) | ((uint32_t)(p.a_par * p.rows_a) << 16);
+                        uint32_t a_row = (((a_base + a_stage * p.a_stage_bytes) >> 4) + (uint32_t)p.tap0) | ((uint32_t)(p.a_par * p.rows_a) << 16);
                         uint32_t b_tap = 0;
                         if (MODE == MODE_FLAT_RESIDENT)
                             b_tap = ((b_base >> 4) + (uint32_t)(g * p.cg * p.n_tile)) | ((uint32_t)p.n_tile << 16);   // this CTA's filter tile only
@@ -1054,7 +1055,7 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
     smem += scatter_smem;
     int want_ctas = 1;
     if (plan->flat) {
-        plan->halo = ((a.R - 1) / 2) * row_vecs(a.W) + (a.S - 1) / 2;      // rows above + columns to the left
+        plan->halo = round_up_i(((a.R - 1) / 2) * row_vecs(a.W) + (a.S - 1) / 2, 2);      // rows above + columns to the left; copies begin at a 32-byte sector
         plan->tps = 1;
         // A 128-position tile is fetched with `halo` rows on either side.  On wide images (the 112-wide stem: 114
         // rows each side of 128) that is most of the traffic into shared memory, so such a layer takes the
@@ -1285,6 +1286,7 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
         p.tap_off[t] = pp * plan.rows_a + plan.halo + (r == 0 ? -p.Wp_in : 0) + (sx == 0 ? -1 : 0);
     }
     p.taps = a.R * a.S; p.cchunks = a.C_pad / 8; p.cg = plan.cg; p.groups = plan.groups;
+    p.tap0 = plan.flat && !a.x_s2d ? plan.halo - (((a.R - 1) / 2) * p.Wp_in + (a.S - 1) / 2) : 0;
     p.halo = plan.halo; p.rows_a = plan.rows_a; p.a_stages = plan.a_stages; p.b_stages = plan.b_stages;
     p.n_tile = plan.n_tile; p.n_tiles = plan.n_tiles; p.tmem_cols = plan.tmem_cols;
     const long long m_tiles = (p.m_total + 127) / 128;

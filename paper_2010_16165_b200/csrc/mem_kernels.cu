@@ -337,12 +337,18 @@ __global__ void pool_sum_kernel(const void* x, int N, int H, int W, int chunks, 
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
-    for (int i = lane; i < HW; i += 32) {
-        const int h = i / W, w = i - h * W;
-        float v[8];
-        load_vec8<BF16>(x, (size_t)j * plane + (size_t)n * P2 + (size_t)(h + 1) * Wp + (w + 1), v);
+    for (int i = lane; i < HW; i += 64) {  // two positions' loads in flight
+        float v[2][8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] += v[e];
+        for (int k = 0; k < 2; ++k) {
+            const int at = min(i + 32 * k, HW - 1), h = at / W, w = at - h * W;
+            load_vec8<BF16>(x, (size_t)j * plane + (size_t)n * P2 + (size_t)(h + 1) * Wp + (w + 1), v[k]);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] += v[0][e];
+        if (i + 32 < HW)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += v[1][e];
     }
     int first = 0;                         // of the channels this lane still carries
 #pragma unroll
@@ -433,13 +439,13 @@ __global__ void __launch_bounds__(32 * kFcWarps, 2) fc_kernel(const float* sums,
     }
 }
 
-// Head, step 2, many images: a block takes 8 * IPL images times 32 classes.  Slabs of 256 channels of the sums and of the FC rows go through
-// shared memory (two on the way behind the one in use), a warp takes 32 channels of each, a lane IPL images times 8 classes of the tile: a
+// Head, step 2, many images: a block takes 8 * IPL images times 32 classes.  Slabs of 128 channels of the sums and of the FC rows go through
+// shared memory (two on the way behind the one in use), a warp takes 16 channels of each, a lane IPL images times 8 classes of the tile: a
 // vector of 4 channels of an image serves 8 classes and one of a class IPL images, so that 12 shared-memory reads feed 64 pairs of
 // FMAs.  (In the kernel above every lane reads its own channels of every image, four wavefronts for 4 classes: both that and the L2
 // reads of the FC matrix, once for every 8 images, took longer than the FMAs.)  Channels are added in pairs (one instruction
 // for two), each warp's in order, then the pair, then the warps' sums in order.
-constexpr int kTileClasses = 32, kTileSlab4 = 64, kTilePitch4 = kTileSlab4 + 1;      // (rows 16 bytes off a multiple of 128: no bank twice)
+constexpr int kTileClasses = 32, kTileSlab4 = 32, kTilePitch4 = kTileSlab4 + 1;      // (rows 16 bytes off a multiple of 128: no bank twice)
 constexpr int kTileStages = 3;
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
@@ -449,14 +455,14 @@ __device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a
 }
 constexpr int fc_tile_smem(int ipl) { return kTileStages * (kTileClasses + 8 * ipl) * kTilePitch4 * (int)sizeof(float4); }
 template <int IPL>
-__global__ void __launch_bounds__(256, 1) fc_tile_kernel(const float* sums, int N, int C_pad, const float* __restrict__ fcw,
+__global__ void __launch_bounds__(256, 2) fc_tile_kernel(const float* sums, int N, int C_pad, const float* __restrict__ fcw,
                                                          const float* __restrict__ fcb, int n_classes, float* __restrict__ logits) {
     extern __shared__ float4 sh4[];        // stages: FC rows, then the images' sums
-    constexpr int kImages = 8 * IPL, kStage4 = (kTileClasses + kImages) * kTilePitch4;
+    constexpr int kRows = 256 / kTileSlab4, kImages = 8 * IPL, kStage4 = (kTileClasses + kImages) * kTilePitch4;
     const int n0 = blockIdx.x * kImages, k0 = (int)(blockIdx.z * gridDim.y + blockIdx.y) * kTileClasses, c4 = C_pad >> 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int slabs = (c4 + kTileSlab4 - 1) / kTileSlab4;
-    // A thread brings the same channel vector of every fourth row.  Rows of the tile that do not exist repeat the last one (nobody reads
+    // A thread brings the same channel vector of every eighth row.  Rows of the tile that do not exist repeat the last one (nobody reads
     // what they give); channels behind the last are zeros.
     const int col = threadIdx.x & (kTileSlab4 - 1), row = threadIdx.x / kTileSlab4;
     const uint32_t mine = (uint32_t)__cvta_generic_to_shared(sh4) + (uint32_t)(row * kTilePitch4 + col) * 16u;
@@ -466,8 +472,8 @@ __global__ void __launch_bounds__(256, 1) fc_tile_kernel(const float* sums, int 
         const int first = (images ? n0 : k0) + row, last = (images ? N : n_classes) - 1;
         const uint32_t to = mine + (stage * kStage4 + (images ? kTileClasses * kTilePitch4 : 0)) * 16u;
 #pragma unroll
-        for (int j = 0; j < (images ? kImages : kTileClasses) / 4; ++j)
-            cp_async16(to + (uint32_t)(4 * j * kTilePitch4) * 16u, from + (size_t)min(first + 4 * j, last) * C_pad, at < c4);
+        for (int j = 0; j < (images ? kImages : kTileClasses) / kRows; ++j)
+            cp_async16(to + (uint32_t)(kRows * j * kTilePitch4) * 16u, from + (size_t)min(first + kRows * j, last) * C_pad, at < c4);
     };
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
     fetch_rows(0, 0, false);               // the FC matrix does not wait for the kernel before

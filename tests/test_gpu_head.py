@@ -1,5 +1,5 @@
 """GPU parity of the average pooling and FC layer: batches at the edges of the image groups (1, 4, 8), classes per warp (1, 2,
-4), tiles of 8, 16 and 32 images times 32 classes, channels around the 2048 and the 256 held at a time, image sizes below and above a warp of positions."""
+4), tiles of 8, 16 and 32 images times 32 classes, channels around the 2048 and the 128 held at a time, image sizes below and above a warp of positions."""
 import numpy as np
 import pytest
 

@@ -771,7 +771,13 @@ void find_chains(fp_handle h, const std::vector<std::vector<Use>>& uses) {
                 off += (ly.blob_bytes + 127) / 128 * 128;
             }
             char msg[256];
-            if (fp::plan_chain_tc(a, &plan, msg, sizeof(msg)) != 0) continue;
+            const bool quad = fp::chain_quad_supported(a);
+            if (quad) {
+                const int step = (fp::kQuadBlobBytes + 127) / 128 * 128;
+                for (int j = 0; j < len; ++j) { a.layers[j].blob_off = j * step; a.layers[j].blob_bytes = fp::kQuadBlobBytes; }
+                off = len * step;
+            }
+            if ((quad ? fp::plan_chain_quad(a, &plan, msg, sizeof(msg)) : fp::plan_chain_tc(a, &plan, msg, sizeof(msg))) != 0) continue;
             Chain ch;
             ch.first_op = i; ch.last_op = i + len - 1; ch.args = a; ch.plan = plan;
             for (int j = 0; j < len; ++j) ch.convs.push_back(h->ops[i + j].idx);
@@ -904,15 +910,15 @@ double layers_cost(fp_handle h) {
     for (const Chain& ch : h->chains) {
         const int groups = (h->max_batch + ch.plan.G - 1) / ch.plan.G, rounds = (groups + (int)sms - 1) / (int)sms;
         for (int l = 0; l < ch.args.n_layers; ++l)
-            us += rounds * ((ch.plan.tiles + 1.5) * (0.194 * ch.args.layers[l].K_pad / 16 + 0.003) + 0.6);
+            us += ch.plan.quad ? rounds * fp::chain_quad_layer_us(ch.plan.tiles) : rounds * ((ch.plan.tiles + 1.5) * (0.194 * ch.args.layers[l].K_pad / 16 + 0.003) + 0.6);
     }
     for (int i = 0; i < (int)h->ops.size(); ++i) {
         if (h->ops[i].kind != 0 || h->op_chain[i] >= 0) continue;
         const FConv& f = h->convs[h->ops[i].idx];
         const Tensor& out = h->tensors[f.out];
-        us += 5.7;
+        us += f.stride == 1 ? 5.7 : 5.3;
         if (f.stride == 1) us += 1.17 * std::ceil((double)fp::used_vecs((int)N, out.H, out.W) / 128) * 9 * (f.C_pad / 16) * std::max(f.K_pad / 2.0, 32 + f.K_pad / 4.0) / (sms * 1900);
-        else us += 2.5e-4 * N * out.H * out.W * (f.C_pad / 16);
+        else us += 9.5e-5 * N * out.H * out.W * (f.C_pad / 16);
     }
     const Tensor& last = h->tensors[h->head_src];
     return us + 2 * 5.7 + 2.6e-5 * N * last.H * last.W * (last.C_pad / 16);
@@ -1250,14 +1256,15 @@ fp_status build_plan(fp_handle h) {
         }
     }
     // One kernel or layer by layer, by the batch that the handle is made for - not by each call's, so that a result does not depend on
-    // the batch it was computed in.  Many layers on many images go layer by layer (unpruned ResNet-110: batch 444 514 us against 705,
-    // 1024 1461 against 1593; ResNet-56 at 0.3: batch 592 393 against 430), few layers or few images as one kernel (ResNet-20: 300
-    // against 355 at batch 1024; ResNet-56 at 0.3, batch 256: 216 against 229).
+    // the batch it was computed in.  Many layers on many images go layer by layer (us, one kernel / runs: unpruned ResNet-110 at batch 200
+    // 442 / 339, ResNet-56 at 0.3 at batch 592 429 / 314), few layers or few images as one kernel (ResNet-20 at batch 296 80 / 94).
     find_net(h, uses);
     const bool one_kernel = h->net_on;
     h->net_on = 0;
     find_chains(h, uses);
-    if (one_kernel && network_cost(h) <= layers_cost(h)) {
+    // (By a margin: a smaller batch on the same handle runs the same form, and a few images take 50-170 us longer layer by layer - ResNet-20,
+    // 8 images, 97 us against 36.  Over 75 networks, ratios and batches the runs so chosen were all the shorter, by 16 us and more.)
+    if (one_kernel && network_cost(h) <= layers_cost(h) + 32.0) {
         h->net_on = 1;
         find_chains(h, uses);
     } else {
@@ -1345,10 +1352,10 @@ fp_status build_plan(fp_handle h) {
             wants.push_back({(void**)&ch.d_blob, ch.blob_bytes});
             for (size_t l = 0; l < ch.convs.size(); ++l) {
                 const FConv& f = h->convs[ch.convs[l]];
-                fp::PackJob j = filters(f, fp::PACK_CHAIN);
-                j.units = j.rows * j.chunks;
+                fp::PackJob j = filters(f, ch.plan.quad ? fp::PACK_QUAD : fp::PACK_CHAIN);
+                j.units = ch.plan.quad ? fp::kQuadFilterBytes / 16 : j.rows * j.chunks;
                 add_job(j, (void**)&ch.d_blob, (size_t)ch.args.layers[l].blob_off);
-                add_job(bias(f), (void**)&ch.d_blob, (size_t)ch.args.layers[l].blob_off + (size_t)9 * f.C_pad * f.K_pad * 2);
+                add_job(bias(f), (void**)&ch.d_blob, (size_t)ch.args.layers[l].blob_off + (ch.plan.quad ? (size_t)fp::kQuadFilterBytes : (size_t)9 * f.C_pad * f.K_pad * 2));
             }
         }
         {
@@ -1625,7 +1632,8 @@ void launch_op(fp_handle h, int op_index, const void* d_input, int batch, float*
         fp::ChainArgs a = ch.args;
         a.N = batch;
         if (a.in_mode) a.x = d_input;
-        fp::launch_chain_tc(ch.plan, a, h->d_status, st);
+        if (ch.plan.quad) fp::launch_chain_quad(ch.plan, a, h->d_status, st);
+        else fp::launch_chain_tc(ch.plan, a, h->d_status, st);
         return;
     }
     if (op.kind == 3) {

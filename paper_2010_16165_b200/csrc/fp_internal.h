@@ -129,7 +129,7 @@ void launch_bank_rank(const SoftBank* banks, const int32_t* filter_bank, int tot
 
 // Packing of a planned graph's filters, biases and FC matrix: all jobs in one launch.  Index arrays (packed row -> fused
 // filter, packed channel -> fused channel, -1 = zeros) are parts of one array, named by their offsets.
-enum { PACK_CONV = 0, PACK_CHAIN = 1, PACK_STEM = 2, PACK_STEM_DIRECT = 3, PACK_FC = 4, PACK_BIAS = 5 };
+enum { PACK_CONV = 0, PACK_CHAIN = 1, PACK_STEM = 2, PACK_STEM_DIRECT = 3, PACK_FC = 4, PACK_BIAS = 5, PACK_QUAD = 6 };
 constexpr int kPackThreads = 256;
 // A block of a convolution's filters: 32 filter rows times a run of units, a unit being as many chunks of 8 channels as have at
 // most nine taps together (eight chunks of a 1x1 filter; of a filter with more taps, nine at a time).  Runs of four where a bank
@@ -314,6 +314,7 @@ struct ChainArgs {
 };
 struct ChainPlan {
     int valid;
+    int quad;             // 1: 2 x 2 pixels a row of the GEMM (chain_quad.cu); of the rest then G, tiles, plane_rows and smem_bytes
     int G;                // images per group (per CTA at a time)
     int tiles;            // 128-position tiles per group
     int plane_rows;       // vectors per channel chunk of an activation buffer
@@ -327,5 +328,12 @@ int chain_layer_blob_bytes(int cchunks, int K_pad);
 bool chain_layer_supported(int H, int W, int K_pad, int C_pad);
 int plan_chain_tc(const ChainArgs& a, ChainPlan* plan, char* err, size_t err_len);
 void launch_chain_tc(const ChainPlan& plan, const ChainArgs& a, int* d_status, cudaStream_t st);
+// The same for layers of 16 filters on images 32 pixels wide (chain_quad.cu): filters of a layer [4 x 4 window pixels][2 chunks][4 outputs x
+// 16 filters][8] bf16, then the 16 fp32 biases.
+constexpr int kQuadFilterBytes = 16 * 2 * 64 * 16, kQuadBlobBytes = kQuadFilterBytes + 64;
+bool chain_quad_supported(const ChainArgs& a);
+int plan_chain_quad(const ChainArgs& a, ChainPlan* plan, char* err, size_t err_len);
+double chain_quad_layer_us(int tiles);         // a layer of a group of that many tiles
+void launch_chain_quad(const ChainPlan& plan, const ChainArgs& a, int* d_status, cudaStream_t st);
 
 }  // namespace fp

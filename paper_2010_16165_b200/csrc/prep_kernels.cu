@@ -261,6 +261,8 @@ __device__ __forceinline__ void store8(const PackJob& j, size_t vec, const float
 //   PACK_CONV   [filter tile][K group][tap][chunk in group][row in tile]: with one tile and one group the plain layout
 //               [tap][chunk][row], otherwise a block per pipeline stage / a contiguous part per filter tile (conv_tc.cu).
 //               Chunks >= chunks1 are the second bank's (a projection shortcut stacked along the channels).
+//   PACK_QUAD   a fused run's layer of 16 filters, 2 x 2 outputs a row: [window pixel][chunk][output][filter], zeros where the pixel is
+//               outside the output's window
 //   PACK_CHAIN  a fused run's layer: per tap row and chunk a stack of 3 * K_pad rows, row 48 * (k / 16) + 16 * s + k % 16
 //               for horizontal tap s (chain_tc.cu)
 // The weights are laid [filter][channel][tap], the banks have the filters innermost: a transposition, through shared memory.
@@ -430,6 +432,17 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const PackJob* __res
     switch (j.kind) {
         case PACK_STEM: pack_stem_vec(j, idx, u); break;
         case PACK_STEM_DIRECT: pack_stem_direct_vec(j, idx, u); break;
+        case PACK_QUAD: {
+            const int k = u & 15, o = u >> 4 & 3, c8 = u >> 6 & 1, w = u >> 7, r = (w >> 2) - (o >> 1), s = (w & 3) - (o & 1), f = idx[j.row + k];
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int c = idx[j.chan + c8 * 8 + e];
+                v[e] = f >= 0 && c >= 0 && r >= 0 && r < 3 && s >= 0 && s < 3 ? j.w[((size_t)f * j.C + c) * 9 + r * 3 + s] : 0.0f;
+            }
+            store8(j, u, v);
+            break;
+        }
         case PACK_FC: {              // out[k][cp] = w[k][chan[cp]] * scale, fp32
             const int chunks = j.chunks, k = u / chunks, c = u - k * chunks;
             float v[8];

@@ -232,7 +232,7 @@ typedef enum {
 } fp_query_what;
 
 enum { FP_KERNEL_CONV_TC = 1, FP_KERNEL_CONV_SPLIT = 2, FP_KERNEL_STEM_POOL = 3, FP_KERNEL_CHAIN_TC = 4, FP_KERNEL_RESIDENT_NET = 5,
-       FP_KERNEL_CONV_SIMT = 6, FP_KERNEL_CONV_PAIR = 7 };   /* fp_op_info::kernel */
+       FP_KERNEL_CONV_SIMT = 6, FP_KERNEL_CONV_PAIR = 7, FP_KERNEL_CHAIN_QUAD = 8 };   /* fp_op_info::kernel */
 
 typedef struct {
     int32_t kind;            /* 0 conv, 1 maxpool, 2 avgpool+fc head, 3 input layout conversion     */

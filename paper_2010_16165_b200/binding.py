@@ -29,7 +29,7 @@ EXPORTS = ["fp_fuse", "fp_prune", "fp_forward", "fp_forward_host", "fp_forward_h
            "fp_debug_expire_wait", "fp_fuse_with_allocator"]
 FP_STATIC_RANK_MAX_FILTERS = 4096
 CONV_KERNELS = ("", "conv_tc_kernel", "conv_split_kernel", "stem_pool_kernel", "chain_tc_kernel", "resident_net_kernel", "conv_simt_kernel",
-                "conv_pair_kernel")
+                "conv_pair_kernel", "chain_quad_kernel")
 
 
 class fp_node(ctypes.Structure):

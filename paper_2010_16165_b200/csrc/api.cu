@@ -1231,7 +1231,7 @@ fp_status build_plan(fp_handle h) {
             // resolution): the projection becomes extra K groups with a centre tap only, read from its own packed bank.
             if (pj < 0 && h->compute == FP_COMPUTE_BF16_TC && !h->keep_outputs && f.res_mode == 1 && f.R == 3 && f.S == 3 &&
                 f.stride == 1 && f.pad == 1 && !f.scatter && !src.split && !out.split && uses[f.res_tid].size() == 1 && f.tc.valid &&
-                f.tc.flat && !f.tc.b_resident && (f.tc.blocked_bank == 0 || f.tc.split) && !(h->stem_packed && f.src == 0)) {
+                f.tc.flat && !f.tc.b_resident && (f.tc.blocked_bank == 3 || f.tc.split) && !(h->stem_packed && f.src == 0)) {
                 const Tensor& rt = h->tensors[f.res_tid];
                 if (rt.producer >= 0 && rt.producer != h->apart && h->ops[rt.producer].kind == 0) {
                     const int cand = h->ops[rt.producer].idx;
@@ -1308,10 +1308,9 @@ fp_status build_plan(fp_handle h) {
             if (h->stem_fused && i == 1) {
                 j.kind = fp::PACK_STEM_DIRECT; j.w2 = f.d_b32;
                 j.units = 32 * f.K_pad; vecs = (size_t)j.units;
-            } else if (h->stem_packed && f.src == 0) {
-                j.kind = fp::PACK_STEM;
-                j.units = 30 * f.K_pad; vecs = (size_t)j.units;
             } else {
+                const bool stem = h->stem_packed && f.src == 0;
+                if (stem) { j.kind = fp::PACK_STEM; j.cg = 10; }
                 if (f.proj_kind == 1) {
                     const FConv& q = h->convs[f.proj];
                     j.w2 = q.d_w32; j.C2 = q.C; j.row2 = q.row_off; j.chan2 = q.chan_off;
@@ -1324,10 +1323,10 @@ fp_status build_plan(fp_handle h) {
                     // the streamed form of the kernel reads its bank block by block, one copy per pipeline stage; gathered and
                     // resident layers with several filter tiles read it tile by tile
                     j.n_tile = f.tc.n_tile; j.rows = f.tc.n_tile * f.tc.n_tiles;
-                    if (f.tc.blocked_bank == 1) j.cg = f.tc.cg;
+                    if (f.tc.blocked_bank != 2) j.cg = f.tc.cg;
                 }
-                j.units = j.rows * j.chunks;
-                vecs = (size_t)j.units * j.RS;
+                j.units = j.rows * (stem ? 30 : j.chunks);
+                vecs = (size_t)j.units * (stem ? 1 : j.RS);
             }
             wants.push_back({&f.d_wp, vecs * 8 * h->act_elem()});
             add_job(j, &f.d_wp, 0);
@@ -1976,7 +1975,7 @@ extern "C" fp_status fp_debug_expire_wait(fp_handle h, void* stream) {
         const Op& op = h->ops[i];
         if (op.kind != 0 || h->op_chain[i] >= 0 || (h->stem_fused && i == 1)) continue;
         const FConv& f = h->convs[op.idx];
-        if (!f.tc.valid || !f.tc.flat || (f.tc.blocked_bank && !f.tc.split) || h->tensors[f.src].split || h->tensors[f.out].split || f.proj >= 0 || f.absorbed || f.pair >= 0 || f.paired) continue;
+        if (!f.tc.valid || !f.tc.flat || ((f.tc.blocked_bank == 1 || f.tc.blocked_bank == 2) && !f.tc.split) || h->tensors[f.src].split || h->tensors[f.out].split || f.proj >= 0 || f.absorbed || f.pair >= 0 || f.paired) continue;
         // the first round of the activation producer is left out, so the MMA-issuing thread's wait for that stage runs
         // out after a millisecond (two million cycles), raises the status word and takes every role of the CTA with it
         fp::launch_conv_tc(f.tc, f.args, h->d_status, (cudaStream_t)stream, 0, 2000000LL);
@@ -2074,7 +2073,7 @@ static void fill_op_info(fp_handle h, int i, fp_op_info* o) {
             o->bytes_fixed += (double)g.K_kept * g.C_kept * e + 4.0 * g.K_kept;
             o->flops_per_image += 2.0 * t.H * t.W * (double)g.K_kept * g.C_kept;
         }
-        o->kernel = h->net_on ? FP_KERNEL_RESIDENT_NET : h->op_chain[i] >= 0 ? FP_KERNEL_CHAIN_TC : h->stem_fused && i == 1 ? FP_KERNEL_STEM_POOL
+        o->kernel = h->net_on ? FP_KERNEL_RESIDENT_NET : h->op_chain[i] >= 0 ? (h->chains[h->op_chain[i]].plan.quad ? FP_KERNEL_CHAIN_QUAD : FP_KERNEL_CHAIN_TC) : h->stem_fused && i == 1 ? FP_KERNEL_STEM_POOL
                   : !f.tc.valid ? FP_KERNEL_CONV_SIMT : f.pair >= 0 || f.paired ? FP_KERNEL_CONV_PAIR : f.tc.split ? FP_KERNEL_CONV_SPLIT : FP_KERNEL_CONV_TC;
         if (f.absorbed || f.paired) { o->flops_per_image = 0.0; o->bytes_per_image = 0.0; o->bytes_fixed = 0.0; }
     } else if (op.kind == 1) {

@@ -258,7 +258,6 @@ conv_tc_kernel(const TcParams p) {
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&ctrl->tmem_base);
 
     const uint4* __restrict__ xv = reinterpret_cast<const uint4*>(p.a.x);
-    const uint4* __restrict__ wv = reinterpret_cast<const uint4*>(p.a.w);
     // channel chunk -> its plane: the chunks behind x2_chunk0 are the second input tensor's
     const uint4* __restrict__ x2v = reinterpret_cast<const uint4*>(p.a.x2);
     const int chunk2 = p.a.x2_chunk0 > 0 ? p.a.x2_chunk0 : 0x7fffffff;
@@ -281,6 +280,52 @@ conv_tc_kernel(const TcParams p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
+    // Activations, in the modes with a ring of their own.  One lane per channel chunk issues that chunk's copy.  (All lanes test the stage's
+    // barrier: one lane testing and a shuffle of the result was measured slower - 41.0 -> 37.7 us on ResNet-50's 1024 -> 308 layer at
+    // batch 128.)  A warp's copies go out one after the other, some 110 cycles each: with streamed filters the warps that have no tile
+    // of a step to issue MMAs for take a share (`me` of n_sharing).
+    const int n_sharing = MODE == MODE_FLAT_STREAM ? 5 - (int)n_issuers : 1;
+    auto produce = [&](int me) {
+        bool ok = true;
+        uint32_t stage = 0, phase = 0;
+        int round = 0;
+        for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x) {
+            const long long f0 = (long long)(p.m_first + p.m_sign * (int)fdiv((uint32_t)tile, p.div_ntiles)) * p.tps * 128;
+            for (int g = 0; g < p.groups + p.groups2; ++g) {
+                const bool w = __all_sync(0xffffffffu, mbar_wait(a_empty0 + 8 * stage, phase ^ 1, abort_flag, wait_limit));
+                if (!w) { ok = false; break; }
+                int cgg = p.cchunks - g * p.cg;
+                if (cgg > p.cg) cgg = p.cg;
+                const uint32_t fb = a_full0 + 8 * stage;
+                const uint32_t dst = a_base + stage * p.a_stage_bytes;
+                if (g >= p.groups) {
+                    // the K groups of the second input tensor (a projection shortcut's input on this layer's grid)
+                    const int g2 = g - p.groups;
+                    cgg = p.cchunks2 - g2 * p.cg;
+                    if (cgg > p.cg) cgg = p.cg;
+                    if (lane == 0 && me == 0) mbar_expect_tx(fb, (uint32_t)(cgg * p.rows_a * 16));
+                    __syncwarp();
+                    const int c = me + n_sharing * lane;
+                    if (c < cgg)
+                        bulk_copy(dst + c * p.rows_a * 16, x2v + (long long)(g2 * p.cg + c) * p.plane_in2 + f0 - p.halo, (uint32_t)(p.rows_a * 16), fb);
+                    ++round;
+                } else if (round++ != p.skip_round) {       // (a diagnostic launch leaves one round out: its stage never fills)
+                    if (lane == 0 && me == 0) mbar_expect_tx(fb, (uint32_t)(p.a_par * cgg * p.rows_a * 16));
+                    __syncwarp();
+                    // one run per channel chunk - or, over a parity-split tensor, one per chunk and parity image
+                    for (int i = me + n_sharing * lane; i < p.a_par * cgg; i += 32 * n_sharing) {
+                        const int c = p.a_par == 1 ? i : i >> 2, pp = p.a_par == 1 ? 0 : i & 3;
+                        bulk_copy(dst + i * p.rows_a * 16,
+                                  chunk_plane(g * p.cg + c) + (long long)pp * p.par_stride + f0 - p.halo,
+                                  (uint32_t)(p.rows_a * 16), fb);
+                    }
+                }
+                __syncwarp();
+                if (++stage == (uint32_t)p.a_stages) { stage = 0; phase ^= 1; }
+            }
+        }
+        if (!ok && lane == 0) raise(ctrl, p.status, 1);
+    };
     if (MODE == MODE_FLAT_UNIFIED && prod >= 0) {
         // ------------------------------ producers, unified stages ------------------------------
         // One stage per (step of tps position tiles, K group): the group's activation rows for all tiles of the step
@@ -331,48 +376,7 @@ conv_tc_kernel(const TcParams p) {
     } else if (warp == 0) {
         // ------------------------------ bulk-copy producer ------------------------------
         if (MODE != MODE_GATHER) {
-            // One lane per channel chunk issues that chunk's copy, so the copies of a K block are issued
-            // side by side instead of one after the other.  (All lanes test the stage's barrier: one lane testing and a
-            // shuffle of the result was measured slower - 41.0 -> 37.7 us on ResNet-50's 1024 -> 308 layer at batch 128.)
-            bool ok = true;
-            uint32_t stage = 0, phase = 0;
-            int round = 0;
-            for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x) {
-                const long long f0 = (long long)(p.m_first + p.m_sign * (int)fdiv((uint32_t)tile, p.div_ntiles)) * p.tps * 128;
-                for (int g = 0; g < p.groups + p.groups2; ++g) {
-                    const bool w = __all_sync(0xffffffffu, mbar_wait(a_empty0 + 8 * stage, phase ^ 1, abort_flag, wait_limit));
-                    if (!w) { ok = false; break; }
-                    int cgg = p.cchunks - g * p.cg;
-                    if (cgg > p.cg) cgg = p.cg;
-                    const uint32_t fb = a_full0 + 8 * stage;
-                    const uint32_t dst = a_base + stage * p.a_stage_bytes;
-                    if (g >= p.groups) {
-                        // the K groups of the second input tensor (a projection shortcut's input on this layer's grid)
-                        const int g2 = g - p.groups;
-                        cgg = p.cchunks2 - g2 * p.cg;
-                        if (cgg > p.cg) cgg = p.cg;
-                        if (lane == 0) mbar_expect_tx(fb, (uint32_t)(cgg * p.rows_a * 16));
-                        __syncwarp();
-                        if (lane < cgg)
-                            bulk_copy(dst + lane * p.rows_a * 16, x2v + (long long)(g2 * p.cg + lane) * p.plane_in2 + f0 - p.halo,
-                                      (uint32_t)(p.rows_a * 16), fb);
-                        ++round;
-                    } else
-                    if (round++ != p.skip_round) {       // (a diagnostic launch leaves one round out: its stage never fills)
-                        if (lane == 0) mbar_expect_tx(fb, (uint32_t)(p.a_par * cgg * p.rows_a * 16));
-                        __syncwarp();
-                        // one run per channel chunk - or, over a parity-split tensor, one per chunk and parity image
-                        for (int i = lane; i < p.a_par * cgg; i += 32) {
-                            const int c = p.a_par == 1 ? i : i >> 2, pp = p.a_par == 1 ? 0 : i & 3;
-                            bulk_copy(dst + i * p.rows_a * 16,
-                                      chunk_plane(g * p.cg + c) + (long long)pp * p.par_stride + f0 - p.halo,
-                                      (uint32_t)(p.rows_a * 16), fb);
-                        }
-                    }
-                    if (++stage == (uint32_t)p.a_stages) { stage = 0; phase ^= 1; }
-                }
-            }
-            if (!ok && lane == 0) raise(ctrl, p.status, 1);
+            produce(0);
         } else {
             // GATHER: filters of each K block into the stage the loader threads fill, one lane per plane
             bool ok = true;
@@ -554,6 +558,8 @@ conv_tc_kernel(const TcParams p) {
                 if (ok && leader) umma_commit(tfull0 + 8 * acc);   // accumulator complete
             }
             if (!ok && leader) raise(ctrl, p.status, 2);
+        } else if (MODE == MODE_FLAT_STREAM) {
+            produce(issuer - (int)n_issuers + 1);
         }
     } else if (warp < 2 + EPI) {
         // ------------------------------ epilogue ----------------------------------
@@ -855,9 +861,10 @@ conv_tc_kernel(const TcParams p) {
     } else if (MODE == MODE_FLAT_STREAM) {
         // ------------------------------ filter producer (streamed filters) --------------
         if (warp == 2 + EPI) {
-            // One filter block per (K group, filter row): [tap of the row][chunk][filter].  When a tile takes all filters
-            // a tap's chunks are one contiguous run of the packed bank: one copy per tap; otherwise one copy per
-            // (tap, chunk), spread over the lanes.
+            // One filter block per (K group, filter row): [tap of the row][chunk][filter], one run of the bank, which is stored in
+            // this order - filter tile by filter tile, K group by K group (ConvPlanTC::blocked_bank 3); a few lanes copy a part each.
+            // (Read from the plain order a block of several filter tiles was a copy per tap and chunk, 30 of them 3300 cycles, twice
+            // what its MMAs take: ResNet-50's 160 -> 160 layers at 14x14, batch 128.)
             uint32_t stage = 0, phase = 0;
             bool ok = true;
             const bool whole = p.n_tiles == 1;
@@ -868,23 +875,17 @@ conv_tc_kernel(const TcParams p) {
                 for (int g = 0; g < p.groups && ok; ++g) {
                     int cgg = p.cchunks - g * p.cg;
                     if (cgg > p.cg) cgg = p.cg;
-                    for (int r = 0; r < p.a.R; ++r) {
+                    const uint32_t bytes = (uint32_t)(p.a.S * cgg * p.n_tile * 16);
+                    const uint8_t* src = reinterpret_cast<const uint8_t*>(p.a.w) + (long long)nt * p.bank_tile_bytes + (long long)p.taps * (g * p.cg) * p.n_tile * 16;
+                    for (int r = 0; r < p.a.R; ++r, src += bytes) {
                         const bool w = __all_sync(0xffffffffu, mbar_wait(b_empty0 + 8 * stage, phase ^ 1, abort_flag, wait_limit));
                         if (!w) { ok = false; break; }
-                        const uint32_t fb = b_full0 + 8 * stage;
-                        const uint32_t dst = b_base + stage * p.b_stage_bytes;
-                        if (lane == 0) mbar_expect_tx(fb, (uint32_t)(p.a.S * cgg * nrows * 16));
+                        const uint32_t fb = b_full0 + 8 * stage, dst = b_base + stage * p.b_stage_bytes;
+                        if (lane == 0) mbar_expect_tx(fb, bytes);
                         __syncwarp();
-                        const uint4* src = wv + ((long long)(r * p.a.S) * p.cchunks + g * p.cg) * p.a.K_pad + nt * p.n_tile;
-                        if (whole) {
-                            if (lane < p.a.S)
-                                bulk_copy(dst + lane * cgg * p.n_tile * 16, src + (long long)lane * p.cchunks * p.a.K_pad, (uint32_t)(cgg * nrows * 16), fb);
-                        } else {
-                            for (int i = lane; i < p.a.S * cgg; i += 32) {
-                                const int sx = i / cgg, c = i - sx * cgg;
-                                bulk_copy(dst + i * p.n_tile * 16, src + ((long long)sx * p.cchunks + c) * p.a.K_pad, (uint32_t)(nrows * 16), fb);
-                            }
-                        }
+                        const uint32_t off = (uint32_t)lane * 16384u;
+                        if (off < bytes) bulk_copy(dst + off, src + off, bytes - off < 16384u ? bytes - off : 16384u, fb);
+                        __syncwarp();
                         if (++stage == (uint32_t)p.b_stages) { stage = 0; phase ^= 1; }
                     }
                 }
@@ -1183,6 +1184,7 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
         } else {
             a_stage = (unsigned)(a_par * plan->cg * plan->rows_a * 16);
             plan->b_resident = 0;
+            plan->blocked_bank = 3;
             plan->b_stages = 4;
             const unsigned b_stage = (unsigned)(a.S * plan->cg * n_tile * 16);
             plan->a_stages = plan->tps > 1 ? 2 : 3;

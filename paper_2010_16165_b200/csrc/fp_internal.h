@@ -185,7 +185,8 @@ struct ConvPlanTC {
                           //    of flat positions (bulk copies); 0: gathered by loader threads
     int b_resident;       // flat only: the whole filter bank stays in shared memory
     int blocked_bank;     // 1: 1x1 layer with unified stages, bank stored block by block; 2: gathered or resident layer with
-                          // several filter tiles, bank stored tile by tile (PackJob either way)
+                          // several filter tiles, bank stored tile by tile; 3: streamed filters, stored as for 1, a row of
+                          // taps of a K group being one copy (PackJob in each case)
     int cg;               // channel chunks (of 8) per K block
     int groups;           // K blocks per filter tap = ceil((C_pad/8) / cg)
     int halo;             // flat: vectors fetched before and after the 128 positions of a tile

@@ -372,8 +372,10 @@ __device__ __forceinline__ void pack_filters(const PackJob& j, const int32_t* __
 // j = s*C + c within a group; everything else zero.  (Input row 2p+1 is held twice, as O of packed row p and as O' of row
 // p+1; it is taken from row p, because below the last image row there is only the zero border.)
 __device__ __forceinline__ void pack_stem_vec(const PackJob& j, const int32_t* __restrict__ idx, int u) {
-    const int k = u % j.K_pad, chunk = u / j.K_pad % 10, dr = u / j.K_pad / 10;
-    const int ks = idx[j.row + k];
+    // [filter tile][K group][tap row][chunk in group][row in tile], as a convolution's bank
+    const int tile = u / (30 * j.n_tile), at = u / j.n_tile - 30 * tile, k = tile * j.n_tile + u % j.n_tile;
+    const int g = at / (3 * j.cg), in_group = at - 3 * j.cg * g, cgg = min(j.cg, 10 - g * j.cg), dr = in_group / cgg, chunk = g * j.cg + in_group % cgg;
+    const int ks = k < j.K_pad ? idx[j.row + k] : -1;
     float v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {

@@ -64,6 +64,7 @@ struct TcParams {
     int n_tile, n_tiles, tmem_cols, total_tiles;
     int m_first, m_sign;                // position tiles are walked 0, 1, ... or from the last one down (ConvArgs::reverse)
     int tpk, kblocks;                   // gather: taps per K block, K blocks per tile
+    int halves, teams;                  // of sixteen epilogue warps: parts of a tile's columns, tiles of a step at a time
     int tps;                            // streamed filters: 128-position tiles per pipeline step (share each filter block)
     int n_producers;                    // streamed filters: producer warps in use (divides a_stages)
     int a_stage_bytes, b_stage_bytes, b_bank_bytes;
@@ -169,7 +170,7 @@ __device__ __forceinline__ void raise(Ctrl* ctrl, int* status, int code) {
 }
 
 // Threads: warp 0 producer, warp 1 MMA, EPI epilogue warps (4, or 8 for wide filter tiles: two warps per
-// TMEM lane quarter, each taking half of the columns), then either 4 loader warps (GATHER) or 4 filter-producer
+// TMEM lane quarter, each taking half of the columns; 16 where a step has several tiles), then either 4 loader warps (GATHER) or 4 filter-producer
 // warps and 3 more MMA warps (FLAT_STREAM).  One thread gets through a (wait, expect, copy) round of the bulk-copy
 // engine in about 500 cycles whatever the copy's size (measured: 4 KB to 32 KB copies all take 530 cycles per round
 // per thread, and the rate scales with the number of threads up to about 100 B/cycle per SM), so the filter blocks
@@ -222,7 +223,7 @@ conv_tc_kernel(const TcParams p) {
             mbar_init(b_full0 + 8 * s, 1);
             mbar_init(b_empty0 + 8 * s, n_issuers);
         }
-        for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, n_issuers); mbar_init(tempty0 + 8 * s, 32 * EPI); }
+        for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, n_issuers); mbar_init(tempty0 + 8 * s, EPI == 16 ? 128 * p.teams * p.halves : 32 * EPI); }
         ctrl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -285,6 +286,14 @@ conv_tc_kernel(const TcParams p) {
     // batch 128.)  A warp's copies go out one after the other, some 110 cycles each: with streamed filters the warps that have no tile
     // of a step to issue MMAs for take a share (`me` of n_sharing).
     const int n_sharing = MODE == MODE_FLAT_STREAM ? 5 - (int)n_issuers : 1;
+    // The first stages of a CTA's first tile are asked for by the epilogue warps, a copy each in turn: a layer that takes 15 us does not begin
+    // a microsecond later because one warp asks for a dozen planes.  (The producer announces their bytes as for the others.  ResNet-34, 17
+    // images of 200 x 200 271.9 -> 269.7 us, ResNet-50, 33 of 179 x 179 533.8 -> 528.9.)
+    const int n_first = MODE == MODE_FLAT_STREAM || MODE == MODE_FLAT_RESIDENT ? (p.groups < p.a_stages ? p.groups : p.a_stages) : 0;
+    auto run_of = [&](int g, int i) {          // of K group g: run i, one per channel chunk - or, over a parity-split tensor, one per chunk and parity image
+        const int c = p.a_par == 1 ? i : i >> 2, pp = p.a_par == 1 ? 0 : i & 3;
+        return chunk_plane(g * p.cg + c) + (long long)pp * p.par_stride - p.halo;
+    };
     auto produce = [&](int me) {
         bool ok = true;
         uint32_t stage = 0, phase = 0;
@@ -312,13 +321,9 @@ conv_tc_kernel(const TcParams p) {
                 } else if (round++ != p.skip_round) {       // (a diagnostic launch leaves one round out: its stage never fills)
                     if (lane == 0 && me == 0) mbar_expect_tx(fb, (uint32_t)(p.a_par * cgg * p.rows_a * 16));
                     __syncwarp();
-                    // one run per channel chunk - or, over a parity-split tensor, one per chunk and parity image
-                    for (int i = me + n_sharing * lane; i < p.a_par * cgg; i += 32 * n_sharing) {
-                        const int c = p.a_par == 1 ? i : i >> 2, pp = p.a_par == 1 ? 0 : i & 3;
-                        bulk_copy(dst + i * p.rows_a * 16,
-                                  chunk_plane(g * p.cg + c) + (long long)pp * p.par_stride + f0 - p.halo,
-                                  (uint32_t)(p.rows_a * 16), fb);
-                    }
+                    if (round > n_first)
+                        for (int i = me + n_sharing * lane; i < p.a_par * cgg; i += 32 * n_sharing)
+                            bulk_copy(dst + i * p.rows_a * 16, run_of(g, i) + f0, (uint32_t)(p.rows_a * 16), fb);
                 }
                 __syncwarp();
                 if (++stage == (uint32_t)p.a_stages) { stage = 0; phase ^= 1; }
@@ -564,7 +569,9 @@ conv_tc_kernel(const TcParams p) {
     } else if (warp < 2 + EPI) {
         // ------------------------------ epilogue ----------------------------------
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter .. +31 belong to this warp
-        const int half = (warp - 2) >> 2;             // with 8 epilogue warps: which half of the columns
+        // eight epilogue warps: two halves of the columns; sixteen: teams that take a step's tiles in turn
+        const int halves = EPI == 16 ? p.halves : EPI / 4, teams = EPI == 16 ? p.teams : 1;
+        const int half = ((warp - 2) >> 2) & (halves - 1), team = EPI == 16 ? ((warp - 2) >> 2) >> (halves - 1) : 0;
         const int row = quarter * 32 + lane;          // accumulator row = position within the tile
         uint32_t acc_phase0 = 0, acc_phase1 = 0;
         int local = 0;
@@ -572,12 +579,24 @@ conv_tc_kernel(const TcParams p) {
         const uint4* __restrict__ res = reinterpret_cast<const uint4*>(p.a.res);
         const __nv_bfloat16* __restrict__ res_s = reinterpret_cast<const __nv_bfloat16*>(p.a.res);
         uint4* __restrict__ y = reinterpret_cast<uint4*>(p.a.y);
-        for (int tile = blockIdx.x; tile < p.total_tiles; tile += gridDim.x, ++local) {
+        if (n_first > 0 && blockIdx.x < p.total_tiles) {
+            const long long f0 = (long long)(p.m_first + p.m_sign * (int)fdiv(blockIdx.x, p.div_ntiles)) * p.tps * 128;
+            int i = warp - 2;
+            for (int g = 0; g < n_first; ++g) {
+                const int runs = p.a_par * (p.cchunks - g * p.cg < p.cg ? p.cchunks - g * p.cg : p.cg);
+                for (; i < runs; i += EPI)
+                    if (lane == 0 && g != p.skip_round)
+                        bulk_copy(a_base + g * p.a_stage_bytes + i * p.rows_a * 16, run_of(g, i) + f0, (uint32_t)(p.rows_a * 16), a_full0 + 8 * g);
+                i -= runs;
+            }
+            __syncwarp();
+        }
+        for (int tile = blockIdx.x; tile < p.total_tiles && team < teams; tile += gridDim.x, ++local) {
             const int step = (int)fdiv((uint32_t)tile, p.div_ntiles), mt = p.m_first + p.m_sign * step;
             const int nt = tile - step * p.n_tiles;
             const int acc = local & 1;
             const uint32_t ph = acc ? acc_phase1 : acc_phase0;
-            for (int t = 0; t < p.tps; ++t) {
+            for (int t = team; t < p.tps; t += teams) {
             const long long f = ((long long)mt * p.tps + t) * 128 + row;
             const bool exists = f < p.m_total;
             const int n = (int)fdiv((uint32_t)f, p.div_p2out);
@@ -599,7 +618,7 @@ conv_tc_kernel(const TcParams p) {
             }
             const long long yvec0 = (long long)(k_base >> 3) * p.plane_y + fy;
             int c_begin = 0, c_end = cols;
-            if (EPI == 8) {
+            if (halves == 2) {
                 const int first = ((cols >> 4) + 1) / 2 * 16;                      // columns of the first half
                 if (half) c_begin = first; else c_end = first;
             }
@@ -614,7 +633,7 @@ conv_tc_kernel(const TcParams p) {
                 for (int i = 0; i < 8; ++i)
                     if (c_begin + i * 8 < c_end) rq[i] = __ldg(res + vec0 + (long long)((c_begin >> 3) + i) * p.plane_out);
             }
-            if (t == 0) {
+            if (t == team) {
                 ok = mbar_wait(tfull0 + 8 * acc, ph, abort_flag, wait_limit);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -627,14 +646,14 @@ conv_tc_kernel(const TcParams p) {
                 res_vec = (long long)n * rP2 + (long long)((hp - 1) * p.a.res_stride + 1) * rWp + ((wq - 1) * p.a.res_stride + 1);
             }
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((acc * p.tps + t) * p.n_tile);
-            if (p.a.scatter) {
+            if (EPI != 16 && p.a.scatter) {
                 // Scattered output: this filter tile owns the output chunks [q_begin, q_end) of the full-width tensor, and its
                 // accumulator columns are the kept filters of those chunks in channel order.  Columns are read 16 at a
                 // time and parked in a per-warp strip of shared memory (a ring of 32 columns per row, row pitch 33 words:
                 // conflict-free); a chunk of 8 output channels then picks its kept channels' columns from there by index -
                 // the same index in every lane - and takes the shortcut alone for the others.
                 int q_begin = schunk0[nt], q_end = schunk0[nt + 1];
-                if (EPI == 8) {
+                if (halves == 2) {
                     const int mid = q_begin + (q_end - q_begin + 1) / 2;
                     if (half) q_begin = mid; else q_end = mid;
                 }
@@ -973,6 +992,7 @@ int round_up_i(int v, int m) { return (v + m - 1) / m * m; }
 
 const void* kernel_for(int mode, int epi) {
     if (mode == MODE_FLAT_RESIDENT) return epi == 8 ? (const void*)conv_tc_kernel<MODE_FLAT_RESIDENT, 8> : (const void*)conv_tc_kernel<MODE_FLAT_RESIDENT, 4>;
+    if (mode == MODE_FLAT_STREAM && epi == 16) return (const void*)conv_tc_kernel<MODE_FLAT_STREAM, 16>;
     if (mode == MODE_FLAT_STREAM) return epi == 8 ? (const void*)conv_tc_kernel<MODE_FLAT_STREAM, 8> : (const void*)conv_tc_kernel<MODE_FLAT_STREAM, 4>;
     if (mode == MODE_FLAT_UNIFIED) return epi == 8 ? (const void*)conv_tc_kernel<MODE_FLAT_UNIFIED, 8> : (const void*)conv_tc_kernel<MODE_FLAT_UNIFIED, 4>;
     return epi == 8 ? (const void*)conv_tc_kernel<MODE_GATHER, 8> : (const void*)conv_tc_kernel<MODE_GATHER, 4>;
@@ -1233,9 +1253,13 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
     // Wide filter tiles get eight epilogue warps, except in gather mode when there are more tiles than SMs: the
     // eight-warp form needs too many registers for a second CTA on the SM, and a second CTA is what hides the
     // loaders' latency there (measured on ResNet-50, batch 128: every strided layer about 30 % faster with four).
-    const int epi = (n_tile >= 64 && (plan->flat || m_tiles * n_tiles <= sms)) ? 8 : 4;
-    plan->epi_warps = epi;
+    int epi = (n_tile >= 64 && (plan->flat || m_tiles * n_tiles <= sms)) ? 8 : 4;
     const int mode = !plan->flat ? MODE_GATHER : bank_fits ? MODE_FLAT_RESIDENT : plan->blocked_bank == 1 ? MODE_FLAT_UNIFIED : MODE_FLAT_STREAM;
+    // A step's tiles are complete together, and a tile takes one team 1500-2500 cycles: behind the last step's, and for narrow tiles always,
+    // that was what a layer waited for.  Sixteen warps are a team per tile (or two of two halves of the columns): ResNet-18 batch 64 294.6 ->
+    // 291.1 us, ResNet-34 batch 64 539 -> 532.
+    if (mode == MODE_FLAT_STREAM && plan->tps > 1 && ctas == 1 && !a.scatter) epi = 16;
+    plan->epi_warps = epi;
     const void* fn = kernel_for(mode, epi);
     // a per-device attribute: set it for the device this plan is made on (cheap, so not cached)
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
@@ -1293,6 +1317,8 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.n_tile = plan.n_tile; p.n_tiles = plan.n_tiles; p.tmem_cols = plan.tmem_cols;
     const long long m_tiles = (p.m_total + 127) / 128;
     p.tps = plan.tps > 0 ? plan.tps : 1;
+    p.halves = p.tps > 2 ? 1 : 2;
+    p.teams = p.tps < 4 / p.halves ? p.tps : 4 / p.halves;
     p.n_producers = plan.a_stages % 4 == 0 ? 4 : plan.a_stages % 3 == 0 ? 3 : plan.a_stages % 2 == 0 ? 2 : 1;
     p.total_tiles = (int)(((m_tiles + p.tps - 1) / p.tps) * plan.n_tiles);
     p.m_first = a.reverse ? p.total_tiles / plan.n_tiles - 1 : 0;

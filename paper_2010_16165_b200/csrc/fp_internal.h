@@ -194,7 +194,7 @@ struct ConvPlanTC {
     int a_stages, b_stages;
     int tpk;              // gather: filter taps per K block (several when the channel count is small)
     int n_tile, n_tiles;  // filters per CTA tile (multiple of 16, <= 256)
-    int epi_warps;        // 4, or 8 for wide filter tiles
+    int epi_warps;        // 4, 8 for wide filter tiles, 16 where several tiles are complete together
     int tps;              // streamed filters: 128-position tiles per pipeline step
     int tmem_cols;
     unsigned smem_bytes;

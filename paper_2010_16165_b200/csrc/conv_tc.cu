@@ -64,6 +64,7 @@ struct TcParams {
     int n_tile, n_tiles, tmem_cols, total_tiles;
     int m_first, m_sign;                // position tiles are walked 0, 1, ... or from the last one down (ConvArgs::reverse)
     int tpk, kblocks;                   // gather: taps per K block, K blocks per tile
+    int b_kept;                         // streamed filters: every block of the bank has a stage of its own and is copied once
     int halves, teams;                  // of sixteen epilogue warps: parts of a tile's columns, tiles of a step at a time
     int tps;                            // streamed filters: 128-position tiles per pipeline step (share each filter block)
     int n_producers;                    // streamed filters: producer warps in use (divides a_stages)
@@ -511,8 +512,8 @@ conv_tc_kernel(const TcParams p) {
                                 accumulate = 1;
                                 b_lo += (uint32_t)(cgg * p.n_tile);
                             }
-                            if (leader) umma_commit(b_empty0 + 8 * b_stage);
-                            if (++b_stage == (uint32_t)p.b_stages) { b_stage = 0; b_phase ^= 1; }
+                            if (leader && !p.b_kept) umma_commit(b_empty0 + 8 * b_stage);
+                            if (++b_stage == (uint32_t)p.b_stages) { b_stage = 0; b_phase ^= p.b_kept ? 0u : 1u; }
                             a_row += (uint32_t)p.Wp_in;
                         }
                         }
@@ -533,8 +534,8 @@ conv_tc_kernel(const TcParams p) {
                         issue_ksteps(leader, cgg >> 1, d_tmem + (uint32_t)(issuer * p.n_tile), a_row, b_lo, 2u * (uint32_t)p.rows_a,
                                      2u * (uint32_t)p.n_tile, idesc, accumulate);
                         accumulate = 1;
-                        if (leader) umma_commit(b_empty0 + 8 * b_stage);
-                        if (++b_stage == (uint32_t)p.b_stages) { b_stage = 0; b_phase ^= 1; }
+                        if (leader && !p.b_kept) umma_commit(b_empty0 + 8 * b_stage);
+                        if (++b_stage == (uint32_t)p.b_stages) { b_stage = 0; b_phase ^= p.b_kept ? 0u : 1u; }
                         if (leader) umma_commit(a_empty0 + 8 * a_stage);
                         if (++a_stage == (uint32_t)p.a_stages) { a_stage = 0; a_phase ^= 1; }
                     }
@@ -887,7 +888,7 @@ conv_tc_kernel(const TcParams p) {
             uint32_t stage = 0, phase = 0;
             bool ok = true;
             const bool whole = p.n_tiles == 1;
-            for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x) {
+            for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += p.b_kept ? p.total_tiles : gridDim.x) {
                 const int nt = tile - (int)fdiv((uint32_t)tile, p.div_ntiles) * p.n_tiles;
                 int nrows = p.a.K_pad - nt * p.n_tile;
                 if (nrows > p.n_tile) nrows = p.n_tile;
@@ -1135,11 +1136,18 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
             // sharing pays even when it leaves only half of the SMs with a CTA (measured on ResNet-18 at batch 64:
             // 368->512 filters at 7x7, 55 us with 164 single-tile CTAs, 32 us with 84 two-tile CTAs).  The search prefers
             // three blocks in flight over two, then more tiles per step, then longer K groups.
+            //
+            // Three tiles where that is one step for every CTA and two are not: its sums then need no second place in tensor memory.
+            // ResNet-18's 28x28 layers at batch 64, 421 tiles on 148 SMs, go in one round of three instead of two of two (291.0 -> 287.9
+            // us, ResNet-34 532.4 -> 525.2); with several rounds of three ResNet-50 batch 128 lost 8 us.
+            auto steps_of = [&](int tps) { return ((m_tiles + tps - 1) / tps) * n_tiles; };
             bool found = false;
             for (int want_b = 3; want_b >= 2 && !found; --want_b)
-                for (int tps = 4; tps >= 1 && !found; tps >>= 1) {
-                    if (2 * tps * n_tile > 512 || tps * 128 + plan->halo + 8 > kGuardVectors) continue;
-                    if (tps > 1 && ((m_tiles + tps - 1) / tps) * n_tiles < sms * 2 / 5) continue;
+                for (int tps : {3, 4, 2, 1}) {
+                    const bool one_step = tps == 3;
+                    if (found || (one_step && (steps_of(3) > sms || steps_of(2) <= sms))) continue;
+                    if ((one_step ? 1 : 2) * tps * n_tile > 512 || tps * 128 + plan->halo + 8 > kGuardVectors) continue;
+                    if (tps > 1 && steps_of(tps) < sms * 2 / 5) continue;
                     const int cg_hi = bank_fits ? plan->cg : (cchunks < 12 ? cchunks : 12), cg_lo = bank_fits ? plan->cg : (cchunks < 4 ? cchunks : 4);
                     for (int cg = cg_hi; cg >= cg_lo && !found; cg -= 2) {
                         const unsigned b_try = (unsigned)(a.S * cg * n_tile * 16), a_try = (unsigned)(cg * run_rows(tps) * 16);
@@ -1206,10 +1214,15 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
             plan->b_resident = 0;
             plan->blocked_bank = 3;
             plan->b_stages = 4;
+            // All blocks of a layer with one filter tile where there is room for them: they stay (ResNet-18, unpruned, 13 images of 253 x
+            // 253 174.0 -> 170.4 us).
+            const int blocks = a.R * plan->groups + (a.x2_C_pad > 0 ? (a.x2_C_pad / 8 + plan->cg - 1) / plan->cg : 0);
             const unsigned b_stage = (unsigned)(a.S * plan->cg * n_tile * 16);
             plan->a_stages = plan->tps > 1 ? 2 : 3;
+            plan->b_kept = n_tiles == 1 && blocks <= kMaxStages && smem + blocks * b_stage + 2u * a_stage <= kSmemMax - 128u;
+            if (plan->b_kept) plan->b_stages = blocks;
             while (plan->a_stages > 2 && smem + plan->b_stages * b_stage + plan->a_stages * a_stage > kSmemMax) --plan->a_stages;
-            while (plan->b_stages > 2 && smem + plan->b_stages * b_stage + plan->a_stages * a_stage > kSmemMax) --plan->b_stages;
+            while (!plan->b_kept && plan->b_stages > 2 && smem + plan->b_stages * b_stage + plan->a_stages * a_stage > kSmemMax) --plan->b_stages;
             smem += (unsigned)round_up_i((int)(plan->b_stages * b_stage), 128) + plan->a_stages * a_stage;
         }
         }
@@ -1239,7 +1252,8 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
         smem += plan->a_stages * stage;
     }
     if (plan->tps < 1) plan->tps = 1;
-    plan->tmem_cols = pow2_at_least(2 * plan->tps * n_tile < 32 ? 32 : 2 * plan->tps * n_tile);
+    const int sums = (plan->tps == 3 ? 1 : 2) * plan->tps * n_tile;          // (three tiles: one step a CTA)
+    plan->tmem_cols = pow2_at_least(sums < 32 ? 32 : sums);
     const int tmem_ctas = 512 / plan->tmem_cols;
     if (smem > kSmemMax) { snprintf(err, err_len, "tile does not fit shared memory (%u bytes)", smem); return 1; }
     // co-resident CTAs must not ask for more than the 512 tensor-memory columns of an SM
@@ -1317,6 +1331,7 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.n_tile = plan.n_tile; p.n_tiles = plan.n_tiles; p.tmem_cols = plan.tmem_cols;
     const long long m_tiles = (p.m_total + 127) / 128;
     p.tps = plan.tps > 0 ? plan.tps : 1;
+    p.b_kept = plan.b_kept && a.R * plan.groups + p.groups2 == plan.b_stages;      // (a projection's blocks come on top: then the stages are a ring)
     p.halves = p.tps > 2 ? 1 : 2;
     p.teams = p.tps < 4 / p.halves ? p.tps : 4 / p.halves;
     p.n_producers = plan.a_stages % 4 == 0 ? 4 : plan.a_stages % 3 == 0 ? 3 : plan.a_stages % 2 == 0 ? 2 : 1;

@@ -65,6 +65,7 @@ struct TcParams {
     int m_first, m_sign;                // position tiles are walked 0, 1, ... or from the last one down (ConvArgs::reverse)
     int tpk, kblocks;                   // gather: taps per K block, K blocks per tile
     int b_kept;                         // streamed filters: every block of the bank has a stage of its own and is copied once
+    int alternate;                      // eight epilogue warps take every other tile by fours
     int halves, teams;                  // of sixteen epilogue warps: parts of a tile's columns, tiles of a step at a time
     int tps;                            // streamed filters: 128-position tiles per pipeline step (share each filter block)
     int n_producers;                    // streamed filters: producer warps in use (divides a_stages)
@@ -224,7 +225,7 @@ conv_tc_kernel(const TcParams p) {
             mbar_init(b_full0 + 8 * s, 1);
             mbar_init(b_empty0 + 8 * s, n_issuers);
         }
-        for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, n_issuers); mbar_init(tempty0 + 8 * s, EPI == 16 ? 128 * p.teams * p.halves : 32 * EPI); }
+        for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, n_issuers); mbar_init(tempty0 + 8 * s, EPI == 16 ? 128 * p.teams * p.halves : p.alternate ? 128 : 32 * EPI); }
         ctrl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -571,11 +572,13 @@ conv_tc_kernel(const TcParams p) {
         // ------------------------------ epilogue ----------------------------------
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter .. +31 belong to this warp
         // eight epilogue warps: two halves of the columns; sixteen: teams that take a step's tiles in turn
-        const int halves = EPI == 16 ? p.halves : EPI / 4, teams = EPI == 16 ? p.teams : 1;
+        // (p.alternate: eight, as two teams that take every other step, each its own accumulators)
+        const int halves = EPI == 16 ? p.halves : EPI == 8 && !p.alternate ? 2 : 1, teams = EPI == 16 ? p.teams : 1;
         const int half = ((warp - 2) >> 2) & (halves - 1), team = EPI == 16 ? ((warp - 2) >> 2) >> (halves - 1) : 0;
+        const int parity = EPI == 8 && p.alternate ? (warp - 2) >> 2 : 0, every = EPI == 8 && p.alternate ? 2 : 1;
         const int row = quarter * 32 + lane;          // accumulator row = position within the tile
         uint32_t acc_phase0 = 0, acc_phase1 = 0;
-        int local = 0;
+        int local = parity;
         bool ok = true;
         const uint4* __restrict__ res = reinterpret_cast<const uint4*>(p.a.res);
         const __nv_bfloat16* __restrict__ res_s = reinterpret_cast<const __nv_bfloat16*>(p.a.res);
@@ -592,7 +595,7 @@ conv_tc_kernel(const TcParams p) {
             }
             __syncwarp();
         }
-        for (int tile = blockIdx.x; tile < p.total_tiles && team < teams; tile += gridDim.x, ++local) {
+        for (int tile = blockIdx.x + parity * gridDim.x; tile < p.total_tiles && team < teams; tile += every * gridDim.x, local += every) {
             const int step = (int)fdiv((uint32_t)tile, p.div_ntiles), mt = p.m_first + p.m_sign * step;
             const int nt = tile - step * p.n_tiles;
             const int acc = local & 1;
@@ -1273,6 +1276,12 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
     // that was what a layer waited for.  Sixteen warps are a team per tile (or two of two halves of the columns): ResNet-18 batch 64 294.6 ->
     // 291.1 us, ResNet-34 batch 64 539 -> 532.
     if (mode == MODE_FLAT_STREAM && plan->tps > 1 && ctas == 1 && !a.scatter) epi = 16;
+    // 3x3 layers with resident filters, where a CTA has more than one tile: two teams that take every other tile.  What an epilogue pays per tile
+    // whatever its width - places, shortcut loads behind the stores of the tile before, the wait - was 1500 of the 3400 cycles of a
+    // 64-filter tile with a shortcut, and longer than the tile's MMAs: ResNet-18 batch 200 732 -> 695 us, batch 64 287 -> 280.  (1x1 layers,
+    // bound by memory, and tiles of fewer filters, whose MMAs are the longer part, lost: ResNet-50 batch 128 1252 -> 1268 us with both,
+    // 1259 with the latter.)
+    plan->alternate = mode == MODE_FLAT_RESIDENT && epi == 8 && taps > 1 && m_tiles * n_tiles > (long long)sms * ctas;
     plan->epi_warps = epi;
     const void* fn = kernel_for(mode, epi);
     // a per-device attribute: set it for the device this plan is made on (cheap, so not cached)
@@ -1331,6 +1340,7 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.n_tile = plan.n_tile; p.n_tiles = plan.n_tiles; p.tmem_cols = plan.tmem_cols;
     const long long m_tiles = (p.m_total + 127) / 128;
     p.tps = plan.tps > 0 ? plan.tps : 1;
+    p.alternate = plan.alternate;
     p.b_kept = plan.b_kept && a.R * plan.groups + p.groups2 == plan.b_stages;      // (a projection's blocks come on top: then the stages are a ring)
     p.halves = p.tps > 2 ? 1 : 2;
     p.teams = p.tps < 4 / p.halves ? p.tps : 4 / p.halves;

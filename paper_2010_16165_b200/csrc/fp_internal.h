@@ -195,6 +195,7 @@ struct ConvPlanTC {
     int tpk;              // gather: filter taps per K block (several when the channel count is small)
     int n_tile, n_tiles;  // filters per CTA tile (multiple of 16, <= 256)
     int epi_warps;        // 4, 8 for wide filter tiles, 16 where several tiles are complete together
+    int alternate;        // eight epilogue warps as two teams that take every other tile
     int tps;              // streamed filters: 128-position tiles per pipeline step
     int b_kept;           // streamed filters: a stage for every block of the bank, copied once
     int tmem_cols;

@@ -1278,10 +1278,10 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
     if (mode == MODE_FLAT_STREAM && plan->tps > 1 && ctas == 1 && !a.scatter) epi = 16;
     // 3x3 layers with resident filters, where a CTA has more than one tile: two teams that take every other tile.  What an epilogue pays per tile
     // whatever its width - places, shortcut loads behind the stores of the tile before, the wait - was 1500 of the 3400 cycles of a
-    // 64-filter tile with a shortcut, and longer than the tile's MMAs: ResNet-18 batch 200 732 -> 695 us, batch 64 287 -> 280.  (1x1 layers,
-    // bound by memory, and tiles of fewer filters, whose MMAs are the longer part, lost: ResNet-50 batch 128 1252 -> 1268 us with both,
-    // 1259 with the latter.)
-    plan->alternate = mode == MODE_FLAT_RESIDENT && epi == 8 && taps > 1 && m_tiles * n_tiles > (long long)sms * ctas;
+    // 64-filter tile with a shortcut, and longer than the tile's MMAs.  ResNet-18 batch 200 732 -> 707 us with tiles of 64 filters and more, 695
+    // with narrower ones over 64 channels and more as well, batch 64 287 -> 284 -> 280.  (Narrow tiles over 48 channels lost, ResNet-50 batch 128 1252
+    // -> 1259, and so did 1x1 layers, which memory bounds: 1268.)
+    if (mode == MODE_FLAT_RESIDENT && (epi == 8 || cchunks >= 8) && taps > 1 && m_tiles * n_tiles > (long long)sms * ctas) { plan->alternate = 1; epi = 8; }
     plan->epi_warps = epi;
     const void* fn = kernel_for(mode, epi);
     // a per-device attribute: set it for the device this plan is made on (cheap, so not cached)

@@ -1,4 +1,4 @@
-"""3x3 layers with streamed filters whose steps have one to four tiles of 128 positions: every operator's output against the validation
+"""3x3 layers with streamed filters whose steps have one to four tiles of 128 positions, and with resident ones: every operator's output against the validation
 convolutions, at batches where a CTA has one step or several, the last one partial, filters that stay and filters that come with every
 step, a projection taken in (its filter blocks on top), wide images."""
 import numpy as np
@@ -30,6 +30,8 @@ def B():
     ((2,), (48,), 232, 9, 0.0),             # 58 pixels wide: steps share the halo, the filters stay
     ((2,), (80,), 248, 33, 0.3),            # 62 pixels wide, several steps a CTA, the last one partial
     ((1,), (256,), 72, 47, 0.0),            # filters that take longer than the MMAs of a tile
+    ((2,), (64,), 120, 25, 0.0),            # filters that stay as a whole, one or two tiles a CTA: teams that take every other tile
+    ((2,), (64,), 120, 61, 0.3),            # the same with narrow tiles, three and four a CTA
 ])
 def test_steps_of_tiles(B, layers, widths, hw, batch, p):
     net = wl.resnet_imagenet_basic(layers, widths, in_hw=hw, n_classes=5, name="steps")

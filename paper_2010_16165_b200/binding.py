@@ -22,12 +22,13 @@ FP_COMPUTE_BF16_TC, FP_COMPUTE_FP32, FP_COMPUTE_BF16_SIMT = 0, 1, 2
 FP_NORM_L1, FP_NORM_L2 = 0, 1
 (FP_Q_N_CONVS, FP_Q_CONV_K_FUSED, FP_Q_CONV_K_KEPT, FP_Q_CONV_C_KEPT, FP_Q_MASK, FP_Q_RANK, FP_Q_N_CLASSES,
  FP_Q_FLOPS, FP_Q_BYTES, FP_Q_N_OPS, FP_Q_OP_INFO, FP_Q_OP_OUTPUT, FP_Q_DEVICE_STATUS, FP_Q_N_LAUNCHES,
- FP_Q_OP_TIMES, FP_Q_CONV_BANK_ELEMS, FP_Q_ALL_MASKS) = range(17)
+ FP_Q_OP_TIMES, FP_Q_CONV_BANK_ELEMS, FP_Q_ALL_MASKS, FP_Q_OP_PLAN) = range(18)
 
 EXPORTS = ["fp_fuse", "fp_prune", "fp_forward", "fp_forward_host", "fp_forward_host_async", "fp_score", "fp_query", "fp_destroy",
            "fp_last_error", "fp_rank_filters_static", "fp_soft_prune_epoch", "fp_soft_prune_finish",
            "fp_debug_expire_wait", "fp_fuse_with_allocator"]
 FP_STATIC_RANK_MAX_FILTERS = 4096
+OP_PLAN_FIELDS = ("tps", "cg", "groups", "groups2", "a_stages", "b_stages", "stays", "epi_warps", "alternate", "n_tile")
 CONV_KERNELS = ("", "conv_tc_kernel", "conv_split_kernel", "stem_pool_kernel", "chain_tc_kernel", "resident_net_kernel", "conv_simt_kernel",
                 "conv_pair_kernel", "chain_quad_kernel")
 
@@ -211,6 +212,11 @@ def fp_query_array(h, what, index, dtype, count):
     out = np.empty(count, dtype=dtype)
     _check(lib().fp_query(h, what, index, out.ctypes.data, out.nbytes))
     return out
+
+
+def fp_query_plan(h, index):
+    """The form that operator `index` has in conv_tc_kernel: OP_PLAN_FIELDS -> int (zeros where another kernel computes it)."""
+    return dict(zip(OP_PLAN_FIELDS, fp_query_array(h, FP_Q_OP_PLAN, index, np.int32, len(OP_PLAN_FIELDS)).tolist()))
 
 
 def fp_query_op(h, index):

@@ -2172,6 +2172,22 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             TRY(need(sizeof(fp_op_info)));
             fill_op_info(h, index, (fp_op_info*)h_out);
             return FP_OK;
+        case FP_Q_OP_PLAN: {
+            if (index < 0 || index >= (int)h->ops.size()) return fail(FP_ERR_ARG, "fp_query: operator %d out of range", index);
+            TRY(need(10 * sizeof(int32_t)));
+            int32_t* o = (int32_t*)h_out;
+            memset(o, 0, 10 * sizeof(int32_t));
+            fp_op_info info;
+            fill_op_info(h, index, &info);
+            if (info.kind != 0 || info.kernel != FP_KERNEL_CONV_TC || h->convs[h->ops[index].idx].absorbed) return FP_OK;
+            const FConv& c = h->convs[h->ops[index].idx];
+            const int groups2 = (c.args.x2_C_pad / 8 + c.tc.cg - 1) / c.tc.cg;
+            const bool stays = c.tc.b_kept && c.R * c.tc.groups + groups2 == c.tc.b_stages;
+            const int32_t plan[10] = {c.tc.tps, c.tc.cg, c.tc.groups, groups2, c.tc.a_stages, c.tc.b_stages, c.tc.b_resident ? 1 : stays ? 2 : 0,
+                                      c.tc.epi_warps, c.tc.alternate, c.tc.n_tile};
+            memcpy(o, plan, sizeof(plan));
+            return FP_OK;
+        }
         case FP_Q_OP_OUTPUT: {
             if (index < 0 || index >= (int)h->ops.size() || h->ops[index].kind == 2)
                 return fail(FP_ERR_ARG, "fp_query: operator %d has no activation output", index);

@@ -220,7 +220,8 @@ conv_tc_kernel(const TcParams p) {
     const int prod = MODE != MODE_FLAT_UNIFIED ? -1 : warp == 0 ? 0 : (warp >= 2 + EPI && warp < 1 + EPI + kProducers) ? warp - (1 + EPI) : -1;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxStages; ++s) {
-            mbar_init(a_full0 + 8 * s, MODE == MODE_GATHER ? 129 : 1);   // gather: 128 loaders + the filter producer
+            // gather: 128 loaders + the filter producer; streamed filters: every warp that copies activations (`produce`)
+            mbar_init(a_full0 + 8 * s, MODE == MODE_GATHER ? 129 : MODE == MODE_FLAT_STREAM ? 5 - n_issuers : 1);
             mbar_init(a_empty0 + 8 * s, n_issuers);
             mbar_init(b_full0 + 8 * s, 1);
             mbar_init(b_empty0 + 8 * s, n_issuers);
@@ -286,10 +287,12 @@ conv_tc_kernel(const TcParams p) {
     // Activations, in the modes with a ring of their own.  One lane per channel chunk issues that chunk's copy.  (All lanes test the stage's
     // barrier: one lane testing and a shuffle of the result was measured slower - 41.0 -> 37.7 us on ResNet-50's 1024 -> 308 layer at
     // batch 128.)  A warp's copies go out one after the other, some 110 cycles each: with streamed filters the warps that have no tile
-    // of a step to issue MMAs for take a share (`me` of n_sharing).
+    // of a step to issue MMAs for take a share (`me` of n_sharing).  Each announces its own share and arrives for every stage, also where it has
+    // no copy of it: a stage cannot be filled, used and emptied past a warp that has yet to look at it, and whose test of the parity would
+    // then take the next phase's for its own.
     const int n_sharing = MODE == MODE_FLAT_STREAM ? 5 - (int)n_issuers : 1;
     // The first stages of a CTA's first tile are asked for by the epilogue warps, a copy each in turn: a layer that takes 15 us does not begin
-    // a microsecond later because one warp asks for a dozen planes.  (The producer announces their bytes as for the others.  ResNet-34, 17
+    // a microsecond later because one warp asks for a dozen planes.  (The producers announce their bytes as for the others.  ResNet-34, 17
     // images of 200 x 200 271.9 -> 269.7 us, ResNet-50, 33 of 179 x 179 533.8 -> 528.9.)
     const int n_first = MODE == MODE_FLAT_STREAM || MODE == MODE_FLAT_RESIDENT ? (p.groups < p.a_stages ? p.groups : p.a_stages) : 0;
     auto run_of = [&](int g, int i) {          // of K group g: run i, one per channel chunk - or, over a parity-split tensor, one per chunk and parity image
@@ -297,6 +300,7 @@ conv_tc_kernel(const TcParams p) {
         return chunk_plane(g * p.cg + c) + (long long)pp * p.par_stride - p.halo;
     };
     auto produce = [&](int me) {
+        auto share = [&](int runs) { return (uint32_t)((runs + n_sharing - 1 - me) / n_sharing * p.rows_a * 16); };      // bytes of runs me, me + n_sharing, ...
         bool ok = true;
         uint32_t stage = 0, phase = 0;
         int round = 0;
@@ -314,14 +318,14 @@ conv_tc_kernel(const TcParams p) {
                     const int g2 = g - p.groups;
                     cgg = p.cchunks2 - g2 * p.cg;
                     if (cgg > p.cg) cgg = p.cg;
-                    if (lane == 0 && me == 0) mbar_expect_tx(fb, (uint32_t)(cgg * p.rows_a * 16));
+                    if (lane == 0) mbar_expect_tx(fb, share(cgg));
                     __syncwarp();
                     const int c = me + n_sharing * lane;
                     if (c < cgg)
                         bulk_copy(dst + c * p.rows_a * 16, x2v + (long long)(g2 * p.cg + c) * p.plane_in2 + f0 - p.halo, (uint32_t)(p.rows_a * 16), fb);
                     ++round;
                 } else if (round++ != p.skip_round) {       // (a diagnostic launch leaves one round out: its stage never fills)
-                    if (lane == 0 && me == 0) mbar_expect_tx(fb, (uint32_t)(p.a_par * cgg * p.rows_a * 16));
+                    if (lane == 0) mbar_expect_tx(fb, share(p.a_par * cgg));
                     __syncwarp();
                     if (round > n_first)
                         for (int i = me + n_sharing * lane; i < p.a_par * cgg; i += 32 * n_sharing)

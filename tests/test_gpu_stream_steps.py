@@ -55,3 +55,52 @@ def test_steps_of_tiles(B, layers, widths, hw, batch, p):
     finally:
         g.close()
         slow.close()
+
+
+def steps_of(o, plan, batch):
+    """Steps of a layer: groups of `tps` tiles of 128 positions (the image's, its zero row and column, those behind the last one), per filter tile."""
+    positions = batch * (o.P + 1) * (o.Q + 1) + o.Q + 2
+    return -(-positions // (128 * plan["tps"])) * -(-o.K_pad // plan["n_tile"])
+
+
+# What is asserted of the operator: its form, chunks of the last K group, and whether a CTA has one step or several.  With streamed filters 5 - tps
+# warps copy activations, each a part of a K group's chunks: none where the group has fewer than that, and none of the first groups.
+@pytest.mark.parametrize("layers, widths, hw, batch, p, scatter, op, form, last, several", [
+    ((2,), (96,), 112, 64, 0.0, 0, 3, dict(tps=3, groups=2, stays=0, epi_warps=16), 4, False),
+    ((1,), (112,), 112, 64, 0.0, 0, 3, dict(tps=3, groups=3, stays=0, epi_warps=16), 2, False),     # two warps, two chunks
+    ((1,), (208,), 56, 200, 0.0, 0, 3, dict(tps=2, groups=4, stays=0, epi_warps=16), 2, True),      # three warps, two chunks
+    ((1,), (160,), 56, 20, 0.3, 1, 4, dict(tps=1, groups=2, stays=0, epi_warps=8), 2, False),       # four warps, two chunks; scattered output
+    ((1,), (192,), 112, 100, 0.7, 0, 3, dict(tps=4, groups=3, stays=0, epi_warps=16), 8, True),     # one warp
+    ((1,), (80,), 112, 100, 0.0, 0, 3, dict(tps=2, groups=1, stays=2, epi_warps=16), 10, True),     # filters that stay
+    ((1,), (48,), 264, 9, 0.0, 0, 3, dict(tps=3, groups=1, stays=2, epi_warps=16), 6, False),       # 66 pixels wide: steps share the halo
+    ((1,), (48,), 264, 30, 0.0, 0, 3, dict(tps=4, groups=1, stays=2, epi_warps=16), 6, True),
+    ((1, 1), (48, 112), 112, 200, 0.0, 0, 7, dict(tps=3, groups=3, groups2=1, stays=0, epi_warps=16), 2, False),     # a projection's 6 chunks
+    ((1, 1), (16, 112), 112, 200, 0.0, 0, 7, dict(tps=3, groups=3, groups2=1, stays=0, epi_warps=16), 2, False),     # ... and its 2
+    ((1, 1), (16, 144), 112, 200, 0.0, 0, 7, dict(tps=2, groups=2, groups2=1, stays=0, epi_warps=16), 8, True),      # three warps, 2 chunks
+    ((1,), (256,), 72, 90, 0.0, 0, 3, dict(tps=2, groups=4, stays=0, epi_warps=16, n_tile=128), 8, True),
+])
+def test_forms(B, layers, widths, hw, batch, p, scatter, op, form, last, several):
+    net = wl.resnet_imagenet_basic(layers, widths, in_hw=hw, n_classes=5, name="forms")
+    w = wl.Workload("forms", net, batch, 31, True, wl.uniform_ratios(p), "uniform")
+    g, slow = Gpu(B, w, B.FP_COMPUTE_BF16_TC, scatter=scatter), Gpu(B, w, B.FP_COMPUTE_BF16_SIMT, keep_outputs=1)
+    try:
+        for x in (g, slow):
+            B.fp_prune(x.h, w.ratios)
+        o, plan = B.op_infos(g.h)[op], B.fp_query_plan(g.h, op)
+        assert {k: plan[k] for k in form} == form
+        assert o.C_pad // 8 - (plan["groups"] - 1) * plan["cg"] == last
+        assert (steps_of(o, plan, batch) > torch.cuda.get_device_properties(0).multi_processor_count) == several
+        logits = g.forward(w.x)
+        slow.forward(w.x)
+        got, want = outputs(B, g, w), outputs(B, slow, w)
+        seen = [i for i, o in enumerate(B.op_infos(g.h)) if o.kind == 0 and got[i] is not None and got[i].shape == want[i].shape]
+        assert op in seen
+        for i in seen:
+            assert close(got[i], want[i]), i
+        for _ in range(20):                                   # nothing depends on who was first (and every forward's status is 0)
+            np.testing.assert_array_equal(g.forward(w.x), logits)
+        for n in (1, batch // 2):
+            np.testing.assert_array_equal(g.forward(w.x[:n]), logits[:n])
+    finally:
+        g.close()
+        slow.close()

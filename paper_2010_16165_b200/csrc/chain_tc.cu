@@ -46,7 +46,7 @@ using namespace tc;
 struct ChainParams {
     ChainArgs a;
     int G, tiles, plane_rows, buf_bytes, wbuf_bytes, tmem_cols, acc_cols, n_groups, stages, split, issuers, ring;
-    int img_pos, w_shift, P2, Wp;
+    int img_pos, P2, Wp;
     FastDiv div_rows;
     long long plane_in, plane_out, plane_res;
     int rP2, rWp;
@@ -113,6 +113,8 @@ __device__ __forceinline__ void issue_tile(bool leader, uint32_t d_tmem, uint32_
     }
 }
 
+// W: the images' width, 8, 16 or 32.  (As a constant: with the width of a shuffle in a register 20 bytes spilled and ResNet-110 lost 1.3 %.)
+template <int W>
 __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_constant__ ChainParams p) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     ChainCtrl* ctrl = reinterpret_cast<ChainCtrl*>(smem_raw);
@@ -155,11 +157,10 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
     __shared__ ChainLayer s_layers[kChainMaxLayers];
     for (int i = threadIdx.x; i < p.a.n_layers * (int)(sizeof(ChainLayer) / 4); i += blockDim.x)
         reinterpret_cast<int*>(s_layers)[i] = reinterpret_cast<const int*>(p.a.layers)[i];
-    // The W guard rows before and after each chunk plane are only read for rows whose results are discarded,
-    // but they must hold finite values (the epilogue masks neighbour terms by multiplying with 0): zero them once.
+    // The W guard rows before and after each chunk plane are only read for rows whose results are discarded: zero them once.
     {
         const int planes = 2 * (p.buf_bytes / (p.plane_rows * 16));
-        const int guard = p.a.W;
+        const int guard = W;
         for (int i = threadIdx.x; i < planes * 2 * guard; i += blockDim.x) {
             const int pl = i / (2 * guard), r = i - pl * 2 * guard;
             const int row = r < guard ? r : p.plane_rows - 2 * guard + r;
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                     const uint32_t src = act0 + (uint32_t)(l & 1) * (uint32_t)p.buf_bytes;
                     // low descriptor words: start address / 16 | (bytes between the two K halves / 16) << 16
                     const uint32_t a_r0 = (src >> 4) | ((uint32_t)p.plane_rows << 16);     // tap row r = 0 starts W rows before the tile
-                    const uint32_t a_r1 = a_r0 + (uint32_t)p.a.W, a_r2 = a_r1 + (uint32_t)p.a.W;
+                    const uint32_t a_r1 = a_r0 + (uint32_t)W, a_r2 = a_r1 + (uint32_t)W;
                     const uint32_t b_r0 = ((wbuf0 + wb * (uint32_t)p.wbuf_bytes) >> 4) | (N << 16);
                     const uint32_t b_r1 = b_r0 + (uint32_t)ly.cchunks * N, b_r2 = b_r1 + (uint32_t)ly.cchunks * N;
                     const uint32_t a_ks = 2u * (uint32_t)p.plane_rows, b_ks = 2u * N;
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         const int unit = grp / split;                 // takes tiles unit, unit + units, ... (the tiles of MMA issuer `unit`)
         const int part = grp - unit * split;          // takes 16-channel groups part, part + split, ...
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter .. +31
-        const int W = p.a.W, H = p.a.H;
+        const int H = p.a.H;
         const int wcol = lane & (W - 1);              // W divides 32: the column of this thread's positions never changes
         const float m_left = wcol > 0 ? 1.0f : 0.0f, m_right = wcol < W - 1 ? 1.0f : 0.0f;
         const int tiles = p.tiles;
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                     for (int q = 0; q < kLoadBatch; ++q) {
                         const int t = tb + q * units;
                         const int f = t * 128 + quarter * 32 + lane;
-                        const int row = f >> p.w_shift;
+                        const int row = (int)((uint32_t)f / W);
                         const int img = (int)fdiv((uint32_t)row, p.div_rows);
                         const int hrow = row - img * (H + 1);
                         const int n = g * p.G + img;
@@ -439,12 +440,14 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                         tmem_ld_wait();
                         // of the 48 columns: [0,16) tap s = 0, wanted by the position on the right; [16,32) the centre
                         // tap; [32,48) tap s = 2, wanted by the position on the left.  The masks drop the neighbour's
-                        // term in the first / last column of an image row (all values involved are finite).
+                        // term in the first / last column of an image row.  The shuffles stay within rows: such a lane gets its own
+                        // term, not one of the row of zeros behind its image, whose sums hold the next image's values - one that
+                        // is not finite would come through a mask of zero.
                         float o[16];
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
-                            const float lf = __shfl_up_sync(0xffffffffu, __uint_as_float(vlc[i]), 1);
-                            const float rt = __shfl_down_sync(0xffffffffu, __uint_as_float(vr[i]), 1);
+                            const float lf = __shfl_up_sync(0xffffffffu, __uint_as_float(vlc[i]), 1, W);
+                            const float rt = __shfl_down_sync(0xffffffffu, __uint_as_float(vr[i]), 1, W);
                             o[i] = fmaf(rt, m_right, fmaf(lf, m_left, __uint_as_float(vlc[16 + i]) + bb[i]));
                         }
                         if (res) {
@@ -471,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                         if (!last) { *slot0 = ov[0]; *slot1 = ov[1]; }
                         else if (pixel) {
                             const int f = t * 128 + quarter * 32 + lane;
-                            const int row = f >> p.w_shift;
+                            const int row = (int)((uint32_t)f / W);
                             const int img = (int)fdiv((uint32_t)row, p.div_rows);
                             const int hrow = row - img * (H + 1);
                             const long long gpos = (long long)(g * p.G + img) * p.P2 + (long long)hrow * p.Wp + (wcol + 1);
@@ -532,6 +535,10 @@ constexpr unsigned kSmemMin = 120u * 1024u;        // more than half an SM: one 
 
 int round_up_i(int v, int m) { return (v + m - 1) / m * m; }
 
+const void* kernel_of(int W) {
+    return W == 8 ? (const void*)chain_tc_kernel<8> : W == 16 ? (const void*)chain_tc_kernel<16> : (const void*)chain_tc_kernel<32>;
+}
+
 }  // namespace
 
 int chain_layer_blob_bytes(int cchunks, int K_pad) { return 3 * cchunks * 3 * K_pad * 16 + K_pad * 4; }
@@ -588,7 +595,7 @@ int plan_chain_tc(const ChainArgs& a, ChainPlan* plan, char* err, size_t err_len
     if (smem < kSmemMin) smem = kSmemMin;
     plan->smem_bytes = smem;
     // a per-device attribute: set it for the device this plan is made on (cheap, so not cached)
-    if (cudaFuncSetAttribute(chain_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
+    if (cudaFuncSetAttribute(kernel_of(a.W), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
         snprintf(err, err_len, "cannot raise the dynamic shared memory limit");
         cudaGetLastError();
         return 1;
@@ -608,7 +615,6 @@ void launch_chain_tc(const ChainPlan& plan, const ChainArgs& a, int* d_status, c
     p.ring = plan.stages / plan.issuers;
     p.n_groups = (a.N + plan.G - 1) / plan.G;
     p.img_pos = (a.H + 1) * a.W;
-    p.w_shift = a.W == 8 ? 3 : a.W == 16 ? 4 : 5;
     p.Wp = row_vecs(a.W); p.P2 = image_vecs(a.H, a.W);
     p.div_rows = make_fastdiv((uint32_t)(a.H + 1));
     p.plane_in = plane_vecs(a.N, a.H, a.W);
@@ -631,7 +637,7 @@ void launch_chain_tc(const ChainPlan& plan, const ChainArgs& a, int* d_status, c
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     void* args[1] = {(void*)&p};
-    cudaLaunchKernelExC(&cfg, (const void*)chain_tc_kernel, args);
+    cudaLaunchKernelExC(&cfg, kernel_of(a.W), args);
 }
 
 }  // namespace fp

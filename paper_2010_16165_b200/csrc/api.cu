@@ -1652,7 +1652,7 @@ void launch_op(fp_handle h, int op_index, const void* d_input, int batch, float*
         fp::launch_maxpool(s.d, o.d, bf16, batch, s.H, s.W, s.C_pad, o.H, o.W, p.R, p.stride, p.pad, st);
     } else {
         const Tensor& s = h->tensors[h->head_src];
-        fp::launch_head(s.d, bf16, batch, s.H, s.W, s.C_pad, h->d_fcw_packed, h->d_fcb, h->n_classes, d_logits, h->d_pool, st);
+        fp::launch_head(s.d, bf16, batch, s.H, s.W, s.C_pad, h->d_fcw_packed, h->d_fcb, h->n_classes, d_logits, h->d_pool, h->max_batch, st);
     }
 }
 

@@ -168,7 +168,7 @@ void launch_input_to_stem_planar(const void* in, int in_is_bf16, void* out, int 
 void launch_maxpool(const void* x, void* y, int is_bf16, int N, int H, int W, int C_pad, int P, int Q, int R,
                     int stride, int pad, cudaStream_t st);
 void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, const float* fcw, const float* fcb,
-                 int n_classes, float* logits, float* pool_scratch, cudaStream_t st);
+                 int n_classes, float* logits, float* pool_scratch, int max_batch, cudaStream_t st);      // max_batch: of the handle
 void launch_planar_to_nchw_f32(const void* x, int is_bf16, float* out, int N, int H, int W, int C_pad, int C_out,
                                int split, cudaStream_t st);
 

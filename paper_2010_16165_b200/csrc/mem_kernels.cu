@@ -372,7 +372,7 @@ __global__ void pool_sum_kernel(const void* x, int N, int H, int W, int chunks, 
 // A block handles IMAGES images (one, four or eight: the sums of images that do not exist would be computed as well), whose channel sums it holds in shared memory, and 8 * CPW classes: a warp walks the FC
 // rows of its CPW classes with 16-byte loads, all images a time.  The first rows are asked for before the channel sums
 // exist (programmatic dependent launch).  Each (image, class) sum has a fixed order: lanes stride over the channels, then a
-// butterfly.  CPW: every sum read from shared memory serves CPW classes, which bounds large batches (128 images x 1000 classes
+// butterfly (the kernels for handles made for many images, below, have another).  CPW: every sum read from shared memory serves CPW classes, which bounds large batches (128 images x 1000 classes
 // x 2048 channels: 7 us of FMAs at full rate, four classes a warp bring the shared-memory reads down to that); one class a warp
 // spreads the FC matrix of a single image over 125 SMs instead of 32.
 constexpr int kFcWarps = 8, kFcSlab4 = 512, kFcPitch4 = kFcSlab4 + 1;       // channels / 4 held at a time, and a zero behind them
@@ -439,13 +439,15 @@ __global__ void __launch_bounds__(32 * kFcWarps, 2) fc_kernel(const float* sums,
     }
 }
 
-// Head, step 2, many images: a block takes 8 * IPL images times 32 classes.  Slabs of 128 channels of the sums and of the FC rows go through
-// shared memory (two on the way behind the one in use), a warp takes 16 channels of each, a lane IPL images times 8 classes of the tile: a
-// vector of 4 channels of an image serves 8 classes and one of a class IPL images, so that 12 shared-memory reads feed 64 pairs of
-// FMAs.  (In the kernel above every lane reads its own channels of every image, four wavefronts for 4 classes: both that and the L2
+// Head, step 2, of a handle made for many images: a block takes 8 * IPL images times 4 * CPL classes.  Slabs of 128 channels of the sums and of the FC rows go through
+// shared memory (two on the way behind the one in use), a warp takes 16 channels of each, a lane IPL images times CPL classes of the tile: a
+// vector of 4 channels of an image serves CPL classes and one of a class IPL images, so that (IPL 4, CPL 8) 12 shared-memory reads feed 64
+// pairs of FMAs.  (In the kernel above every lane reads its own channels of every image, four wavefronts for 4 classes: both that and the L2
 // reads of the FC matrix, once for every 8 images, took longer than the FMAs.)  Channels are added in pairs (one instruction
-// for two), each warp's in order, then the pair, then the warps' sums in order.
-constexpr int kTileClasses = 32, kTileSlab4 = 32, kTilePitch4 = kTileSlab4 + 1;      // (rows 16 bytes off a multiple of 128: no bank twice)
+// for two), each warp's in order, then the pair, then the warps' sums in order: another order than the kernel's above, the same for every
+// IPL and CPL.  Which of the two kernels a handle uses goes by the batch it is made for, so that an image's logits do not depend on the
+// call it came in.
+constexpr int kTileSlab4 = 32, kTilePitch4 = kTileSlab4 + 1;      // (rows 16 bytes off a multiple of 128: no bank twice)
 constexpr int kTileStages = 3;
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
@@ -453,12 +455,12 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
 __device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
-constexpr int fc_tile_smem(int ipl) { return kTileStages * (kTileClasses + 8 * ipl) * kTilePitch4 * (int)sizeof(float4); }
-template <int IPL>
+constexpr int fc_tile_smem(int ipl, int cpl) { return kTileStages * (4 * cpl + 8 * ipl) * kTilePitch4 * (int)sizeof(float4); }
+template <int IPL, int CPL>
 __global__ void __launch_bounds__(256, 2) fc_tile_kernel(const float* sums, int N, int C_pad, const float* __restrict__ fcw,
                                                          const float* __restrict__ fcb, int n_classes, float* __restrict__ logits) {
     extern __shared__ float4 sh4[];        // stages: FC rows, then the images' sums
-    constexpr int kRows = 256 / kTileSlab4, kImages = 8 * IPL, kStage4 = (kTileClasses + kImages) * kTilePitch4;
+    constexpr int kRows = 256 / kTileSlab4, kImages = 8 * IPL, kTileClasses = 4 * CPL, kStage4 = (kTileClasses + kImages) * kTilePitch4;
     const int n0 = blockIdx.x * kImages, k0 = (int)(blockIdx.z * gridDim.y + blockIdx.y) * kTileClasses, c4 = C_pad >> 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int slabs = (c4 + kTileSlab4 - 1) / kTileSlab4;
@@ -483,11 +485,11 @@ __global__ void __launch_bounds__(256, 2) fc_tile_kernel(const float* sums, int 
     commit();
     if (slabs > 1) fetch_rows(1, 1, true);
     commit();
-    unsigned long long acc[IPL][8];
+    unsigned long long acc[IPL][CPL];
 #pragma unroll
     for (int i = 0; i < IPL; ++i)
 #pragma unroll
-        for (int t = 0; t < 8; ++t) acc[i][t] = 0ull;
+        for (int t = 0; t < CPL; ++t) acc[i][t] = 0ull;
     const int li = lane & 7, lc = lane >> 3;      // image li + 8 i, class lc + 4 t
     uint32_t stage = 0;
     for (int slab = 0; slab < slabs; ++slab) {
@@ -507,7 +509,7 @@ __global__ void __launch_bounds__(256, 2) fc_tile_kernel(const float* sums, int 
 #pragma unroll
             for (int i = 0; i < IPL; ++i) sv[i] = s[8 * i * kTilePitch4 + c];
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
+            for (int t = 0; t < CPL; ++t) {
                 const ulonglong2 wv = w[4 * t * kTilePitch4 + c];
 #pragma unroll
                 for (int i = 0; i < IPL; ++i) {
@@ -523,7 +525,7 @@ __global__ void __launch_bounds__(256, 2) fc_tile_kernel(const float* sums, int 
 #pragma unroll
     for (int i = 0; i < IPL; ++i)
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
+        for (int t = 0; t < CPL; ++t) {
             const float2 v = *reinterpret_cast<const float2*>(&acc[i][t]);
             part[(warp * kImages + li + 8 * i) * (kTileClasses + 1) + lc + 4 * t] = v.x + v.y;
         }
@@ -535,6 +537,59 @@ __global__ void __launch_bounds__(256, 2) fc_tile_kernel(const float* sums, int 
         for (int k = 0; k < 8; ++k) v += part[(k * kImages + i) * (kTileClasses + 1) + t];
         if (n0 + i < N && k0 + t < n_classes) logits[(size_t)(n0 + i) * n_classes + k0 + t] = v + (fcb ? fcb[k0 + t] : 0.0f);
     }
+}
+
+// Head, step 2, of a call of up to four images on a handle made for many: the tiles' sums in the tiles' order, for one image a block and without the
+// tiles' passes through shared memory.  Eight lanes share a class; a lane does what a warp does there, 16 channels of every 128, and the eight
+// sums are added in order.  Half of 2048 channels of the FC rows are on the way before the channel sums exist.  What bounds it is that
+// latency: a forward of one image (ResNet-18 at 32x32 on a handle made for 24, 512 channels; ResNet-50 at 32x32 made for 64, 2048 channels) takes
+// 78.1 and 186.3 us, with tiles of 8 images times 8 classes 82.5 and 191.5, with the first of these kernels, whose order is another, 78.3 and
+// 182.9; four images 81.2 and 189.6, 84.0 and 191.1, 80.3 and 187.0.  At eight images the tiles are as fast (82.0, 190.5).
+constexpr int kFewImages = 4, kFewWarps = 2, kFewAhead = 8, kFewSlabs = 16;           // slabs of FC rows on the way, of sums held at a time
+__global__ void __launch_bounds__(32 * kFewWarps) fc_few_kernel(const float* sums, int N, int C_pad, const float* __restrict__ fcw,
+                                                               const float* __restrict__ fcb, int n_classes, float* __restrict__ logits) {
+    constexpr int kPitch4 = kTileSlab4 + kTileSlab4 / 4;   // of a slab: behind a lane's four vectors 16 bytes, so that eight lanes meet no bank twice
+    __shared__ float4 sh[kFewSlabs * kPitch4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = lane & 7, c4 = C_pad >> 2, slabs = (c4 + kTileSlab4 - 1) / kTileSlab4;
+    const int n = blockIdx.x, k = ((int)(blockIdx.z * gridDim.y + blockIdx.y) * kFewWarps + warp) * 4 + (lane >> 3);
+    const float4* row = reinterpret_cast<const float4*>(fcw + (size_t)min(k, n_classes - 1) * C_pad) + 4 * part;
+    float4 w[kFewAhead][4];
+    auto fetch = [&](int slab, int i) {    // zeros behind the last channel
+#pragma unroll
+        for (int c = 0; c < 4; ++c) w[i][c] = kTileSlab4 * slab + 4 * part + c < c4 ? __ldg(row + kTileSlab4 * slab + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    };
+#pragma unroll
+    for (int i = 0; i < kFewAhead; ++i) fetch(i, i);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    unsigned long long acc = 0ull;
+    for (int first = 0; first < slabs; first += kFewSlabs) {
+        const int n_slabs = min(kFewSlabs, slabs - first);
+        const float4* from = reinterpret_cast<const float4*>(sums + (size_t)n * C_pad) + first * kTileSlab4;
+        if (first) __syncthreads();        // the slabs before have been used
+#pragma unroll 8
+        for (int v = threadIdx.x; v < n_slabs * kTileSlab4; v += 32 * kFewWarps)
+            sh[v + (v >> 2)] = first * kTileSlab4 + v < c4 ? from[v] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        __syncthreads();
+        for (int slab = 0; slab < n_slabs; slab += kFewAhead) {      // (which divides kFewSlabs)
+#pragma unroll
+            for (int i = 0; i < kFewAhead; ++i) {
+                if (slab + i >= n_slabs) break;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const ulonglong2 wv = *reinterpret_cast<const ulonglong2*>(&w[i][c]);
+                    const ulonglong2 sv = *reinterpret_cast<const ulonglong2*>(&sh[(slab + i) * kPitch4 + 5 * part + c]);
+                    fma2(acc, sv.x, wv.x);
+                    fma2(acc, sv.y, wv.y);
+                }
+                fetch(first + slab + i + kFewAhead, i);
+            }
+        }
+    }
+    const float mine = __uint_as_float((uint32_t)acc) + __uint_as_float((uint32_t)(acc >> 32));
+    float v = 0.0f;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) v += __shfl_sync(0xffffffffu, mine, (lane & 24) + p);
+    if (part == 0 && k < n_classes) logits[(size_t)n * n_classes + k] = v + (fcb ? fcb[k] : 0.0f);
 }
 
 template <bool BF16>
@@ -601,7 +656,7 @@ void launch_maxpool(const void* x, void* y, int is_bf16, int N, int H, int W, in
 }
 
 void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, const float* fcw, const float* fcb,
-                 int n_classes, float* logits, float* pool_scratch, cudaStream_t st) {
+                 int n_classes, float* logits, float* pool_scratch, int max_batch, cudaStream_t st) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cudaLaunchAttribute attr[1];
@@ -616,28 +671,34 @@ void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, con
     cudaLaunchKernelEx(&cfg, is_bf16 ? pool_sum_kernel<true> : pool_sum_kernel<false>, x, N, H, W, chunks, pool_scratch);
     // classes per warp: one while that is what fills the GPU, four once there are blocks enough
     typedef void (*Fc)(const float*, int, int, const float*, const float*, int, float*);
-    // many images: tiles of 32, 16 or 8 images times 32 classes, the widest that gives most SMs one
-    const int tile_blocks = (n_classes + kTileClasses - 1) / kTileClasses;
-    int ipl = 4;
-    while (ipl > 1 && (N + 8 * ipl - 1) / (8 * ipl) * tile_blocks < sm_count() * 2 / 3) ipl >>= 1;
-    const bool tiled = N >= 16 && n_classes >= kTileClasses;
-    const int images = tiled ? 8 * ipl : N == 1 ? 1 : N <= 4 ? 4 : 8, groups = (N + images - 1) / images;
+    // A handle made for many images: tiles of 32, 16 or 8 images times 32 classes, or 8 times 8, the widest that gives most SMs one; a kernel
+    // of the same order of sums for a few images.  By the handle's batch, not the call's: an image's logits are the same bits in every call.
+    const bool tiled = max_batch >= 16 && n_classes >= 32;
+    int ipl = 4, cpl = 8;
+    auto tiles = [&] { return (N + 8 * ipl - 1) / (8 * ipl) * ((n_classes + 4 * cpl - 1) / (4 * cpl)); };
+    while (ipl > 1 && tiles() < sm_count() * 2 / 3) ipl >>= 1;
+    if (tiles() < sm_count() * 2 / 3) cpl = 2;
+    const bool few = tiled && N <= kFewImages;
+    const int images = few ? 1 : tiled ? 8 * ipl : N == 1 ? 1 : N <= 4 ? 4 : 8, groups = (N + images - 1) / images;
     const int cpw = images < 8 ? 1 : groups * ((n_classes + 31) / 32) >= 2 * sm_count() ? 4 : groups * ((n_classes + 15) / 16) >= sm_count() ? 2 : 1;
-    const Fc fn = tiled ? (ipl == 4 ? (Fc)fc_tile_kernel<4> : ipl == 2 ? (Fc)fc_tile_kernel<2> : (Fc)fc_tile_kernel<1>)
+    const Fc fn = few ? (Fc)fc_few_kernel
+                : tiled ? (ipl == 4 ? (Fc)fc_tile_kernel<4, 8> : ipl == 2 ? (Fc)fc_tile_kernel<2, 8> : cpl == 8 ? (Fc)fc_tile_kernel<1, 8> : (Fc)fc_tile_kernel<1, 2>)
                 : cpw == 4 ? (Fc)fc_kernel<8, 4, 2> : cpw == 2 ? (Fc)fc_kernel<8, 2, 4> : images == 8 ? (Fc)fc_kernel<8, 1, 8>
                 : images == 4 ? (Fc)fc_kernel<4, 1, 8> : (Fc)fc_kernel<1, 1, 16>;
     // (65535 blocks are the most along y; a matrix of more classes goes on along z)
-    const unsigned class_blocks = tiled ? (unsigned)tile_blocks : (unsigned)((n_classes + kFcWarps * cpw - 1) / (kFcWarps * cpw)), along_y = std::min(class_blocks, 65535u);
+    const int classes = few ? 4 * kFewWarps : tiled ? 4 * cpl : kFcWarps * cpw;      // of a block
+    const unsigned class_blocks = (unsigned)((n_classes + classes - 1) / classes), along_y = std::min(class_blocks, 65535u);
     cfg.gridDim = dim3((unsigned)groups, along_y, (class_blocks + along_y - 1) / along_y);
-    cfg.dynamicSmemBytes = tiled ? (size_t)fc_tile_smem(ipl) : (size_t)images * kFcPitch4 * sizeof(float4);
+    if (few) cfg.blockDim = dim3(32 * kFewWarps);
+    cfg.dynamicSmemBytes = few ? 0 : tiled ? (size_t)fc_tile_smem(ipl, cpl) : (size_t)images * kFcPitch4 * sizeof(float4);
     static std::atomic<bool> raised[64];   // per device, once (threads may all be the first)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !raised[dev]) {
         for (Fc f : {(Fc)fc_kernel<8, 1, 8>, (Fc)fc_kernel<8, 2, 4>, (Fc)fc_kernel<8, 4, 2>})
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * kFcPitch4 * sizeof(float4)));
-        cudaFuncSetAttribute(fc_tile_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(4));
-        cudaFuncSetAttribute(fc_tile_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(2));
-        cudaFuncSetAttribute(fc_tile_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(1));
+        cudaFuncSetAttribute(fc_tile_kernel<4, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(4, 8));
+        cudaFuncSetAttribute(fc_tile_kernel<2, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(2, 8));
+        cudaFuncSetAttribute(fc_tile_kernel<1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(1, 8));
         if (dev >= 0 && dev < 64) raised[dev] = true;
     }
     cudaLaunchKernelEx(&cfg, fn, (const float*)pool_scratch, N, C_pad, fcw, fcb, n_classes, logits);

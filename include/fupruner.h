@@ -231,7 +231,8 @@ typedef enum {
     FP_Q_OP_PLAN = 17,       /* int32[10]: the form of operator `index` where conv_tc_kernel computes it, zeros elsewhere: tiles of
                                 128 positions a step, channel chunks a K group, K groups, K groups of a projection taken in,
                                 stages of activations, of filters, filters that stay (1: as a whole, 2: a stage a block), epilogue
-                                warps, 1 where they are two teams that take every other tile, filters a tile (debug) */
+                                warps, 1 where they are two teams that take every other tile (in a call of the last
+                                batch), filters a tile (debug) */
     FP_Q_CONV_BANK_ELEMS = 15 /* int64: weights in the fused fp32 bank of conv `index` (K_fused*C_fused*R*S), 0 if absorbed */
 } fp_query_what;
 

@@ -1308,6 +1308,33 @@ int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len)
     return 0;
 }
 
+namespace {
+
+// (nobody reads behind the last image of a split tensor)
+long long positions_of(const ConvArgs& a) { return a.y_split ? (long long)a.N * image_vecs(a.P, a.Q) : used_vecs(a.N, a.P, a.Q); }
+
+int tiles_of(const ConvPlanTC& plan, const ConvArgs& a) {
+    const int tps = plan.tps > 0 ? plan.tps : 1;
+    const long long m_tiles = (positions_of(a) + 127) / 128;
+    return (int)(((m_tiles + tps - 1) / tps) * plan.n_tiles);
+}
+
+int grid_of(const ConvPlanTC& plan, int tiles) {
+    int grid = sm_count() * plan.ctas_per_sm;
+    if (grid > tiles) grid = tiles;
+    if (plan.b_resident && plan.n_tiles > 1 && grid > plan.n_tiles) grid -= grid % plan.n_tiles;   // a CTA's tiles share a filter tile
+    return grid < 1 ? 1 : grid;
+}
+
+}  // namespace
+
+// Where a call brings so few images that every CTA has one tile, all eight warps finish it: a second team would have none.  (us, two teams /
+// eight warps: ResNet-18 on a handle made for 64, 1 image 192.8 / 189.5, 8 199.0 / 196.4, 32 the same; ResNet-34 384.1 / 381.0, 397.2 / 395.0.)
+bool conv_tc_alternates(const ConvPlanTC& plan, const ConvArgs& a) {
+    const int tiles = tiles_of(plan, a);
+    return plan.alternate && tiles > grid_of(plan, tiles);
+}
+
 void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cudaStream_t st, int skip_round, long long wait_cycles) {
     if (plan.split > 0) { launch_conv_split(plan, a, d_status, st, skip_round, wait_cycles); return; }
     TcParams p;
@@ -1320,13 +1347,12 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.cchunks2 = a.x2_C_pad / 8;
     p.groups2 = a.x2_C_pad > 0 ? (p.cchunks2 + plan.cg - 1) / plan.cg : 0;
     p.plane_out = plane_vecs(a.N, a.P, a.Q);
-    p.m_total = used_vecs(a.N, a.P, a.Q);
+    p.m_total = positions_of(a);
     p.plane_y = p.plane_out;
     if (a.y_split) {
         p.y_split = 1; p.y_Wh2 = row_vecs((a.Q + 1) / 2); p.y_P2h = image_vecs((a.P + 1) / 2, (a.Q + 1) / 2);
         p.plane_y = plane_vecs(4 * a.N, (a.P + 1) / 2, (a.Q + 1) / 2);
         p.y_edges = (a.P & 1) || (a.Q & 1);
-        p.m_total = (long long)a.N * p.P2_out;       // (nobody reads behind the last image of a split tensor)
     }
     p.a_par = a.x_s2d ? 4 : 1;
     p.par_stride = (long long)a.N * p.P2_in;
@@ -1342,14 +1368,12 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.tap0 = plan.flat && !a.x_s2d ? plan.halo - (((a.R - 1) / 2) * p.Wp_in + (a.S - 1) / 2) : 0;
     p.halo = plan.halo; p.rows_a = plan.rows_a; p.a_stages = plan.a_stages; p.b_stages = plan.b_stages;
     p.n_tile = plan.n_tile; p.n_tiles = plan.n_tiles; p.tmem_cols = plan.tmem_cols;
-    const long long m_tiles = (p.m_total + 127) / 128;
     p.tps = plan.tps > 0 ? plan.tps : 1;
-    p.alternate = plan.alternate;
     p.b_kept = plan.b_kept && a.R * plan.groups + p.groups2 == plan.b_stages;      // (a projection's blocks come on top: then the stages are a ring)
     p.halves = p.tps > 2 ? 1 : 2;
     p.teams = p.tps < 4 / p.halves ? p.tps : 4 / p.halves;
     p.n_producers = plan.a_stages % 4 == 0 ? 4 : plan.a_stages % 3 == 0 ? 3 : plan.a_stages % 2 == 0 ? 2 : 1;
-    p.total_tiles = (int)(((m_tiles + p.tps - 1) / p.tps) * plan.n_tiles);
+    p.total_tiles = tiles_of(plan, a);
     p.m_first = a.reverse ? p.total_tiles / plan.n_tiles - 1 : 0;
     p.m_sign = a.reverse ? -1 : 1;
     const int gplanes = plan.groups > 1 ? plan.cg : plan.tpk * p.cchunks;      // gather: planes per stage
@@ -1366,10 +1390,8 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.div_ntiles = make_fastdiv((uint32_t)plan.n_tiles);
     p.div_p2out = make_fastdiv((uint32_t)p.P2_out);
     p.div_qp = make_fastdiv((uint32_t)p.Qp);
-    int grid = sm_count() * plan.ctas_per_sm;
-    if (grid > p.total_tiles) grid = p.total_tiles;
-    if (plan.b_resident && plan.n_tiles > 1 && grid > plan.n_tiles) grid -= grid % plan.n_tiles;   // a CTA's tiles share a filter tile
-    if (grid < 1) grid = 1;
+    const int grid = grid_of(plan, p.total_tiles);
+    p.alternate = conv_tc_alternates(plan, a);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)grid);

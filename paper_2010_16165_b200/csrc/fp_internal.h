@@ -195,7 +195,7 @@ struct ConvPlanTC {
     int tpk;              // gather: filter taps per K block (several when the channel count is small)
     int n_tile, n_tiles;  // filters per CTA tile (multiple of 16, <= 256)
     int epi_warps;        // 4, 8 for wide filter tiles, 16 where several tiles are complete together
-    int alternate;        // eight epilogue warps as two teams that take every other tile
+    int alternate;        // eight epilogue warps as two teams that take every other tile, in launches of more tiles than CTAs
     int tps;              // streamed filters: 128-position tiles per pipeline step
     int b_kept;           // streamed filters: a stage for every block of the bank, copied once
     int tmem_cols;
@@ -209,6 +209,7 @@ bool plan_conv_split(const ConvArgs& a, ConvPlanTC* plan);
 void launch_conv_split(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cudaStream_t st, int skip_round, long long wait_cycles);
 // Returns 0 on success, otherwise writes a message.
 int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len);
+bool conv_tc_alternates(const ConvPlanTC& plan, const ConvArgs& a);      // ConvPlanTC::alternate, in a launch with these arguments
 // skip_round / wait_cycles: diagnostic launch (see fp_debug_expire_wait): the activation producer of a stride-1 layer leaves
 // out one round of copies and every wait gives up after wait_cycles SM clock cycles; -1 / 0 for a normal launch
 void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cudaStream_t st, int skip_round = -1,

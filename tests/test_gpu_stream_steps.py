@@ -104,3 +104,40 @@ def test_forms(B, layers, widths, hw, batch, p, scatter, op, form, last, several
     finally:
         g.close()
         slow.close()
+
+
+@pytest.mark.parametrize("layers, widths, hw, batch, p, op, n_tile", [
+    ((2,), (64,), 120, 61, 0.0, 3, 64),        # two CTAs on an SM
+    ((2,), (64,), 120, 61, 0.3, 3, 48),        # a narrow tile: the halves have 32 and 16 columns
+    ((2,), (64,), 120, 61, 0.8, 3, 16),        # 16 columns: the second half has none
+    ((2,), (80,), 248, 33, 0.3, 4, 80),        # with a shortcut
+    ((1, 1), (48, 112), 112, 90, 0.0, 5, 112), # over parity images
+])
+def test_teams_by_tile_where_a_call_has_tiles_for_both(B, layers, widths, hw, batch, p, op, n_tile):
+    """Two teams of epilogue warps take every other tile of a CTA; a call whose CTAs have one tile each has both teams finish it."""
+    net = wl.resnet_imagenet_basic(layers, widths, in_hw=hw, n_classes=5, name="teams")
+    w = wl.Workload("teams", net, batch, 37, True, wl.uniform_ratios(p), "uniform")
+    g, slow = Gpu(B, w, B.FP_COMPUTE_BF16_TC), Gpu(B, w, B.FP_COMPUTE_BF16_SIMT, keep_outputs=1)
+    try:
+        for x in (g, slow):
+            B.fp_prune(x.h, w.ratios)
+        full = g.forward(w.x)
+        plan = B.fp_query_plan(g.h, op)
+        assert (plan["stays"], plan["epi_warps"], plan["alternate"], plan["n_tile"]) == (1, 8, 1, n_tile)
+        o = B.op_infos(g.h)[op]
+        few = 128 * 148 // ((o.P + 1) * (o.Q + 1)) // 2                # half as many tiles as SMs
+        for n in (1, few, few + 1, batch - 1):
+            got = g.forward(w.x[:n])
+            assert B.fp_query_plan(g.h, op)["alternate"] == (n == batch - 1)
+            np.testing.assert_array_equal(got, full[:n])
+        for x in (g, slow):
+            x.forward(w.x[:few])
+        wf = wl.Workload("teams", net, few, 37, True, wl.uniform_ratios(p), "uniform")
+        got, want = outputs(B, g, wf), outputs(B, slow, wf)
+        assert got[op] is not None and got[op].shape == want[op].shape
+        for i, v in got.items():
+            if v is not None and want.get(i) is not None and v.shape == want[i].shape:
+                assert close(v, want[i]), i
+    finally:
+        g.close()
+        slow.close()

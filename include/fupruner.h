@@ -229,7 +229,7 @@ typedef enum {
                                 convolutions in one call - int32[N_CONVS] filters per convolution (0 if absorbed),
                                 int32[n] ranks, uint8[n] masks, in description order                   */
     FP_Q_OP_PLAN = 17,       /* int32[10]: the form of operator `index` where conv_tc_kernel computes it, zeros elsewhere: tiles of
-                                128 positions a step, channel chunks a K group, K groups, K groups of a projection taken in,
+                                128 positions a step (in a call of the last batch), channel chunks a K group, K groups, K groups of a projection taken in,
                                 stages of activations, of filters, filters that stay (1: as a whole, 2: a stage a block), epilogue
                                 warps, 1 where they are two teams that take every other tile (in a call of the last
                                 batch), filters a tile (debug) */

@@ -2185,7 +2185,7 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             const bool stays = c.tc.b_kept && c.R * c.tc.groups + groups2 == c.tc.b_stages;
             fp::ConvArgs args = c.args;
             args.N = (h->last_batch > 0 ? h->last_batch : h->max_batch) * c.n_mult;
-            const int32_t plan[10] = {c.tc.tps, c.tc.cg, c.tc.groups, groups2, c.tc.a_stages, c.tc.b_stages, c.tc.b_resident ? 1 : stays ? 2 : 0,
+            const int32_t plan[10] = {fp::conv_tc_step_tiles(c.tc, args), c.tc.cg, c.tc.groups, groups2, c.tc.a_stages, c.tc.b_stages, c.tc.b_resident ? 1 : stays ? 2 : 0,
                                       c.tc.epi_warps, fp::conv_tc_alternates(c.tc, args), c.tc.n_tile};
             memcpy(o, plan, sizeof(plan));
             return FP_OK;

@@ -1313,11 +1313,9 @@ namespace {
 // (nobody reads behind the last image of a split tensor)
 long long positions_of(const ConvArgs& a) { return a.y_split ? (long long)a.N * image_vecs(a.P, a.Q) : used_vecs(a.N, a.P, a.Q); }
 
-int tiles_of(const ConvPlanTC& plan, const ConvArgs& a) {
-    const int tps = plan.tps > 0 ? plan.tps : 1;
-    const long long m_tiles = (positions_of(a) + 127) / 128;
-    return (int)(((m_tiles + tps - 1) / tps) * plan.n_tiles);
-}
+long long steps_with(const ConvPlanTC& plan, const ConvArgs& a, int tps) { return ((positions_of(a) + 127) / 128 + tps - 1) / tps * plan.n_tiles; }
+
+int tiles_of(const ConvPlanTC& plan, const ConvArgs& a) { return (int)steps_with(plan, a, conv_tc_step_tiles(plan, a)); }
 
 int grid_of(const ConvPlanTC& plan, int tiles) {
     int grid = sm_count() * plan.ctas_per_sm;
@@ -1327,6 +1325,14 @@ int grid_of(const ConvPlanTC& plan, int tiles) {
 }
 
 }  // namespace
+
+// Three tiles a step are taken where that is one round over the SMs and two are not (plan_conv_tc).  A call of fewer images than the handle is
+// made for goes in steps of two where those are one round, as it would on a smaller handle: fewer tiles in a row, over more SMs.  (Stages and
+// sums of two tiles fit where three do, the K groups stay, so the sums are the same bits.  us, three / two: ResNet-18 on a handle made for 200, 1 image 259.4 / 227.8, 32 314.1 / 279.8, 100
+// 474.7 / 442.4; ResNet-34 made for 64, 8 images 396.8 / 371.0, 32 446.8 / 426.0.)
+int conv_tc_step_tiles(const ConvPlanTC& plan, const ConvArgs& a) {
+    return plan.tps == 3 && steps_with(plan, a, 2) <= sm_count() ? 2 : plan.tps > 0 ? plan.tps : 1;
+}
 
 // Where a call brings so few images that every CTA has one tile, all eight warps finish it: a second team would have none.  (us, two teams /
 // eight warps: ResNet-18 on a handle made for 64, 1 image 192.8 / 189.5, 8 199.0 / 196.4, 32 the same; ResNet-34 384.1 / 381.0, 397.2 / 395.0.)
@@ -1366,9 +1372,10 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     }
     p.taps = a.R * a.S; p.cchunks = a.C_pad / 8; p.cg = plan.cg; p.groups = plan.groups;
     p.tap0 = plan.flat && !a.x_s2d ? plan.halo - (((a.R - 1) / 2) * p.Wp_in + (a.S - 1) / 2) : 0;
-    p.halo = plan.halo; p.rows_a = plan.rows_a; p.a_stages = plan.a_stages; p.b_stages = plan.b_stages;
+    p.halo = plan.halo; p.a_stages = plan.a_stages; p.b_stages = plan.b_stages;
     p.n_tile = plan.n_tile; p.n_tiles = plan.n_tiles; p.tmem_cols = plan.tmem_cols;
-    p.tps = plan.tps > 0 ? plan.tps : 1;
+    p.tps = conv_tc_step_tiles(plan, a);
+    p.rows_a = plan.rows_a - (plan.tps > 0 ? plan.tps - p.tps : 0) * 128;
     p.b_kept = plan.b_kept && a.R * plan.groups + p.groups2 == plan.b_stages;      // (a projection's blocks come on top: then the stages are a ring)
     p.halves = p.tps > 2 ? 1 : 2;
     p.teams = p.tps < 4 / p.halves ? p.tps : 4 / p.halves;
@@ -1377,7 +1384,7 @@ void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cu
     p.m_first = a.reverse ? p.total_tiles / plan.n_tiles - 1 : 0;
     p.m_sign = a.reverse ? -1 : 1;
     const int gplanes = plan.groups > 1 ? plan.cg : plan.tpk * p.cchunks;      // gather: planes per stage
-    p.a_stage_bytes = plan.flat ? plan.cg * p.a_par * plan.rows_a * 16 : gplanes * 128 * 16;
+    p.a_stage_bytes = plan.flat ? plan.cg * p.a_par * p.rows_a * 16 : gplanes * 128 * 16;
     p.b_stage_bytes = plan.blocked_bank == 1 ? p.taps * plan.cg * plan.n_tile * 16 : plan.flat ? a.S * plan.cg * plan.n_tile * 16 : gplanes * plan.n_tile * 16;
     p.bank_tile_bytes = (long long)p.taps * p.cchunks * plan.n_tile * 16;
     p.tpk = plan.tpk > 0 ? plan.tpk : 1;

@@ -209,7 +209,9 @@ bool plan_conv_split(const ConvArgs& a, ConvPlanTC* plan);
 void launch_conv_split(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cudaStream_t st, int skip_round, long long wait_cycles);
 // Returns 0 on success, otherwise writes a message.
 int plan_conv_tc(const ConvArgs& a, ConvPlanTC* plan, char* err, size_t err_len);
-bool conv_tc_alternates(const ConvPlanTC& plan, const ConvArgs& a);      // ConvPlanTC::alternate, in a launch with these arguments
+// ConvPlanTC::tps and ::alternate, in a launch with these arguments
+int conv_tc_step_tiles(const ConvPlanTC& plan, const ConvArgs& a);
+bool conv_tc_alternates(const ConvPlanTC& plan, const ConvArgs& a);
 // skip_round / wait_cycles: diagnostic launch (see fp_debug_expire_wait): the activation producer of a stride-1 layer leaves
 // out one round of copies and every wait gives up after wait_cycles SM clock cycles; -1 / 0 for a normal launch
 void launch_conv_tc(const ConvPlanTC& plan, const ConvArgs& a, int* d_status, cudaStream_t st, int skip_round = -1,

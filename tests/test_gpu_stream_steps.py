@@ -141,3 +141,39 @@ def test_teams_by_tile_where_a_call_has_tiles_for_both(B, layers, widths, hw, ba
     finally:
         g.close()
         slow.close()
+
+
+@pytest.mark.parametrize("layers, widths, hw, batch, p, op, few, epi_warps", [
+    ((1,), (112,), 112, 64, 0.0, 3, 40, 16),
+    ((1, 1), (48, 112), 112, 200, 0.0, 7, 100, 16),      # a projection's K group behind the layer's own
+    ((1,), (48,), 264, 9, 0.0, 3, 8, 16),                # filters that stay
+    ((1,), (512,), 28, 200, 0.3, 3, 100, 16),            # 7 x 7 pixels, three filter tiles
+    ((1,), (512,), 28, 200, 0.3, 4, 100, 8),             # ... with a scattered output
+])
+def test_steps_of_two_tiles_in_a_smaller_call_than_steps_of_three_are_for(B, layers, widths, hw, batch, p, op, few, epi_warps):
+    net = wl.resnet_imagenet_basic(layers, widths, in_hw=hw, n_classes=5, name="fewer")
+    w = wl.Workload("fewer", net, batch, 47, True, wl.uniform_ratios(p), "uniform")
+    g, slow = Gpu(B, w, B.FP_COMPUTE_BF16_TC), Gpu(B, w, B.FP_COMPUTE_BF16_SIMT, keep_outputs=1)
+    try:
+        for x in (g, slow):
+            B.fp_prune(x.h, w.ratios)
+        full = g.forward(w.x)
+        plan = B.fp_query_plan(g.h, op)
+        assert (plan["tps"], plan["epi_warps"]) == (3, epi_warps)
+        o, sms = B.op_infos(g.h)[op], torch.cuda.get_device_properties(0).multi_processor_count
+        assert steps_of(o, dict(plan, tps=2), few) <= sms
+        for n in (1, 2, few, few + 1, batch - 1):
+            got = g.forward(w.x[:n])
+            assert B.fp_query_plan(g.h, op)["tps"] == (2 if steps_of(o, dict(plan, tps=2), n) <= sms else 3)
+            np.testing.assert_array_equal(got, full[:n])
+        for x in (g, slow):
+            x.forward(w.x[:few])
+        wf = wl.Workload("fewer", net, few, 47, True, wl.uniform_ratios(p), "uniform")
+        got, want = outputs(B, g, wf), outputs(B, slow, wf)
+        assert got[op] is not None and got[op].shape == want[op].shape
+        for i, v in got.items():
+            if v is not None and want.get(i) is not None and v.shape == want[i].shape:
+                assert close(v, want[i]), i
+    finally:
+        g.close()
+        slow.close()

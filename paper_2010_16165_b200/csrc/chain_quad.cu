@@ -5,8 +5,8 @@
 //   accumulator columns and 32 shuffles for 16 values, a chain of some 2400 cycles per 128 pixels, four of which are in flight: 520
 //   cycles a tile of 128 pixels, against 130 of its MMAs.  Here the tensor pipe does the adding and the epilogue is the shorter half.
 //   GEMM view     A row is a block of 2 x 2 pixels, N = 4 pixels x 16 filters, K = the 4 x 4 pixels the block's windows cover x 16 channels:
-//                 16 MMAs of M 128, N 64, K 16 for 512 pixels.  7 of the 16 x 4 (pixel, output) places are outside the window and hold
-//                 zero filters; an MMA of N = 64 costs the pipe little more than one of N = 16 (48 cycles against 39, the fetch of
+//                 16 MMAs of M 128, N 64, K 16 for 512 pixels.  28 of the 16 x 4 (pixel, output) places are outside the output's window
+//                 (7 of its 16 pixels each) and hold zero filters; an MMA of N = 64 costs the pipe little more than one of N = 16 (48 cycles against 39, the fetch of
 //                 the 128 x 16 operand), so that is 192 cycles per 128 pixels where nine MMAs of N = 16 take 350.
 //   Layout        planar-8 per parity: plane (row parity, column parity, chunk) holds the blocks' pixels of that parity at
 //                 img * (H/2 + 1)(W/2 + 1) + (i + 1)(W/2 + 1) + (j + 1), zeros above and to the left of an image and behind the last.
@@ -25,6 +25,7 @@
 //   Measured      ResNet-110's 37 layers of 1024 images 695 -> 400 us, of 148 images 105 -> 88 us (a layer of one image's three tiles is
 //                 4500 cycles, of two images' five 5100: the chain of MMAs, commit and epilogue behind a tile's neighbours).
 //   Waits         bounded as in conv_tc.cu.
+#include "chain_quad_layout.h"
 #include "fp_internal.h"
 #include "tc_common.cuh"
 
@@ -37,21 +38,11 @@ namespace {
 
 using namespace tc;
 
-constexpr int kN = 64, kStages = 8, kIssuers = 4, kGroups = 4, kWindow = 16;
+constexpr int kN = 64, kStages = kQuadStages, kIssuers = 4, kGroups = 4, kWindow = 16;
 constexpr int kFilterBytes = kQuadFilterBytes, kBlobBytes = kQuadBlobBytes;
 constexpr int kIssuer0 = 4 * kGroups, kThreads = 32 * (kIssuer0 + kIssuers);
 constexpr int kHandOver = 6;                             // the MMA behind which the next warp may begin: it needs some 400 cycles to get there
-constexpr int kMaxTiles = 8;
-constexpr unsigned kSmemMax = 232448u - 2048u;           // (the layer table is static)
-
-struct QuadCtrl {
-    uint64_t w_full[2], w_empty[2], sum_full[kStages], sum_empty[kStages], tile_done[2][kMaxTiles], group_sync;
-    uint32_t tmem_base;
-    int abort_flag;
-    uint32_t next_tile;                                  // whose MMAs are issued next
-    int pad_[3];
-};
-static_assert(sizeof(QuadCtrl) % 16 == 0, "buffers behind the control block must stay 16-byte aligned");
+constexpr int kMaxTiles = kQuadMaxTiles;
 
 struct QuadParams {
     ChainArgs a;
@@ -166,11 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_quad_kernel(const __grid_co
                     const uint32_t d = tmem + stage * (uint32_t)kN, at = a0 + (uint32_t)(t * 128);
 #pragma unroll
                     for (int w = 0; w < kWindow; ++w) {
-                        const int iy = w >> 2, ix = w & 3;
-                        // the plane of the window pixel's parity, from the block row and column it lies in
-                        const uint32_t plane = (uint32_t)((((iy + 1) & 1) * 2 + ((ix + 1) & 1)) * 2) * rows;
-                        const uint32_t row = (iy == 0 ? 0u - pitch : iy == 3 ? pitch : 0u) + (ix == 0 ? 0u - 1u : ix == 3 ? 1u : 0u);
-                        umma_bf16_lo_if(leader, d, at + plane + row, b0 + (uint32_t)(w * 2 * kN), idesc, w ? 1u : 0u);
+                        umma_bf16_lo_if(leader, d, at + quad_window_plane(w, rows) + quad_window_row(w, pitch), b0 + (uint32_t)(w * 2 * kN), idesc, w ? 1u : 0u);
                         if (w == kHandOver && leader) *next_tile = q + 1;
                     }
                     if (leader) umma_commit(sum_full0 + 8 * stage);
@@ -347,25 +334,16 @@ __global__ void __launch_bounds__(kThreads, 1) chain_quad_kernel(const __grid_co
     }
 }
 
-// blocks of G images with their borders, and the zeros behind the last
-int plane_rows(int G, int H, int W) { return (G * (H / 2 + 1) * (W / 2 + 1) + W / 2 + 2 + 7) / 8 * 8; }
-// Two buffers of eight planes, and behind them what the last tile's operands read past the last plane: its rows up to a multiple of 128, and
-// a row and a block below them.  (The rows before the first plane lie in the filters.)
-unsigned smem_for(int G, int H, int W) {
-    const unsigned rows = (unsigned)plane_rows(G, H, W), read = (rows + 127) / 128 * 128 + (unsigned)(W / 2 + 1) + 1;
-    return (unsigned)sizeof(QuadCtrl) + 128u + 2u * kBlobBytes + (15u * rows + read) * 16u;
-}
-
 }  // namespace
 
 // Runs whose layers have 16 filters and channels (padded), on images 32 pixels wide and of even height.  (The first layer may not add a
 // tensor: the run's second buffer is not loaded.)  There it was the shorter form at every batch: 37 layers, us of chain_tc.cu -> of
 // this one, 32 images 103 -> 86, 149 174 -> 103, 444 234 -> 201, 592 343 -> 201, 1024 695 -> 400.
 bool chain_quad_supported(const ChainArgs& a) {
-    if (a.W != 32 || a.H % 2 || a.H < 2 || a.res_mode || a.in_C > 16) return false;
+    if (a.W != 32 || a.H % 2 || a.H < 2 || a.res_mode) return false;
     for (int l = 0; l < a.n_layers; ++l)
         if (a.layers[l].K_pad != 16 || a.layers[l].cchunks != 2) return false;
-    return smem_for(1, a.H, a.W) <= kSmemMax;
+    return quad_smem(1, a.H, a.W) <= kQuadSmemMax;
 }
 
 // A layer of one image's 3 tiles takes 2.38 us, of two images' 5 2.75 us: two images a CTA wherever that saves a round.
@@ -376,20 +354,20 @@ int plan_chain_quad(const ChainArgs& a, ChainPlan* plan, char* err, size_t err_l
     int best = 0;
     double best_cost = 0;
     for (int G = 1; G <= a.N; ++G) {
-        const int tiles = (plane_rows(G, a.H, a.W) + 127) / 128;
-        if (smem_for(G, a.H, a.W) > kSmemMax || tiles > kMaxTiles) break;
+        const int tiles = quad_tiles(quad_plane_rows(G, a.H, a.W));
+        if (quad_smem(G, a.H, a.W) > kQuadSmemMax || tiles > kMaxTiles) break;
         const int groups = (a.N + G - 1) / G;
         const double cost = ((groups + sm_count() - 1) / sm_count()) * chain_quad_layer_us(tiles);
         if (!best || cost <= best_cost) { best = G; best_cost = cost; }
     }
-    if (!best || cudaFuncSetAttribute(chain_quad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) {
+    if (!best || cudaFuncSetAttribute(chain_quad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQuadSmemMax) != cudaSuccess) {
         cudaGetLastError();
         snprintf(err, err_len, "one image does not fit shared memory");
         return 1;
     }
-    plan->quad = 1; plan->G = best; plan->plane_rows = plane_rows(best, a.H, a.W);
-    plan->tiles = (plan->plane_rows + 127) / 128;
-    plan->smem_bytes = smem_for(best, a.H, a.W);
+    plan->quad = 1; plan->G = best; plan->plane_rows = quad_plane_rows(best, a.H, a.W);
+    plan->tiles = quad_tiles(plan->plane_rows);
+    plan->smem_bytes = quad_smem(best, a.H, a.W);
     if (plan->smem_bytes < 120u * 1024u) plan->smem_bytes = 120u * 1024u;      // one CTA per SM: tensor memory is never contended
     plan->valid = 1;
     return 0;
@@ -401,7 +379,7 @@ void launch_chain_quad(const ChainPlan& plan, const ChainArgs& a, int* d_status,
     p.a = a;
     p.G = plan.G; p.tiles = plan.tiles; p.rows = plan.plane_rows;
     p.n_groups = (a.N + plan.G - 1) / plan.G;
-    p.pitch = a.W / 2 + 1; p.image = (a.H / 2 + 1) * p.pitch;
+    p.pitch = quad_pitch(a.W); p.image = (a.H / 2 + 1) * p.pitch;
     p.div_image = make_fastdiv((uint32_t)p.image); p.div_pitch = make_fastdiv((uint32_t)p.pitch);
     p.Wp = row_vecs(a.W); p.P2 = image_vecs(a.H, a.W);
     p.plane_in = p.plane_out = plane_vecs(a.N, a.H, a.W);

@@ -671,18 +671,26 @@ void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, con
     cudaLaunchKernelEx(&cfg, is_bf16 ? pool_sum_kernel<true> : pool_sum_kernel<false>, x, N, H, W, chunks, pool_scratch);
     // classes per warp: one while that is what fills the GPU, four once there are blocks enough
     typedef void (*Fc)(const float*, int, int, const float*, const float*, int, float*);
-    // A handle made for many images: tiles of 32, 16 or 8 images times 32 classes, or 8 times 8, the widest that gives most SMs one; a kernel
-    // of the same order of sums for a few images.  By the handle's batch, not the call's: an image's logits are the same bits in every call.
+    // A handle made for many images: tiles, and a kernel of the same order of sums for a few images.  By the handle's batch, not the call's: an
+    // image's logits are the same bits in every call.
     const bool tiled = max_batch >= 16 && n_classes >= 32;
-    int ipl = 4, cpl = 8;
-    auto tiles = [&] { return (N + 8 * ipl - 1) / (8 * ipl) * ((n_classes + 4 * cpl - 1) / (4 * cpl)); };
-    while (ipl > 1 && tiles() < sm_count() * 2 / 3) ipl >>= 1;
-    if (tiles() < sm_count() * 2 / 3) cpl = 2;
+    // The widest tile of which there are enough: a wide one reads least, but its block works longest, and the last blocks' time is the
+    // kernel's.  (Forward of ResNet-50 at 32x32 with 1000 classes, us, tiles of 8 x 8, 8 x 16, 16 x 16, 16 x 32, 32 x 32 images x classes, in brackets
+    // the kernel above: 16 images 187.1, 190.3, 188.7, 192.4, 201.3 (187.7); 32 207.0, 204.2, 208.4, 215.2, 230.1 (202.2); 48 221.8, 218.5, 217.8, 224.4,
+    // 240.2 (219.1); 64 241.1, 238.3, 233.2, 231.2, 254.5 (235.5); 100 275.7, 270.5, 264.2, 263.5, 280.8 (265.4); 128 316.5, 306.9, 299.6, 293.7, 308.0
+    // (296.8); 200 379.1, 361.8, 348.2, 340.7, 346.1 (345.3); 256 425.9, 405.0, 384.7, 378.5, 373.3 (385.2).)
+    static const struct { int ipl, cpl; float blocks_per_sm; } kTiles[] = {{4, 8, 1.7f}, {2, 8, 0.85f}, {2, 4, 1.2f}, {1, 4, 1.2f}, {1, 2, 0.0f}};
+    int ipl = 0, cpl = 0;
+    for (const auto& t : kTiles) {
+        ipl = t.ipl; cpl = t.cpl;
+        if ((N + 8 * ipl - 1) / (8 * ipl) * (float)((n_classes + 4 * cpl - 1) / (4 * cpl)) >= t.blocks_per_sm * sm_count()) break;
+    }
     const bool few = tiled && N <= kFewImages;
     const int images = few ? 1 : tiled ? 8 * ipl : N == 1 ? 1 : N <= 4 ? 4 : 8, groups = (N + images - 1) / images;
     const int cpw = images < 8 ? 1 : groups * ((n_classes + 31) / 32) >= 2 * sm_count() ? 4 : groups * ((n_classes + 15) / 16) >= sm_count() ? 2 : 1;
     const Fc fn = few ? (Fc)fc_few_kernel
-                : tiled ? (ipl == 4 ? (Fc)fc_tile_kernel<4, 8> : ipl == 2 ? (Fc)fc_tile_kernel<2, 8> : cpl == 8 ? (Fc)fc_tile_kernel<1, 8> : (Fc)fc_tile_kernel<1, 2>)
+                : tiled ? (ipl == 4 ? (Fc)fc_tile_kernel<4, 8> : ipl == 2 ? (cpl == 8 ? (Fc)fc_tile_kernel<2, 8> : (Fc)fc_tile_kernel<2, 4>)
+                                  : cpl == 4 ? (Fc)fc_tile_kernel<1, 4> : (Fc)fc_tile_kernel<1, 2>)
                 : cpw == 4 ? (Fc)fc_kernel<8, 4, 2> : cpw == 2 ? (Fc)fc_kernel<8, 2, 4> : images == 8 ? (Fc)fc_kernel<8, 1, 8>
                 : images == 4 ? (Fc)fc_kernel<4, 1, 8> : (Fc)fc_kernel<1, 1, 16>;
     // (65535 blocks are the most along y; a matrix of more classes goes on along z)
@@ -698,7 +706,7 @@ void launch_head(const void* x, int is_bf16, int N, int H, int W, int C_pad, con
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * kFcPitch4 * sizeof(float4)));
         cudaFuncSetAttribute(fc_tile_kernel<4, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(4, 8));
         cudaFuncSetAttribute(fc_tile_kernel<2, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(2, 8));
-        cudaFuncSetAttribute(fc_tile_kernel<1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(1, 8));
+        cudaFuncSetAttribute(fc_tile_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, fc_tile_smem(2, 4));
         if (dev >= 0 && dev < 64) raised[dev] = true;
     }
     cudaLaunchKernelEx(&cfg, fn, (const float*)pool_scratch, N, C_pad, fcw, fcb, n_classes, logits);

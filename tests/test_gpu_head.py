@@ -1,5 +1,5 @@
 """GPU parity of the average pooling and FC layer: batches at the edges of the image groups (1, 4, 8), classes per warp (1, 2,
-4), tiles of 8, 16 and 32 images times 32 classes and of 8 times 8, channels around the 2048 and the 128 held at a time, image sizes below and above a warp of positions."""
+4), tiles of 8 to 32 images times 8 to 32 classes, channels around the 2048 and the 128 held at a time, image sizes below and above a warp of positions."""
 import numpy as np
 import pytest
 
@@ -31,7 +31,8 @@ def one_layer(batch, hw, channels, classes):
 @pytest.mark.parametrize("batch, hw, channels, classes", [
     (1, 7, 2048, 1000), (1, 4, 2064, 11), (2, 9, 72, 1003), (4, 3, 4112, 9), (5, 7, 512, 1000), (8, 2, 24, 1),
     (9, 7, 2032, 130), (24, 5, 136, 1000), (83, 3, 520, 1000), (97, 3, 2080, 801),
-    (16, 2, 1024, 32), (33, 2, 272, 70), (64, 2, 16, 1000), (129, 2, 784, 1001),      # tiles of 8 images and 8 classes, of 16 and of 32 images
+    (16, 2, 1024, 32), (33, 2, 272, 70), (64, 2, 16, 1000), (129, 2, 784, 1001),      # tiles of 8 images x 8 classes, of 16 x 32
+    (31, 2, 144, 1000), (48, 2, 272, 1003), (257, 2, 144, 1000),                      # of 8 x 16, 16 x 16 and 32 x 32
 ])
 @pytest.mark.parametrize("compute", ["fp32", "tc"])
 def test_head_matches_oracle(B, fpo, batch, hw, channels, classes, compute):
@@ -44,7 +45,7 @@ def test_head_matches_oracle(B, fpo, batch, hw, channels, classes, compute):
         g.close()
 
 
-@pytest.mark.parametrize("made, hw, channels, classes", [(40, 3, 272, 1000), (300, 2, 144, 70), (16, 4, 2048, 33), (15, 4, 2048, 1000), (64, 2, 528, 31), (20, 2, 2080, 100), (33, 2, 1040, 45), (16, 3, 16, 540_001)])
+@pytest.mark.parametrize("made, hw, channels, classes", [(40, 3, 272, 1000), (300, 2, 144, 70), (16, 4, 2048, 33), (15, 4, 2048, 1000), (64, 2, 528, 31), (20, 2, 2080, 100), (33, 2, 1040, 45), (16, 3, 16, 540_001), (270, 2, 272, 1000)])
 @pytest.mark.parametrize("compute", ["fp32", "tc"])
 def test_logits_do_not_depend_on_the_batch_of_the_call(B, made, hw, channels, classes, compute):
     """One handle, calls on both sides of 16 images and of the tiles' widths: an image's logits are the same bits in each."""
@@ -52,7 +53,7 @@ def test_logits_do_not_depend_on_the_batch_of_the_call(B, made, hw, channels, cl
     g = Gpu(B, w, B.FP_COMPUTE_FP32 if compute == "fp32" else B.FP_COMPUTE_BF16_TC)
     try:
         full = g.forward(w.x)
-        for n in sorted({n for n in (1, 2, 4, 5, 8, 9, 15, 16, 17, 24, 33, 129, made - 1) if n < made}):
+        for n in sorted({n for n in (1, 2, 4, 5, 8, 9, 15, 16, 17, 24, 33, 48, 129, made - 1) if n < made}):
             np.testing.assert_array_equal(g.forward(w.x[:n]), full[:n], err_msg=str(n))
     finally:
         g.close()

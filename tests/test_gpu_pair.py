@@ -42,7 +42,7 @@ def test_layers_that_run_as_pairs(B, layers, widths, hw, batch, ratios, pairs):
         for x in (g, kept):
             B.fp_prune(x.h, w.ratios)
         logits = g.forward(w.x)
-        kept.forward(w.x)
+        assert close(logits, kept.forward(w.x))                          # (of what a forward stores; the outputs below are stored whole)
         infos = B.op_infos(g.h)
         assert sum(o.kind == 0 and B.CONV_KERNELS[o.kernel] == "conv_pair_kernel" for o in infos) >= 2 * pairs
         got, want = outputs(B, g, w), outputs(B, kept, w)
@@ -66,3 +66,33 @@ def test_a_smaller_batch_than_the_handle_is_made_for(B):
             np.testing.assert_array_equal(g.forward(w.x[:n]), logits[:n])
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("width, blocks, hw, batch", [
+    (16, 2, 24, 40),       # one group of 64 channels
+    (20, 2, 23, 41),       # groups of 64 and 16
+    (48, 3, 17, 70),       # three groups, filters that stay
+    (96, 2, 14, 131),      # six groups, filters with every tile
+])
+def test_a_pair_computes_what_its_two_layers_do(B, width, blocks, hw, batch):
+    """Blocks without projections, so that both handles give the pair the same inputs: every operator's output is the same bits as
+    that of a launch of its own."""
+    net = wl.Net(3, hw, hw, "pairs_alone")
+    x = net.relu(net.bn(net.conv(-1, 4 * width, 3, 1, 1, 0), 4 * width))
+    for b in range(blocks):
+        x = wl._bottleneck(net, x, 4 * width, width, 1, False, b)
+    net.fc(net.gavgpool(x, 4 * width), 5, 4 * width)
+    net.n_blocks = blocks
+    w = wl.Workload("pairs_alone", net, batch, 59, True, wl.uniform_ratios(0.0), "none")
+    g, kept = Gpu(B, w, B.FP_COMPUTE_BF16_TC), Gpu(B, w, B.FP_COMPUTE_BF16_TC, keep_outputs=1)
+    try:
+        infos = B.op_infos(g.h)
+        assert sum(o.kind == 0 and B.CONV_KERNELS[o.kernel] == "conv_pair_kernel" for o in infos) == 2 * (blocks - 1)
+        np.testing.assert_array_equal(g.forward(w.x), kept.forward(w.x))
+        got, want = outputs(B, g, w), outputs(B, kept, w)
+        for i, o in enumerate(infos):
+            if o.kind == 0:
+                np.testing.assert_array_equal(got[i], want[i], err_msg=str(i))
+    finally:
+        g.close()
+        kept.close()

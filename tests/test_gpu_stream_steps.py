@@ -22,16 +22,17 @@ def B():
     return binding
 
 
+# (Which forms these sizes have is said here as of today and not asserted; test_forms and what is behind it do.)
 @pytest.mark.parametrize("layers, widths, hw, batch, p", [
     ((2,), (96,), 112, 64, 0.0),            # 421 tiles: one step of three a CTA
-    ((2,), (96,), 112, 23, 0.0),            # a tile or two a step
-    ((2,), (160,), 100, 57, 0.1),           # two filter tiles or three tiles of 144 filters
-    ((1, 1), (64, 112), 120, 70, 0.0),      # a projection's blocks behind the layer's own
-    ((2,), (48,), 232, 9, 0.0),             # 58 pixels wide: steps share the halo, the filters stay
-    ((2,), (80,), 248, 33, 0.3),            # 62 pixels wide, several steps a CTA, the last one partial
-    ((1,), (256,), 72, 47, 0.0),            # filters that take longer than the MMAs of a tile
-    ((2,), (64,), 120, 25, 0.0),            # filters that stay as a whole, one or two tiles a CTA: teams that take every other tile
-    ((2,), (64,), 120, 61, 0.3),            # the same with narrow tiles, three and four a CTA
+    ((2,), (96,), 112, 23, 0.0),            # few enough for the split form
+    ((2,), (160,), 100, 57, 0.1),           # two filter tiles, steps of two
+    ((1, 1), (64, 112), 120, 70, 0.0),      # filters that stay, teams; strided layers and the second stage in the split form
+    ((2,), (48,), 232, 9, 0.0),             # 58 pixels wide, filters that stay
+    ((2,), (80,), 248, 33, 0.3),            # 62 pixels wide, filters that stay, several tiles a CTA, the last one partial
+    ((1,), (256,), 72, 47, 0.0),            # split form, filters that take longer than the MMAs of a tile
+    ((2,), (64,), 120, 25, 0.0),            # filters that stay as a whole, a tile a CTA
+    ((2,), (64,), 120, 61, 0.3),            # the same with narrow tiles, three and four a CTA: teams that take every other tile
 ])
 def test_steps_of_tiles(B, layers, widths, hw, batch, p):
     net = wl.resnet_imagenet_basic(layers, widths, in_hw=hw, n_classes=5, name="steps")

@@ -889,10 +889,13 @@ NetParts network_parts(fp_handle h, int batch) {
     return parts;
 }
 
-// Microseconds of a forward of the largest batch, as one kernel and layer by layer (runs of layers where there are any): fitted to 524
-// timings of networks of 7 to 109 layers, 8 to 64 filters wide, pruned at 0 to 0.6, batches from 148 (4 % rms each).  One kernel: every
+// Microseconds of a forward of the largest batch, as one kernel and layer by layer (runs of layers where there are any).  One kernel: every
 // round over the GPU costs the planner's cycles and the ends of the layers.  Layer by layer: a launch, and per run the rounds of its
-// groups times the tiles' chains; single layers by their MMAs, strided ones by the gathered positions.
+// groups times the tiles' chains; single layers by their MMAs, strided ones by the gathered positions.  The terms were fitted to 524
+// timings of networks of 7 to 109 layers, 8 to 64 filters wide, pruned at 0 to 0.6, batches from 148 (4 % rms each), but for two that
+// were set when their kernels changed: that of runs of 16 filters (chain_quad_layer_us, from timings of groups of one image and of two)
+// and that of strided layers (9.5e-5 and 5.3 instead of 2.5e-4 and 5.7).  The whole has been checked by its choices since, not by its rms
+// (build_plan, where the margin is).
 double network_cost(fp_handle h) {
     double us = 6.1;
     for (const NetPart& part : network_parts(h, h->max_batch)) {
@@ -2246,7 +2249,8 @@ extern "C" fp_status fp_query(fp_handle h, int32_t what, int32_t index, void* h_
             CK(cudaDeviceSynchronize());
             if (!h->keep_outputs) {
                 // Buffers are reused once their last reader has run, so the tensor may have been overwritten since:
-                // run the forward's launches up to this operator again (same input, same kernels) and stop there.
+                // run the forward's launches up to this operator again (same input, same kernels; only that parity-split tensors, of
+                // which a forward may write what is read, are written with all their pixels) and stop there.
                 if (!h->last_input) return fail(FP_ERR_ARG, "fp_query: no forward has run yet");
                 h->whole_outputs = 1;
                 for (int j = 0; j <= index; ++j) launch_op(h, j, h->last_input, h->last_batch, h->d_logits_stage, 0);

@@ -24,6 +24,8 @@
 //   Pipelining    as chain_tc.cu: eight accumulator stages, a barrier pair per tile says when its outputs are there, layers overlap.
 //   Measured      ResNet-110's 37 layers of 1024 images 695 -> 400 us, of 148 images 105 -> 88 us (a layer of one image's three tiles is
 //                 4500 cycles, of two images' five 5100: the chain of MMAs, commit and epilogue behind a tile's neighbours).
+//   Not finite    An infinity or a NaN reaches every output of the blocks whose 4 x 4 pixels hold it, also those it is multiplied by a zero
+//                 filter for.  It stays within its image: above, below and between images' columns lie zeros.
 //   Waits         bounded as in conv_tc.cu.
 #include "chain_quad_layout.h"
 #include "fp_internal.h"

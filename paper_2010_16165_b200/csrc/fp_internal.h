@@ -10,8 +10,15 @@
 // plane = N * P2 + W + 2 rounded up to whole cache lines.
 // So each chunk is one contiguous plane over the whole batch; a run of consecutive "flat
 // positions" f = n*P2 + (h+1)*(W+1) + (w+1) is contiguous in memory for every chunk, and the
-// 3x3 neighbourhood of position f is f + dr*(W+1) + ds.  Every kernel that writes a tensor
-// writes all of its positions, zeros on the border, so the border never has to be cleared.
+// 3x3 neighbourhood of position f is f + dr*(W+1) + ds.  Every kernel that writes a whole tensor
+// writes all of its positions, zeros on the border, so the border never has to be cleared.  What rounds a
+// plane up to whole lines, and the guard vectors, are defined nowhere.
+// Of a parity-split tensor (ConvArgs::y_split) less is written: not the border row of the images of even rows,
+// nor the border column of those of even columns, nor anything behind the last image - and with
+// PairArgs::y_quarter the parity-00 images alone.  Buffers are reused, so those places hold other tensors' values,
+// which need not be finite.  A reader may fetch them, as rows of an operand, but has to leave the results they give
+// where they are (by position; a product with zero would not do): the strided convolutions read no such place for a
+// position of theirs that exists, 1x1 layers give each position's to that position.
 // (With a border on all four sides, which was the layout before, 7x7 pixels took 81 positions instead
 // of 64, 14x14 256 instead of 225, 28x28 900 instead of 841: work of every convolution and bytes of every tensor.)
 // Buffers carry `kGuardVectors` vectors of slack before and after the data, because tiles of

@@ -18,12 +18,13 @@ struct QuadCtrl {
 static_assert(sizeof(QuadCtrl) % 16 == 0, "buffers behind the control block must stay 16-byte aligned");
 
 // Vectors of a row of blocks, and of a plane of G images: blocks with their borders, and the zeros behind the last.
-__host__ __device__ constexpr int quad_pitch(int W) { return W / 2 + 1; }
+constexpr int quad_pitch(int W) { return W / 2 + 1; }
 constexpr int quad_plane_rows(int G, int H, int W) { return (G * (H / 2 + 1) * quad_pitch(W) + W / 2 + 2 + 7) / 8 * 8; }
 constexpr int quad_tiles(int plane_rows) { return (plane_rows + 127) / 128; }
 // Where window pixel w = 4 iy + ix of a block is: the plane of its parity, `rows` vectors a plane, from the block row and column it lies in.
-__host__ __device__ constexpr uint32_t quad_window_plane(int w, uint32_t rows) { return (uint32_t)(((((w >> 2) + 1) & 1) * 2 + (((w & 3) + 1) & 1)) * 2) * rows; }
-__host__ __device__ constexpr uint32_t quad_window_row(int w, uint32_t pitch) {
+// (The kernel has these two written out.)
+constexpr uint32_t quad_window_plane(int w, uint32_t rows) { return (uint32_t)(((((w >> 2) + 1) & 1) * 2 + (((w & 3) + 1) & 1)) * 2) * rows; }
+constexpr uint32_t quad_window_row(int w, uint32_t pitch) {
     return ((w >> 2) == 0 ? 0u - pitch : (w >> 2) == 3 ? pitch : 0u) + ((w & 3) == 0 ? 0u - 1u : (w & 3) == 3 ? 1u : 0u);
 }
 // Two buffers of eight planes, and behind them what the last tile's operands read past the last plane: its rows up to a multiple of 128, and
